@@ -326,3 +326,19 @@ def test_learner_iterations_from_a_cuda_graph_with_device_bookkeeping(oracle):
             assert torch.equal(view, cands[where[slot]]["target_logits"])
     ring.device_end()
     ring.close()
+
+
+@pytest.mark.parametrize("row_bytes", [1, 2, 4, 6, 8, 36, 200, 256, 264, 1800, 4096, 4104, 70000])
+@pytest.mark.parametrize("n", [1, 33, 1000])
+def test_gather_rows_of_every_width(row_bytes, n):
+    """Rows of one element up to several warps' chunks, in every element width, counts that leave a ragged last round."""
+    import paper_1912_00167_b200 as ip
+    g = torch.Generator(device="cuda").manual_seed(row_bytes + n)
+    src = torch.randint(0, 256, (301, row_bytes), dtype=torch.uint8, device="cuda", generator=g)
+    idx = torch.randint(0, 301, (n,), dtype=torch.int32, device="cuda", generator=g)
+    guard = torch.full((n * row_bytes + 512,), 0xA5, dtype=torch.uint8, device="cuda")
+    dst = guard[256:256 + n * row_bytes].view(n, row_bytes)
+    ip.impact_gather_rows(src, idx, dst)
+    torch.cuda.synchronize()
+    assert torch.equal(dst, src[idx.long()])
+    assert bool((guard[:256] == 0xA5).all()) and bool((guard[256 + n * row_bytes:] == 0xA5).all())
