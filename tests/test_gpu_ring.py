@@ -328,6 +328,43 @@ def test_learner_iterations_from_a_cuda_graph_with_device_bookkeeping(oracle):
     ring.close()
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("N,K", [(1, 2), (31, 1), (33, 2), (64, 1), (100, 3), (1024, 1)])
+def test_device_step_at_the_edges_of_its_slot_words(oracle, mode, N, K):
+    """The slots' flags are walked 32 to a word: sets of slots that end inside, at and after a word, from empty to
+    full and back, give the oracle's trace.  The field is no multiple of 16 bytes."""
+    import paper_1912_00167_b200 as ip
+    nbytes, n_cand = 4 * 1021, 3
+    cands = [torch.randint(0, 2 ** 31 - 1, (1021,), dtype=torch.int32, device="cuda") for _ in range(n_cand)]
+    ring = ip.ImpactBuffer(N, K, [nbytes], seed=N + 7, sample_mode=mode)
+    ref = oracle.Ring(N, K, mode, seed=N + 7)
+    table = torch.tensor([[c.data_ptr(), 0] for c in cands], dtype=torch.int64, device="cuda")
+    record = ip.new_loss_inputs_record()
+    push = ring.prepare_device_step(push_sources=table)
+    draw = ring.prepare_device_step({"actions": 0}, record=record)
+    ring.device_begin()
+    rng = np.random.default_rng(N)
+    want, where, pushes = [], {}, 0
+    script = ["push"] * (N + 1) + ["push" if rng.random() < 0.4 else "draw" for _ in range(min(2 * N + 20, 1200))]
+    for op in script:
+        (push if op == "push" else draw)()
+        if op == "push":
+            st, slot = ref.push()
+            want.append((1, -5 if st == ref.FULL else 0, -1 if st == ref.FULL else slot, 0))
+            if st != ref.FULL:
+                where[slot] = pushes % n_cand
+                pushes += 1
+        else:
+            st, slot, k = ref.sample()
+            want.append((2, -4, -1, 0) if st == ref.EMPTY else (2, 0, slot, k))
+    assert ring.device_events() == want[-4096:]
+    for slot, c in where.items():
+        assert torch.equal(ring.slot_view(slot, 0, torch.int32, (1021,)), cands[c])
+    assert ring.live() == ref.live()
+    ring.device_end()
+    ring.close()
+
+
 @pytest.mark.parametrize("row_bytes", [1, 2, 4, 6, 8, 36, 200, 256, 264, 1800, 4096, 4104, 70000])
 @pytest.mark.parametrize("n", [1, 33, 1000])
 def test_gather_rows_of_every_width(row_bytes, n):
