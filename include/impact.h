@@ -206,11 +206,10 @@ int32_t impact_loss_workspace_status(const void* workspace, size_t workspace_byt
  * Outputs must not alias inputs.
  * workspace: device scratch of at least impact_loss_workspace_bytes(B,T) bytes, cleared
  *   once with impact_loss_workspace_init.
- * Limits: 1 <= A <= 512; B*T*A < 2^40.  No input is clamped or sanitised: NaN/Inf inputs
- * give NaN/Inf outputs wherever the arithmetic above carries them -- and, because trajectories
- * shorter than 128 steps are worked on several to a tile with the recursion cut between them by
- * a factor of zero, possibly also in the trajectories that precede the affected one within its
- * tile (floor(128 / T) consecutive trajectories).  No wait depends on a value: nothing hangs.
+ * Limits: 1 <= A <= 512; B*T*A < 2^40.  (Without room for the tiles' aggregates in the workspace,
+ * T < 2^32 - 4096.)  No input is clamped or sanitised: NaN/Inf inputs give NaN/Inf outputs wherever
+ * the arithmetic above carries them, which is never beyond the trajectory that holds them (and the
+ * batch means).  No wait depends on a value: nothing hangs.
  * Errors: INVALID_ARG, UNSUPPORTED, WORKSPACE_TOO_SMALL, CUDA (launch failure).
  */
 int32_t impact_loss_fwd_bwd(
@@ -309,9 +308,7 @@ int32_t impact_loss_fwd_bwd_gaussian(
  * impact_loss_fwd_bwd with a workspace for those.
  *
  * The first call on a device looks up the array's device address (a driver query, with that
- * device current); make that first call outside any stream capture.  Every call enqueues a
- * small clear of the counter before its kernel, since the array still holds what the
- * previous call left.  All calls on a device share the one array: two calls whose kernels
+ * device current); make that first call outside any stream capture.  All calls on a device share the one array: two calls whose kernels
  * may run at the same time (different streams, or different host threads without ordering)
  * corrupt each other's sums.  Keep them on one stream or order them with events.
  * The array's error word (see impact_loss_workspace_status) is sticky across calls: read it,

@@ -1,0 +1,1131 @@
+// The categorical IMPACT loss + gradient kernel and its launch rules (one kernel template for every action count).
+//
+// One block per SM.  A producer warp streams the block's tiles -- consecutive steps of the row-major [B*T, A] logits --
+// through a ring of shared-memory stages by bulk asynchronous copies; C consumer groups of four warps take every C-th
+// tile as it lands, one thread per step for the recursion and 1 to 32 lanes per step for the row passes, and every
+// warp sends its own gradient rows off by a bulk store while later tiles are still arriving.
+//
+// Two ways to lay the batch out over the grid:
+//   flat  (kLong = false): a block owns a contiguous range of whole trajectories and walks its rows from the END, a tile
+//         of NT rows at a time, with no regard to where trajectories begin: a step that ends its trajectory has the
+//         affine map (0, b), so the recursion is cut there by itself.  Where a trajectory crosses a tile boundary, the
+//         value at the later tile's first step passes to the earlier tile through a mailbox in shared memory; only that
+//         one multiply-add per tile is serial.  (Packing whole trajectories into tiles instead leaves a fifth of the
+//         lanes idle at T = 50 or 100.)
+//   long  (kLong = true): tiles of one trajectory on neighbouring blocks, for few long trajectories; the recursion
+//         crosses tiles through their affine aggregates, published in the workspace (see the kernel's carry step).
+#pragma once
+
+#include "impact_device.cuh"
+#include "impact_internal.h"
+#include "impact_loss_params.h"
+
+namespace impact {
+
+// ---- geometry ---------------------------------------------------------------------------------------------------
+struct Tile {
+    long long row0;  // first row of the tile (of the whole batch)
+    int nrows;       // rows of the slab that are loaded
+    int r;           // long: number of the tile counted from its trajectory's end
+    long long traj;  // long: the trajectory
+};
+// What a block of a flat launch owns.
+struct BlockRange {
+    long long traj0, r0, r1;  // first trajectory, first row, end of rows
+    long long base;           // row of the first tile's first slot: r0, or up to seven rows before it
+    int tiles;
+};
+__device__ __forceinline__ BlockRange block_range(const CatGeometry& g) {
+    BlockRange b;
+    const long long q = g.B / gridDim.x, rem = g.B - q * gridDim.x, x = blockIdx.x;
+    b.traj0 = x * q + (x < rem ? x : rem);
+    const long long ntraj = q + (x < rem ? 1 : 0);
+    b.r0 = b.traj0 * g.T;
+    b.r1 = b.r0 + ntraj * g.T;
+    // tiles start on multiples of eight rows, where every row pitch is a multiple of 16 bytes, unless that costs a tile
+    const int shift = (int)(b.r0 & 7);
+    const long long rows = b.r1 - b.r0;
+    const long long tiles = (rows + g.nt - 1) / g.nt;
+    const bool fits = rows + shift <= tiles * g.nt;
+    b.base = fits ? b.r0 - shift : b.r0;
+    b.tiles = (int)tiles;
+    return b;
+}
+// The block's n-th tile in the order in which it works on them.
+template <bool kLong>
+__device__ __forceinline__ Tile tile_at(const CatGeometry& g, const BlockRange& b, int n, int nt) {
+    Tile t;
+    if (kLong) {
+        const long long x = (long long)blockIdx.x + (long long)n * gridDim.x;
+        if (g.tile_major) {  // the last tiles of all trajectories first, then the tiles before them, ...
+            t.r = (int)((unsigned long long)x / (unsigned long long)g.B);
+            t.traj = x - (long long)t.r * g.B;
+        } else {  // trajectory by trajectory, each from its last tile backwards
+            t.traj = (long long)((unsigned long long)x / (unsigned int)g.ntiles);
+            t.r = (int)(x - t.traj * g.ntiles);
+        }
+        const long long t0 = (long long)(g.ntiles - 1 - t.r) * nt;
+        const long long left = g.T - t0;
+        t.nrows = left < nt ? (int)left : nt;
+        t.row0 = t.traj * g.T + t0;
+    } else {
+        t.row0 = b.base + (long long)(b.tiles - 1 - n) * nt;
+        const long long left = b.r1 - t.row0;
+        t.nrows = left < nt ? (int)left : nt;
+        t.r = 0;
+        t.traj = 0;
+    }
+    return t;
+}
+__device__ __forceinline__ int tiles_of_block(const CatGeometry& g, const BlockRange& b, bool is_long) {
+    if (!is_long) return b.tiles;
+    const long long total = g.B * g.ntiles;
+    return (int)((total - blockIdx.x + gridDim.x - 1) / gridDim.x);
+}
+
+// A slab in shared memory: nt rows of `row_bytes`, plus 32 bytes of padding, because a tile's rows sit at the same
+// offset inside their 16-byte granule as in global memory (0..15 bytes after the slab's start) and the copy that
+// brings them is widened to whole granules (see dev::widen_range).
+__host__ __device__ constexpr size_t slab_pitch(size_t nt, size_t row_bytes) { return nt * row_bytes + 32; }
+__host__ __device__ constexpr size_t cat_stage_bytes(size_t nt, size_t A, size_t in_elem, size_t out_elem) {
+    const size_t raw = 2 * slab_pitch(nt, A * in_elem) + (in_elem == out_elem ? 0 : slab_pitch(nt, A * out_elem));
+    return (raw + 127) / 128 * 128;
+}
+
+// ---- row access -------------------------------------------------------------------------------------------------
+// kV neighbouring elements of a row in shared memory, in their storage type, as one access.
+template <typename ST, int kV> struct Vec;
+template <> struct Vec<float, 1> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) { f[0] = *reinterpret_cast<const float*>(p); }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) { *reinterpret_cast<float*>(p) = f[0]; }
+};
+template <> struct Vec<float, 2> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) {
+        const float2 v = *reinterpret_cast<const float2*>(p);
+        f[0] = v.x; f[1] = v.y;
+    }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) { *reinterpret_cast<float2*>(p) = make_float2(f[0], f[1]); }
+};
+template <> struct Vec<float, 4> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w;
+    }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
+        *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]);
+    }
+};
+template <> struct Vec<__nv_bfloat16, 1> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) {
+        f[0] = __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(p) << 16);
+    }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
+        *reinterpret_cast<__nv_bfloat16*>(p) = __float2bfloat16_rn(f[0]);
+    }
+};
+template <> struct Vec<__nv_bfloat16, 2> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) {
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
+        f[0] = __uint_as_float(w << 16); f[1] = __uint_as_float(w & 0xFFFF0000u);
+    }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
+        *reinterpret_cast<uint32_t*>(p) = dev::Pack<__nv_bfloat16>::two(f[0], f[1]);
+    }
+};
+template <> struct Vec<__nv_bfloat16, 4> {
+    static __device__ __forceinline__ void ld(const unsigned char* p, float* f) {
+        const uint2 w = *reinterpret_cast<const uint2*>(p);
+        f[0] = __uint_as_float(w.x << 16); f[1] = __uint_as_float(w.x & 0xFFFF0000u);
+        f[2] = __uint_as_float(w.y << 16); f[3] = __uint_as_float(w.y & 0xFFFF0000u);
+    }
+    static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
+        *reinterpret_cast<uint2*>(p) = make_uint2(dev::Pack<__nv_bfloat16>::two(f[0], f[1]), dev::Pack<__nv_bfloat16>::two(f[2], f[3]));
+    }
+};
+// Overwrites one element after vector stores to the same row; an explicit shared-memory store keeps it ordered behind
+// them.
+template <typename ST>
+__device__ __forceinline__ void put_element(unsigned char* row, int col, float x) {
+    if constexpr (sizeof(ST) == 4) {
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(dev::smem_addr(row) + (uint32_t)col * 4u), "f"(x) : "memory");
+    } else {
+        const unsigned short h = __bfloat16_as_ushort(__float2bfloat16_rn(x));
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(dev::smem_addr(row) + (uint32_t)col * 2u), "h"(h) : "memory");
+    }
+}
+template <typename ST>
+__device__ __forceinline__ float get_element(const unsigned char* row, int col) {
+    float f;
+    Vec<ST, 1>::ld(row + col * (int)sizeof(ST), &f);
+    return f;
+}
+
+// ---- the recursion's scan ---------------------------------------------------------------------------------------
+// Suffix composition of the lanes' affine maps: lane l ends up with f_l o f_{l+1} o ... o f_{l + limit}, where limit is
+// what is left of the lane's trajectory (or of the warp): nothing of another trajectory enters, not even times zero.
+__device__ __forceinline__ void warp_suffix_compose(float& a, float& b, int limit) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float a2 = __shfl_down_sync(0xffffffffu, a, off);
+        const float b2 = __shfl_down_sync(0xffffffffu, b, off);
+        asm("{\n\t.reg .pred p;\n\tsetp.ge.s32 p, %4, %5;\n\t"
+            "@p fma.rn.f32 %1, %0, %3, %1;\n\t"
+            "@p mul.rn.f32 %0, %0, %2;\n\t}"
+            : "+f"(a), "+f"(b) : "f"(a2), "f"(b2), "r"(limit), "r"(off));
+    }
+}
+
+// ---- a step's scalars -------------------------------------------------------------------------------------------
+// Log-probabilities are kept in base 2 (as the row passes form them): every exponential of a difference is then one
+// instruction, and only the worker's log-probability has to be scaled.  (Products and sums are spelled out where the
+// compiler could fuse them one way in one instantiation and another way in the next: every kernel that can serve a call
+// gives the same bits.)
+struct Step {
+    float l2_theta, l2_target, l2_worker;
+    float reward, discount, value, value_next;
+    bool ends;              // last step of its trajectory: the trace stops, V_{t+1} is the bootstrap value
+    float rho = 0.0f;       // truncated importance weight (set by recursion_map)
+    float adv_next = 0.0f;  // A_{t+1} (set from the scan)
+};
+// Truncated importance weights and the affine map of the advantage recursion (Section 2.2; Section 3.1).  Returns
+// whether the weight exceeded rho_bar.
+template <bool kPlain>
+__device__ __forceinline__ bool step_map(Step& s, const LossScalars& k, float& a, float& b) {
+    const float x = ((!kPlain && k.is_source == 1) ? s.l2_theta : s.l2_target) - s.l2_worker;
+    const float w = (!kPlain && k.is_source == 2) ? 1.0f : dev::exp2_fast(x);  // 2: plain GAE, no importance weights
+    const float rho = fminf(k.rho_bar, w);
+    s.rho = rho;
+    const float c = fminf(k.c_bar, w);
+    b = __fmul_rn(rho, __fadd_rn(fmaf(s.discount, s.value_next, s.reward), -s.value));
+    a = s.ends ? 0.0f : __fmul_rn(__fmul_rn(k.lambda_, s.discount), c);
+    return w > k.rho_bar;
+}
+// Ratio of Section 4.1 and the eps-clipped surrogate of Appendix E.  Returns the weight adv * R of the policy-gradient
+// term (0 where the clip removes it).
+template <bool kPlain>
+__device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars& k, float adv, float& surr, float& ratio,
+                                                bool& clipped) {
+    if (!kPlain && k.objective == 1) {
+        // IMPALA's actor update (Section 2.2): weight rho_t (r_t + gamma_t v_{t+1} - V_t) on
+        // grad log pi_theta, v the V-trace target V + A (the bootstrap value after the last step)
+        const float v_next = s.value_next + (s.ends ? 0.0f : s.adv_next);
+        const float w = __fmul_rn(s.rho, __fadd_rn(fmaf(s.discount, v_next, s.reward), -s.value));
+        surr = __fmul_rn(w, s.l2_theta * 0.6931471805599453f);
+        ratio = s.rho;
+        clipped = false;
+        return w;
+    }
+    float d = fmaxf(s.l2_target, s.l2_worker - k.log2_rho_tw);
+    if (!kPlain) {
+        if (k.ratio_mode == 1) d = s.l2_target;
+        else if (k.ratio_mode == 2) d = s.l2_worker;
+    }
+    const float R = dev::exp2_fast(s.l2_theta - d);
+    const float Rc = fminf(fmaxf(R, k.clip_lo), k.clip_hi);
+    const float Ra = __fmul_rn(R, adv);
+    surr = fminf(Ra, __fmul_rn(Rc, adv));
+    clipped = (adv > 0.0f && R > k.clip_hi) || (adv < 0.0f && R < k.clip_lo);
+    ratio = R;
+    return clipped ? 0.0f : Ra;
+}
+
+// ---- waits ------------------------------------------------------------------------------------------------------
+// The first look is inline (the barrier's own wait usually covers it); what follows is out of the way of the loop.
+static __device__ __noinline__ bool stage_wait_rest(uint64_t* bar, uint32_t parity, int* abort_flag) {
+    return dev::mbarrier_wait(bar, parity, abort_flag);
+}
+__device__ __forceinline__ bool stage_wait(uint64_t* bar, uint32_t parity, int* abort_flag) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(dev::smem_addr(bar)), "r"(parity) : "memory");
+    return __all_sync(0xffffffffu, done) ? true : stage_wait_rest(bar, parity, abort_flag);
+}
+__device__ __forceinline__ void arrive_if(uint64_t* bar, bool who) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(dev::smem_addr(bar)), "r"((uint32_t)who) : "memory");
+}
+
+// ---- the mailbox of a flat launch -------------------------------------------------------------------------------
+// The block's n-th tile leaves the value at its first step in slot n mod 32 as one 8-byte (value, n + 1) pair; tile
+// n + 1 reads it there.  A slot is not written again before it has been read: tile n + 32 is requested only after
+// tile n + 32 - S was handed back by its four warps, S <= 24 stages, tiles are requested in order, and a warp of tile
+// n + 1 reads the mailbox before it hands its stage back; a block with no more tiles than stages never uses a slot twice.
+constexpr int kMailSlots = 32;
+static_assert(kWsMaxStages < kMailSlots, "see above");
+__device__ __forceinline__ void mail_put(uint64_t* mail, int n, float value) {
+    const uint64_t v = ((uint64_t)(uint32_t)(n + 1) << 32) | (uint64_t)__float_as_uint(value);
+    asm volatile("st.volatile.shared.b64 [%0], %1;" ::"r"(dev::smem_addr(mail + (n & (kMailSlots - 1)))), "l"(v) : "memory");
+}
+static __device__ __noinline__ float mail_wait(uint32_t at, uint32_t tag, int* abort_flag) {
+    uint64_t v = 0;
+    for (unsigned int tries = 0; tries < (1u << 24); ++tries) {
+        asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+        if ((uint32_t)(v >> 32) == tag) return __uint_as_float((uint32_t)v);
+        if (*reinterpret_cast<volatile int*>(abort_flag)) return 0.0f;
+    }
+    *reinterpret_cast<volatile int*>(abort_flag) = 1;
+    return 0.0f;
+}
+__device__ __forceinline__ float mail_get(const uint64_t* mail, int n, int* abort_flag) {
+    const uint32_t at = dev::smem_addr(mail + (n & (kMailSlots - 1)));
+    uint64_t v;
+    asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+    const bool here = (uint32_t)(v >> 32) == (uint32_t)(n + 1);
+    return __all_sync(0xffffffffu, here) ? __uint_as_float((uint32_t)v) : mail_wait(at, (uint32_t)(n + 1), abort_flag);
+}
+
+// Sends rows [lo, hi) of a warp's share [wrow, wrow + ntw) of a tile (`slab` and `out` point at the tile's first row in
+// shared and in global memory).  Out of line: it serves the ends of a block's range and row pitches that do not keep a
+// warp's rows on 16-byte boundaries.
+static __device__ __noinline__ void send_rows_general(unsigned char* out, const unsigned char* slab, int pitch, int wrow,
+                                                      int ntw, int lo, int hi, bool wrote) {
+    lo = max(lo, wrow);
+    hi = min(hi, wrow + ntw);
+    const uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) * (uint32_t)pitch : 0u;
+    dev::warp_send_bytes(out + (long long)lo * pitch, slab + lo * pitch, bytes, wrote);
+}
+
+// ---- shape of the row passes ------------------------------------------------------------------------------------
+// kA > 0: the action count, known at compile time; a row belongs to one lane, which keeps its exponentials.
+// kA = 0 (narrow): at most 16 actions, one lane per row as well, the count a run-time value.
+// kA < 0 (wide): any count; a row belongs to L = 2 ... 32 lanes that hold up to 16 elements each (vector i of lane g is
+//   the row's vector i L + g, which spreads a warp's accesses over the banks without padding), and a warp works on its
+//   NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the warp is worked on in pass p by lanes [q L, q L + L)
+//   and owned -- for everything that is per step -- by lane q L + p of them, so results never move between lanes.
+//   The gradient pass forms the exponentials again instead of holding P rows in registers.
+constexpr int kMaxLaneElems = 16;
+// Is the j-th of a lane's elements part of the row?
+__device__ __forceinline__ bool element_exists(int j, int part, int vstep, int kv, int A) {
+    return (j / kv) * vstep + part * kv < A;
+}
+
+// The record of impact_buffer_device_step, read past L1 (an earlier launch may have left an older version there).
+__device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss_inputs* rec) {
+    const ulonglong2* q = reinterpret_cast<const ulonglong2*>(rec);
+    const ulonglong2 a = __ldcg(q), b = __ldcg(q + 1), c = __ldcg(q + 2), d = __ldcg(q + 3);
+    const unsigned long long e = __ldcg(reinterpret_cast<const unsigned long long*>(q + 4));
+    LossInputPointers in;
+    in.learner_logits = reinterpret_cast<const void*>(a.x);
+    in.target_logits = reinterpret_cast<const void*>(a.y);
+    in.worker_logp = reinterpret_cast<const float*>(b.x);
+    in.actions = reinterpret_cast<const int32_t*>(b.y);
+    in.rewards = reinterpret_cast<const float*>(c.x);
+    in.discounts = reinterpret_cast<const float*>(c.y);
+    in.values = reinterpret_cast<const float*>(d.x);
+    in.bootstrap = reinterpret_cast<const float*>(d.y);
+    in.target_copy = reinterpret_cast<void*>(e);
+    return in;
+}
+
+// kPlain: the configuration of the paper's experiments -- no KL term, the clipped surrogate with the default ratio and
+// importance weights, no optional outputs -- with those branches compiled out.
+//
+// Barrier protocol of the persistent kernels (S stages, at most W tiles in flight, lanes <= S - W):
+//   full[s]     one arrival (a producer lane's, with the bytes the tile's two copies will deliver): stage s holds
+//               the rows of its current tile.
+//   empty[s]    one arrival per consumer warp, after that warp's stores have finished reading the stage.
+// A wait names a phase by its PARITY, which is only unambiguous while the waiter is at most one phase ahead of the
+// barrier: asked about phase k while phase k-1 is still open, the barrier answers "complete".  The producer
+// therefore issues tiles STRICTLY in order, and tile n only after (a) tile n-W has landed and
+// (b) every consumer warp has released tile n-S.  From that:
+//   * consumer of tile n waits on full[n % S] for phase n/S.  It got there after consuming tile n-C, so n-C was
+//     issued, so (in order) tile n-S+W <= n-C was issued, so by (a) tile n-S -- phase n/S - 1 of the same stage --
+//     had landed: the barrier is in phase n/S or later.  It cannot be beyond n/S + 1 open, because tile n+S is not
+//     issued before this consumer releases tile n (b).  (This is where S >= W + C is needed.)
+//   * producer's look at full[(n-W) % S] for phase (n-W)/S: tile n-W was issued, so by (b) tile n-W-S was consumed,
+//     hence had landed: phase (n-W)/S - 1 is complete; tile n-W+S > n is not issued yet.
+//   * producer's look at empty[n % S] for phase n/S - 1: tile n-S was issued, so by (b) phase n/S - 2 is complete;
+//     phase n/S needs the consumers of tile n, which is not issued yet.
+// Without the in-order rule (lanes that found their own tile ready first went first) the first argument fails for
+// tiles of one round: a consumer could be handed a stage whose previous tile had not landed, read stale rows,
+// release the stage early, and the phases slipped until one of the bounded waits ran out.
+template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
+__global__ void __launch_bounds__(C * 128 + 32, 1)
+impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid_constant__ CatShape sh) {
+    constexpr bool kWide = kA < 0, kFixed = kA > 0;
+    constexpr int E = kFixed ? kA : kMaxLaneElems;
+    constexpr int NV = (E + kV - 1) / kV;       // vectors per lane at most
+    constexpr int NP = (E + 1) / 2;             // pairs: Blackwell's packed fp32 add / mul / fma work on two lanes at once
+    constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+    constexpr float kLowest = -3.402823466e38f;  // stands for an element that is not there: its exponential is 0
+    static_assert(!kFixed || kA % kV == 0, "whole vectors");
+    const int A = kFixed ? kA : p.A;
+    const int NT = kFixed ? 128 : sh.nt;
+    const int NTW = NT >> 2;  // rows of a tile that one warp works on
+    const int S = sh.stages, W = sh.in_flight;
+    const int in_row = A * (int)sizeof(LT), out_row = A * (int)sizeof(GT);
+    const int in_pitch = (int)slab_pitch(NT, in_row);
+    const int stage_bytes = (int)cat_stage_bytes(NT, A, sizeof(LT), sizeof(GT));
+
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kWsMaxStages], empty_bar[kWsMaxStages];
+    __shared__ __align__(8) uint64_t mail[kMailSlots];
+    __shared__ unsigned int tickets_s, tag_s;  // (see dev::draw_ticket_and_publish)
+    __shared__ float2 warp_agg[C][2][4];       // (two sets, used in turn: a tile's scan has one barrier)
+    __shared__ __align__(16) float red[C][4][8];
+    __shared__ int abort_s;
+    __shared__ float carry_s[C];
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const LossScalars& k = p.k;
+    const CatGeometry& g = p.geo;
+    const BlockRange br = block_range(g);
+    const int n_tiles = tiles_of_block(g, br, kLong);
+    const long long total_rows = g.B * g.T;
+    // The tensors this launch reads: the call's own arguments (kernel parameters, read where they are used), or --
+    // kIndirect: the call names a record in device memory that an earlier kernel of the stream fills (the circular
+    // buffer's bookkeeping on the device) -- that record's, fetched once the stream dependency has resolved and kept
+    // in shared memory (the producer warp alone fetches the record, before the block-wide barrier that releases the
+    // consumer warps: with every warp of the grid fetching it -- 3 000 warps asking one cache line at the same
+    // moment -- the first tile was requested 3.6 us late)
+    __shared__ LossInputPointers in_s;
+#define IMPACT_IN(field) (kIndirect ? in_s.field : p.field)
+
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (known to be the same for the whole warp)
+    if (warp >= C * 4) {
+        // ---- producer warp ----------------------------------------------------------------------------------
+        const int n_first = n_tiles < W ? n_tiles : W;
+        // First of all, while the kernel before this one on the stream is still finishing, the warp asks L2 for
+        // the block's first tiles (logits and per-step scalars), unless the launch's companion kernel has done so
+        // already: the pages are mapped and the bytes on their way when the dependency resolves.
+        if (sh.n_prefetch > 0) {
+            const void* base = nullptr;
+            long long pitch = 4;
+            if (lane == 0) { base = IMPACT_IN(learner_logits); pitch = in_row; }
+            else if (lane == 1) { base = IMPACT_IN(target_logits); pitch = in_row; }
+            else if (lane == 2) base = IMPACT_IN(actions);
+            else if (lane == 3) base = IMPACT_IN(worker_logp);
+            else if (lane == 4) base = IMPACT_IN(rewards);
+            else if (lane == 5) base = IMPACT_IN(discounts);
+            else if (lane == 6) base = IMPACT_IN(values);
+            const int n_pf = n_tiles < sh.n_prefetch ? n_tiles : sh.n_prefetch;
+            for (int n = 0; n < n_pf; ++n) {
+                const Tile t = tile_at<kLong>(g, br, n, NT);
+                if (base) dev::prefetch_range_l2(base, t.row0 * pitch, (uint32_t)(t.nrows * pitch), total_rows * pitch);
+            }
+        }
+        // then the barriers
+        if (lane < S) {
+            dev::mbarrier_init_nofence(&full_bar[lane], 1);
+            dev::mbarrier_init_nofence(&empty_bar[lane], 4);  // one arrival per consumer warp
+        }
+        mail[lane] = 0ull;
+        if (lane == 0) { abort_s = 0; tickets_s = 0u; }
+        dev::fence_mbarrier_init();
+        __syncwarp();
+
+        // One slab of a tile into stage s: a bulk copy of the 16-byte granules that enclose the tile's rows
+        // (dev::widen_range).  The lane with the learner's slab makes the barrier's one arrival, announcing the
+        // bytes of both slabs; where the tensors end inside the last granule, it also fetches that granule's bytes
+        // of both slabs by ordinary loads, fenced towards the copy engine because the consumers may send the target
+        // rows on from the stage by a bulk store.
+        const long long tensor_bytes = total_rows * in_row;
+        struct SlabRequest {
+            unsigned char* d0;        // the learner's slab of the stage (the target's lies in_pitch further)
+            const unsigned char* gl;  // first granule of the tile in the learner's logits
+            const unsigned char* gt;  // ... in the target's
+            uint32_t span, tail;      // dev::WideRange
+        };
+        auto request_for = [&](int n, int s) {
+            const Tile t = tile_at<kLong>(g, br, n, NT);
+            const dev::WideRange w = dev::widen_range(t.row0 * (long long)in_row, (uint32_t)t.nrows * in_row, tensor_bytes);
+            SlabRequest r;
+            r.d0 = smem_raw + s * stage_bytes;  // the tile's first row starts (row0 * in_row) mod 16 bytes in
+            r.gl = static_cast<const unsigned char*>(IMPACT_IN(learner_logits)) + w.first;
+            r.gt = static_cast<const unsigned char*>(IMPACT_IN(target_logits)) + w.first;
+            r.span = w.span;
+            r.tail = w.tail;
+            return r;
+        };
+        auto send_slab = [&](const SlabRequest& r, int s, bool target) {
+            uint64_t* const bar = &full_bar[s];
+            if (target) {
+                if (r.span) dev::bulk_load(r.d0 + in_pitch, r.gt, r.span, bar);
+                return;
+            }
+            if (r.tail) {
+                for (uint32_t i = 0; i < r.tail; ++i) {
+                    r.d0[r.span + i] = r.gl[r.span + i];
+                    r.d0[in_pitch + r.span + i] = r.gt[r.span + i];
+                }
+                dev::fence_async_shared();
+            }
+            if (r.span) {
+                dev::mbarrier_expect_tx(bar, 2 * r.span);
+                dev::bulk_load(r.d0, r.gl, r.span, bar);
+            } else {
+                dev::mbarrier_arrive(bar);
+            }
+        };
+        // Tiles leave in rounds: lane l < 16 owns the round's l-th tile and requests its learner slab, lane l + 16
+        // requests the same tile's target slab, so that all requests of a round leave in the same few instructions
+        // (one thread gets at most four bulk requests under way, and needs about a third of a microsecond per
+        // tile; a lane per request reaches the HBM rate).
+        const int sub = lane & 15;
+        const bool second = lane >= 16;
+        // the first W tiles need no wait (tile n goes to stage n): their requests are worked out now and leave the
+        // moment the stream's previous kernel is done, before the rest of the block has even started
+        SlabRequest first = request_for(sub < n_first ? sub : 0, sub);
+
+        grid_dependency_wait();
+
+        if (kIndirect) {  // (the addresses were not known before)
+            if (lane == 0) in_s = fetch_loss_inputs(p.indirect);
+            __syncwarp();
+            first = request_for(sub < n_first ? sub : 0, sub);
+        }
+        if (sub < n_first) send_slab(first, sub, second);
+        __syncthreads();  // the barriers are set up: the consumer warps may use them
+        const unsigned int tag = dev::launch_tag(p.counter);  // (asked for now, needed after the last tile has left)
+        // The rest.  Tile n goes to stage n % S once that stage's previous tile has left (the "empty" phase before
+        // this one) and tile n - W has landed (at most W tiles in flight).  The owners look at their barriers side by
+        // side (one thread taking tile after tile through blocking waits costs a third of a microsecond per tile, too
+        // much for small tiles: measured 33 us against 25 us on a million steps of six actions), but a tile is sent
+        // only when every earlier tile of the round has been sent or is sent in the same instruction: tiles leave in
+        // order.
+        const int lanes = sh.lanes;
+        for (int base = n_first; base < n_tiles; base += lanes) {
+            const int n = base + sub;
+            bool pending = sub < lanes && n < n_tiles;
+            const int cyc = n / S, s = n - cyc * S;
+            const int wcyc = (n - W) / S, ws = (n - W) - wcyc * S;
+            const SlabRequest req = request_for(pending ? n : 0, s);
+            for (unsigned int spin = 0; spin < (1u << 22); ++spin) {
+                const bool ready = !second && pending && (cyc == 0 || dev::mbarrier_test(&empty_bar[s], (uint32_t)(cyc - 1) & 1u)) &&
+                                   dev::mbarrier_test(&full_bar[ws], (uint32_t)wcyc & 1u);
+                const unsigned int waiting = __ballot_sync(0xffffffffu, !second && pending && !ready);
+                bool go = ready && (waiting & ((1u << sub) - 1u)) == 0u;
+                go = __shfl_sync(0xffffffffu, go, sub);  // the owner decides for both lanes of its tile
+                if (go && pending) {
+                    send_slab(req, s, second);
+                    pending = false;
+                }
+                if (!__any_sync(0xffffffffu, pending)) break;
+                if (*reinterpret_cast<volatile int*>(&abort_s)) break;
+                __nanosleep(32);
+            }
+            if (__any_sync(0xffffffffu, pending)) {  // a stage never came back, or a tile never landed
+                if (lane == 0) {
+                    atomicExch(p.counter + 1, 1u);
+                    *reinterpret_cast<volatile int*>(&abort_s) = 1;
+                }
+                break;
+            }
+        }
+        __syncwarp();
+        // ---- then it leaves this launch's tag for whoever publishes the block's sums, and draws its own ticket
+        if (lane == 0) tag_s = tag;
+        dev::draw_ticket_and_publish<C, 4>(&tickets_s, &tag_s, red, p.tagged_rows);
+        return;
+    }
+
+    // ---- consumer groups ------------------------------------------------------------------
+    // What is the same for a whole warp (the tile, the stage, addresses) is kept apart from what differs by lane, so
+    // that it is worked out once per warp: a tile costs about as many instructions outside the row passes as in them.
+    const int grp = warp >> 2, gwarp = warp & 3;
+    const int gtid = gwarp * 32 + lane;
+    const int bar_id = grp + 1;
+    const int wrow = gwarp * NTW;  // the warp's first row in a tile
+    const bool want_kl = !kPlain && (k.kl_coef != 0.0f);
+
+    // the lane's part in the row passes (wide: see above), and the row of a tile that it owns
+    const int log_l = kWide ? sh.log_lanes : 0;
+    const int L = 1 << log_l;
+    const int passes = kWide ? sh.passes : 1;
+    const int part = kWide ? (lane & (L - 1)) : 0;
+    // (a lane that owns no row stands for the one after it: the identity map, in that row's trajectory)
+    const int lrow = wrow + (kWide ? (lane >> log_l) * passes + min(part, passes) : lane);
+    const bool owner = kWide ? part < passes : true;
+    const int vstep = kWide ? (kV << log_l) : kV;  // elements from a lane's vector to its next
+    const int nvec = kFixed ? NV : (A + vstep - 1) / vstep;  // (of the lane with the most)
+
+    // The tile: which of its rows are this block's (flat) or exist at all (long), and where its first row sits.  In a
+    // flat launch only a block's first tile ends early, only its last one can begin late, and from one of the group's
+    // tiles to its next (C tiles further back) every position changes by a constant.
+    struct Now {
+        long long row0, traj;
+        int lo, hi, r;
+    };
+    auto tile_now = [&](int n) {
+        const Tile t = tile_at<kLong>(g, br, n < n_tiles ? n : 0, NT);
+        Now w;
+        w.row0 = t.row0; w.traj = t.traj; w.r = t.r;
+        w.lo = (!kLong && n == n_tiles - 1) ? (int)(br.r0 - br.base) : 0;
+        w.hi = n < n_tiles ? t.nrows : 0;
+        return w;
+    };
+    const unsigned int back = (unsigned int)(C * NT);
+    Now tl = tile_now(grp);
+    // (flat) how many steps follow the lane's step in its trajectory, and the trajectory (of the block's)
+    const unsigned int T32 = (unsigned int)g.T;  // (flat: T < 2^32, checked on the host)
+    const unsigned int back_traj = kLong ? 0u : back / T32, back_rest = kLong ? 0u : back - back_traj * T32;
+    unsigned int to_end = 0, traj = 0;
+    if constexpr (!kLong) {
+        const long long row = tl.row0 + lrow;
+        const unsigned long long rho = row > br.r0 ? (unsigned long long)(row - br.r0) : 0ull;
+        const unsigned long long q = rho / T32;
+        to_end = T32 - 1u - (unsigned int)(rho - q * T32);
+        traj = (unsigned int)q;
+    }
+    auto to_next_tile = [&](int n_next) {
+        if constexpr (kLong) {
+            tl = tile_now(n_next);
+        } else {
+            tl.row0 -= back;
+            tl.lo = n_next == n_tiles - 1 ? (int)(br.r0 - br.base) : 0;
+            tl.hi = NT;
+            to_end += back_rest;
+            const bool wrapped = to_end >= T32 || to_end < back_rest;
+            to_end -= wrapped ? T32 : 0u;
+            traj -= back_traj + (wrapped ? 1u : 0u);
+        }
+    };
+    auto is_mine = [&](const Now& t) { return owner && lrow >= t.lo && lrow < t.hi; };
+    auto ends_here = [&](const Now& t) { return kLong ? (t.r == 0 && lrow == t.hi - 1) : to_end == 0; };
+
+    struct StepRaw {
+        int a;
+        float l_worker, reward, discount, value, value_next;
+    };
+    auto load_scalars = [&](const Now& t, bool inner) {
+        StepRaw x;
+        // (loads that name the global space: a pointer taken from the device record is a generic one to the
+        // compiler, and a generic load has to be complete before the next store to shared memory -- that put the
+        // whole trip to L2 into every tile, 10.9 us a launch against 6.8)
+        auto fetch = [&]() {
+            x.a = __ldg(IMPACT_IN(actions) + t.row0 + lrow);
+            x.l_worker = __ldg(IMPACT_IN(worker_logp) + t.row0 + lrow);
+            x.reward = __ldg(IMPACT_IN(rewards) + t.row0 + lrow);
+            x.discount = __ldg(IMPACT_IN(discounts) + t.row0 + lrow);
+            const float* const v = IMPACT_IN(values) + t.row0 + lrow;
+            x.value = __ldg(v);
+            x.value_next = __ldg(ends_here(t) ? IMPACT_IN(bootstrap) + (kLong ? t.traj : br.traj0 + (long long)traj) : v + 1);
+        };
+        if (inner) {  // every row is there, and so is the one after the last
+            fetch();
+        } else {
+            x.a = 0; x.l_worker = 0.0f; x.reward = 0.0f; x.discount = 0.0f; x.value = 0.0f; x.value_next = 0.0f;
+            if (is_mine(t)) fetch();
+        }
+        return x;
+    };
+    // (a lane that owns no row reads that of the row it stands for, which may be the first of the next tile)
+    auto is_inner = [&](const Now& t, int n) { return !kLong && !kWide && n > 0 && t.lo == 0; };
+
+    float t_surr = 0.0f, t_val = 0.0f, t_ent = 0.0f, t_ratio = 0.0f, t_kl = 0.0f;
+    int n_clip = 0, n_trunc = 0;
+    // The group's sums, once final: a butterfly per warp into `red`, then the warp's ticket; the last ticket of
+    // the block publishes its row (fixed order throughout).
+    auto hand_over_sums = [&]() {
+        dev::hand_over_warp_sums<C, 4>(t_surr, t_val, t_ent, t_ratio, t_kl, want_kl,
+                                       __reduce_add_sync(0xffffffffu, n_clip), __reduce_add_sync(0xffffffffu, n_trunc),
+                                       red[grp][gwarp], &tickets_s, &tag_s, red, p.tagged_rows);
+    };
+
+    const bool reuse = n_tiles > S;  // a block with no more tiles than stages never needs a stage back
+    // a warp's rows of a whole tile lie on 16-byte boundaries (flat: tiles are nt rows apart)
+    const uint32_t m_in0 = ((uint32_t)br.base * (uint32_t)in_row) & 15u, m_out0 = ((uint32_t)br.base * (uint32_t)out_row) & 15u;
+    const bool rows_aligned = ((((kLong ? 0 : (int)(br.base & 15)) * out_row) | (NTW * out_row)) & 15) == 0 &&
+                              (!kLong || ((g.T * out_row) & 15) == 0);
+
+    grid_dependency_wait();
+    StepRaw cur;
+    if (!kIndirect) cur = load_scalars(tl, is_inner(tl, grp));
+    __syncthreads();  // the producer warp has set up the barriers (and fetched the device record)
+    if (kIndirect) cur = load_scalars(tl, is_inner(tl, grp));
+    int s = grp % S, s_prev = 0;
+    uint32_t ph = (uint32_t)(grp / S) & 1u;
+    int turn = 0;  // which of the group's two sets of warp aggregates this tile uses
+
+    for (int n = grp; n < n_tiles; n += C) {
+        // this warp's previous rows have left shared memory: hand the stage back.  (Only where stages are used
+        // more than once: the wait for the store's reads sits between two tiles of the warp.)
+        if (reuse && n != grp) {
+            dev::bulk_store_wait_read();
+            arrive_if(&empty_bar[s_prev], lane == 0);
+        }
+        // (long) one early look at the aggregates of the later tiles of this tile's trajectory: with many
+        // trajectories they were published a round ago, and reading them now keeps that trip to L2 off the path
+        // between this tile's scan and its gradients (only where tiles are numbered tile-major; the values are first
+        // looked at after the scan)
+        const long long gtile = (long long)blockIdx.x + (long long)n * gridDim.x;
+        const long long agg_stride = g.tile_major ? 2 * g.B : 2;  // slots between a tile's aggregate and that of the tile after it in time
+        const bool peeked = kLong && g.tile_major && gwarp == 0 && tl.r > lane;
+        unsigned long long early_a = 0, early_b = 0;
+        if (peeked) dev::load_aggregate(p.tile_aggregates + 2 * gtile, agg_stride, tl.r - lane, early_a, early_b);
+        // every thread waits for the stage itself (a bounded wait: on a time-out the flag is set and the
+        // thread goes on with whatever the stage holds, so that all barriers below still pair up)
+        if (!stage_wait(&full_bar[s], ph, &abort_s)) atomicExch(p.counter + 1, 1u);
+
+        // rows keep their place inside their 16-byte granule: the tile's first row starts (row0 * pitch) mod 16
+        // bytes into the slab
+        unsigned char* const stage = smem_raw + s * stage_bytes;
+        // (flat: tiles are a multiple of eight rows apart, so this is the same for all of the block's)
+        const uint32_t m_in = kLong ? ((uint32_t)tl.row0 * (uint32_t)in_row) & 15u : m_in0;
+        const uint32_t m_out = (sizeof(LT) == sizeof(GT)) ? m_in : (kLong ? ((uint32_t)tl.row0 * (uint32_t)out_row) & 15u : m_out0);
+        unsigned char* const s0 = stage + m_in;    // learner logits
+        unsigned char* const s1 = s0 + in_pitch;   // target logits
+        unsigned char* const so = (sizeof(LT) == sizeof(GT)) ? s0 : stage + 2 * in_pitch + m_out;
+        // (first traversal of a batch) the target rows go to the circular buffer as well, each warp's rows
+        // straight from the stage, which nothing writes to
+        if (IMPACT_IN(target_copy))
+            send_rows_general(static_cast<unsigned char*>(IMPACT_IN(target_copy)) + tl.row0 * (long long)in_row, s1,
+                              in_row, wrow, NTW, tl.lo, tl.hi, false);
+
+        // ---- row passes (every lane; rows that are not the tile's hold stale bytes and are masked)
+        float2 e[kWide ? 1 : NP];  // the learner row's exponentials, kept for the gradient pass
+        // Per row: log2 e times the largest logit (m2), log2 of the exponentials' sum (lg); learner: 1 / that sum and the
+        // mean logit.  m2 and lg are kept apart: adding them first would round their sum, the largest of the numbers
+        // that a log-probability is made of.
+        float m2_t = 0.0f, lg_t = 0.0f, m2_l = 0.0f, lg_l = 0.0f, inv_s = 0.0f, mean_z = 0.0f, kl = 0.0f;
+        // a row of the lane's pass: where it starts in its slab, at the lane's first vector
+        auto row_of = [&](int pass) { return wrow + (kWide ? (lane >> log_l) * passes + pass : lane); };
+        auto load_row = [&](const unsigned char* slab, int r, float2 (&z)[NP]) {
+            const unsigned char* at = slab + r * in_row + part * (kV * (int)sizeof(LT));
+            float f[2 * NP];
+#pragma unroll
+            for (int j = 0; j < 2 * NP; ++j) f[j] = kLowest;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const bool there = kFixed || (kWide ? i * vstep + part * kV < A : i * kV < A);
+                if (there) Vec<LT, kV>::ld(at + i * vstep * (int)sizeof(LT), f + i * kV);
+            }
+#pragma unroll
+            for (int j = 0; j < NP; ++j) z[j] = make_float2(f[2 * j], f[2 * j + 1]);
+        };
+        auto row_max2 = [&](const float2 (&z)[NP]) {
+            float m0 = fmaxf(z[0].x, z[0].y), m1 = m0;
+#pragma unroll
+            for (int j = 1; j < NP; ++j) {
+                if (j & 1) m1 = fmaxf(m1, fmaxf(z[j].x, z[j].y));
+                else m0 = fmaxf(m0, fmaxf(z[j].x, z[j].y));
+            }
+            return fmaxf(m0, m1);
+        };
+        // pairs that hold elements (a uniform count): what lies beyond is not worked on
+        const int n_pairs = kFixed ? NP : (nvec * kV + 1) / 2;
+        const float2 log2e2 = make_float2(kLog2e, kLog2e);
+        for (int pass = 0; pass < (kWide ? passes : 1); ++pass) {
+            const int r = row_of(pass);
+            float2 z[NP];
+            // target row: its log2-sum-exp (base 2, of z log2 e)
+            load_row(s1, r, z);
+            float m_t = row_max2(z);
+            if (kWide) for (int o = 1; o < L; o <<= 1) m_t = fmaxf(m_t, __shfl_xor_sync(0xffffffffu, m_t, o));
+            const float m2t = __fmul_rn(m_t, kLog2e);
+            float2 sum2 = make_float2(0.0f, 0.0f);
+            {
+                const float2 neg_m2 = make_float2(-m2t, -m2t);
+#pragma unroll
+                for (int j = 0; j < NP; ++j) {
+                    if (!kFixed && j >= n_pairs) continue;
+                    const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);  // (z - m) log2 e
+                    const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
+                    sum2 = __fadd2_rn(sum2, ex);
+                }
+            }
+            float sum_t = sum2.x + sum2.y;
+            // learner row: log2-sum-exp, sum_j e_j z_j
+            load_row(s0, r, z);
+            float m_l = row_max2(z);
+            if (kWide) for (int o = 1; o < L; o <<= 1) m_l = fmaxf(m_l, __shfl_xor_sync(0xffffffffu, m_l, o));
+            const float m2 = __fmul_rn(m_l, kLog2e);
+            sum2 = make_float2(0.0f, 0.0f);
+            float2 sez2 = make_float2(0.0f, 0.0f);
+            {
+                const float2 neg_m2 = make_float2(-m2, -m2);
+#pragma unroll
+                for (int j = 0; j < NP; ++j) {
+                    if (!kFixed && j >= n_pairs) continue;
+                    const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);
+                    const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
+                    sum2 = __fadd2_rn(sum2, ex);
+                    sez2 = __ffma2_rn(ex, z[j], sez2);
+                    if constexpr (!kWide) e[j] = ex;
+                }
+            }
+            float sum_l = sum2.x + sum2.y, sez = sez2.x + sez2.y;
+            if (kWide) {
+                for (int o = 1; o < L; o <<= 1) {
+                    sum_t += __shfl_xor_sync(0xffffffffu, sum_t, o);
+                    sum_l += __shfl_xor_sync(0xffffffffu, sum_l, o);
+                    sez += __shfl_xor_sync(0xffffffffu, sez, o);
+                }
+            }
+            const float lgt = dev::log2_fast(sum_t), lgl = dev::log2_fast(sum_l);
+            const float is = dev::rcp_fast(sum_l);
+            float klr = 0.0f;
+            if (want_kl) {
+                float2 zt[NP];
+                load_row(s1, r, zt);
+                const float lt2 = __fadd_rn(m2t, lgt), ll2 = __fadd_rn(m2, lgl);
+#pragma unroll
+                for (int j = 0; j < NP; ++j) {
+                    if (!kFixed && j >= n_pairs) continue;
+                    const float ax = fmaf(zt[j].x, kLog2e, -lt2), ay = fmaf(zt[j].y, kLog2e, -lt2);
+                    const float ex = dev::exp2_fast(ax), ey = dev::exp2_fast(ay);
+                    const float dx = (ax - fmaf(z[j].x, kLog2e, -ll2)) * kLn2, dy = (ay - fmaf(z[j].y, kLog2e, -ll2)) * kLn2;
+                    // (an element that is not there: its two logarithms are both -inf, and it adds nothing)
+                    const bool has_x = kFixed || element_exists(2 * j, part, vstep, kV, A);
+                    const bool has_y = (kFixed && 2 * j + 1 < E) || (!kFixed && element_exists(2 * j + 1, part, vstep, kV, A));
+                    if (has_x) klr = fmaf(ex, dx, klr);
+                    if (has_y) klr = fmaf(ey, dy, klr);
+                }
+                if (kWide) for (int o = 1; o < L; o <<= 1) klr += __shfl_xor_sync(0xffffffffu, klr, o);
+            }
+            if (!kWide || part == pass) {
+                m2_t = m2t; lg_t = lgt; m2_l = m2; lg_l = lgl; inv_s = is; mean_z = __fmul_rn(sez, is); kl = klr;
+            }
+        }
+        // ---- the step's own scalars (its owner lane)
+        const int act = min(max(cur.a, 0), A - 1);
+        Step st;
+        st.l2_worker = __fmul_rn(cur.l_worker, kLog2e);
+        st.reward = cur.reward;
+        st.discount = cur.discount;
+        st.value = cur.value;
+        st.value_next = cur.value_next;
+        st.ends = ends_here(tl);
+        const int orow = kWide && !owner ? wrow : lrow;  // (a lane that owns no row looks at the warp's first)
+        st.l2_target = fmaf(get_element<LT>(s1 + orow * in_row, act), kLog2e, -m2_t) - lg_t;
+        st.l2_theta = fmaf(get_element<LT>(s0 + orow * in_row, act), kLog2e, -m2_l) - lg_l;
+        // H = -sum_j pi_j lp_j = (m + ln S) - sum_j e_j z_j / S
+        const float ent = fmaf(__fadd_rn(m2_l, lg_l), kLn2, -mean_z);
+        float fa, fb;
+        const bool truncated = step_map<kPlain>(st, k, fa, fb);
+        const bool mine = is_mine(tl);
+        if (!mine) { fa = 1.0f; fb = 0.0f; }
+        // (flat) the slot of the tile, or beyond, where the step's trajectory ends
+        const int reach = lrow + (int)min(to_end, 1024u);
+        int limit = 31 - lane;
+        if constexpr (!kLong) {
+            const int left = reach - wrow;  // ... counted from the warp's first row
+            limit = min(limit, (kWide ? (left / passes << log_l) + left % passes : left) - lane);
+        }
+
+        // the next tile's scalars travel while this tile is worked on
+        const Now here = tl;
+        to_next_tile(n + C);
+        if (n + C < n_tiles) cur = load_scalars(tl, is_inner(tl, n + C));
+
+        // ---- the recursion: maps composed from the tile's end
+        warp_suffix_compose(fa, fb, limit);
+        if (lane == 0) warp_agg[grp][turn][gwarp] = make_float2(fa, fb);
+        asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
+        float adv, after;  // A of the step, and (lane 31) of the step after the warp's last
+        if constexpr (!kLong) {
+            // what follows the warp's last step, as far as the step's trajectory reaches
+            float x = 0.0f;
+            // (a lane that owns no row passes the value on to the one before it, as the advantage of the step after it)
+            const bool goes_on = (owner ? mine : n > 0) && reach >= NT;
+            if (__any_sync(0xffffffffu, goes_on)) {
+                const float m = mail_get(mail, n - 1, &abort_s);
+                x = goes_on ? m : 0.0f;
+            }
+#pragma unroll
+            for (int w = 3; w > 0; --w) {
+                const float2 f = warp_agg[grp][turn][w];
+                if (w > gwarp && reach >= w * NTW) x = fmaf(f.x, x, f.y);
+            }
+            adv = fmaf(fa, x, fb);
+            after = x;
+            if (gtid == 0) mail_put(mail, n, adv);
+        } else {
+            // maps instead of values: (ma, mb) takes the value that enters the tile's last step to A of this step,
+            // (la, lb) to A of the step after this warp's last
+            float la = 1.0f, lb = 0.0f;
+#pragma unroll
+            for (int w = 3; w > 0; --w) {
+                const float2 f = warp_agg[grp][turn][w];
+                if (w > gwarp) { lb = fmaf(f.x, lb, f.y); la = f.x * la; }
+            }
+            const float ma = fa * la, mb = fmaf(fa, lb, fb);
+            if (gtid == 0) dev::publish_tile_aggregate(p.tile_aggregates + 2 * gtile, ma, mb, dev::launch_tag(p.counter));
+            float carry = 0.0f;
+            if (here.r > 0) {  // uniform over the group
+                if (gwarp == 0) {
+                    const float c = dev::compose_later_aggregates(p.tile_aggregates + 2 * gtile, agg_stride, here.r,
+                                                                  dev::launch_tag(p.counter), &abort_s, peeked,
+                                                                  early_a, early_b);
+                    if (lane == 0) carry_s[grp] = c;
+                }
+                asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
+                carry = carry_s[grp];
+            }
+            adv = fmaf(ma, carry, mb);
+            after = fmaf(la, carry, lb);
+        }
+        if constexpr (!kPlain) {
+            const float below = __shfl_down_sync(0xffffffffu, adv, 1);
+            st.adv_next = (lane == 31) ? after : below;
+        }
+        turn ^= 1;
+
+        float surr, ratio;
+        bool clipped;
+        const float wpg = step_surrogate<kPlain>(st, k, adv, surr, ratio, clipped);
+        if (mine) {
+            t_surr += surr;
+            t_val = fmaf(0.5f * adv, adv, t_val);
+            t_ent += ent;
+            t_ratio += ratio;
+            if (!kPlain) t_kl += kl;
+            n_clip += clipped ? 1 : 0;  // (per thread; added up over the warp when the sums are handed over)
+            n_trunc += truncated ? 1 : 0;
+        }
+        // the group's sums are final after its last tile's scan: handed over here, they are published while
+        // that tile's gradient pass runs
+        if (n + C >= n_tiles) hand_over_sums();
+
+        // ---- gradients: row_j = e_j (ga z_j + gb) [- kl_coef pi_target_j / M], then the taken action's entry
+        const float w1 = __fmul_rn(wpg, k.inv_M), ce = k.ent_over_M, ck = kPlain ? 0.0f : k.kl_over_M;
+        const float ga = __fmul_rn(ce, inv_s), gb = __fmul_rn(__fadd_rn(fmaf(-ce, mean_z, w1), ck), inv_s);
+        for (int pass = 0; pass < (kWide ? passes : 1); ++pass) {
+            const int r = row_of(pass);
+            float pga = ga, pgb = gb, pm2 = m2_l, plt = kPlain ? 0.0f : __fadd_rn(m2_t, lg_t);
+            if (kWide) {
+                const int from = (lane & ~(L - 1)) + pass;
+                pga = __shfl_sync(0xffffffffu, ga, from);
+                pgb = __shfl_sync(0xffffffffu, gb, from);
+                pm2 = __shfl_sync(0xffffffffu, m2_l, from);
+                if (want_kl) plt = __shfl_sync(0xffffffffu, __fadd_rn(m2_t, lg_t), from);
+            }
+            const float2 ga2 = make_float2(pga, pga), gb2 = make_float2(pgb, pgb);
+            const float2 neg_m2 = make_float2(-pm2, -pm2);
+            const float2 neg_lse2 = make_float2(-plt, -plt), nck2 = make_float2(-ck, -ck);
+            const unsigned char* const zrow = s0 + r * in_row + part * (kV * (int)sizeof(LT));
+            const unsigned char* const trow = s1 + r * in_row + part * (kV * (int)sizeof(LT));
+            unsigned char* const orow_ = so + r * out_row + part * (kV * (int)sizeof(GT));
+            // vector by vector (two at a time where a vector is one element: the arithmetic is on pairs)
+            constexpr int kStep = kV == 1 ? 2 : 1, kElems = kStep * kV;
+#pragma unroll
+            for (int i = 0; i < NV; i += kStep) {
+                float z[kElems], o[kElems], zt[kElems];
+                bool there[kStep];
+#pragma unroll
+                for (int u = 0; u < kStep; ++u)
+                    there[u] = kFixed ? i + u < NV : (kWide ? (i + u) * vstep + part * kV < A : (i + u) * kV < A);
+                if (!kFixed && !kWide && !there[0]) continue;  // (uniform)
+#pragma unroll
+                for (int u = 0; u < kStep; ++u) {
+#pragma unroll
+                    for (int v = 0; v < kV; ++v) z[u * kV + v] = 0.0f, zt[u * kV + v] = 0.0f;
+                    if (there[u]) {
+                        Vec<LT, kV>::ld(zrow + (i + u) * vstep * (int)sizeof(LT), z + u * kV);
+                        if (want_kl) Vec<LT, kV>::ld(trow + (i + u) * vstep * (int)sizeof(LT), zt + u * kV);
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < kElems; v += 2) {
+                    const float2 z2 = make_float2(z[v], z[v + 1]);
+                    float2 ex;
+                    if constexpr (kWide) {
+                        const float2 t2 = __ffma2_rn(z2, log2e2, neg_m2);
+                        ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
+                    } else {
+                        ex = e[(i * kV + v) / 2];
+                    }
+                    float2 gr = __fmul2_rn(ex, __ffma2_rn(z2, ga2, gb2));
+                    if (want_kl) {
+                        const float2 tt = __ffma2_rn(make_float2(zt[v], zt[v + 1]), log2e2, neg_lse2);
+                        gr = __ffma2_rn(nck2, make_float2(dev::exp2_fast(tt.x), dev::exp2_fast(tt.y)), gr);
+                    }
+                    o[v] = gr.x;
+                    o[v + 1] = gr.y;
+                }
+#pragma unroll
+                for (int u = 0; u < kStep; ++u)
+                    if (there[u]) Vec<GT, kV>::st(orow_ + (i + u) * vstep * (int)sizeof(GT), o + u * kV);
+            }
+        }
+        const float pi_a = dev::exp2_fast(st.l2_theta);
+        float g_a = fmaf(pi_a, fmaf(ce, fmaf(st.l2_theta, kLn2, ent), w1), -w1);
+        if (want_kl) g_a = fmaf(ck, pi_a - dev::exp2_fast(st.l2_target), g_a);
+        if (mine) {
+            p.dvalues[here.row0 + lrow] = __fmul_rn(k.dvalue_over_adv, adv);  // V - Vhat = -A
+            if (!kPlain) {
+                if (p.vtarget) p.vtarget[here.row0 + lrow] = st.value + adv;
+                if (p.advantage) p.advantage[here.row0 + lrow] = adv;
+            }
+        }
+        if (kWide) __syncwarp();  // (other lanes wrote the row that this one corrects)
+        if (owner) put_element<GT>(so + lrow * out_row, act, g_a);
+        // ---- each warp sends its own rows: no barrier across the group
+        {
+            unsigned char* const out = static_cast<unsigned char*>(p.dlogits) + here.row0 * (long long)out_row;
+            if (here.lo == 0 && here.hi == NT && rows_aligned) {  // whole granules: the usual case
+                dev::fence_async_shared();
+                __syncwarp();
+                if (lane == 0) dev::bulk_store(out + wrow * out_row, so + wrow * out_row, (uint32_t)(NTW * out_row));
+            } else {
+                send_rows_general(out, so, out_row, wrow, NTW, here.lo, here.hi, true);
+            }
+        }
+        s_prev = s;
+        s += C;
+        if (s >= S) { s -= S; ph ^= 1u; }  // (C <= S wherever a group has a second tile)
+    }
+
+    // a group without tiles still hands over its (zero) sums, so that every row of the grid is defined
+    if (grp >= n_tiles) hand_over_sums();
+    // ---- one group of the grid (block 0's, the one that runs out of tiles first and so is polling long before the
+    // last rows appear) collects every block's row as it appears and writes the loss terms
+    if (blockIdx.x == 0 && grp == n_tiles % C) {
+        if (!dev::reduce_tagged_rows<128>(p.tagged_rows, (int)gridDim.x, dev::launch_tag(p.counter), p.counter,
+                                          p.loss_terms, k.vf_coef, k.ent_coef, k.kl_coef, k.steps_total,
+                                          gtid, bar_id, &abort_s))
+            if (gtid == 0) atomicExch(p.counter + 1, 1u);
+    }
+    if (lane == 0) dev::bulk_store_wait_read();  // shared memory must outlive the stores' reads
+#undef IMPACT_IN
+}
+
+// ------------------------------------------------------------------------------------------
+// Launch
+// ------------------------------------------------------------------------------------------
+template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
+int32_t launch_categorical(CatParams p, int nt, int log_lanes, const DeviceInfo* di, cudaStream_t stream) {
+    auto kernel = impact_loss_categorical_kernel<LT, GT, kA, C, kV, kPlain, kLong, kIndirect>;
+    const size_t stage = cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT));
+    p.geo.nt = nt;
+    p.geo.ntiles = kLong ? (int)((p.geo.T + nt - 1) / nt) : 1;
+    long long grid, tiles, tiles_per_block;
+    if (kLong) {
+        tiles = p.geo.B * p.geo.ntiles;
+        grid = tiles < di->sm_count ? tiles : di->sm_count;
+        tiles_per_block = (tiles + grid - 1) / grid;
+    } else {
+        // a block per tile's worth of whole trajectories, or per trajectory, up to one per SM
+        const long long per_tile = p.geo.T < nt ? nt / p.geo.T : 1;
+        grid = (p.geo.B + per_tile - 1) / per_tile;
+        if (grid > di->sm_count) grid = di->sm_count;
+        const long long trajs = (p.geo.B + grid - 1) / grid;
+        tiles_per_block = (trajs * p.geo.T + nt - 1) / nt;
+        tiles = tiles_per_block * grid;
+    }
+    if (grid > kMaxTaggedRows) return IMPACT_ERR_UNSUPPORTED;  // one tagged row per block
+    // tile-major once every block has a trajectory of its own: the aggregates a tile needs are then a round old
+    p.geo.tile_major = (kLong && p.geo.B >= grid) ? 1 : 0;
+    CatShape sh = {};
+    sh.nt = nt;
+    sh.log_lanes = log_lanes;
+    sh.passes = (nt / 4 << log_lanes) / 32;
+    ws_ring_shape(stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di->max_smem_optin, tiles_per_block, &sh.stages, &sh.in_flight);
+    if (sh.stages < 1 || sh.in_flight < 1) return IMPACT_ERR_UNSUPPORTED;
+    const int spare = sh.stages - sh.in_flight;  // producer lanes that request tiles side by side
+    sh.lanes = spare < 4 ? (spare < 1 ? 1 : spare) : 4;
+    const size_t smem = (size_t)sh.stages * stage;
+    static thread_local int configured_device = -1;
+    if (configured_device != di->device) {  // once per device: room for the largest ring any window setting asks for
+        IMPACT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, di->max_smem_optin - 4096));
+        configured_device = di->device;
+    }
+    // (rows wider than 32 actions: the companion gains nothing with fp32 logits and doubles a launch with bf16 ones
+    // -- 27 against 14 us at 65 536 steps --, so such launches ask for their first tiles themselves)
+    WsPlan plan = ws_plan(tiles, grid, (size_t)nt * (2 * p.A * sizeof(LT) + 20), sh.in_flight, p.A <= 32);
+    if (kIndirect) { plan.companion = false; plan.prefetch_tiles = 0; }  // (addresses unknown on the host)
+    if (plan.companion) {
+        const int32_t st = launch_companion(p, (int)sizeof(LT), kLong, plan.prefetch_tiles, (int)grid, stream);
+        if (st != IMPACT_OK) return st;
+    } else {
+        sh.n_prefetch = plan.prefetch_tiles;
+    }
+    IMPACT_CUDA_TRY(launch_serialized(kernel, dim3((unsigned)grid), dim3(C * 128 + 32), smem, stream, p, sh));
+    return IMPACT_OK;
+}
+
+// Long trajectories go to neighbouring blocks while there are too few of them to give every block about four (and the
+// caller's scratch has room for the tiles' aggregates); from there on blocks that own whole trajectories are as busy,
+// without any exchange between blocks.
+inline bool splits_trajectories(const CatParams& p, int nt, const DeviceInfo* di) {
+    return p.geo.T > nt && nt >= kMinTileRows && p.tile_aggregates && p.geo.B < 4ll * di->sm_count;
+}
+// (a flat launch counts a trajectory's steps in 32 bits)
+inline bool fits_flat(const CatParams& p) { return p.geo.T < (1ll << 32) - 4096; }
+
+// Consumer groups: four with every switch compiled in; five in the default configuration; six there for small action
+// sets, which are bound by arithmetic, not bytes.
+template <typename LT, typename GT, int A, int kV>
+int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    constexpr int C = 4, CP = A <= 9 ? 6 : 5;
+    const bool plain = p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
+                       p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 &&
+                       !p.vtarget && !p.advantage;
+    if (p.indirect) {  // compiled for trajectories that fit a tile only
+        if (p.geo.T > 128) return IMPACT_ERR_UNSUPPORTED;
+        return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, true>(p, 128, 0, di, stream)
+                     : launch_categorical<LT, GT, A, C, kV, false, false, true>(p, 128, 0, di, stream);
+    }
+    if (splits_trajectories(p, 128, di) || !fits_flat(p)) {
+        if (!p.tile_aggregates) return IMPACT_ERR_UNSUPPORTED;
+        return launch_categorical<LT, GT, A, C, kV, false, true, false>(p, 128, 0, di, stream);
+    }
+    return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, 128, 0, di, stream)
+                 : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, 128, 0, di, stream);
+}
+
+// How many lanes of a warp's accesses to rows of `row_bytes`, `group` lanes to a row, meet on the same banks.
+inline int bank_ways(size_t row_bytes, int rows_between, int group, int access_bytes) {
+    const size_t stride = row_bytes * (size_t)rows_between, window = (size_t)group * access_bytes;
+    const int rows_at_once = 128 / access_bytes / group;
+    if (rows_at_once <= 1) return 1;
+    size_t step = stride % 128;  // gcd(stride, 128)
+    step = step ? (step & (~step + 1)) : 128;
+    return step >= window ? (int)(step / window) : 1;
+}
+
+template <typename LT, typename GT, int kV>
+int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    constexpr int C = 4;
+    const size_t row = p.A * sizeof(LT);
+    if (p.A <= kMaxLaneElems && bank_ways(row, 1, 1, kV * (int)sizeof(LT)) <= 2) {
+        if (p.indirect) return IMPACT_ERR_UNSUPPORTED;
+        if (splits_trajectories(p, 128, di) || !fits_flat(p)) {
+            if (!p.tile_aggregates) return IMPACT_ERR_UNSUPPORTED;
+            return launch_categorical<LT, GT, 0, C, kV, false, true, false>(p, 128, 0, di, stream);
+        }
+        return launch_categorical<LT, GT, 0, C, kV, false, false, false>(p, 128, 0, di, stream);
+    }
+    // Rows of more than a lane: tiles of up to 36 KB (a ring of six stages, four of them being worked on), then the
+    // fewest lanes that hold a row and do not meet on the banks more than two at a time.
+    int nt = 128;
+    while (nt > 8 && cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT)) > 36 * 1024) nt /= 2;
+    int log_l = 1;
+    auto lanes_suffice = [&](int l) {
+        if ((nt / 4 << l) < 32 || ((long long)kMaxLaneElems << l) < p.A) return false;
+        return l == 5 || bank_ways(row, (nt / 4 << l) / 32, 1 << l, kV * (int)sizeof(LT)) <= 2;
+    };
+    while (!lanes_suffice(log_l)) ++log_l;
+    if (p.indirect) {
+        if constexpr (kV == 4) {
+            if (p.A == 64 && p.geo.T <= 64)
+                return launch_categorical<LT, GT, -1, C, kV, false, false, true>(p, nt, log_l, di, stream);
+        }
+        return IMPACT_ERR_UNSUPPORTED;
+    }
+    if (splits_trajectories(p, nt, di) || !fits_flat(p)) {
+        if (!p.tile_aggregates || nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
+        return launch_categorical<LT, GT, -1, C, kV, false, true, false>(p, nt, log_l, di, stream);
+    }
+    return launch_categorical<LT, GT, -1, C, kV, false, false, false>(p, nt, log_l, di, stream);
+}
+
+template <typename LT, typename GT>
+int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    switch (p.A) {  // (the Atari action sets)
+        case 4: return run_fixed<LT, GT, 4, 4>(p, di, stream);
+        case 6: return run_fixed<LT, GT, 6, 2>(p, di, stream);
+        case 9: return run_fixed<LT, GT, 9, 1>(p, di, stream);
+        case 18: return run_fixed<LT, GT, 18, 2>(p, di, stream);
+        default: break;
+    }
+    if (p.A % 4 == 0) return run_runtime_width<LT, GT, 4>(p, di, stream);
+    if (p.A % 2 == 0) return run_runtime_width<LT, GT, 2>(p, di, stream);
+    return run_runtime_width<LT, GT, 1>(p, di, stream);
+}
+
+}  // namespace impact

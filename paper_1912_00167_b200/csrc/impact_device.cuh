@@ -575,6 +575,8 @@ struct LossScalars {
     float rho_bar, c_bar, clip_lo, clip_hi;
     float vf_coef, ent_coef, kl_coef, lambda_, log_rho_tw;
     float inv_M;
+    // products and conversions of the above that a step would otherwise form for itself
+    float ent_over_M, kl_over_M, dvalue_over_adv, log2_rho_tw;
     int is_source, ratio_mode, objective;
     double steps_total;  // M: the steps the means are taken over (this call's, or the whole batch's when it is split)
 };

@@ -1,0 +1,89 @@
+// Parameters of the loss kernels, shared by the host entry points and the translation units that instantiate kernels
+// (not part of the ABI).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "impact.h"
+#include "impact_device.cuh"
+#include "impact_internal.h"
+
+namespace impact {
+
+using dev::LossScalars;
+
+constexpr int kWsMaxStages = 24;      // stages of a persistent kernel's ring at most
+constexpr int kMaxGridBlocks = 4096;  // upper bound on blocks of a loss launch (sizes the workspace)
+constexpr size_t kCounterBytes = 256; // words after the partials: [0] completion counter, [1] error flag, [2] launch number
+constexpr int kMaxTaggedRows = 1024;  // rows of eight (value, tag) pairs after the counter words: one per block of a persistent kernel
+constexpr int kMinTileRows = 64;      // the smallest tile of a launch that publishes its tiles' aggregates
+
+// How a categorical batch is laid out over the grid (see impact_categorical.cuh).
+struct CatGeometry {
+    long long B, T;
+    int nt;          // rows of a tile
+    int ntiles;      // long: tiles per trajectory
+    int tile_major;  // long: order of the grid's tiles
+};
+
+struct CatParams {
+    const void* learner_logits;
+    const void* target_logits;
+    const float* worker_logp;
+    const int32_t* actions;
+    const float* rewards;
+    const float* discounts;
+    const float* values;
+    const float* bootstrap;
+    float* loss_terms;
+    void* dlogits;
+    float* dvalues;
+    float* vtarget;
+    float* advantage;
+    unsigned int* counter;
+    unsigned long long* tagged_rows;      // rows of (value, launch tag) pairs, see dev::publish_tagged
+    unsigned long long* tile_aggregates;  // long launches: two (value, launch tag) pairs per tile (NULL = no room for them)
+    void* target_copy;  // where the target logits are written as well (NULL = nowhere)
+    const impact_loss_inputs* indirect;  // device record that overrides the nine input pointers above (NULL = none)
+    CatGeometry geo;
+    LossScalars k;
+    int A;
+};
+
+// The rest of a categorical launch's shape.
+struct CatShape {
+    int nt, stages, in_flight, lanes, n_prefetch;
+    int log_lanes, passes;  // rows wider than a lane (see impact_categorical.cuh)
+};
+
+struct LossInputPointers {
+    const void* learner_logits;
+    const void* target_logits;
+    const float* worker_logp;
+    const int32_t* actions;
+    const float* rewards;
+    const float* discounts;
+    const float* values;
+    const float* bootstrap;
+    void* target_copy;
+};
+
+// Picks the kernel for a categorical call (`p` complete except for geo) and launches it.
+template <typename LT, typename GT>
+int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
+
+// Tiles the producer keeps in flight and stages of the ring, for tiles of `tile_in_bytes` bytes of logits.
+void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max_smem, long long tiles_per_block,
+                   int* stages, int* in_flight);
+// How many tiles per block are asked for in L2 ahead of time, and by whom.
+struct WsPlan {
+    int prefetch_tiles;  // tiles per block asked for in L2 ahead of time
+    bool companion;      // by a companion kernel enqueued before the loss kernel (else by the loss kernel's first warp)
+};
+WsPlan ws_plan(long long tiles, long long grid, size_t tile_bytes, int in_flight, bool allow_companion);
+
+// The companion of a categorical launch of `grid` blocks: asks L2 for each block's first `n_tiles` tiles.
+int32_t launch_companion(const CatParams& p, int elem_bytes, bool is_long, int n_tiles, int grid, cudaStream_t stream);
+
+}  // namespace impact

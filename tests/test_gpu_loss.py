@@ -560,3 +560,80 @@ def test_prepared_calls_keep_their_tensors_alive():
         call, addresses = make()
         held = {x.data_ptr() for x in call._keep if isinstance(x, torch.Tensor)}
         assert set(addresses) <= held
+
+
+WIDTHS = [1, 2, 3, 5, 7, 8, 10, 12, 15, 16, 17, 20, 31, 32, 33, 48, 63, 65, 96, 100, 127, 128, 130, 200, 255, 256, 300, 511, 512]
+
+
+@pytest.mark.parametrize("A", WIDTHS)
+def test_every_width_of_the_row_passes(oracle, A):
+    """Action counts on both sides of every change of layout (elements per access, lanes per row, rows per tile), with
+    more trajectories than blocks, so that trajectories cross the tiles of a block; fp32 and bf16, each with the
+    other's gradients too."""
+    T = 50 if A <= 128 else 21
+    batch = ii.categorical_batch(331 if A <= 128 else 301, T, A, seed=6000 + A, p_done=0.02)
+    full = LossHyper(rho_bar=1.3, c_bar=1.1, clip_eps=0.25, vf_coef=0.7, ent_coef=0.02, kl_coef=0.1, lam=0.97, rho_tw=2.0)
+    P.check_categorical(oracle, batch, full, target_copy=True)
+    P.check_categorical(oracle, batch, full, torch.bfloat16, torch.float32, target_copy=True)
+    P.check_categorical(oracle, batch, full, torch.bfloat16, torch.bfloat16, rtol=P.RTOL_BF16, atol=P.ATOL_BF16)
+    P.check_categorical(oracle, batch, full, torch.float32, torch.bfloat16, rtol=P.RTOL_BF16, atol=P.ATOL_BF16)
+
+
+def _off_the_truncation_bound(batch, rho_bar):
+    """Steps whose importance weight lies so close to rho_bar that fp32 and fp64 may count it on different sides are
+    moved off it: log-probabilities of magnitude up to 16 carry two roundings each in fp32 (2 * 2 * 16 * 2^-24 < 4e-6),
+    and one step more or less is already 1 / (B T) of the truncated share."""
+    z = batch["target_logits"].astype(np.float64)
+    lse = np.log(np.exp(z - z.max(-1, keepdims=True)).sum(-1)) + z.max(-1)
+    l_target = np.take_along_axis(z, batch["actions"][..., None].astype(int), -1)[..., 0] - lse
+    near = np.abs(l_target - batch["worker_logp"].astype(np.float64) - np.log(rho_bar)) < 4e-6
+    batch["worker_logp"] = np.where(near, batch["worker_logp"] - 0.01, batch["worker_logp"]).astype(np.float32)
+    return batch
+
+
+@pytest.mark.parametrize("B,T", [(1000, 1), (999, 3), (600, 31), (449, 50), (400, 100), (300, 127), (311, 128), (170, 129),
+                                 (149, 200), (640, 257), (700, 300)])
+@pytest.mark.parametrize("A", [6, 18, 7, 40])
+def test_trajectories_that_cross_the_tiles_of_a_block(oracle, B, T, A):
+    """Blocks own whole trajectories and walk their rows in tiles that begin and end anywhere: trajectories shorter
+    than a warp, than a tile, of a tile and longer; ranges that start off the multiples of eight rows; blocks with one
+    trajectory more than others.  Without optional outputs (the default configuration's kernel) and with every switch."""
+    batch = ii.categorical_batch(B, T, A, seed=6500 + B + T + A, p_done=0.02)
+    plain = LossHyper(rho_bar=1.0, c_bar=1.0, clip_eps=0.3, vf_coef=0.5, ent_coef=0.01, kl_coef=0.0, rho_tw=1.0)
+    full = LossHyper(rho_bar=1.3, c_bar=1.1, clip_eps=0.25, vf_coef=0.7, ent_coef=0.02, kl_coef=0.1, lam=0.97, rho_tw=2.0)
+    P.check_categorical(oracle, _off_the_truncation_bound(batch, 1.0), plain, extra=False)
+    P.check_categorical(oracle, _off_the_truncation_bound(batch, 1.3), full)
+    impala = LossHyper(objective=1, rho_bar=1.3, c_bar=1.1, lam=0.97, ent_coef=0.02)  # (reads A of the following step)
+    P.check_categorical(oracle, batch, impala)
+
+
+@pytest.mark.parametrize("B,T,A", [(450, 50, 6), (450, 50, 18), (450, 50, 7), (450, 50, 40), (600, 20, 18), (160, 300, 18)])
+def test_a_non_finite_value_stays_in_its_trajectory(B, T, A):
+    """The recursion is cut between trajectories, not multiplied by zero: an infinite reward or a NaN logit leaves every
+    other trajectory's outputs as they are, bit for bit, wherever the tiles of a block begin and end."""
+    import paper_1912_00167_b200 as ip
+    batch = ii.categorical_batch(B, T, A, seed=71 + A, p_done=0.0)
+    clean = {k: torch.from_numpy(v).cuda() for k, v in batch.items()}
+    dirty = {k: v.clone() for k, v in clean.items()}
+    hit = [0, 3, 4, B // 2, B - 1]
+    for i, b in enumerate(hit):
+        if i % 2:
+            dirty["rewards"][b, (7 * i) % T] = float("inf")
+        else:
+            dirty["learner_logits"][b, (5 * i) % T, A - 1] = float("nan")
+            dirty["target_logits"][b, T - 1, 0] = float("nan")
+    res = []
+    for t in (clean, dirty):
+        out = dict(loss_terms=torch.zeros(8, device="cuda"), dlogits=torch.zeros(B, T, A, device="cuda"),
+                   dvalues=torch.zeros(B, T, device="cuda"))
+        ws = ip.new_workspace(B, T)
+        ip.impact_loss_fwd_bwd(t["learner_logits"], t["target_logits"], t["worker_logp"], t["actions"], t["rewards"],
+                               t["discounts"], t["values"], t["bootstrap_values"], ip.Coefficients(clip_eps=0.3),
+                               workspace=ws, **out)
+        torch.cuda.synchronize()
+        assert ip.impact_loss_workspace_status(ws) == 0
+        res.append(out)
+    others = [b for b in range(B) if b not in hit]
+    for k in ("dlogits", "dvalues"):
+        assert torch.equal(res[0][k][others], res[1][k][others])
+        assert not torch.isfinite(res[1][k][hit]).all()
