@@ -291,17 +291,21 @@ static __device__ __noinline__ void send_rows_general(unsigned char* out, const 
 
 // ---- shape of the row passes ------------------------------------------------------------------------------------
 // kA > 0: the action count, known at compile time; a row belongs to one lane, which keeps its exponentials.
-// kA = 0 (narrow): at most 16 actions, one lane per row as well, the count a run-time value.
-// kA < 0 (wide): any count; a row belongs to L = 2 ... 32 lanes that hold up to 16 elements each (vector i of lane g is
-//   the row's vector i L + g, which spreads a warp's accesses over the banks without padding), and a warp works on its
-//   NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the warp is worked on in pass p by lanes [q L, q L + L)
-//   and owned -- for everything that is per step -- by lane q L + p of them, so results never move between lanes.
-//   The gradient pass forms the exponentials again instead of holding P rows in registers.
-constexpr int kMaxLaneElems = 16;
-// Is the j-th of a lane's elements part of the row?
-__device__ __forceinline__ bool element_exists(int j, int part, int vstep, int kv, int A) {
-    return (j / kv) * vstep + part * kv < A;
-}
+// kA = kNarrow16, kNarrow32: at most 16 or 32 actions, one lane per row as well, the count a run-time value.
+// kA = kWideRows: any count; a row belongs to L = 2 ... 32 lanes that hold up to 32 elements each (vector i of lane g is
+//   the row's vector i L + g), and a warp works on its NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the
+//   warp is worked on in pass p by lanes [q L, q L + L) and owned -- for everything that is per step -- by lane q L + p
+//   of them, so results never move between lanes.  The gradient pass forms the exponentials again instead of holding P
+//   rows in registers.  (Fewest lanes: a pass costs a warp about a hundred instructions besides its elements'.)
+//
+// Rows keep their dense layout in shared memory.  kV = 4 or 2: elements per access, where they divide the count.
+// kV = 1 stands for odd counts: a row is then one element and pairs, the element in front where the row starts on an odd
+// one (so that the pairs are aligned) and behind where it starts on an even one.  (fp32 and a count known at compile
+// time: element by element -- such rows meet on no bank, their pairs on two; 250 000 steps of 9 actions with every
+// switch in use take 11.8 us instead of 12.4.)  Where rows meet on the same banks
+// (pitches with a large power of two), lanes take their vectors in rotated order; maxima and sums do not mind.
+constexpr int kNarrow16 = 0, kNarrow32 = -2, kWideRows = -1;
+constexpr int kWideElems = 32;  // elements of a row that a lane holds at most
 
 // The record of impact_buffer_device_step, read past L1 (an earlier launch may have left an older version there).
 __device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss_inputs* rec) {
@@ -346,13 +350,15 @@ __device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss
 template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid_constant__ CatShape sh) {
-    constexpr bool kWide = kA < 0, kFixed = kA > 0;
-    constexpr int E = kFixed ? kA : kMaxLaneElems;
-    constexpr int NV = (E + kV - 1) / kV;       // vectors per lane at most
-    constexpr int NP = (E + 1) / 2;             // pairs: Blackwell's packed fp32 add / mul / fma work on two lanes at once
+    constexpr bool kWide = kA == kWideRows, kFixed = kA > 0;
+    constexpr bool kSingles = kV == 1 && kFixed && sizeof(LT) == 4;  // rows element by element
+    constexpr bool kOdd = kV == 1 && !kSingles;
+    constexpr int VW = kV == 1 ? 2 : kV;  // elements of a vector
+    constexpr int NV = (kFixed ? kA : (kA == kNarrow16 ? 16 : kWideElems)) / VW;  // vectors per lane at most
+    constexpr int NP = NV * VW / 2 + (kV == 1 ? 1 : 0);  // pairs: Blackwell's packed fp32 add / mul / fma work on two at once
     constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
     constexpr float kLowest = -3.402823466e38f;  // stands for an element that is not there: its exponential is 0
-    static_assert(!kFixed || kA % kV == 0, "whole vectors");
+    static_assert(!kFixed || kA % VW == (kV == 1 ? 1 : 0), "whole vectors");
     const int A = kFixed ? kA : p.A;
     const int NT = kFixed ? 128 : sh.nt;
     const int NTW = NT >> 2;  // rows of a tile that one warp works on
@@ -540,8 +546,9 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     // (a lane that owns no row stands for the one after it: the identity map, in that row's trajectory)
     const int lrow = wrow + (kWide ? (lane >> log_l) * passes + min(part, passes) : lane);
     const bool owner = kWide ? part < passes : true;
-    const int vstep = kWide ? (kV << log_l) : kV;  // elements from a lane's vector to its next
-    const int nvec = kFixed ? NV : (A + vstep - 1) / vstep;  // (of the lane with the most)
+    const int row_vecs = A / VW;  // vectors of a row (odd counts: and one element)
+    const int nvec = kFixed ? NV : (row_vecs + L - 1) >> log_l;  // of the lane with the most
+    const int rot = (kV == 4 && !kFixed) ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
 
     // The tile: which of its rows are this block's (flat) or exist at all (long), and where its first row sits.  In a
     // flat launch only a block's first tile ends early, only its last one can begin late, and from one of the group's
@@ -682,39 +689,53 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         // mean logit.  m2 and lg are kept apart: adding them first would round their sum, the largest of the numbers
         // that a log-probability is made of.
         float m2_t = 0.0f, lg_t = 0.0f, m2_l = 0.0f, lg_l = 0.0f, inv_s = 0.0f, mean_z = 0.0f, kl = 0.0f;
-        // a row of the lane's pass: where it starts in its slab, at the lane's first vector
         auto row_of = [&](int pass) { return wrow + (kWide ? (lane >> log_l) * passes + pass : lane); };
+        // byte offset of the lane's i-th vector from the row's first (of `elem`-byte elements)
+        auto vec_at = [&](int i, int elem) {
+            const int step = (VW * elem) << log_l;
+            return (kV == 4 && !kFixed) ? ((i * step) ^ (rot * step)) : i * step;
+        };
+        auto vec_there = [&](int i) { return kFixed || (kWide ? (i << log_l) + part < row_vecs : i < row_vecs); };
+        // (odd counts) does the row start on an odd element?  Tiles are an even number of rows apart.
+        const uint32_t tile_odd = kOdd ? (uint32_t)(kLong ? tl.row0 : br.base) & 1u : 0u;
+        auto first_of = [&](int r) { return kOdd ? (int)((tile_odd + (uint32_t)r) & 1u) : 0; };  // of the vectors
+        auto single_of = [&](int r) { return first_of(r) ? 0 : A - 1; };                         // the element beside them
         auto load_row = [&](const unsigned char* slab, int r, float2 (&z)[NP]) {
-            const unsigned char* at = slab + r * in_row + part * (kV * (int)sizeof(LT));
+            const unsigned char* const row = slab + r * in_row;
+            const unsigned char* const at = row + (first_of(r) + part * VW) * (int)sizeof(LT);
             float f[2 * NP];
 #pragma unroll
             for (int j = 0; j < 2 * NP; ++j) f[j] = kLowest;
+            if constexpr (kSingles) {
 #pragma unroll
-            for (int i = 0; i < NV; ++i) {
-                const bool there = kFixed || (kWide ? i * vstep + part * kV < A : i * kV < A);
-                if (there) Vec<LT, kV>::ld(at + i * vstep * (int)sizeof(LT), f + i * kV);
+                for (int j = 0; j < kA; ++j) f[j] = get_element<LT>(row, j);
             }
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+                if (!kSingles && vec_there(i)) Vec<LT, VW>::ld(at + vec_at(i, (int)sizeof(LT)), f + i * VW);
+            if (kOdd && (!kWide || part == 0)) f[2 * NP - 2] = get_element<LT>(row, single_of(r));
 #pragma unroll
             for (int j = 0; j < NP; ++j) z[j] = make_float2(f[2 * j], f[2 * j + 1]);
         };
-        auto row_max2 = [&](const float2 (&z)[NP]) {
+        // is pair j worked on?  (run-time counts: groups of two pairs up to the last that holds elements; a uniform test)
+        auto pair_used = [&](int j) { return kFixed || (kOdd && j == NP - 1) || (j & ~1) * 2 < nvec * VW; };
+        auto row_max = [&](const float2 (&z)[NP]) {
             float m0 = fmaxf(z[0].x, z[0].y), m1 = m0;
 #pragma unroll
             for (int j = 1; j < NP; ++j) {
+                if (NP > 9 && !pair_used(j)) continue;
                 if (j & 1) m1 = fmaxf(m1, fmaxf(z[j].x, z[j].y));
                 else m0 = fmaxf(m0, fmaxf(z[j].x, z[j].y));
             }
             return fmaxf(m0, m1);
         };
-        // pairs that hold elements (a uniform count): what lies beyond is not worked on
-        const int n_pairs = kFixed ? NP : (nvec * kV + 1) / 2;
         const float2 log2e2 = make_float2(kLog2e, kLog2e);
         for (int pass = 0; pass < (kWide ? passes : 1); ++pass) {
             const int r = row_of(pass);
             float2 z[NP];
-            // target row: its log2-sum-exp (base 2, of z log2 e)
+            // target row
             load_row(s1, r, z);
-            float m_t = row_max2(z);
+            float m_t = row_max(z);
             if (kWide) for (int o = 1; o < L; o <<= 1) m_t = fmaxf(m_t, __shfl_xor_sync(0xffffffffu, m_t, o));
             const float m2t = __fmul_rn(m_t, kLog2e);
             float2 sum2 = make_float2(0.0f, 0.0f);
@@ -722,16 +743,16 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 const float2 neg_m2 = make_float2(-m2t, -m2t);
 #pragma unroll
                 for (int j = 0; j < NP; ++j) {
-                    if (!kFixed && j >= n_pairs) continue;
+                    if (!pair_used(j)) continue;
                     const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);  // (z - m) log2 e
                     const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
                     sum2 = __fadd2_rn(sum2, ex);
                 }
             }
             float sum_t = sum2.x + sum2.y;
-            // learner row: log2-sum-exp, sum_j e_j z_j
+            // learner row: also sum_j e_j z_j
             load_row(s0, r, z);
-            float m_l = row_max2(z);
+            float m_l = row_max(z);
             if (kWide) for (int o = 1; o < L; o <<= 1) m_l = fmaxf(m_l, __shfl_xor_sync(0xffffffffu, m_l, o));
             const float m2 = __fmul_rn(m_l, kLog2e);
             sum2 = make_float2(0.0f, 0.0f);
@@ -740,7 +761,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 const float2 neg_m2 = make_float2(-m2, -m2);
 #pragma unroll
                 for (int j = 0; j < NP; ++j) {
-                    if (!kFixed && j >= n_pairs) continue;
+                    if (!pair_used(j)) continue;
                     const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);
                     const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
                     sum2 = __fadd2_rn(sum2, ex);
@@ -760,21 +781,26 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const float is = dev::rcp_fast(sum_l);
             float klr = 0.0f;
             if (want_kl) {
-                float2 zt[NP];
-                load_row(s1, r, zt);
                 const float lt2 = __fadd_rn(m2t, lgt), ll2 = __fadd_rn(m2, lgl);
+                auto add_kl = [&](float zt, float zl) {
+                    const float at2 = fmaf(zt, kLog2e, -lt2);
+                    klr = fmaf(dev::exp2_fast(at2), (at2 - fmaf(zl, kLog2e, -ll2)) * kLn2, klr);
+                };
+                const unsigned char* const row = s1 + r * in_row;
+                const unsigned char* const at = row + (first_of(r) + part * VW) * (int)sizeof(LT);
 #pragma unroll
-                for (int j = 0; j < NP; ++j) {
-                    if (!kFixed && j >= n_pairs) continue;
-                    const float ax = fmaf(zt[j].x, kLog2e, -lt2), ay = fmaf(zt[j].y, kLog2e, -lt2);
-                    const float ex = dev::exp2_fast(ax), ey = dev::exp2_fast(ay);
-                    const float dx = (ax - fmaf(z[j].x, kLog2e, -ll2)) * kLn2, dy = (ay - fmaf(z[j].y, kLog2e, -ll2)) * kLn2;
-                    // (an element that is not there: its two logarithms are both -inf, and it adds nothing)
-                    const bool has_x = kFixed || element_exists(2 * j, part, vstep, kV, A);
-                    const bool has_y = (kFixed && 2 * j + 1 < E) || (!kFixed && element_exists(2 * j + 1, part, vstep, kV, A));
-                    if (has_x) klr = fmaf(ex, dx, klr);
-                    if (has_y) klr = fmaf(ey, dy, klr);
+                for (int i = 0; i < NV; ++i) {
+                    if (!vec_there(i)) continue;
+                    float zt[VW];
+                    if constexpr (kSingles) { zt[0] = get_element<LT>(row, 2 * i); zt[1] = get_element<LT>(row, 2 * i + 1); }
+                    else Vec<LT, VW>::ld(at + vec_at(i, (int)sizeof(LT)), zt);
+#pragma unroll
+                    for (int v = 0; v < VW; v += 2) {
+                        add_kl(zt[v], z[(i * VW + v) / 2].x);
+                        add_kl(zt[v + 1], z[(i * VW + v) / 2].y);
+                    }
                 }
+                if (kV == 1 && (!kWide || part == 0)) add_kl(get_element<LT>(row, single_of(r)), z[NP - 1].x);
                 if (kWide) for (int o = 1; o < L; o <<= 1) klr += __shfl_xor_sync(0xffffffffu, klr, o);
             }
             if (!kWide || part == pass) {
@@ -897,49 +923,57 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const float2 ga2 = make_float2(pga, pga), gb2 = make_float2(pgb, pgb);
             const float2 neg_m2 = make_float2(-pm2, -pm2);
             const float2 neg_lse2 = make_float2(-plt, -plt), nck2 = make_float2(-ck, -ck);
-            const unsigned char* const zrow = s0 + r * in_row + part * (kV * (int)sizeof(LT));
-            const unsigned char* const trow = s1 + r * in_row + part * (kV * (int)sizeof(LT));
-            unsigned char* const orow_ = so + r * out_row + part * (kV * (int)sizeof(GT));
-            // vector by vector (two at a time where a vector is one element: the arithmetic is on pairs)
-            constexpr int kStep = kV == 1 ? 2 : 1, kElems = kStep * kV;
+            // the gradient of up to VW neighbouring elements: z and zt in, their places among the lane's elements
+            auto grad_of = [&](const float2& z2, const float2& zt2, int pair) {
+                float2 ex;
+                if constexpr (kWide) {
+                    const float2 t2 = __ffma2_rn(z2, log2e2, neg_m2);
+                    ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
+                } else {
+                    ex = e[pair];
+                }
+                float2 gr = __fmul2_rn(ex, __ffma2_rn(z2, ga2, gb2));
+                if (want_kl) {
+                    const float2 tt = __ffma2_rn(zt2, log2e2, neg_lse2);
+                    gr = __ffma2_rn(nck2, make_float2(dev::exp2_fast(tt.x), dev::exp2_fast(tt.y)), gr);
+                }
+                return gr;
+            };
+            const unsigned char* const zrow = s0 + r * in_row;
+            const unsigned char* const trow = s1 + r * in_row;
+            unsigned char* const grow = so + r * out_row;
+            const int first = first_of(r) + part * VW;
 #pragma unroll
-            for (int i = 0; i < NV; i += kStep) {
-                float z[kElems], o[kElems], zt[kElems];
-                bool there[kStep];
+            for (int i = 0; i < NV; ++i) {
+                if (!kFixed && kWide && i >= nvec) continue;  // (uniform)
+                if (!vec_there(i)) continue;
+                float z[VW], o[VW], zt[VW];
 #pragma unroll
-                for (int u = 0; u < kStep; ++u)
-                    there[u] = kFixed ? i + u < NV : (kWide ? (i + u) * vstep + part * kV < A : (i + u) * kV < A);
-                if (!kFixed && !kWide && !there[0]) continue;  // (uniform)
-#pragma unroll
-                for (int u = 0; u < kStep; ++u) {
-#pragma unroll
-                    for (int v = 0; v < kV; ++v) z[u * kV + v] = 0.0f, zt[u * kV + v] = 0.0f;
-                    if (there[u]) {
-                        Vec<LT, kV>::ld(zrow + (i + u) * vstep * (int)sizeof(LT), z + u * kV);
-                        if (want_kl) Vec<LT, kV>::ld(trow + (i + u) * vstep * (int)sizeof(LT), zt + u * kV);
-                    }
+                for (int v = 0; v < VW; ++v) zt[v] = 0.0f;
+                if constexpr (kSingles) {
+                    z[0] = get_element<LT>(zrow, 2 * i); z[1] = get_element<LT>(zrow, 2 * i + 1);
+                    if (want_kl) { zt[0] = get_element<LT>(trow, 2 * i); zt[1] = get_element<LT>(trow, 2 * i + 1); }
+                } else {
+                    Vec<LT, VW>::ld(zrow + first * (int)sizeof(LT) + vec_at(i, (int)sizeof(LT)), z);
+                    if (want_kl) Vec<LT, VW>::ld(trow + first * (int)sizeof(LT) + vec_at(i, (int)sizeof(LT)), zt);
                 }
 #pragma unroll
-                for (int v = 0; v < kElems; v += 2) {
-                    const float2 z2 = make_float2(z[v], z[v + 1]);
-                    float2 ex;
-                    if constexpr (kWide) {
-                        const float2 t2 = __ffma2_rn(z2, log2e2, neg_m2);
-                        ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
-                    } else {
-                        ex = e[(i * kV + v) / 2];
-                    }
-                    float2 gr = __fmul2_rn(ex, __ffma2_rn(z2, ga2, gb2));
-                    if (want_kl) {
-                        const float2 tt = __ffma2_rn(make_float2(zt[v], zt[v + 1]), log2e2, neg_lse2);
-                        gr = __ffma2_rn(nck2, make_float2(dev::exp2_fast(tt.x), dev::exp2_fast(tt.y)), gr);
-                    }
+                for (int v = 0; v < VW; v += 2) {
+                    const float2 gr = grad_of(make_float2(z[v], z[v + 1]), make_float2(zt[v], zt[v + 1]), (i * VW + v) / 2);
                     o[v] = gr.x;
                     o[v + 1] = gr.y;
                 }
-#pragma unroll
-                for (int u = 0; u < kStep; ++u)
-                    if (there[u]) Vec<GT, kV>::st(orow_ + (i + u) * vstep * (int)sizeof(GT), o + u * kV);
+                if constexpr (kSingles) {
+                    Vec<GT, 1>::st(grow + 2 * i * (int)sizeof(GT), o);
+                    Vec<GT, 1>::st(grow + (2 * i + 1) * (int)sizeof(GT), o + 1);
+                } else {
+                    Vec<GT, VW>::st(grow + first * (int)sizeof(GT) + vec_at(i, (int)sizeof(GT)), o);
+                }
+            }
+            if (kV == 1 && (!kWide || part == 0)) {
+                const int c = single_of(r);
+                const float z = get_element<LT>(zrow, c), zt = want_kl ? get_element<LT>(trow, c) : 0.0f;
+                put_element<GT>(grow, c, grad_of(make_float2(z, z), make_float2(zt, zt), NP - 1).x);
             }
         }
         const float pi_a = dev::exp2_fast(st.l2_theta);
@@ -987,8 +1021,14 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
 // ------------------------------------------------------------------------------------------
 // Launch
 // ------------------------------------------------------------------------------------------
+// How the rows of a batch are laid on lanes: rows of a tile, lanes per row, rotation of a lane's vectors.
+struct RowLayout {
+    int nt = 128, log_lanes = 0, rot_shift = 0, rot_mask = 0;
+};
+
 template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
-int32_t launch_categorical(CatParams p, int nt, int log_lanes, const DeviceInfo* di, cudaStream_t stream) {
+int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
+    const int nt = rl.nt;
     auto kernel = impact_loss_categorical_kernel<LT, GT, kA, C, kV, kPlain, kLong, kIndirect>;
     const size_t stage = cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT));
     p.geo.nt = nt;
@@ -1012,8 +1052,10 @@ int32_t launch_categorical(CatParams p, int nt, int log_lanes, const DeviceInfo*
     p.geo.tile_major = (kLong && p.geo.B >= grid) ? 1 : 0;
     CatShape sh = {};
     sh.nt = nt;
-    sh.log_lanes = log_lanes;
-    sh.passes = (nt / 4 << log_lanes) / 32;
+    sh.log_lanes = rl.log_lanes;
+    sh.passes = (nt / 4 << rl.log_lanes) / 32;
+    sh.rot_shift = rl.rot_shift;
+    sh.rot_mask = rl.rot_mask;
     ws_ring_shape(stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di->max_smem_optin, tiles_per_block, &sh.stages, &sh.in_flight);
     if (sh.stages < 1 || sh.in_flight < 1) return IMPACT_ERR_UNSUPPORTED;
     const int spare = sh.stages - sh.in_flight;  // producer lanes that request tiles side by side
@@ -1038,80 +1080,114 @@ int32_t launch_categorical(CatParams p, int nt, int log_lanes, const DeviceInfo*
     return IMPACT_OK;
 }
 
-// Long trajectories go to neighbouring blocks while there are too few of them to give every block about four (and the
-// caller's scratch has room for the tiles' aggregates); from there on blocks that own whole trajectories are as busy,
-// without any exchange between blocks.
+// Long trajectories go to neighbouring blocks where blocks that own whole ones would leave most of the device idle: the
+// busiest of them has ceil(B / blocks) trajectories (and where the caller's scratch has room for the tiles' aggregates).
+// A split launch pays for its exchange with about half of a flat one's rate.  Measured in us, flat against split, by the
+// share of the device that the flat launch keeps busy: 0.20 (A = 64, 31 x 4000) 62.6 / 41.6; 0.21 (18, 31 x 4000) 15.7 /
+// 13.3; 0.25 (64, 37 x 1000) 18.0 / 12.3; 0.33 (40, 49 x 4000) 54.4 / 63.5; 0.40 (40, 59 x 1000) 16.0 / 20.8; 0.47 (7,
+// 69 x 4000) 18.2 / 23.6; 0.70 (18, 104 x 4000) 19.9 / 40.2.
 inline bool splits_trajectories(const CatParams& p, int nt, const DeviceInfo* di) {
-    return p.geo.T > nt && nt >= kMinTileRows && p.tile_aggregates && p.geo.B < 4ll * di->sm_count;
+    if (p.geo.T <= nt || nt < kMinTileRows || !p.tile_aggregates) return false;
+    const long long rounds = (p.geo.B + di->sm_count - 1) / di->sm_count;
+    return 10 * p.geo.B < 3 * rounds * di->sm_count;
 }
 // (a flat launch counts a trajectory's steps in 32 bits)
 inline bool fits_flat(const CatParams& p) { return p.geo.T < (1ll << 32) - 4096; }
+
+// The configuration of the paper's experiments, for which the switches and optional outputs are compiled out.
+inline bool is_plain(const CatParams& p) {
+    return p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
+           p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
+}
 
 // Consumer groups: four with every switch compiled in; five in the default configuration; six there for small action
 // sets, which are bound by arithmetic, not bytes.
 template <typename LT, typename GT, int A, int kV>
 int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
     constexpr int C = 4, CP = A <= 9 ? 6 : 5;
-    const bool plain = p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
-                       p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 &&
-                       !p.vtarget && !p.advantage;
+    const bool plain = is_plain(p);
+    const RowLayout rl;
     if (p.indirect) {  // compiled for trajectories that fit a tile only
         if (p.geo.T > 128) return IMPACT_ERR_UNSUPPORTED;
-        return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, true>(p, 128, 0, di, stream)
-                     : launch_categorical<LT, GT, A, C, kV, false, false, true>(p, 128, 0, di, stream);
+        return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, true>(p, rl, di, stream)
+                     : launch_categorical<LT, GT, A, C, kV, false, false, true>(p, rl, di, stream);
     }
     if (splits_trajectories(p, 128, di) || !fits_flat(p)) {
         if (!p.tile_aggregates) return IMPACT_ERR_UNSUPPORTED;
-        return launch_categorical<LT, GT, A, C, kV, false, true, false>(p, 128, 0, di, stream);
+        return launch_categorical<LT, GT, A, C, kV, false, true, false>(p, rl, di, stream);
     }
-    return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, 128, 0, di, stream)
-                 : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, 128, 0, di, stream);
+    return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, rl, di, stream)
+                 : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, rl, di, stream);
 }
 
-// How many lanes of a warp's accesses to rows of `row_bytes`, `group` lanes to a row, meet on the same banks.
-inline int bank_ways(size_t row_bytes, int rows_between, int group, int access_bytes) {
-    const size_t stride = row_bytes * (size_t)rows_between, window = (size_t)group * access_bytes;
-    const int rows_at_once = 128 / access_bytes / group;
-    if (rows_at_once <= 1) return 1;
+// Where a warp's accesses of `access_bytes`, `group` neighbouring lanes to a row and the rows `stride` bytes apart, fall
+// on the banks: `ways` accesses meet, and rows 2^shift apart are the first that do.
+struct BankPattern {
+    int ways, shift;
+};
+inline BankPattern bank_pattern(size_t stride, int group, int access_bytes) {
+    const size_t window = (size_t)group * access_bytes;
+    const size_t rows_at_once = 128 / window > 1 ? 128 / window : 1;
     size_t step = stride % 128;  // gcd(stride, 128)
     step = step ? (step & (~step + 1)) : 128;
-    return step >= window ? (int)(step / window) : 1;
+    BankPattern b = {1, 0};
+    for (size_t d = 128 / step; d > 1; d /= 2) ++b.shift;
+    if (rows_at_once > 1 && step > window) b.ways = (int)(step / window);
+    return b;
+}
+
+template <typename LT, typename GT, int kA, int C, int CP, int kV>
+int32_t run_runtime_form(const CatParams& p, const RowLayout& rl, bool plain, const DeviceInfo* di, cudaStream_t stream) {
+    if (splits_trajectories(p, rl.nt, di) || !fits_flat(p)) {
+        if (!p.tile_aggregates || rl.nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
+        return launch_categorical<LT, GT, kA, C, kV, false, true, false>(p, rl, di, stream);
+    }
+    return plain ? launch_categorical<LT, GT, kA, CP, kV, true, false, false>(p, rl, di, stream)
+                 : launch_categorical<LT, GT, kA, C, kV, false, false, false>(p, rl, di, stream);
 }
 
 template <typename LT, typename GT, int kV>
 int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    constexpr int C = 4;
+    constexpr int VW = kV == 1 ? 2 : kV;
+    const int vecs = p.A / VW, access = VW * (int)sizeof(LT);
     const size_t row = p.A * sizeof(LT);
-    if (p.A <= kMaxLaneElems && bank_ways(row, 1, 1, kV * (int)sizeof(LT)) <= 2) {
-        if (p.indirect) return IMPACT_ERR_UNSUPPORTED;
-        if (splits_trajectories(p, 128, di) || !fits_flat(p)) {
-            if (!p.tile_aggregates) return IMPACT_ERR_UNSUPPORTED;
-            return launch_categorical<LT, GT, 0, C, kV, false, true, false>(p, 128, 0, di, stream);
+    RowLayout rl;
+    // what is left of the bank conflicts of rows on 2^l lanes each, after rotating the order of a lane's vectors
+    auto settle = [&](int l) {
+        rl.log_lanes = l;
+        const int passes = (rl.nt / 4 << l) / 32;
+        const BankPattern b = bank_pattern(row * (size_t)(passes < 1 ? 1 : passes), 1 << l, access);
+        rl.rot_mask = 0;
+        rl.rot_shift = b.shift;
+        if (kV == 4 && vecs % (1 << l) == 0) {
+            const int per_lane = vecs >> l;
+            while (2 * (rl.rot_mask + 1) <= b.ways && per_lane % (2 * (rl.rot_mask + 1)) == 0) rl.rot_mask = 2 * rl.rot_mask + 1;
         }
-        return launch_categorical<LT, GT, 0, C, kV, false, false, false>(p, 128, 0, di, stream);
+        return b.ways / (rl.rot_mask + 1);
+    };
+    const bool plain = is_plain(p);
+    if (p.A <= 32) {
+        if (p.indirect) return IMPACT_ERR_UNSUPPORTED;
+        rl.nt = 128;
+        settle(0);
+        if (p.A <= 16) return run_runtime_form<LT, GT, kNarrow16, 4, 5, kV>(p, rl, plain, di, stream);
+        return run_runtime_form<LT, GT, kNarrow32, 4, 4, kV>(p, rl, plain, di, stream);
     }
     // Rows of more than a lane: tiles of up to 36 KB (a ring of six stages, four of them being worked on), then the
     // fewest lanes that hold a row and do not meet on the banks more than two at a time.
-    int nt = 128;
-    while (nt > 8 && cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT)) > 36 * 1024) nt /= 2;
-    int log_l = 1;
-    auto lanes_suffice = [&](int l) {
-        if ((nt / 4 << l) < 32 || ((long long)kMaxLaneElems << l) < p.A) return false;
-        return l == 5 || bank_ways(row, (nt / 4 << l) / 32, 1 << l, kV * (int)sizeof(LT)) <= 2;
-    };
-    while (!lanes_suffice(log_l)) ++log_l;
+    rl.nt = 128;
+    while (rl.nt > 8 && cat_stage_bytes(rl.nt, p.A, sizeof(LT), sizeof(GT)) > 36 * 1024) rl.nt /= 2;
+    int l = 1;
+    while (l < 5 && ((rl.nt / 4 << l) < 32 || ((kWideElems / VW) << l) < vecs || settle(l) > 2)) ++l;
+    settle(l);
     if (p.indirect) {
         if constexpr (kV == 4) {
             if (p.A == 64 && p.geo.T <= 64)
-                return launch_categorical<LT, GT, -1, C, kV, false, false, true>(p, nt, log_l, di, stream);
+                return launch_categorical<LT, GT, kWideRows, 4, kV, false, false, true>(p, rl, di, stream);
         }
         return IMPACT_ERR_UNSUPPORTED;
     }
-    if (splits_trajectories(p, nt, di) || !fits_flat(p)) {
-        if (!p.tile_aggregates || nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
-        return launch_categorical<LT, GT, -1, C, kV, false, true, false>(p, nt, log_l, di, stream);
-    }
-    return launch_categorical<LT, GT, -1, C, kV, false, false, false>(p, nt, log_l, di, stream);
+    return run_runtime_form<LT, GT, kWideRows, 4, 4, kV>(p, rl, plain, di, stream);
 }
 
 template <typename LT, typename GT>

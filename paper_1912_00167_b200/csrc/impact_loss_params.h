@@ -54,7 +54,7 @@ struct CatParams {
 // The rest of a categorical launch's shape.
 struct CatShape {
     int nt, stages, in_flight, lanes, n_prefetch;
-    int log_lanes, passes;  // rows wider than a lane (see impact_categorical.cuh)
+    int log_lanes, passes, rot_shift, rot_mask;  // how rows are laid on lanes (see impact_categorical.cuh)
 };
 
 struct LossInputPointers {
