@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 
 import torch
@@ -78,13 +79,25 @@ class impact_loss_inputs(ctypes.Structure):
                [(n, ctypes.c_int32) for n in ("status", "slot", "k_before", "pad")]
 
 
+def _pack_format(cls) -> str:
+    """The struct-module format of a ctypes structure (native alignment; a nested structure starts on its own)."""
+    codes = {ctypes.c_void_p: "P", ctypes.c_float: "f", ctypes.c_int32: "i", ctypes.c_int64: "q", ctypes.c_size_t: "N"}
+    align = "0q" if ctypes.alignment(cls) == 8 else ""
+    return align + "".join(codes[t] if t in codes else _pack_format(t) for _, t in cls._fields_) + align
+
+
+# impact_loss_call as bytes in one go: filling the ctypes structure field by field costs a call 4 us, this 1 us
+_CALL = struct.Struct("@" + _pack_format(impact_loss_call))
+assert _CALL.size == ctypes.sizeof(impact_loss_call)
+
 _lib = None
+_call_packed = None
 _vp, _i32, _i64, _f32, _sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_float, ctypes.c_size_t
 
 
 def load_library() -> ctypes.CDLL:
     """Loads libimpact.so; raises if it has not been built (there is no other code path)."""
-    global _lib
+    global _lib, _call_packed
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -152,6 +165,10 @@ def load_library() -> ctypes.CDLL:
     lib.impact_set_option.argtypes = [_i32, _i64]
     lib.impact_get_option.restype = _i64
     lib.impact_get_option.argtypes = [_i32]
+    # the same entry point by a function object of its own that takes the structure as bytes
+    _call_packed = lib["impact_loss_fwd_bwd_call"]
+    _call_packed.restype = _i32
+    _call_packed.argtypes = [ctypes.c_char_p, _vp]
     _lib = lib
     return lib
 
@@ -195,8 +212,14 @@ def _dev(t: torch.Tensor | None, dtype, shape, name: str, optional: bool = False
     return t.data_ptr()
 
 
+# (the stream's handle without the Python object around it, where this torch has that: 0.1 us instead of 0.7)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -253,24 +276,27 @@ _TORCH_DTYPE = {DTYPE_F32: torch.float32, DTYPE_BF16: torch.bfloat16}
 _DTYPE_CODE = {torch.float32: DTYPE_F32, torch.bfloat16: DTYPE_BF16}
 
 
+_SIMPLE = (_vp, _i32, _i64, _f32, _sz)
+
+
 class PreparedCall:
     """A C call with its arguments marshalled once; `()` re-issues it on the given stream.  `keep` holds whatever
     the marshalled pointers point into (the C structs and every tensor of the call), so that the call can be
     re-issued for as long as it exists."""
 
     def __init__(self, fn, args, what, keep):
-        self._fn, self._args, self._what, self._keep = fn, list(args), what, keep
+        # every argument but the last, the stream, as the ctypes object that it is converted to anyway
+        conv = [a if a is None or t not in _SIMPLE or isinstance(a, t) else t(a) for a, t in zip(args, fn.argtypes)]
+        self._fn, self._args, self._what, self._keep = fn, tuple(conv[:-1]), what, keep
 
     def __call__(self, stream=None) -> None:
-        self._args[-1] = _stream(stream)
-        st = self._fn(*self._args)
+        st = self._fn(*self._args, _stream(stream))
         if st != OK:
             _check(st, self._what)
 
     def on_stream(self, cuda_stream: int) -> None:
         """Same as `()`, for a raw cudaStream_t value (skips the torch stream lookup)."""
-        self._args[-1] = cuda_stream
-        st = self._fn(*self._args)
+        st = self._fn(*self._args, cuda_stream)
         if st != OK:
             _check(st, self._what)
 
@@ -329,10 +355,47 @@ def prepare_loss_fwd_bwd_from_record(record: torch.Tensor, B: int, T: int, A: in
                         (call, record, loss_terms, dlogits, dvalues, vtarget, advantage, workspace))
 
 
+def _fits(t, dtype, shape) -> bool:
+    """What _dev checks, as one expression (it also tells what is wrong)."""
+    return t.dtype is dtype and t.is_cuda and t.shape == shape and t.is_contiguous()
+
+
 def impact_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values,
                         bootstrap_values, coef: Coefficients, *, loss_terms, dlogits, dvalues,
                         vtarget=None, advantage=None, workspace, target_logits_copy=None, stream=None) -> None:
     """Enqueues the categorical IMPACT loss + gradients on `stream` (see include/impact.h)."""
+    # The usual call: every argument as it should be, checked in a row and packed at once.  Anything else goes the way
+    # of a prepared call, which names the argument at fault.
+    try:
+        shape = learner_logits.shape
+        B, T, A = shape
+        bt, f32, ldt, gdt = (B, T), torch.float32, learner_logits.dtype, dlogits.dtype
+        usual = (_fits(learner_logits, ldt, shape) and _fits(target_logits, ldt, shape) and _fits(worker_logp, f32, bt)
+                 and _fits(actions, torch.int32, bt) and _fits(rewards, f32, bt) and _fits(discounts, f32, bt)
+                 and _fits(values, f32, bt) and _fits(bootstrap_values, f32, (B,)) and _fits(loss_terms, f32, (NUM_TERMS,))
+                 and _fits(dlogits, gdt, shape) and _fits(dvalues, f32, bt)
+                 and (vtarget is None or _fits(vtarget, f32, bt)) and (advantage is None or _fits(advantage, f32, bt))
+                 and workspace.dtype is torch.uint8 and workspace.is_cuda and workspace.is_contiguous()
+                 and (target_logits_copy is None or _fits(target_logits_copy, ldt, shape)))
+        packed = _CALL.pack(
+            learner_logits.data_ptr(), target_logits.data_ptr(), worker_logp.data_ptr(), actions.data_ptr(),
+            rewards.data_ptr(), discounts.data_ptr(), values.data_ptr(), bootstrap_values.data_ptr(),
+            coef.rho_bar, coef.c_bar, coef.clip_eps, _DTYPE_CODE[ldt],
+            coef.vf_coef, coef.ent_coef, coef.kl_coef, coef.lam, coef.rho_tw, coef.is_source, coef.ratio_mode,
+            _DTYPE_CODE[gdt], coef.objective, coef.global_steps, A, B, T,
+            loss_terms.data_ptr(), dlogits.data_ptr(), dvalues.data_ptr(),
+            0 if vtarget is None else vtarget.data_ptr(), 0 if advantage is None else advantage.data_ptr(),
+            workspace.data_ptr(), workspace.numel(),
+            0 if target_logits_copy is None else target_logits_copy.data_ptr(), 0) if usual else None
+    except (AttributeError, KeyError, TypeError, ValueError, OverflowError, struct.error):
+        packed = None
+    if packed is not None:
+        if _lib is None:
+            load_library()
+        st = _call_packed(packed, _stream(stream))
+        if st != OK:
+            _check(st, "impact_loss_fwd_bwd_call")
+        return
     prepare_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values,
                          bootstrap_values, coef, loss_terms=loss_terms, dlogits=dlogits, dvalues=dvalues,
                          vtarget=vtarget, advantage=advantage, workspace=workspace,
@@ -457,6 +520,12 @@ class ImpactBuffer:
         self._h = h
         self._slot = _i32(-1)
         self._k = _i32(-1)
+        self._slot_ref, self._k_ref = ctypes.byref(self._slot), ctypes.byref(self._k)
+        # where the library puts a slot's fields, and the storage seen as other types (slot_view)
+        if storage is not None:
+            self._field_at = [self.slot_ptr(0, f) - storage.data_ptr() for f in range(self.n_fields)]
+            self._slot_bytes = self.slot_ptr(1, 0) - self.slot_ptr(0, 0) if N > 1 else 0
+            self._typed = {}
 
     @staticmethod
     def storage_bytes(N: int, field_bytes) -> int:
@@ -471,7 +540,7 @@ class ImpactBuffer:
             if t is None:
                 arr[f] = None
                 continue
-            nbytes = t.numel() * t.element_size()
+            nbytes = t.nbytes
             if nbytes != self.field_bytes[f] or not t.is_contiguous():
                 raise ValueError(f"field {f}: expected {self.field_bytes[f]} dense bytes, got {nbytes}")
             arr[f] = t.data_ptr()
@@ -483,7 +552,7 @@ class ImpactBuffer:
         if any(host) and not all(host):
             raise ValueError("push sources must be all on the device or all on the host")
         loc = SRC_DEVICE if (not host or host[0]) else SRC_HOST
-        st = self._lib.impact_buffer_push(self._h, self._ptr_array(fields), loc, ctypes.byref(self._slot),
+        st = self._lib.impact_buffer_push(self._h, self._ptr_array(fields), loc, self._slot_ref,
                                           _stream(stream))
         if _check(st, "impact_buffer_push", allow=(ERR_FULL,)) == ERR_FULL:
             return None
@@ -496,7 +565,7 @@ class ImpactBuffer:
             if not all(t is None or t.is_cuda for t in gather_dst):
                 raise ValueError("gather destinations must be CUDA tensors")
             arr = self._ptr_array(gather_dst)
-        st = self._lib.impact_buffer_sample(self._h, ctypes.byref(self._slot), ctypes.byref(self._k), arr,
+        st = self._lib.impact_buffer_sample(self._h, self._slot_ref, self._k_ref, arr,
                                             _stream(stream))
         if _check(st, "impact_buffer_sample", allow=(ERR_EMPTY,)) == ERR_EMPTY:
             return None
@@ -518,6 +587,18 @@ class ImpactBuffer:
         """Zero-copy tensor over one field of a slot (needs torch-owned storage)."""
         if self._storage is None:
             raise ValueError("slot_view needs torch-owned storage")
+        # one view instead of three where the shape fills the field exactly, dense and in whole elements
+        if 0 <= slot < self.N and 0 <= field < self.n_fields and type(shape) in (tuple, torch.Size):
+            size, n, strides = dtype.itemsize, 1, []
+            for d in reversed(shape):
+                strides.append(n)
+                n *= d
+            off = slot * self._slot_bytes + self._field_at[field]
+            if n * size == self.field_bytes[field] and min(shape, default=1) > 0 and self._storage.dtype is torch.uint8:
+                typed = self._typed.get(dtype)
+                if typed is None:
+                    typed = self._typed[dtype] = self._storage[:self._storage.numel() // size * size].view(dtype)
+                return typed.as_strided(shape, strides[::-1], typed.storage_offset() + off // size)
         off = self.slot_ptr(slot, field) - self._storage.data_ptr()
         n = self.field_bytes[field]
         return self._storage[off:off + n].view(dtype).view(*shape)

@@ -85,3 +85,29 @@ def test_ring_bookkeeping_runs_on_caller_storage_without_a_gpu(lib, oracle):
         if st == 0:
             assert (slot.value, k.value) == (rslot, rk)
     assert lib.impact_buffer_destroy(h) == 0
+
+
+def test_a_call_packed_as_bytes_is_the_structure(lib):
+    """The direct call packs impact_loss_call in one go: the bytes are those of the ctypes structure, field by field."""
+    from paper_1912_00167_b200 import binding as b
+    head = [11 * (i + 1) for i in range(8)] + [1.5, 2.5, 3.5, 1]
+    coef = [0.5, 0.25, 0.125, 4.0, 5.0, 1, 2, 1, 0, 12345678901]
+    tail = [7, 8, 9, 1001, 1002, 1003, 0, 1005, 1006, 777, 0, 0]
+    want = bytes(b.impact_loss_call(*head, b.impact_coefficients(*coef), *tail))
+    assert b._CALL.pack(*head, *coef, *tail) == want
+    assert b._call_packed(want, None) == -1  # it reaches the library, which refuses the unaligned addresses
+
+
+def test_the_direct_call_names_the_argument_at_fault(lib):
+    """Arguments that the quick check turns away get the ordinary check's error."""
+    import torch
+    from paper_1912_00167_b200 import binding as b
+    f = lambda *s: torch.zeros(*s)  # (CPU tensors: there is no CPU path)
+    with pytest.raises(ValueError, match="learner_logits must be a CUDA tensor"):
+        b.impact_loss_fwd_bwd(f(2, 3, 4), f(2, 3, 4), f(2, 3), f(2, 3).int(), f(2, 3), f(2, 3), f(2, 3), f(2),
+                              b.Coefficients(), loss_terms=f(8), dlogits=f(2, 3, 4), dvalues=f(2, 3),
+                              workspace=torch.zeros(10, dtype=torch.uint8))
+    with pytest.raises(ValueError, match="logits must be float32 or bfloat16"):
+        b.impact_loss_fwd_bwd(f(2, 3, 4).double(), f(2, 3, 4), f(2, 3), f(2, 3).int(), f(2, 3), f(2, 3), f(2, 3), f(2),
+                              b.Coefficients(), loss_terms=f(8), dlogits=f(2, 3, 4), dvalues=f(2, 3),
+                              workspace=torch.zeros(10, dtype=torch.uint8))
