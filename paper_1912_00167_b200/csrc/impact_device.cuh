@@ -269,248 +269,6 @@ __device__ __forceinline__ float warp_sum4(float a, float b, float c, float d) {
     return x;
 }
 
-// Walks (row, col) positions of a dense [rows, W] slab in steps of a fixed element count.
-struct RowCol {
-    int r, c;
-    __device__ __forceinline__ void init(int e, int W) { r = e / W; c = e - r * W; }
-    __device__ __forceinline__ void advance(int dq, int dr, int W) {
-        r += dq; c += dr;
-        if (c >= W) { c -= W; ++r; }
-    }
-};
-
-// Stage `nelem` consecutive elements of `src`, starting at element `base`, into shared
-// rows of stride `Ws` floats (element e of the slab lands at [e / W][e % W]).
-template <typename ST, int NT>
-__device__ __forceinline__ void stage_slab(float* __restrict__ dst, const ST* __restrict__ src,
-                                           long long base, int nelem, int W, int Ws) {
-    constexpr int VE = Pack<ST>::kElems;
-    const int tid = threadIdx.x;
-    int done = 0;
-    if ((base % VE) == 0) {
-        const int nvec = nelem / VE;
-        const uint4* s4 = reinterpret_cast<const uint4*>(src + base);
-        const int dq = (NT * VE) / W, dr = (NT * VE) % W;
-        RowCol rc; rc.init(tid * VE, W);
-        int v = tid;
-        constexpr int U = 4;
-        for (; v + (U - 1) * NT < nvec; v += U * NT) {
-            uint4 x[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) x[u] = ld_stream16(s4 + v + u * NT);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float f[VE];
-                Pack<ST>::unpack(x[u], f);
-                int rr = rc.r, cc = rc.c;
-#pragma unroll
-                for (int j = 0; j < VE; ++j) {
-                    dst[rr * Ws + cc] = f[j];
-                    if (++cc == W) { cc = 0; ++rr; }
-                }
-                rc.advance(dq, dr, W);
-            }
-        }
-        for (; v < nvec; v += NT) {
-            uint4 x = ld_stream16(s4 + v);
-            float f[VE];
-            Pack<ST>::unpack(x, f);
-            int rr = rc.r, cc = rc.c;
-#pragma unroll
-            for (int j = 0; j < VE; ++j) {
-                dst[rr * Ws + cc] = f[j];
-                if (++cc == W) { cc = 0; ++rr; }
-            }
-            rc.advance(dq, dr, W);
-        }
-        done = nvec * VE;
-    }
-    if (done + tid < nelem) {  // unaligned slab, or the last few elements of an aligned one
-        const int dq = NT / W, dr = NT % W;
-        RowCol rc; rc.init(done + tid, W);
-        for (int e = done + tid; e < nelem; e += NT) {
-            dst[rc.r * Ws + rc.c] = Pack<ST>::to_float(src[base + e]);
-            rc.advance(dq, dr, W);
-        }
-    }
-}
-
-// The reverse of stage_slab: write the shared rows back to a dense global slab.
-template <typename ST, int NT>
-__device__ __forceinline__ void unstage_slab(ST* __restrict__ dst, const float* __restrict__ src,
-                                             long long base, int nelem, int W, int Ws) {
-    constexpr int VE = Pack<ST>::kElems;
-    const int tid = threadIdx.x;
-    int done = 0;
-    if ((base % VE) == 0) {
-        const int nvec = nelem / VE;
-        uint4* d4 = reinterpret_cast<uint4*>(dst + base);
-        const int dq = (NT * VE) / W, dr = (NT * VE) % W;
-        RowCol rc; rc.init(tid * VE, W);
-        for (int v = tid; v < nvec; v += NT) {
-            float f[VE];
-            int rr = rc.r, cc = rc.c;
-#pragma unroll
-            for (int j = 0; j < VE; ++j) {
-                f[j] = src[rr * Ws + cc];
-                if (++cc == W) { cc = 0; ++rr; }
-            }
-            st_stream16(d4 + v, Pack<ST>::pack(f));
-            rc.advance(dq, dr, W);
-        }
-        done = nvec * VE;
-    }
-    if (done + tid < nelem) {
-        const int dq = NT / W, dr = NT % W;
-        RowCol rc; rc.init(done + tid, W);
-        for (int e = done + tid; e < nelem; e += NT) {
-            dst[base + e] = Pack<ST>::from_float(src[rc.r * Ws + rc.c]);
-            rc.advance(dq, dr, W);
-        }
-    }
-}
-
-// ---- backward recursion as a suffix scan of affine maps ----------------------------------
-// Each thread i holds the map f_i(x) = a*x + b of its time step
-// (A_i = delta_i + (lambda gamma_i c_i) A_{i+1}).  Returns A_i = f_i(f_{i+1}(... f_{NT-1}(carry))).
-// Affine maps compose associatively, so the recursion is a scan: shuffles inside a warp,
-// one shared-memory hop across warps.  Contains one __syncthreads().
-// `next` receives A_{i+1}, the value the thread's own map was applied to (the carry for the last row).
-template <int NT>
-__device__ __forceinline__ float suffix_affine_scan(float a, float b, float carry, float2* warp_agg, float& next) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float a2 = __shfl_down_sync(0xffffffffu, a, off);
-        const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-        if (lane + off < 32) {
-            b = fmaf(a, b2, b);
-            a = a * a2;
-        }
-    }
-    if (lane == 0) warp_agg[warp] = make_float2(a, b);
-    __syncthreads();
-    float x = carry;
-#pragma unroll 1
-    for (int w = NT / 32 - 1; w > warp; --w) {
-        const float2 g = warp_agg[w];
-        x = fmaf(g.x, x, g.y);
-    }
-    const float result = fmaf(a, x, b);
-    const float below = __shfl_down_sync(0xffffffffu, result, 1);
-    next = (lane == 31) ? x : below;
-    return result;
-}
-
-// The same scan inside a group of NT threads that synchronises on named barrier `bar_id`
-// (trajectories never continue past a tile here, so there is no carry).
-template <int NT>
-__device__ __forceinline__ float suffix_affine_scan_group(float a, float b, float2* warp_agg, float& next, int bar_id) {
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (NT - 1)) >> 5;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float a2 = __shfl_down_sync(0xffffffffu, a, off);
-        const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-        if (lane + off < 32) {
-            b = fmaf(a, b2, b);
-            a = a * a2;
-        }
-    }
-    if (lane == 0) warp_agg[warp] = make_float2(a, b);
-    asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(NT) : "memory");
-    float x = 0.0f;
-#pragma unroll
-    for (int w = NT / 32 - 1; w > 0; --w) {
-        const float2 g = warp_agg[w];
-        if (w > warp) x = fmaf(g.x, x, g.y);
-    }
-    const float result = fmaf(a, x, b);
-    const float below = __shfl_down_sync(0xffffffffu, result, 1);
-    next = (lane == 31) ? x : below;
-    return result;
-}
-
-// The same scan with R rows per thread: a group of NTH threads covers NTH * R consecutive steps, warp w the steps
-// [32 R w, 32 R (w + 1)), lane l of it the steps 32 R w + 32 i + l for i < R (a lane's rows are 32 apart, which
-// keeps its accesses to rows of shared memory on the banks a single row per lane would use).  a[i], b[i] are the
-// rows' maps; res[i] receives A of row i, next[i] the value row i's map was applied to (0 after the last step).
-template <int NTH, int R>
-__device__ __forceinline__ void suffix_affine_scan_rows(float (&a)[R], float (&b)[R], float2* warp_agg, float (&res)[R],
-                                                        float (&next)[R], int bar_id) {
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (NTH - 1)) >> 5;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float a2 = __shfl_down_sync(0xffffffffu, a[i], off);
-            const float b2 = __shfl_down_sync(0xffffffffu, b[i], off);
-            if (lane + off < 32) {
-                b[i] = fmaf(a[i], b2, b[i]);
-                a[i] = a[i] * a2;
-            }
-        }
-    }
-    // inside the warp: the maps of the later sub-segments follow those of the earlier ones
-#pragma unroll
-    for (int i = R - 2; i >= 0; --i) {
-        const float ta = __shfl_sync(0xffffffffu, a[i + 1], 0), tb = __shfl_sync(0xffffffffu, b[i + 1], 0);
-        b[i] = fmaf(a[i], tb, b[i]);
-        a[i] = a[i] * ta;
-    }
-    float x = 0.0f;
-    if constexpr (NTH > 32) {
-        if (lane == 0) warp_agg[warp] = make_float2(a[0], b[0]);
-        asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(NTH) : "memory");
-#pragma unroll
-        for (int w = NTH / 32 - 1; w > 0; --w) {
-            const float2 g = warp_agg[w];
-            if (w > warp) x = fmaf(g.x, x, g.y);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < R; ++i) res[i] = fmaf(a[i], x, b[i]);
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const float below = __shfl_down_sync(0xffffffffu, res[i], 1);
-        float first_after = x;  // what follows this sub-segment's last row
-        if (i + 1 < R) first_after = __shfl_sync(0xffffffffu, res[i + 1], 0);
-        next[i] = (lane == 31) ? first_after : below;
-    }
-}
-
-// The scan as maps, for tiles that do not know yet what enters their last step: (ma, mb) is the
-// composition of the maps of this thread's step and all later steps of the tile, (la, lb) that of
-// all steps after this thread's warp (the identity for the last warp).  Thread 0's (ma, mb) is the
-// tile's aggregate.
-template <int NT>
-__device__ __forceinline__ void suffix_affine_maps_group(float a, float b, float2* warp_agg, float& ma, float& mb,
-                                                         float& la, float& lb, int bar_id) {
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (NT - 1)) >> 5;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float a2 = __shfl_down_sync(0xffffffffu, a, off);
-        const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-        if (lane + off < 32) {
-            b = fmaf(a, b2, b);
-            a = a * a2;
-        }
-    }
-    if (lane == 0) warp_agg[warp] = make_float2(a, b);
-    asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(NT) : "memory");
-    la = 1.0f;
-    lb = 0.0f;
-#pragma unroll
-    for (int w = NT / 32 - 1; w > 0; --w) {
-        const float2 g = warp_agg[w];
-        if (w > warp) {  // (la, lb) <- g o (la, lb)
-            lb = fmaf(g.x, lb, g.y);
-            la = g.x * la;
-        }
-    }
-    ma = a * la;
-    mb = fmaf(a, lb, b);
-}
-
 __device__ __forceinline__ void publish_tagged(unsigned long long* slot, float value, unsigned int tag);
 
 // A tile's aggregate map, published as two (value, launch tag) pairs (see publish_tagged).
@@ -591,233 +349,53 @@ struct StepIn {
     float adv_next = 0.0f;  // A_{t+1} (set from the scan)
 };
 
-// Truncated importance weights and the affine map of the advantage recursion
-// (Section 2.2; Section 3.1).  Returns whether exp(x) exceeded rho_bar.
 // exp of a log-probability difference.  Arguments are a few units at most, where the
 // multiply-then-exp2 form stays within ~3e-7 relative of the correctly rounded result.
 __device__ __forceinline__ float exp_of_logratio(float x) { return exp2_fast(x * 1.4426950408889634f); }
 
+// Truncated importance weights and the affine map of the advantage recursion
+// (Section 2.2; Section 3.1).  Returns whether exp(x) exceeded rho_bar.  kPlain: the default configuration
+// (importance weights pi_target / pi_worker, ratio R3, clipped surrogate), without the run-time switches.
+// (Products and sums are spelled out so that both forms give the same bits.)
+template <bool kPlain>
 __device__ __forceinline__ bool recursion_map(StepIn& s, const LossScalars& k, float& a, float& b) {
-    const float x = (k.is_source == 1 ? s.l_theta : s.l_target) - s.l_worker;
-    const float w = (k.is_source == 2) ? 1.0f : exp_of_logratio(x);  // 2: plain GAE, no importance weights
+    const float x = ((!kPlain && k.is_source == 1) ? s.l_theta : s.l_target) - s.l_worker;
+    const float w = (!kPlain && k.is_source == 2) ? 1.0f : exp_of_logratio(x);  // 2: plain GAE, no importance weights
     const float rho = fminf(k.rho_bar, w);
     s.rho = rho;
     const float c = fminf(k.c_bar, w);
-    b = rho * (s.reward + s.discount * s.value_next - s.value);
-    a = s.last_step ? 0.0f : k.lambda_ * s.discount * c;
+    b = __fmul_rn(rho, __fadd_rn(fmaf(s.discount, s.value_next, s.reward), -s.value));
+    a = s.last_step ? 0.0f : __fmul_rn(__fmul_rn(k.lambda_, s.discount), c);
     return w > k.rho_bar;
 }
 
 // Ratio of Section 4.1 and the eps-clipped surrogate of Appendix E.  Returns the weight
 // adv * R of the policy-gradient term (0 where the clip removes it).
+template <bool kPlain>
 __device__ __forceinline__ float surrogate(const StepIn& s, const LossScalars& k, float adv,
                                            float& surr, float& ratio, bool& clipped) {
-    if (k.objective == 1) {
+    if (!kPlain && k.objective == 1) {
         // IMPALA's actor update (Section 2.2): weight rho_t (r_t + gamma_t v_{t+1} - V_t) on
         // grad log pi_theta, v the V-trace target V + A (the bootstrap value after the last step)
         const float v_next = s.value_next + (s.last_step ? 0.0f : s.adv_next);
-        const float w = s.rho * (s.reward + s.discount * v_next - s.value);
-        surr = w * (s.l_theta + s.l_shift);
+        const float w = __fmul_rn(s.rho, __fadd_rn(fmaf(s.discount, v_next, s.reward), -s.value));
+        surr = __fmul_rn(w, s.l_theta + s.l_shift);
         ratio = s.rho;
         clipped = false;
         return w;
     }
-    float d;
-    if (k.ratio_mode == 1) d = s.l_target;
-    else if (k.ratio_mode == 2) d = s.l_worker;
-    else d = fmaxf(s.l_target, s.l_worker - k.log_rho_tw);
+    float d = fmaxf(s.l_target, s.l_worker - k.log_rho_tw);
+    if (!kPlain) {
+        if (k.ratio_mode == 1) d = s.l_target;
+        else if (k.ratio_mode == 2) d = s.l_worker;
+    }
     const float R = exp_of_logratio(s.l_theta - d);
     const float Rc = fminf(fmaxf(R, k.clip_lo), k.clip_hi);
-    surr = fminf(R * adv, Rc * adv);
+    const float Ra = __fmul_rn(R, adv);
+    surr = fminf(Ra, __fmul_rn(Rc, adv));
     clipped = (adv > 0.0f && R > k.clip_hi) || (adv < 0.0f && R < k.clip_lo);
     ratio = R;
-    return clipped ? 0.0f : adv * R;
-}
-
-// The two functions above for the default configuration (importance weights pi_target / pi_worker,
-// ratio R3, clipped surrogate), without the run-time switches.
-__device__ __forceinline__ bool recursion_map_plain(StepIn& s, const LossScalars& k, float& a, float& b) {
-    const float w = exp_of_logratio(s.l_target - s.l_worker);
-    const float rho = fminf(k.rho_bar, w);
-    s.rho = rho;
-    const float c = fminf(k.c_bar, w);
-    b = rho * (s.reward + s.discount * s.value_next - s.value);
-    a = s.last_step ? 0.0f : k.lambda_ * s.discount * c;
-    return w > k.rho_bar;
-}
-__device__ __forceinline__ float surrogate_plain(const StepIn& s, const LossScalars& k, float adv, float& surr,
-                                                 float& ratio, bool& clipped) {
-    const float d = fmaxf(s.l_target, s.l_worker - k.log_rho_tw);
-    const float R = exp_of_logratio(s.l_theta - d);
-    const float Rc = fminf(fmaxf(R, k.clip_lo), k.clip_hi);
-    surr = fminf(R * adv, Rc * adv);
-    clipped = (adv > 0.0f && R > k.clip_hi) || (adv < 0.0f && R < k.clip_lo);
-    ratio = R;
-    return clipped ? 0.0f : adv * R;
-}
-
-// Sum the kNumSums per-thread values over the block (fixed order) and add them to `acc`,
-// which only thread 0 keeps.  `red` is [NT/32][8] shared floats.  The caller must place a
-// __syncthreads() between the write phase and the read phase: call stage 1, sync, stage 2.
-template <int NT>
-__device__ __forceinline__ void block_sums_stage1(float (&v)[kNumSums], float (*red)[8]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < kNumSums; ++j) {
-        float x = v[j];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) red[warp][j] = x;
-    }
-}
-template <int NT>
-__device__ __forceinline__ void block_sums_stage2(float (&acc)[kNumSums], float (*red)[8]) {
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int j = 0; j < kNumSums; ++j) {
-            float x = 0.0f;
-            for (int w = 0; w < NT / 32; ++w) x += red[w][j];
-            acc[j] += x;
-        }
-    }
-}
-
-// Last step of every loss kernel: publish this block's sums, and let the block that
-// finishes last add all blocks' sums in index order (fp64) and write the eight loss terms.
-// `counter` must be 0 on entry to the kernel and is 0 again on exit.
-template <int NT>
-__device__ __forceinline__ void finish_loss_terms(const float (&acc)[kNumSums], float* partials,
-                                                  unsigned int* counter, float* loss_terms,
-                                                  const LossScalars& k, double M) {
-    __shared__ bool is_last;
-    __shared__ double dred[NT / 32][kNumSums];
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int j = 0; j < kNumSums; ++j) partials[(size_t)blockIdx.x * 8 + j] = acc[j];
-        __threadfence();
-        const unsigned int ticket = atomicAdd(counter, 1u);
-        is_last = (ticket == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    double s[kNumSums];
-#pragma unroll
-    for (int j = 0; j < kNumSums; ++j) s[j] = 0.0;
-    for (unsigned int blk = threadIdx.x; blk < gridDim.x; blk += NT) {
-        const float4 p0 = __ldcg(reinterpret_cast<const float4*>(partials + (size_t)blk * 8));
-        const float4 p1 = __ldcg(reinterpret_cast<const float4*>(partials + (size_t)blk * 8 + 4));
-        s[0] += p0.x; s[1] += p0.y; s[2] += p0.z; s[3] += p0.w;
-        s[4] += p1.x; s[5] += p1.y; s[6] += p1.z;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < kNumSums; ++j) {
-        double x = s[j];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) dred[warp][j] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[kNumSums];
-#pragma unroll
-        for (int j = 0; j < kNumSums; ++j) {
-            double x = 0.0;
-            for (int w = 0; w < NT / 32; ++w) x += dred[w][j];
-            t[j] = x / M;
-        }
-        const double l_pi = -t[0], l_v = t[1], ent = t[2], kl = t[3];
-        loss_terms[0] = (float)(l_pi + (double)k.vf_coef * l_v - (double)k.ent_coef * ent +
-                                (double)k.kl_coef * kl);
-        loss_terms[1] = (float)l_pi;
-        loss_terms[2] = (float)l_v;
-        loss_terms[3] = (float)ent;
-        loss_terms[4] = (float)kl;
-        loss_terms[5] = (float)t[4];
-        loss_terms[6] = (float)t[5];
-        loss_terms[7] = (float)t[6];
-        *counter = 0u;
-    }
-}
-
-// ---- early publication of a block's sums ---------------------------------------------------
-// Thread 0 calls this as soon as its block's last sums are final, long before the block's
-// stores are done: the fence and the counter's round trip then overlap the rest of the
-// block's work instead of extending it.  Returns the block's ticket (0-based arrival order).
-__device__ __forceinline__ unsigned int publish_block_sums(const float (&acc)[kNumSums], float* partials,
-                                                           unsigned int* counter) {
-    float4* row = reinterpret_cast<float4*>(partials + (size_t)blockIdx.x * 8);
-    row[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    row[1] = make_float4(acc[4], acc[5], acc[6], 0.0f);
-    // one acq_rel atomic: releases this block's row and, for the block that draws the last ticket,
-    // acquires every other block's (their atomics on the counter form the release sequence)
-    unsigned int ticket;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(ticket) : "l"(counter) : "memory");
-    return ticket;
-}
-// Run by every thread of the block that drew the last ticket: add all blocks' sums in index
-// order (fp64), write the eight loss terms, and leave the counter at 0 for the next launch.
-template <int NT>
-__device__ __noinline__ void reduce_published_sums(const float* partials, unsigned int* counter, float* loss_terms,
-                                                      float vf_coef, float ent_coef, float kl_coef, double M) {
-    __shared__ double dred[NT / 32][kNumSums];
-    // thread 0 acquired the rows with its ticket and a block barrier lies between that and here;
-    // the loads below go to L2 (ld.cg), so no further fence is needed
-    double s[kNumSums];
-#pragma unroll
-    for (int j = 0; j < kNumSums; ++j) s[j] = 0.0;
-    // rows in batches of eight per thread, all loads of a batch in flight together
-    constexpr int kBatch = 8;
-    for (unsigned int first = threadIdx.x; first < gridDim.x; first += NT * kBatch) {
-        float4 p0[kBatch], p1[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            const unsigned int blk = first + u * NT;
-            if (blk < gridDim.x) {
-                p0[u] = __ldcg(reinterpret_cast<const float4*>(partials + (size_t)blk * 8));
-                p1[u] = __ldcg(reinterpret_cast<const float4*>(partials + (size_t)blk * 8 + 4));
-            } else {
-                p0[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                p1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            s[0] += p0[u].x; s[1] += p0[u].y; s[2] += p0[u].z; s[3] += p0[u].w;
-            s[4] += p1[u].x; s[5] += p1[u].y; s[6] += p1[u].z;
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < kNumSums; ++j) {
-        double x = s[j];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) dred[warp][j] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double inv_m = 1.0 / M;
-        double t[kNumSums];
-#pragma unroll
-        for (int j = 0; j < kNumSums; ++j) {
-            double x = 0.0;
-            for (int w = 0; w < NT / 32; ++w) x += dred[w][j];
-            t[j] = x * inv_m;
-        }
-        const double l_pi = -t[0], l_v = t[1], ent = t[2], kl = t[3];
-        loss_terms[0] = (float)(l_pi + (double)vf_coef * l_v - (double)ent_coef * ent +
-                                (double)kl_coef * kl);
-        loss_terms[1] = (float)l_pi;
-        loss_terms[2] = (float)l_v;
-        loss_terms[3] = (float)ent;
-        loss_terms[4] = (float)kl;
-        loss_terms[5] = (float)t[4];
-        loss_terms[6] = (float)t[5];
-        loss_terms[7] = (float)t[6];
-        *counter = 0u;
-    }
+    return clipped ? 0.0f : Ra;
 }
 
 // ---- sums published as tagged rows (persistent kernel) --------------------------------------

@@ -19,8 +19,8 @@ constexpr size_t kCounterBytes = 256; // words after the partials: [0] completio
 constexpr int kMaxTaggedRows = 1024;  // rows of eight (value, tag) pairs after the counter words: one per block of a persistent kernel
 constexpr int kMinTileRows = 64;      // the smallest tile of a launch that publishes its tiles' aggregates
 
-// How a categorical batch is laid out over the grid (see impact_categorical.cuh).
-struct CatGeometry {
+// How a batch is laid out over the grid (see impact_flat.cuh).
+struct BatchGeometry {
     long long B, T;
     int nt;          // rows of a tile
     int ntiles;      // long: tiles per trajectory
@@ -46,13 +46,38 @@ struct CatParams {
     unsigned long long* tile_aggregates;  // long launches: two (value, launch tag) pairs per tile (NULL = no room for them)
     void* target_copy;  // where the target logits are written as well (NULL = nowhere)
     const impact_loss_inputs* indirect;  // device record that overrides the nine input pointers above (NULL = none)
-    CatGeometry geo;
+    BatchGeometry geo;
     LossScalars k;
     int A;
 };
 
-// The rest of a categorical launch's shape.
-struct CatShape {
+struct GaussParams {
+    const float* learner_mean;
+    const float* learner_logstd;
+    const float* target_mean;
+    const float* target_logstd;
+    const float* actions;
+    const float* worker_logp;
+    const float* rewards;
+    const float* discounts;
+    const float* values;
+    const float* bootstrap;
+    float* loss_terms;
+    float* dmean;
+    float* dlogstd;
+    float* dvalues;
+    float* vtarget;
+    float* advantage;
+    unsigned int* counter;
+    unsigned long long* tagged_rows;
+    unsigned long long* tile_aggregates;
+    BatchGeometry geo;
+    LossScalars k;
+    int D;
+};
+
+// The rest of a launch's shape.
+struct LaunchForm {
     int nt, stages, in_flight, lanes, n_prefetch;
     int log_lanes, passes, rot_shift, rot_mask;  // how rows are laid on lanes (see impact_categorical.cuh)
 };
@@ -72,6 +97,8 @@ struct LossInputPointers {
 // Picks the kernel for a categorical call (`p` complete except for geo) and launches it.
 template <typename LT, typename GT>
 int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
+
+int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
 
 // Tiles the producer keeps in flight and stages of the ring, for tiles of `tile_in_bytes` bytes of logits.
 void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max_smem, long long tiles_per_block,

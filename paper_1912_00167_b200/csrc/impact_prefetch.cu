@@ -1,6 +1,6 @@
 // The companion kernel that asks L2 for a categorical loss launch's first tiles while the kernel before it on the
 // stream is still running.
-#include "impact_categorical.cuh"
+#include "impact_flat.cuh"
 
 namespace impact {
 namespace {
@@ -15,7 +15,7 @@ struct PrefetchList {
     int row_bytes[kArrays];
     int n_tiles_max;  // tiles of a block that are asked for (from its first)
     int is_long;
-    CatGeometry geo;
+    BatchGeometry geo;
 };
 
 // Enqueued right before the loss launch and of as many blocks, it becomes resident next to the blocks of whatever

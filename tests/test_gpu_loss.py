@@ -637,3 +637,26 @@ def test_a_non_finite_value_stays_in_its_trajectory(B, T, A):
     for k in ("dlogits", "dvalues"):
         assert torch.equal(res[0][k][others], res[1][k][others])
         assert not torch.isfinite(res[1][k][hit]).all()
+
+
+@pytest.mark.parametrize("D", [1, 2, 4, 5, 8, 12, 16, 18, 20, 33, 34, 35, 64, 68, 69, 100, 128, 137, 138, 200, 256])
+def test_gaussian_every_width_of_the_row_pass(oracle, D):
+    """Dimensions on both sides of every change of layout (rows per tile, lanes per row, elements per access), with
+    trajectories that cross the tiles of a block; the default configuration's form and the one with every switch."""
+    B, T = (331, 50) if D <= 64 else (301, 21)
+    batch = ii.gaussian_batch(B, T, D, seed=8000 + D, p_done=0.02)
+    P.check_gaussian(oracle, batch, LossHyper(clip_eps=0.3, vf_coef=0.5, ent_coef=0.01, kl_coef=0.0))
+    P.check_gaussian(oracle, batch, LossHyper(rho_bar=1.2, c_bar=1.0, clip_eps=0.3, vf_coef=0.5, ent_coef=0.01, kl_coef=0.05,
+                                              lam=0.99, rho_tw=2.0))
+    P.check_gaussian(oracle, batch, LossHyper(objective=1))
+
+
+@pytest.mark.parametrize("B,T,D", [(3, 4500, 5), (2, 1000, 20), (5, 1300, 40), (400, 100, 3), (170, 129, 6), (160, 300, 17),
+                                   (640, 257, 24), (1000, 1, 17), (999, 3, 50)])
+def test_gaussian_trajectories_across_tiles_and_blocks(oracle, B, T, D):
+    """Few long trajectories (tiles on neighbouring blocks, or swept by one block where tiles are small) and many of
+    every length (blocks own whole ones)."""
+    batch = ii.gaussian_batch(B, T, D, seed=8500 + B + T + D, p_done=0.003)
+    P.check_gaussian(oracle, batch, LossHyper(rho_bar=1.2, c_bar=1.0, clip_eps=0.3, vf_coef=0.5, ent_coef=0.01, kl_coef=0.05,
+                                              lam=0.99, rho_tw=2.0))
+    P.check_gaussian(oracle, batch, LossHyper(clip_eps=0.3, kl_coef=0.0, lam=0.99))
