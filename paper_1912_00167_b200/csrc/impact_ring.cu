@@ -256,17 +256,35 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
         const uint32_t word = __ballot_sync(0xFFFFFFFFu, s < v.N && __ldcg(v.valid + s) != 0);
         if (lane == 0) live_s[s >> 5] = word;
     }
+    // (the candidate's pointers are on their way while the slots are worked out)
+    unsigned long long cand = 0;
     if (tid < 32 && sources && lane <= v.n_fields)
-        cand_s[lane] = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(
-            sources + (size_t)(hd.pushes % (uint64_t)n_candidates) * (size_t)(v.n_fields + 1) + lane)));
+        cand = __ldcg(reinterpret_cast<const unsigned long long*>(
+            sources + (size_t)(hd.pushes % (uint64_t)n_candidates) * (size_t)(v.n_fields + 1) + lane));
     __syncthreads();
     uint32_t live = 0;
-    int32_t slot = -1;
+    int32_t slot = -1, pick = -1, drawn_count = 0;
+    unsigned long long drawn_fresh = 0;
     if (tid < 32) {
         live = live_s[lane];
         const int32_t left = v.N - 32 * lane;  // slots that exist in this lane's word
         const uint32_t exist = left >= 32 ? 0xFFFFFFFFu : (left > 0 ? (1u << left) - 1u : 0u);
         if (sources) slot = first_at_or_after(~live & exist, hd.write_cursor);
+        if (slot >= 0 && lane == (slot >> 5)) live |= 1u << (slot & 31);
+        // the draw too is worked out by every block, so that what is kept with the drawn slot has arrived by the time
+        // the last block is known
+        const uint32_t n_live = (uint32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
+        if (do_sample && n_live > 0)
+            pick = v.mode == IMPACT_SAMPLE_UNIFORM  // floor(u * live / 2^64)
+                       ? nth_member(live, (uint32_t)__umul64hi(splitmix64_at_dev(v.seed, hd.draws), (uint64_t)n_live))
+                       : first_at_or_after(live, hd.read_cursor);
+        if (pick >= 0 && pick != slot) {
+            drawn_count = __ldcg(v.count + pick);
+            drawn_fresh = __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh + pick));
+        }
+        if (lane <= v.n_fields) cand_s[lane] = reinterpret_cast<const void*>(cand);
+        __syncwarp();
+        if (pick == slot) drawn_fresh = reinterpret_cast<unsigned long long>(cand_s[v.n_fields]);  // (drawn as it is pushed)
         if (lane == 0) {
             int n = 0;
             unsigned long long units = 0;
@@ -282,7 +300,7 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
                 }
             }
             plan_s.n = n;
-            // this block has read all of the state it will ever read, unless it turns out to be the last
+            // this block has read all of the state (the release orders those reads before the ticket)
             unsigned int ticket;
             asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(ticket) : "l"(&v.hd->tickets) : "memory");
             last_s = ticket == gridDim.x - 1;
@@ -295,7 +313,6 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
     // ---- the bookkeeping, by the first warp of the last block
     if (sources) {
         if (slot >= 0) {
-            if (lane == (slot >> 5)) live |= 1u << (slot & 31);
             if (lane == 0) {
                 v.fresh[slot] = reinterpret_cast<uint64_t>(cand_s[v.n_fields]);
                 v.valid[slot] = 1;
@@ -308,23 +325,15 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
         hd.n_events += 1;
     }
     if (do_sample) {
-        const uint32_t n_live = (uint32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
-        int32_t pick = -1;
-        if (n_live > 0) {
-            if (v.mode == IMPACT_SAMPLE_UNIFORM) {
-                const uint64_t u = splitmix64_at_dev(v.seed, hd.draws++);
-                pick = nth_member(live, (uint32_t)__umul64hi(u, (uint64_t)n_live));  // floor(u * live / 2^64)
-            } else {
-                pick = first_at_or_after(live, hd.read_cursor);
-                hd.read_cursor = (pick + 1) % v.N;
-            }
+        if (pick >= 0) {
+            if (v.mode == IMPACT_SAMPLE_UNIFORM) hd.draws += 1;
+            else hd.read_cursor = (pick + 1) % v.N;
         }
         if (lane == 0) {
             int32_t k_before = 0;
             if (pick >= 0) {
-                k_before = pick == slot ? 0 : __ldcg(v.count + pick);
-                const void* const fresh = pick == slot ? cand_s[v.n_fields] : reinterpret_cast<const void*>(__ldcg(
-                                              reinterpret_cast<const unsigned long long*>(v.fresh + pick)));
+                k_before = drawn_count;
+                const void* const fresh = reinterpret_cast<const void*>(drawn_fresh);
                 v.count[pick] = k_before + 1;
                 if (k_before + 1 >= v.K) v.valid[pick] = 0;
                 auto field = [&](int32_t f) -> const void* {
