@@ -595,6 +595,9 @@ int32_t run_gaussian_width(const GaussParams& p, const DeviceInfo* di, cudaStrea
     if (kV == 4 && vecs % (1 << rl.log_lanes) == 0)
         while (2 * (rl.rot_mask + 1) <= b.ways && (vecs >> rl.log_lanes) % (2 * (rl.rot_mask + 1)) == 0)
             rl.rot_mask = 2 * rl.rot_mask + 1;
+    // (five groups where rows are short, tiles small and a tile's time is arithmetic: D = 1 49.5 -> 43.5 us, 5 70 -> 57 on
+    // 100 to 300 MB; at 12 to 14 dimensions they lose up to a third, at 8 they are even)
+    if (p.D <= 8) return run_gaussian_form<0, 4, 5, kV>(p, rl, di, stream);
     return run_gaussian_form<0, 3, 3, kV>(p, rl, di, stream);
 }
 
