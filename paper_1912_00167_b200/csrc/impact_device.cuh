@@ -1,18 +1,13 @@
-// Device building blocks of the fused IMPACT loss kernels (sm_100a).
+// Device building blocks of the fused IMPACT loss kernels (sm_100a): bulk copies and their barriers, fast
+// exponentials, the importance weights and the surrogate, published aggregates and sums.
 //
-// Work decomposition shared by all loss kernels:
-//   * one thread per time step ("row"); a tile is up to NT consecutive rows of the row-major
-//     [B*T, width] tensors, which is one contiguous slab of global memory;
-//   * short trajectories (T <= NT) are packed, floor(NT/T) whole trajectories per tile; long
-//     ones are cut into tiles that are linked by one scalar (swept from the END backwards inside
-//     one block) or by published affine aggregates (tiles on different blocks) -- either way
-//     every byte is read once;
-//   * slabs reach shared memory by bulk asynchronous copies (one instruction per slab) and
-//     keep their dense layout; gradients overwrite the staged rows in place and leave by bulk
-//     stores;
-//   * sums are reduced in a fixed order: per thread, per warp, per block, and across blocks
-//     either by the last block to arrive (ticket) or, in the persistent kernels, by one
-//     collecting group that reads every block's tagged row.
+// Work decomposition shared by the loss kernels (see impact_flat.cuh):
+//   * a tile is a number of consecutive steps ("rows") of the row-major [B*T, width] tensors, which is one contiguous
+//     slab of global memory; each byte is read once;
+//   * slabs reach shared memory by bulk asynchronous copies (one instruction per slab) and keep their dense layout;
+//     gradients overwrite the staged rows in place and leave by bulk stores;
+//   * sums are reduced in a fixed order: per thread, per warp, per block, and across blocks by one collecting group
+//     that reads every block's tagged row.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -24,50 +19,10 @@ namespace dev {
 
 constexpr int kNumSums = 7;  // surrogate, value, entropy, kl, clipped, rho-truncated, ratio
 
-// ---- 16-byte vectors of storage elements ---------------------------------------------
-template <typename T> struct Pack;
-template <> struct Pack<float> {
-    static constexpr int kElems = 4;
-    static __device__ __forceinline__ void unpack(const uint4& v, float (&f)[4]) {
-        f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);
-        f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
-    }
-    static __device__ __forceinline__ uint4 pack(const float (&f)[4]) {
-        return make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]),
-                          __float_as_uint(f[2]), __float_as_uint(f[3]));
-    }
-    static __device__ __forceinline__ float to_float(float x) { return x; }
-    static __device__ __forceinline__ float from_float(float x) { return x; }
-};
-template <> struct Pack<__nv_bfloat16> {
-    static constexpr int kElems = 8;
-    static __device__ __forceinline__ void unpack(const uint4& v, float (&f)[8]) {
-        // a bf16 is the upper half of an fp32: widening is a shift, exact
-        f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xFFFF0000u);
-        f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xFFFF0000u);
-        f[4] = __uint_as_float(v.z << 16); f[5] = __uint_as_float(v.z & 0xFFFF0000u);
-        f[6] = __uint_as_float(v.w << 16); f[7] = __uint_as_float(v.w & 0xFFFF0000u);
-    }
-    static __device__ __forceinline__ uint32_t two(float lo, float hi) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // round to nearest even
-        return *reinterpret_cast<uint32_t*>(&h);
-    }
-    static __device__ __forceinline__ uint4 pack(const float (&f)[8]) {
-        return make_uint4(two(f[0], f[1]), two(f[2], f[3]), two(f[4], f[5]), two(f[6], f[7]));
-    }
-    static __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
-    static __device__ __forceinline__ __nv_bfloat16 from_float(float x) { return __float2bfloat16_rn(x); }
-};
-
-__device__ __forceinline__ uint4 ld_stream16(const uint4* p) {
-    uint4 v;
-    asm volatile("ld.global.cs.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ void st_stream16(uint4* p, const uint4& v) {
-    asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};"
-                 :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+// Two fp32 values as a pair of bf16, rounded to nearest even.
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<uint32_t*>(&h);
 }
 
 // ---- bulk asynchronous copies (the 1-D form of the tensor memory accelerator) -----------
@@ -77,10 +32,6 @@ __device__ __forceinline__ void st_stream16(uint4* p, const uint4& v) {
 // bulk async-groups.  No multicast and no cluster: every copy is local to the block.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbarrier_init(uint64_t* bar, uint32_t arrivals) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(arrivals) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 // Initialisation of many barriers: each without a fence, then one fence_mbarrier_init() by every
 // initialising thread before the block-wide barrier that precedes their first use.
@@ -95,25 +46,6 @@ __device__ __forceinline__ void mbarrier_expect_tx(uint64_t* bar, uint32_t bytes
 __device__ __forceinline__ void mbarrier_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
-// Waits for the phase with the given parity to complete.  The wait is bounded: if the
-// bytes never arrive the caller gets `false` instead of a hang.
-__device__ __forceinline__ bool mbarrier_wait(uint64_t* bar, uint32_t parity) {
-    const uint32_t addr = smem_addr(bar);
-    // each try may sleep up to the hint and a failed try backs off 64 ns: the wait gives up after
-    // somewhere between ~0.07 s and ~1.1 s, far beyond any copy's latency, far short of a hang
-    constexpr uint32_t kSuspendHintNs = 1000;
-    for (uint32_t tries = 0; tries < (1u << 20); ++tries) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(addr), "r"(parity), "r"(kSuspendHintNs) : "memory");
-        if (done) return true;
-        __nanosleep(64);  // a failed try returns early on this part: back off instead of spinning
-    }
-    return false;
-}
 // One look at the barrier, without waiting: has the phase with the given parity completed?
 __device__ __forceinline__ bool mbarrier_test(uint64_t* bar, uint32_t parity) {
     uint32_t done;
@@ -124,9 +56,9 @@ __device__ __forceinline__ bool mbarrier_test(uint64_t* bar, uint32_t parity) {
         : "=r"(done) : "r"(smem_addr(bar)), "r"(parity) : "memory");
     return done != 0;
 }
-// The same wait for blocks in which several warps wait on one another's barriers: it also gives up
-// (at once) when `*abort_flag` is set, and sets it when it gives up itself, so that one wait that
-// runs out ends every other wait of the block instead of each running out in turn.
+// Waits for the phase with the given parity to complete.  The wait is bounded: if the bytes never arrive the caller
+// gets `false` instead of a hang.  It also gives up (at once) when `*abort_flag` is set, and sets it when it gives up
+// itself, so that one wait that runs out ends every other wait of the block instead of each running out in turn.
 __device__ __forceinline__ bool mbarrier_wait(uint64_t* bar, uint32_t parity, int* abort_flag) {
     const uint32_t addr = smem_addr(bar);
     // (no suspend hint and no sleep between tries: the wait sits between a tile's landing and the first

@@ -125,7 +125,7 @@ template <> struct Vec<__nv_bfloat16, 2> {
         f[0] = __uint_as_float(w << 16); f[1] = __uint_as_float(w & 0xFFFF0000u);
     }
     static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
-        *reinterpret_cast<uint32_t*>(p) = dev::Pack<__nv_bfloat16>::two(f[0], f[1]);
+        *reinterpret_cast<uint32_t*>(p) = dev::bf16_pair(f[0], f[1]);
     }
 };
 template <> struct Vec<__nv_bfloat16, 4> {
@@ -135,7 +135,7 @@ template <> struct Vec<__nv_bfloat16, 4> {
         f[2] = __uint_as_float(w.y << 16); f[3] = __uint_as_float(w.y & 0xFFFF0000u);
     }
     static __device__ __forceinline__ void st(unsigned char* p, const float* f) {
-        *reinterpret_cast<uint2*>(p) = make_uint2(dev::Pack<__nv_bfloat16>::two(f[0], f[1]), dev::Pack<__nv_bfloat16>::two(f[2], f[3]));
+        *reinterpret_cast<uint2*>(p) = make_uint2(dev::bf16_pair(f[0], f[1]), dev::bf16_pair(f[2], f[3]));
     }
 };
 // Overwrites one element after vector stores to the same row; an explicit shared-memory store keeps it ordered behind
