@@ -68,16 +68,76 @@ __global__ void __launch_bounds__(256) multi_copy_kernel(const __grid_constant__
     copy_segments(s);
 }
 
-// dst[i, :] = src[idx[i], :], rows of `units` elements of type V.
+// dst[i, :] = src[idx[i], :], rows of `units` elements of type V, at least 16 bytes, and a destination on a 16-byte boundary.
 //
-// The destination is walked flat, a grid's width at a time, so that every lane has an element whatever the row's width,
-// and a thread's place in its row is carried along instead of divided out: from one of its elements to the next the row
-// advances by stride / units and the place by stride % units.  With 64 warps to an SM one element of a thread under way is
-// enough for elements of up to 4 bytes, two for wider ones (four and eight are slower).  40 MB in rows of 12, 96, 132, 200,
-// 1800 and 4096 bytes take 28.7, 15.6, 22.1, 17.0, 16.5 and 14.8 us.  Rows laid on as many lanes as cover them, a power of
-// two, took 59, 23, 36, 23, 17.6 and 16.0: idle lanes; a 64-bit division per element, 16- or 4-byte elements and one under
-// way, took 36, 17, 32, 32, 32 and 15.4.  Slower than the former only for rows of an odd number of words beyond 4 KB (22.4
-// against 21.5 at 4100 bytes).
+// The destination is walked flat in granules of 16 bytes, a grid's width at a time, so that every lane has one whatever the
+// row's width.  A granule is put together from elements of one row or, where a row ends inside it, of two; both rows'
+// indices are asked for side by side.  A thread's row and place in it are carried along: from one of its granules to the
+// next the row advances by stride_rows and the place by stride_rest; the one division is done while the kernel before this
+// one drains.  Bound by HBM from 64-byte rows on (a granule at a time keeps 2048 threads' loads under way on every SM; two
+// where granules are single loads, four are slower).  40 MB in rows of 17, 36, 132, 200, 1800 and 4096 bytes take 66, 21.4,
+// 16.9, 16.1, 15.1 and 14.5 us, 4.2 MB in rows of 200 and 204 bytes 3.5 and 3.6; element by element (below) 72, 24.2, 22.1,
+// 17.0, 16.5, 14.9, 4.5 and 5.7.
+template <typename V, int U>
+__global__ void __launch_bounds__(256, 8) gather_granules_kernel(const V* __restrict__ src, const int32_t* __restrict__ idx,
+                                                                 unsigned int n, int n_src_rows, unsigned int units,
+                                                                 unsigned int stride_rows, unsigned int stride_rest,
+                                                                 V* __restrict__ dst) {
+    constexpr int N = 16 / (int)sizeof(V);  // elements of a granule
+    union Granule {
+        uint4 all;
+        V part[N];
+    };
+    const unsigned long long total = (unsigned long long)n * units;  // elements
+    const unsigned long long granules = total / N;
+    const unsigned int stride = gridDim.x * blockDim.x;
+    unsigned long long v = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned int i = (unsigned int)(v * N / units), c = (unsigned int)(v * N - (unsigned long long)i * units);
+    grid_dependency_wait();
+    auto row_at = [&](unsigned int k) {
+        const int r = __ldg(idx + k);
+        return src + (unsigned long long)(unsigned int)min(max(r, 0), n_src_rows - 1) * units;
+    };
+    for (; v < granules; v += (unsigned long long)U * stride) {
+        const V *first[U], *second[U];
+        unsigned int left[U];  // elements of the granule that its first row still has
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            left[u] = units - c;
+            first[u] = second[u] = src;
+            if (v + (unsigned long long)u * stride < granules) {
+                first[u] = row_at(i) + c;
+                // (asked for in any case, the same index where the row goes on: no branch that waits for the first)
+                if constexpr (N > 1) second[u] = row_at(left[u] < N ? i + 1 : i) - left[u];
+            }
+            i += stride_rows;
+            c += stride_rest;
+            if (c >= units) { c -= units; ++i; }
+        }
+        Granule x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (v + (unsigned long long)u * stride < granules) {
+#pragma unroll
+                for (int e = 0; e < N; ++e) x[u].part[e] = __ldg((e < (int)left[u] ? first[u] : second[u]) + e);
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (v + (unsigned long long)u * stride < granules)
+                reinterpret_cast<uint4*>(dst)[v + (unsigned long long)u * stride] = x[u].all;
+    }
+    // what is left of the last granule (by threads that had none, in a grid of one round)
+    const unsigned long long free_thread = blockIdx.x * blockDim.x + threadIdx.x - (granules + 16 <= stride ? granules : 0);
+    if (free_thread < total - granules * N) {
+        const unsigned long long at = granules * N + free_thread;
+        const unsigned int k = (unsigned int)(at / units);
+        dst[at] = __ldg(row_at(k) + (at - (unsigned long long)k * units));
+    }
+}
+
+// The same element by element, for rows narrower than a granule, of which one would hold several, and destinations that lie
+// on a smaller boundary; two elements of 8 bytes and more of a thread are under way, one of the narrower ones.  40 MB in rows
+// of 12 bytes take 28.7 us.
 template <typename V, int U>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const V* __restrict__ src, const int32_t* __restrict__ idx,
                                                           long long n, long long n_src_rows, long long units,
@@ -751,16 +811,39 @@ extern "C" int32_t impact_buffer_import_state(impact_buffer* h, const void* blob
     return IMPACT_OK;
 }
 
+template <typename V, int U>
+static int32_t launch_granules(const V* src, const int32_t* idx, unsigned int n, int n_src_rows, unsigned int units, V* dst,
+                               const DeviceInfo* di, cudaStream_t cs) {
+    constexpr unsigned int per = 16 / sizeof(V);
+    const unsigned long long granules = (unsigned long long)n * units / per;
+    const int blocks = blocks_for(granules + 16, U, di);  // (16: threads for what is left of the last granule)
+    const unsigned long long stride = (unsigned long long)blocks * 256 * per;
+    IMPACT_CUDA_TRY(launch_serialized(gather_granules_kernel<V, U>, dim3(blocks), dim3(256), 0, cs, src, idx, n, n_src_rows,
+                                      units, (unsigned int)(stride / units), (unsigned int)(stride % units), dst));
+    return IMPACT_OK;
+}
+
 template <typename V>
 static int32_t launch_gather(const void* src, const int32_t* idx, int64_t n, int64_t n_src_rows, size_t row_bytes,
                              void* dst, const DeviceInfo* di, cudaStream_t cs) {
-    constexpr int U = sizeof(V) >= 8 ? 2 : 1;
     const long long units = (long long)(row_bytes / sizeof(V));
+    const V* const from = static_cast<const V*>(src);
+    V* const to = static_cast<V*>(dst);
+    constexpr long long most = 1ll << 31;  // (what the granules' counters hold)
+    // (elements of 4 and 8 bytes: a fifth and more of the granules of rows below 32 bytes hold an end, 25.4 / 27.4 us at 20
+    // bytes; narrower elements gain all the same, 45 / 40 at 18)
+    const bool wide_enough = sizeof(V) == 4 || sizeof(V) == 8 ? row_bytes >= 32 : row_bytes >= 16;
+    if (wide_enough && aligned16(dst) && n < most && n_src_rows < most && (long long)row_bytes < most) {
+        if constexpr (sizeof(V) == 16)  // (two under way where a thread has more than one: 4 MB 4.3 us against 4.7; less 1.5 / 1.4)
+            if (n * units > (long long)di->sm_count * 8 * 256)
+                return launch_granules<V, 2>(from, idx, (unsigned int)n, (int)n_src_rows, (unsigned int)units, to, di, cs);
+        return launch_granules<V, 1>(from, idx, (unsigned int)n, (int)n_src_rows, (unsigned int)units, to, di, cs);
+    }
+    constexpr int U = sizeof(V) >= 8 ? 2 : 1;
     const int blocks = blocks_for((unsigned long long)n * (unsigned long long)units, U, di);
     const long long stride = (long long)blocks * 256;
-    IMPACT_CUDA_TRY(launch_serialized(gather_rows_kernel<V, U>, dim3(blocks), dim3(256), 0, cs, static_cast<const V*>(src), idx,
-                                      (long long)n, (long long)n_src_rows, units, stride / units, stride % units,
-                                      static_cast<V*>(dst)));
+    IMPACT_CUDA_TRY(launch_serialized(gather_rows_kernel<V, U>, dim3(blocks), dim3(256), 0, cs, from, idx, (long long)n,
+                                      (long long)n_src_rows, units, stride / units, stride % units, to));
     return IMPACT_OK;
 }
 

@@ -379,3 +379,20 @@ def test_gather_rows_of_every_width(row_bytes, n):
     torch.cuda.synchronize()
     assert torch.equal(dst, src[idx.long()])
     assert bool((guard[:256] == 0xA5).all()) and bool((guard[256 + n * row_bytes:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("row_bytes", [15, 16, 17, 18, 24, 31, 32, 34, 36, 40, 48, 200, 1802])
+@pytest.mark.parametrize("n,offset", [(1, 0), (7, 0), (5000, 0), (40000, 0), (5000, 8), (5000, 4)])
+def test_gather_rows_around_the_granules(row_bytes, n, offset):
+    """Rows that end inside a granule of 16 bytes or fill it, one round of the grid and several, destinations on smaller
+    boundaries, indices beyond either end (clamped)."""
+    import paper_1912_00167_b200 as ip
+    g = torch.Generator(device="cuda").manual_seed(row_bytes + n + offset)
+    src = torch.randint(0, 256, (57, row_bytes), dtype=torch.uint8, device="cuda", generator=g)
+    idx = torch.randint(-3, 60, (n,), dtype=torch.int32, device="cuda", generator=g)
+    guard = torch.full((n * row_bytes + 512,), 0xA5, dtype=torch.uint8, device="cuda")
+    dst = guard[256 + offset:256 + offset + n * row_bytes].view(n, row_bytes)
+    ip.impact_gather_rows(src, idx, dst)
+    torch.cuda.synchronize()
+    assert torch.equal(dst, src[idx.long().clamp(0, 56)])
+    assert bool((guard[:256 + offset] == 0xA5).all()) and bool((guard[256 + offset + n * row_bytes:] == 0xA5).all())
