@@ -32,7 +32,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     # (no unique symbols: a process that loads two copies of the library -- two versions, say -- would share what each kernel
     # remembers of its own configuration, and the second copy's launches would fail)
-    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC,-fno-gnu-unique",
+    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xfatbin", "-compress-all",
+             "-Xcompiler", "-fPIC,-fno-gnu-unique",
              "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if verbose:
         flags += ["-Xptxas", "-v"]

@@ -74,8 +74,8 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 }
 
 // ---- shape of the row passes ------------------------------------------------------------------------------------
-// kA > 0: the action count, known at compile time; a row belongs to one lane, which keeps its exponentials.
-// kA = kNarrow16, kNarrow32: at most 16 or 32 actions, one lane per row as well, the count a run-time value.
+// kA > 0: the action count, known at compile time (1 to 16 and 18); a row belongs to one lane, which keeps its exponentials.
+// kA = kNarrow32: at most 32 actions, one lane per row as well, the count a run-time value.
 // kA = kWideRows: any count; a row belongs to L = 2 ... 32 lanes that hold up to 32 elements each (vector i of lane g is
 //   the row's vector i L + g), and a warp works on its NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the
 //   warp is worked on in pass p by lanes [q L, q L + L) and owned -- for everything that is per step -- by lane q L + p
@@ -88,8 +88,12 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 // time: element by element -- such rows meet on no bank, their pairs on two; 250 000 steps of 9 actions with every
 // switch in use take 11.8 us instead of 12.4.)  Where rows meet on the same banks
 // (pitches with a large power of two), lanes take their vectors in rotated order; maxima and sums do not mind.
-constexpr int kNarrow16 = 0, kNarrow32 = -2, kWideRows = -1;
+constexpr int kNarrow32 = -2, kWideRows = -1;
 constexpr int kWideElems = 32;  // elements of a row that a lane holds at most
+__host__ __device__ constexpr bool is_atari(int A) { return A == 4 || A == 6 || A == 9 || A == 18; }
+// Trajectories of 2^32 steps and more that no room for aggregates lets split: with more actions than this they are wider
+// than any device's memory.
+constexpr int kLongestRows = 3;
 
 // The record of impact_buffer_device_step, read past L1 (an earlier launch may have left an older version there).
 __device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss_inputs* rec) {
@@ -116,15 +120,16 @@ template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLo
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid_constant__ LaunchForm sh) {
     constexpr bool kWide = kA == kWideRows, kFixed = kA > 0;
+    constexpr bool kRotated = kV == 4 && (!kFixed || kA % 8 == 0);  // (rows of 4 and 12 actions meet on no bank)
     constexpr bool kSingles = kV == 1 && kFixed && sizeof(LT) == 4;  // rows element by element
     constexpr bool kOdd = kV == 1 && !kSingles;
     constexpr int VW = kV == 1 ? 2 : kV;  // elements of a vector
-    constexpr int NV = (kFixed ? kA : (kA == kNarrow16 ? 16 : kWideElems)) / VW;  // vectors per lane at most
+    constexpr int NV = (kFixed ? kA : kWideElems) / VW;  // vectors per lane at most
     constexpr int NP = NV * VW / 2 + (kV == 1 ? 1 : 0);  // pairs: Blackwell's packed fp32 add / mul / fma work on two at once
     constexpr float kLowest = -3.402823466e38f;  // stands for an element that is not there: its exponential is 0
     static_assert(!kFixed || kA % VW == (kV == 1 ? 1 : 0), "whole vectors");
     const int A = kFixed ? kA : p.A;
-    const int NT = kFixed ? 128 : sh.nt;
+    const int NT = kWide ? sh.nt : 128;
     const int NTW = NT >> 2;  // rows of a tile that one warp works on
     const int S = sh.stages, W = sh.in_flight;
     const int in_row = A * (int)sizeof(LT), out_row = A * (int)sizeof(GT);
@@ -312,7 +317,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     const bool owner = kWide ? part < passes : true;
     const int row_vecs = A / VW;  // vectors of a row (odd counts: and one element)
     const int nvec = kFixed ? NV : (row_vecs + L - 1) >> log_l;  // of the lane with the most
-    const int rot = (kV == 4 && !kFixed) ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
+    const int rot = kRotated ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
 
     // The tile (in a flat launch only a block's first tile ends early, only its last one can begin late, and from one of
     // the group's tiles to its next, C tiles further back, every position changes by a constant).
@@ -320,7 +325,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     const unsigned int back = (unsigned int)(C * NT);
     TileRows tl = tile_now(grp);
     // (flat) the place of the lane's step
-    using Steps = typename std::conditional<kA == kNarrow16 && !kPlain, unsigned long long, unsigned int>::type;
+    using Steps = typename std::conditional<kFixed && kA <= kLongestRows && !kPlain, unsigned long long, unsigned int>::type;
     const Steps Tn = (Steps)g.T;
     const unsigned int back_traj = kLong ? 0u : (unsigned int)(back / Tn);
     const Steps back_rest = kLong ? (Steps)0 : back - back_traj * Tn;
@@ -443,7 +448,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         // byte offset of the lane's i-th vector from the row's first (of `elem`-byte elements)
         auto vec_at = [&](int i, int elem) {
             const int step = (VW * elem) << log_l;
-            return (kV == 4 && !kFixed) ? ((i * step) ^ (rot * step)) : i * step;
+            return kRotated ? ((i * step) ^ (rot * step)) : i * step;
         };
         auto vec_there = [&](int i) { return kFixed || (kWide ? (i << log_l) + part < row_vecs : i < row_vecs); };
         // (odd counts) does the row start on an odd element?  Tiles are an even number of rows apart.
@@ -761,7 +766,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     if (grp >= n_tiles) hand_over_sums();
     // ---- one group of the grid (block 0's, the one that runs out of tiles first and so is polling long before the
     // last rows appear) collects every block's row as it appears and writes the loss terms
-    // (in fp64, but for the compiled action counts on trajectories that fit a tile or are split, which add in fp32 as they
+    // (in fp64, but for the Atari action sets on trajectories that fit a tile or are split, which add in fp32 as they
     // always did: fp64 costs 0.15 to 0.3 us at the end of a launch)
     if (blockIdx.x == 0 && grp == n_tiles % C) {
         auto collect = [&](auto zero) {
@@ -770,7 +775,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                                                               k.steps_total, gtid, bar_id, &abort_s))
                 if (gtid == 0) atomicExch(p.counter + 1, 1u);
         };
-        if (!kFixed || (!kLong && g.T > 128)) collect(0.0);
+        if (!is_atari(kA) || (!kLong && g.T > 128)) collect(0.0);
         else collect(0.0f);
     }
     if (lane == 0) dev::bulk_store_wait_read();  // shared memory must outlive the stores' reads
@@ -822,24 +827,44 @@ inline bool is_plain(const CatParams& p) {
            p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
 }
 
+// How a warp's rows on 2^l lanes each meet on the banks, and the rotation that lanes of vectors of four elements take them in.
+// Returns the accesses that still meet.
+template <typename LT, int kV>
+int settle_rows(RowLayout& rl, int A, int l) {
+    constexpr int VW = kV == 1 ? 2 : kV;
+    rl.log_lanes = l;
+    const int passes = (rl.nt / 4 << l) / 32, vecs = A / VW;
+    const BankPattern b = bank_pattern(A * sizeof(LT) * (size_t)(passes < 1 ? 1 : passes), 1 << l, VW * (int)sizeof(LT));
+    rl.rot_mask = 0;
+    rl.rot_shift = b.shift;
+    if (kV == 4 && vecs % (1 << l) == 0) {
+        const int per_lane = vecs >> l;
+        while (2 * (rl.rot_mask + 1) <= b.ways && per_lane % (2 * (rl.rot_mask + 1)) == 0) rl.rot_mask = 2 * rl.rot_mask + 1;
+    }
+    return b.ways / (rl.rot_mask + 1);
+}
+
 // Consumer groups: four with every switch compiled in; five in the default configuration; six there for small action
 // sets, which are bound by arithmetic, not bytes.
-template <typename LT, typename GT, int A, int kV>
+template <typename LT, typename GT, int A>
 int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    constexpr int C = 4, CP = A <= 9 ? 6 : 5;
-    const bool plain = is_plain(p);
-    const RowLayout rl;
+    constexpr int C = 4, CP = A <= 9 ? 6 : 5, kV = A % 4 == 0 ? 4 : A % 2 == 0 ? 2 : 1;
+    const bool plain = is_plain(p), fits = fits_flat(p.geo);
+    RowLayout rl;
+    settle_rows<LT, kV>(rl, A, 0);
     if (p.indirect) {  // compiled for trajectories that fit a tile only
-        if (p.geo.T > 128) return IMPACT_ERR_UNSUPPORTED;
-        return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, true>(p, rl, di, stream)
-                     : launch_categorical<LT, GT, A, C, kV, false, false, true>(p, rl, di, stream);
+        if constexpr (is_atari(A)) {
+            if (p.geo.T > 128) return IMPACT_ERR_UNSUPPORTED;
+            return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, true>(p, rl, di, stream)
+                         : launch_categorical<LT, GT, A, C, kV, false, false, true>(p, rl, di, stream);
+        }
+        return IMPACT_ERR_UNSUPPORTED;
     }
-    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0) || !fits_flat(p.geo)) {
-        if (!p.tile_aggregates) return IMPACT_ERR_UNSUPPORTED;
+    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0) || (!fits && p.tile_aggregates))
         return launch_categorical<LT, GT, A, C, kV, false, true, false>(p, rl, di, stream);
-    }
-    return plain ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, rl, di, stream)
-                 : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, rl, di, stream);
+    if (!fits && A > kLongestRows) return IMPACT_ERR_UNSUPPORTED;
+    return plain && fits ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, rl, di, stream)
+                         : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, rl, di, stream);
 }
 
 // Rows of a tile where a row takes more than a lane: tiles of up to 36 KB (a ring of six stages, four of them being worked
@@ -874,8 +899,7 @@ int32_t run_runtime_form(const CatParams& p, const RowLayout& rl, bool plain, co
         }
         return launch_categorical<LT, GT, kA, C, kV, false, true, false>(p, rl, di, stream);
     }
-    if (!fits && kA != kNarrow16) return IMPACT_ERR_UNSUPPORTED;
-    plain = plain && fits;
+    if (!fits) return IMPACT_ERR_UNSUPPORTED;
     return plain ? launch_categorical<LT, GT, kA, CP, kV, true, false, false>(p, rl, di, stream)
                  : launch_categorical<LT, GT, kA, C, kV, false, false, false>(p, rl, di, stream);
 }
@@ -883,28 +907,14 @@ int32_t run_runtime_form(const CatParams& p, const RowLayout& rl, bool plain, co
 template <typename LT, typename GT, int kV>
 int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
     constexpr int VW = kV == 1 ? 2 : kV;
-    const int vecs = p.A / VW, access = VW * (int)sizeof(LT);
-    const size_t row = p.A * sizeof(LT);
+    const int vecs = p.A / VW;
     RowLayout rl;
-    // what is left of the bank conflicts of rows on 2^l lanes each, after rotating the order of a lane's vectors
-    auto settle = [&](int l) {
-        rl.log_lanes = l;
-        const int passes = (rl.nt / 4 << l) / 32;
-        const BankPattern b = bank_pattern(row * (size_t)(passes < 1 ? 1 : passes), 1 << l, access);
-        rl.rot_mask = 0;
-        rl.rot_shift = b.shift;
-        if (kV == 4 && vecs % (1 << l) == 0) {
-            const int per_lane = vecs >> l;
-            while (2 * (rl.rot_mask + 1) <= b.ways && per_lane % (2 * (rl.rot_mask + 1)) == 0) rl.rot_mask = 2 * rl.rot_mask + 1;
-        }
-        return b.ways / (rl.rot_mask + 1);
-    };
+    auto settle = [&](int l) { return settle_rows<LT, kV>(rl, p.A, l); };
     const bool plain = is_plain(p);
     if (p.A <= 32) {
         if (p.indirect) return IMPACT_ERR_UNSUPPORTED;
         rl.nt = 128;
         settle(0);
-        if (p.A <= 16) return run_runtime_form<LT, GT, kNarrow16, 4, 5, kV>(p, rl, plain, di, stream);
         return run_runtime_form<LT, GT, kNarrow32, 4, 4, kV>(p, rl, plain, di, stream);
     }
     // Rows of more than a lane: the fewest lanes that hold a row and do not meet on the banks more than two at a time.
@@ -923,14 +933,19 @@ int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t
 }
 
 template <typename LT, typename GT>
-int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    switch (p.A) {  // (the Atari action sets)
-        case 4: return run_fixed<LT, GT, 4, 4>(p, di, stream);
-        case 6: return run_fixed<LT, GT, 6, 2>(p, di, stream);
-        case 9: return run_fixed<LT, GT, 9, 1>(p, di, stream);
-        case 18: return run_fixed<LT, GT, 18, 2>(p, di, stream);
-        default: break;
+int32_t run_compiled_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    switch (p.A) {
+#define IMPACT_FIXED(n) case n: return run_fixed<LT, GT, n>(p, di, stream)
+        IMPACT_FIXED(1); IMPACT_FIXED(2); IMPACT_FIXED(3); IMPACT_FIXED(4); IMPACT_FIXED(5); IMPACT_FIXED(6);
+        IMPACT_FIXED(7); IMPACT_FIXED(8); IMPACT_FIXED(9); IMPACT_FIXED(10); IMPACT_FIXED(11); IMPACT_FIXED(12);
+        IMPACT_FIXED(13); IMPACT_FIXED(14); IMPACT_FIXED(15); IMPACT_FIXED(16); IMPACT_FIXED(18);
+#undef IMPACT_FIXED
+        default: return IMPACT_ERR_UNSUPPORTED;
     }
+}
+
+template <typename LT, typename GT>
+int32_t run_runtime_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
     if (p.A % 4 == 0) return run_runtime_width<LT, GT, 4>(p, di, stream);
     if (p.A % 2 == 0) return run_runtime_width<LT, GT, 2>(p, di, stream);
     return run_runtime_width<LT, GT, 1>(p, di, stream);

@@ -337,8 +337,7 @@ inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt,
     const int percent = wide_row == 0 ? 30 : (wide_row >= 48 && rounds > 1) ? 60 : 45;
     return 100 * g.B < percent * rounds * di->sm_count;
 }
-// Flat launches count a trajectory's steps in 32 bits, but for the form of at most sixteen actions with every switch
-// compiled in: longer trajectories are wider than any device's memory with more than two actions.
+// Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.
 inline bool fits_flat(const BatchGeometry& g) { return g.T < (1ll << 32) - 4096; }
 
 // Where a warp's accesses of `access_bytes`, `group` neighbouring lanes to a row and the rows `stride` bytes apart, fall
