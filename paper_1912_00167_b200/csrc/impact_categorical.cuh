@@ -803,13 +803,16 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     sh.lanes = ls.lanes;
     const size_t smem = (size_t)sh.stages * stage;
     static thread_local int configured_device = -1;
-    if (configured_device != di->device) {  // once per device: room for the largest ring any window setting asks for
-        IMPACT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, di->max_smem_optin - 4096));
+    if (configured_device != di->device) {
+        IMPACT_CUDA_TRY(configure_ring_kernel(kernel, di));
         configured_device = di->device;
     }
     // (rows wider than 32 actions: the companion gains nothing with fp32 logits and doubles a launch with bf16 ones
     // -- 27 against 14 us at 65 536 steps --, so such launches ask for their first tiles themselves)
-    WsPlan plan = ws_plan(ls.tiles, ls.grid, (size_t)nt * (2 * p.A * sizeof(LT) + 20), sh.in_flight, p.A <= 32);
+    // (nor where four groups have a tile each, all of which are asked for at once: 5 to 8 % slower at 600 x 128 steps)
+    const long long rows = p.geo.B * p.geo.T;
+    const bool one_round = C == 4 && 2 * rows < 9 * ls.grid * nt;
+    WsPlan plan = ws_plan(ls.tiles, ls.grid, (size_t)nt * (2 * p.A * sizeof(LT) + 20), sh.in_flight, p.A <= 32 && !one_round);
     if (kIndirect) { plan.companion = false; plan.prefetch_tiles = 0; }  // (addresses unknown on the host)
     if (plan.companion) {
         const int32_t st = launch_companion(p, (int)sizeof(LT), kLong, plan.prefetch_tiles, (int)ls.grid, stream);
