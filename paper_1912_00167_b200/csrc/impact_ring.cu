@@ -263,23 +263,30 @@ __device__ __forceinline__ int32_t nth_member(uint32_t word, uint32_t j) {
 // first free slot at or after the write cursor (none free: nothing happens, the event says FULL); (2) a live slot is
 // drawn and the inputs of the loss call are resolved into `inputs`.
 //
-// One launch does both.  Every block reads the state for itself (past L1: an earlier launch may have left an older
-// version there) and finds the slot of the push, which is all that its share of the copy needs; then it draws a ticket.
-// The block with the last ticket knows that every block has read the state, so it alone does the bookkeeping and writes
-// the new state -- nothing waits.  The launch is a chain of latencies (its start, the state, the candidate's pointers,
-// the copy): as two launches, one warp's bookkeeping and then the copy from a plan in device memory, it took 6.5 us of
-// a 16.3 us learner iteration of 131 072 steps.
-__global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ RingDeviceView v, const impact_ring_field_map map,
-                                                        const void* learner_logits, const float* values,
-                                                        const float* bootstrap_values, const void* const* sources,
-                                                        int32_t n_candidates, int32_t do_sample,
-                                                        impact_loss_inputs* inputs) {
+// One launch does both.  Every block reads the state for itself (past L1: an earlier launch may have left an older version
+// there) and works out the push's slot and the draw; then it draws a ticket.  The block with the last ticket knows that every
+// block has read the state, so it alone does the bookkeeping and writes the new state -- nothing waits.  The launch is a
+// chain of latencies: its start, the state, the ticket, its end.  So all of the state is asked for at once, what is kept
+// with each slot and the candidates' pointers among it (where they are no more than a block's threads), not only what turns
+// out to be needed; and blocks are few, because their tickets come from one word.  (An iteration of 131 072 steps of 18
+// actions, K = 4, with its loss: 12.1 us; 12.6 with two blocks per SM that asked for the drawn slot's count and pointer and
+// for the candidate's pointers once they knew which.  L2 asked for the drawn slot's fields in here: 12.2.)
+constexpr int kStepThreads = 512;
+__global__ void __launch_bounds__(kStepThreads) ring_step_kernel(const __grid_constant__ RingDeviceView v, const impact_ring_field_map map,
+                                                                 const void* learner_logits, const float* values,
+                                                                 const float* bootstrap_values, const void* const* sources,
+                                                                 int32_t n_candidates, int32_t do_sample,
+                                                                 impact_loss_inputs* inputs) {
     grid_dependency_wait();
     __shared__ uint32_t live_s[kMaxDeviceSlots / 32];
+    __shared__ int32_t count_s[kMaxDeviceSlots];
+    __shared__ unsigned long long fresh_s[kMaxDeviceSlots];
     __shared__ CopySegments plan_s;
-    __shared__ const void* cand_s[kMaxFields + 1];
+    __shared__ const void* cand_s[kStepThreads];
     __shared__ int32_t last_s;
     const int tid = threadIdx.x, lane = tid & 31;
+    const int width = v.n_fields + 1;  // pointers of a candidate
+    const bool all_candidates = sources && (long long)n_candidates * width <= kStepThreads;
     // (the header by every thread of the first warp: one request)
     RingDeviceHeader hd;
     if (tid < 32) {
@@ -288,51 +295,59 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
         hd.write_cursor = (int32_t)h0.x; hd.read_cursor = (int32_t)h0.y; hd.n_events = h0.z; hd.tickets = 0;
         hd.draws = ((uint64_t)h1.y << 32) | h1.x; hd.pushes = ((uint64_t)h1.w << 32) | h1.z;
     }
-    for (int32_t base = 0; base < kMaxDeviceSlots; base += (int32_t)blockDim.x) {
+    const void* cand = nullptr;
+    if (all_candidates && tid < n_candidates * width)
+        cand = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(sources) + tid));
+    for (int32_t base = 0; base < kMaxDeviceSlots; base += kStepThreads) {
         const int32_t s = base + tid;
         if (base >= v.N) {
             if (lane == 0) live_s[s >> 5] = 0u;
             continue;
         }
-        const uint32_t word = __ballot_sync(0xFFFFFFFFu, s < v.N && __ldcg(v.valid + s) != 0);
+        const bool there = s < v.N;
+        const int32_t valid = there ? __ldcg(v.valid + s) : 0;
+        const int32_t count = there ? __ldcg(v.count + s) : 0;
+        const unsigned long long fresh = there ? __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh) + s) : 0ull;
+        const uint32_t word = __ballot_sync(0xFFFFFFFFu, valid != 0);
         if (lane == 0) live_s[s >> 5] = word;
+        if (there) { count_s[s] = count; fresh_s[s] = fresh; }
     }
-    // (the candidate's pointers are on their way while the slots are worked out)
-    unsigned long long cand = 0;
-    if (tid < 32 && sources && lane <= v.n_fields)
-        cand = __ldcg(reinterpret_cast<const unsigned long long*>(
-            sources + (size_t)(hd.pushes % (uint64_t)n_candidates) * (size_t)(v.n_fields + 1) + lane));
+    if (all_candidates) cand_s[tid] = cand;
     __syncthreads();
     uint32_t live = 0;
     int32_t slot = -1, pick = -1, drawn_count = 0;
-    unsigned long long drawn_fresh = 0;
+    const void* drawn_fresh = nullptr;
+    int first_cand = 0;  // of the candidate's pointers in cand_s
     if (tid < 32) {
         live = live_s[lane];
         const int32_t left = v.N - 32 * lane;  // slots that exist in this lane's word
         const uint32_t exist = left >= 32 ? 0xFFFFFFFFu : (left > 0 ? (1u << left) - 1u : 0u);
         if (sources) slot = first_at_or_after(~live & exist, hd.write_cursor);
-        if (slot >= 0 && lane == (slot >> 5)) live |= 1u << (slot & 31);
-        // the draw too is worked out by every block, so that what is kept with the drawn slot has arrived by the time
-        // the last block is known
+        if (slot >= 0) {
+            const uint64_t c = hd.pushes % (uint64_t)n_candidates;
+            if (all_candidates) first_cand = (int)c * width;
+            else if (lane < width) cand_s[lane] = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(sources) + c * (uint64_t)width + lane));
+            __syncwarp();
+            if (lane == (slot >> 5)) live |= 1u << (slot & 31);
+        }
+        // the draw too is worked out by every block, so that it is done by the time the last one is known
         const uint32_t n_live = (uint32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
         if (do_sample && n_live > 0)
             pick = v.mode == IMPACT_SAMPLE_UNIFORM  // floor(u * live / 2^64)
                        ? nth_member(live, (uint32_t)__umul64hi(splitmix64_at_dev(v.seed, hd.draws), (uint64_t)n_live))
                        : first_at_or_after(live, hd.read_cursor);
-        if (pick >= 0 && pick != slot) {
-            drawn_count = __ldcg(v.count + pick);
-            drawn_fresh = __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh + pick));
+        if (pick >= 0) {  // (drawn as it is pushed: nothing is kept with it yet)
+            drawn_count = pick == slot ? 0 : count_s[pick];
+            drawn_fresh = pick == slot ? cand_s[first_cand + v.n_fields] : reinterpret_cast<const void*>(fresh_s[pick]);
         }
-        if (lane <= v.n_fields) cand_s[lane] = reinterpret_cast<const void*>(cand);
-        __syncwarp();
-        if (pick == slot) drawn_fresh = reinterpret_cast<unsigned long long>(cand_s[v.n_fields]);  // (drawn as it is pushed)
         if (lane == 0) {
             int n = 0;
             unsigned long long units = 0;
             if (slot >= 0) {
                 for (int f = 0; f < v.n_fields; ++f) {
-                    if (!cand_s[f]) continue;
-                    plan_s.src[n] = static_cast<const char*>(cand_s[f]);
+                    const void* const from = cand_s[first_cand + f];
+                    if (!from) continue;
+                    plan_s.src[n] = static_cast<const char*>(from);
                     plan_s.dst[n] = v.storage + (unsigned long long)slot * v.slot_stride + v.field_offset[f];
                     plan_s.bytes[n] = v.field_bytes[f];
                     units += (v.field_bytes[f] + 15ull) / 16ull;
@@ -355,7 +370,7 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
     if (sources) {
         if (slot >= 0) {
             if (lane == 0) {
-                v.fresh[slot] = reinterpret_cast<uint64_t>(cand_s[v.n_fields]);
+                v.fresh[slot] = reinterpret_cast<uint64_t>(cand_s[first_cand + v.n_fields]);
                 v.valid[slot] = 1;
                 v.count[slot] = 0;
             }
@@ -374,7 +389,7 @@ __global__ void __launch_bounds__(256) ring_step_kernel(const __grid_constant__ 
             int32_t k_before = 0;
             if (pick >= 0) {
                 k_before = drawn_count;
-                const void* const fresh = reinterpret_cast<const void*>(drawn_fresh);
+                const void* const fresh = drawn_fresh;
                 v.count[pick] = k_before + 1;
                 if (k_before + 1 >= v.K) v.valid[pick] = 0;
                 auto field = [&](int32_t f) -> const void* {
@@ -725,12 +740,12 @@ extern "C" int32_t impact_buffer_device_step(impact_buffer* h, const impact_ring
     if (push_sources) {
         unsigned long long units = 0;
         for (int f = 0; f < h->n_fields; ++f) units += (h->field_bytes[f] + 15) / 16;
-        // (a grid of two blocks per SM: most steps find every slot live and copy nothing, and an empty launch should
-        // cost as little as possible)
-        blocks = blocks_for(units, 4, di);
-        if (blocks > 2 * di->sm_count) blocks = 2 * di->sm_count;
+        // (a block per SM: most steps find every slot live and copy nothing, and an empty launch should cost as little as
+        // possible)
+        blocks = blocks_for(units, 4, di, kStepThreads);
+        if (blocks > di->sm_count) blocks = di->sm_count;
     }
-    IMPACT_CUDA_TRY(launch_serialized(ring_step_kernel, dim3(blocks), dim3(256), 0, cs, v, m, learner_logits, values,
+    IMPACT_CUDA_TRY(launch_serialized(ring_step_kernel, dim3(blocks), dim3(kStepThreads), 0, cs, v, m, learner_logits, values,
                                       bootstrap_values, push_sources, n_candidates, inputs_out ? 1 : 0, inputs_out));
     return IMPACT_OK;
 }
