@@ -7,6 +7,7 @@ GPU or a non-zero status raises.
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 import struct
 from dataclasses import dataclass
@@ -92,12 +93,13 @@ assert _CALL.size == ctypes.sizeof(impact_loss_call)
 
 _lib = None
 _call_packed = None
+_loss_direct = None  # the direct loss call's arguments checked in native code (csrc/marshal.cpp)
 _vp, _i32, _i64, _f32, _sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_float, ctypes.c_size_t
 
 
 def load_library() -> ctypes.CDLL:
     """Loads libimpact.so; raises if it has not been built (there is no other code path)."""
-    global _lib, _call_packed
+    global _lib, _call_packed, _loss_direct
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -169,6 +171,9 @@ def load_library() -> ctypes.CDLL:
     _call_packed = lib["impact_loss_fwd_bwd_call"]
     _call_packed.restype = _i32
     _call_packed.argtypes = [ctypes.c_char_p, _vp]
+    marshal = importlib.import_module("._marshal", __package__)
+    marshal.bind(ctypes.cast(lib.impact_loss_fwd_bwd_call, _vp).value)
+    _loss_direct = marshal.loss
     _lib = lib
     return lib
 
@@ -364,8 +369,18 @@ def impact_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rew
                         bootstrap_values, coef: Coefficients, *, loss_terms, dlogits, dvalues,
                         vtarget=None, advantage=None, workspace, target_logits_copy=None, stream=None) -> None:
     """Enqueues the categorical IMPACT loss + gradients on `stream` (see include/impact.h)."""
-    # The usual call: every argument as it should be, checked in a row and packed at once.  Anything else goes the way
-    # of a prepared call, which names the argument at fault.
+    # The usual call: plain tensors, every argument as it should be, checked in native code.  What that leaves (None) --
+    # subclasses, numbers of other types, arguments at fault -- is checked here in a row and packed at once; what still is
+    # not as it should be goes the way of a prepared call, which names the argument at fault.
+    if _lib is None:
+        load_library()
+    st = _loss_direct(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values, bootstrap_values, coef,
+                      loss_terms, dlogits, dvalues, vtarget, advantage, workspace, target_logits_copy,
+                      None if stream is None else _stream(stream))
+    if st is not None:
+        if st != OK:
+            _check(st, "impact_loss_fwd_bwd_call")
+        return
     try:
         shape = learner_logits.shape
         B, T, A = shape
@@ -390,8 +405,6 @@ def impact_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rew
     except (AttributeError, KeyError, TypeError, ValueError, OverflowError, struct.error):
         packed = None
     if packed is not None:
-        if _lib is None:
-            load_library()
         st = _call_packed(packed, _stream(stream))
         if st != OK:
             _check(st, "impact_loss_fwd_bwd_call")

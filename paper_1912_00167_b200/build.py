@@ -1,10 +1,11 @@
-"""Builds libimpact.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libimpact.so (the C-ABI library) in-tree with nvcc for sm_100a, and the binding's native part beside it."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 import tempfile
 from concurrent.futures import ThreadPoolExecutor
 
@@ -12,6 +13,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libimpact.so")
+MARSHAL = os.path.join(PKG, "_marshal.so")
 
 
 def sources() -> list[str]:
@@ -19,11 +21,26 @@ def sources() -> list[str]:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(MARSHAL)):
         return True
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.cpp")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
     deps += glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps)
+    return any(os.path.getmtime(d) > min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL)) for d in deps)
+
+
+def build_marshal() -> None:
+    """The native part of the Python binding (csrc/marshal.cpp), against the headers and libraries of the installed torch."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    tmp = MARSHAL + ".tmp.%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fno-gnu-unique", "-DNDEBUG",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), "-I", os.path.join(ROOT, "include"),
+                           "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(root, "include"),
+                           "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                           "-isystem", os.path.join(cuda, "include"), os.path.join(CSRC, "marshal.cpp"), "-o", tmp,
+                           "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, MARSHAL)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -44,7 +61,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
             subprocess.check_call([nvcc, *flags, "-c", "-o", obj, src])
             return obj
         with ThreadPoolExecutor(max_workers=os.cpu_count() or 1) as pool:
+            marshal = pool.submit(build_marshal)
             done = list(pool.map(compile_one, sources()))
+            marshal.result()
         subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp, *done])
     os.replace(tmp, LIB)
     return LIB
