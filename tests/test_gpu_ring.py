@@ -396,3 +396,34 @@ def test_gather_rows_around_the_granules(row_bytes, n, offset):
     torch.cuda.synchronize()
     assert torch.equal(dst, src[idx.long().clamp(0, 56)])
     assert bool((guard[:256 + offset] == 0xA5).all()) and bool((guard[256 + offset + n * row_bytes:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("sizes", [(4, 20, 5000), (16, 6400, 6401, 115200), (300000, 200000, 24272), (300000, 200000, 24304)])
+@pytest.mark.parametrize("memory", ["pinned", "pageable", "pinned off a boundary", "mixed", "absent"])
+def test_push_from_host_memory_of_every_kind(sizes, memory):
+    """Host batches that a kernel reads in place (pinned, on 16-byte boundaries, up to 512 KB) and those that are copied: both
+    give the bytes, and a buffer may be refilled once the push is complete."""
+    import paper_1912_00167_b200 as ip
+
+    def host(n, i):
+        t = torch.empty(n + 64, dtype=torch.uint8)
+        if memory != "pageable" and not (memory == "mixed" and i == 1):
+            t = t.pin_memory()
+        return t[4:4 + n] if memory == "pinned off a boundary" else t[:n]
+
+    src = [host(n, i) for i, n in enumerate(sizes)]
+    ring = ip.ImpactBuffer(2, 1, list(sizes), sample_mode=ip.binding.SAMPLE_ROUND_ROBIN)
+    for round_ in range(3):
+        want = [torch.randint(0, 256, (n,), dtype=torch.uint8) for n in sizes]
+        for s, w in zip(src, want):
+            s.copy_(w)
+        given = [None if memory == "absent" and i == 1 else s for i, s in enumerate(src)]
+        slot = ring.push(given)
+        torch.cuda.synchronize()
+        for s in src:
+            s.fill_(7)
+        got = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in sizes]
+        assert ring.sample(gather_dst=got) == (slot, 0)
+        for i, (g, w) in enumerate(zip(got, want)):
+            assert given[i] is None or torch.equal(g.cpu(), w)
+    ring.close()
