@@ -543,45 +543,52 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const float is = dev::reciprocal(sum_l);
             float klr = 0.0f, ist = 0.0f;
             if (want_kl) {
-                // kept: KL = sum_j e^t_j ((zt_j - m_t) - (zl_j - m_l)) / S_t + ln S_l - ln S_t.  What the logits of a row have
-                // in common cancels before anything is rounded at its size.
-                // otherwise: in natural units, action by action.
-                // (An action masked by the type's lowest value in both rows counts 0 times a finite difference in both; in
-                // base 2 its log-probabilities overflow and the difference is no number.)
-                const float lse_t = fmaf(lgt, kLn2, m_t), lse_l = fmaf(lgl, kLn2, m_l);
-                float2 skl2 = make_float2(0.0f, 0.0f);
-                auto add_kl = [&](const float2& zt, const float2& zl, int pair) {
-                    if constexpr (kKeepTarget) {
-                        const float2 dt = __fadd2_rn(zt, make_float2(-m_t, -m_t)), dl = __fadd2_rn(zl, make_float2(-m_l, -m_l));
-                        skl2 = __ffma2_rn(et[pair], __ffma2_rn(dl, make_float2(-1.0f, -1.0f), dt), skl2);
-                    } else {
-                        auto one = [&](float a, float b) {
-                            const float lpt = __fadd_rn(a, -lse_t);
-                            klr = fmaf(dev::exp2_fast(__fmul_rn(lpt, kLog2e)), __fadd_rn(lpt, -__fadd_rn(b, -lse_l)), klr);
-                        };
-                        one(zt.x, zl.x);
-                        if (kV != 1 || pair != NP - 1) one(zt.y, zl.y);
-                    }
-                };
                 const unsigned char* const row = s1 + r * in_row;
                 const unsigned char* const at = row + (first_of(r) + part * VW) * (int)sizeof(LT);
-#pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    if (!vec_there(i)) continue;
-                    float zt[VW];
+                auto target_vec = [&](int i, float (&zt)[VW]) {
                     if constexpr (kSingles) { zt[0] = get_element<LT>(row, 2 * i); zt[1] = get_element<LT>(row, 2 * i + 1); }
                     else Vec<LT, VW>::ld(at + vec_at(i, (int)sizeof(LT)), zt);
-#pragma unroll
-                    for (int v = 0; v < VW; v += 2) add_kl(make_float2(zt[v], zt[v + 1]), z[(i * VW + v) / 2], (i * VW + v) / 2);
-                }
-                if (kV == 1 && (!kWide || part == 0)) {  // (the pair's other element is in neither row)
-                    const float zt = get_element<LT>(row, single_of(r));
-                    add_kl(make_float2(zt, kLowest), make_float2(z[NP - 1].x, kLowest), NP - 1);
-                }
-                if (kWide) for (int o = 1; o < L; o <<= 1) klr += __shfl_xor_sync(0xffffffffu, klr, o);
+                };
+                // (An action masked by the type's lowest value in both rows counts 0 times a finite difference in both forms; in
+                // base 2 its log-probabilities overflow and the difference is no number.)
                 if constexpr (kKeepTarget) {
+                    // KL = sum_j e^t_j ((zt_j - m_t) - (zl_j - m_l)) / S_t + ln S_l - ln S_t.  What the logits of a row have in
+                    // common cancels before anything is rounded at its size.
+                    float2 skl2 = make_float2(0.0f, 0.0f);
+                    auto add_kl = [&](const float2& zt, const float2& zl, int pair) {
+                        const float2 dt = __fadd2_rn(zt, make_float2(-m_t, -m_t)), dl = __fadd2_rn(zl, make_float2(-m_l, -m_l));
+                        skl2 = __ffma2_rn(et[pair], __ffma2_rn(dl, make_float2(-1.0f, -1.0f), dt), skl2);
+                    };
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) {
+                        float zt[VW];
+                        target_vec(i, zt);
+#pragma unroll
+                        for (int v = 0; v < VW; v += 2) add_kl(make_float2(zt[v], zt[v + 1]), z[(i * VW + v) / 2], (i * VW + v) / 2);
+                    }
+                    if (kV == 1)  // (the pair's other element is in neither row)
+                        add_kl(make_float2(get_element<LT>(row, single_of(r)), kLowest), make_float2(z[NP - 1].x, kLowest), NP - 1);
                     ist = dev::reciprocal(sum_t);
                     klr = fmaf(skl2.x + skl2.y, ist, __fmul_rn(lgl - lgt, kLn2));
+                } else {  // in natural units, action by action
+                    const float lse_t = fmaf(lgt, kLn2, m_t), lse_l = fmaf(lgl, kLn2, m_l);
+                    auto add_kl = [&](float zt, float zl) {
+                        const float lpt = __fadd_rn(zt, -lse_t);
+                        klr = fmaf(dev::exp2_fast(__fmul_rn(lpt, kLog2e)), __fadd_rn(lpt, -__fadd_rn(zl, -lse_l)), klr);
+                    };
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) {
+                        if (!vec_there(i)) continue;
+                        float zt[VW];
+                        target_vec(i, zt);
+#pragma unroll
+                        for (int v = 0; v < VW; v += 2) {
+                            add_kl(zt[v], z[(i * VW + v) / 2].x);
+                            add_kl(zt[v + 1], z[(i * VW + v) / 2].y);
+                        }
+                    }
+                    if (kV == 1 && (!kWide || part == 0)) add_kl(get_element<LT>(row, single_of(r)), z[NP - 1].x);
+                    if (kWide) for (int o = 1; o < L; o <<= 1) klr += __shfl_xor_sync(0xffffffffu, klr, o);
                 }
             }
             if (!kWide || part == pass) {
