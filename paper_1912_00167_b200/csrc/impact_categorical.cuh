@@ -74,8 +74,7 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 }
 
 // ---- shape of the row passes ------------------------------------------------------------------------------------
-// kA > 0: the action count, known at compile time (1 to 16 and 18); a row belongs to one lane, which keeps its exponentials.
-// kA = kNarrow32: at most 32 actions, one lane per row as well, the count a run-time value.
+// kA > 0: the action count, known at compile time (1 to 32); a row belongs to one lane, which keeps its exponentials.
 // kA = kWideRows: any count; a row belongs to L = 2 ... 32 lanes that hold up to 32 elements each (vector i of lane g is
 //   the row's vector i L + g), and a warp works on its NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the
 //   warp is worked on in pass p by lanes [q L, q L + L) and owned -- for everything that is per step -- by lane q L + p
@@ -88,7 +87,7 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 // time: element by element -- such rows meet on no bank, their pairs on two; 250 000 steps of 9 actions with every
 // switch in use take 11.8 us instead of 12.4.)  Where rows meet on the same banks
 // (pitches with a large power of two), lanes take their vectors in rotated order; maxima and sums do not mind.
-constexpr int kNarrow32 = -2, kWideRows = -1;
+constexpr int kWideRows = -1;
 constexpr int kWideElems = 32;  // elements of a row that a lane holds at most
 __host__ __device__ constexpr bool is_atari(int A) { return A == 4 || A == 6 || A == 9 || A == 18; }
 // Trajectories of 2^32 steps and more that no room for aggregates lets split: with more actions than this they are wider
@@ -885,10 +884,11 @@ int settle_rows(RowLayout& rl, int A, int l) {
 }
 
 // Consumer groups: four with every switch compiled in; five in the default configuration; six there for small action
-// sets, which are bound by arithmetic, not bytes.
+// sets, which are bound by arithmetic, not bytes.  One and two fewer where the rows' exponentials take 19 to 32 registers
+// (128 to a thread with three groups, 96 with four).
 template <typename LT, typename GT, int A>
 int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    constexpr int C = 4, CP = A <= 9 ? 6 : 5, kV = A % 4 == 0 ? 4 : A % 2 == 0 ? 2 : 1;
+    constexpr int C = A <= 18 ? 4 : 3, CP = A <= 9 ? 6 : A <= 18 ? 5 : 4, kV = A % 4 == 0 ? 4 : A % 2 == 0 ? 2 : 1;
     const bool plain = is_plain(p), fits = fits_flat(p.geo);
     RowLayout rl;
     settle_rows<LT, kV>(rl, A, 0);
@@ -951,12 +951,6 @@ int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t
     RowLayout rl;
     auto settle = [&](int l) { return settle_rows<LT, kV>(rl, p.A, l); };
     const bool plain = is_plain(p);
-    if (p.A <= 32) {
-        if (p.indirect) return IMPACT_ERR_UNSUPPORTED;
-        rl.nt = 128;
-        settle(0);
-        return run_runtime_form<LT, GT, kNarrow32, 4, 4, kV>(p, rl, plain, di, stream);
-    }
     // Rows of more than a lane: the fewest lanes that hold a row and do not meet on the banks more than two at a time.
     rl.nt = wide_tile_rows(p.geo, p.tile_aggregates, p.A, sizeof(LT), sizeof(GT), di);
     int l = 1;
@@ -979,6 +973,16 @@ int32_t run_compiled_count(const CatParams& p, const DeviceInfo* di, cudaStream_
         IMPACT_FIXED(1); IMPACT_FIXED(2); IMPACT_FIXED(3); IMPACT_FIXED(4); IMPACT_FIXED(5); IMPACT_FIXED(6);
         IMPACT_FIXED(7); IMPACT_FIXED(8); IMPACT_FIXED(9); IMPACT_FIXED(10); IMPACT_FIXED(11); IMPACT_FIXED(12);
         IMPACT_FIXED(13); IMPACT_FIXED(14); IMPACT_FIXED(15); IMPACT_FIXED(16); IMPACT_FIXED(18);
+        default: return IMPACT_ERR_UNSUPPORTED;
+    }
+}
+
+template <typename LT, typename GT>
+int32_t run_larger_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    switch (p.A) {
+        IMPACT_FIXED(17); IMPACT_FIXED(19); IMPACT_FIXED(20); IMPACT_FIXED(21); IMPACT_FIXED(22); IMPACT_FIXED(23);
+        IMPACT_FIXED(24); IMPACT_FIXED(25); IMPACT_FIXED(26); IMPACT_FIXED(27); IMPACT_FIXED(28); IMPACT_FIXED(29);
+        IMPACT_FIXED(30); IMPACT_FIXED(31); IMPACT_FIXED(32);
 #undef IMPACT_FIXED
         default: return IMPACT_ERR_UNSUPPORTED;
     }

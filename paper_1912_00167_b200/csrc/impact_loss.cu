@@ -165,7 +165,8 @@ extern "C" int32_t impact_loss_workspace_status(const void* workspace, size_t wo
 
 template <typename LT, typename GT>
 static int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t s) {
-    return is_compiled_count(p.A) ? run_compiled_count<LT, GT>(p, di, s) : run_runtime_count<LT, GT>(p, di, s);
+    return is_compiled_count(p.A) ? run_compiled_count<LT, GT>(p, di, s)
+           : is_larger_count(p.A) ? run_larger_count<LT, GT>(p, di, s) : run_runtime_count<LT, GT>(p, di, s);
 }
 static int32_t run_typed(const CatParams& p, bool logits_bf16, bool grads_bf16, const DeviceInfo* di, cudaStream_t s) {
     if (!logits_bf16 && !grads_bf16) return run_categorical<float, float>(p, di, s);

@@ -97,11 +97,16 @@ struct LossInputPointers {
 };
 
 // Picks the kernel for a categorical call (`p` complete except for geo.nt and what follows it) and launches it.  Every count
-// up to 16, and 18, is compiled in: told at run time, a row of 1 to 16 actions takes a warp some 200 to 350 instructions more
-// for tests of what is there (a million steps of 7 actions in fp32 24.3 against 20.2 us, of 2 actions 46.9 against 30.1).
+// up to 32 is compiled in, in two kinds of translation units: told at run time, a row of 1 to 16 actions takes a warp some 200
+// to 350 instructions more for tests of what is there (926 000 steps of 7 actions in fp32 24.3 against 20.2 us, 2.1 million of
+// 2 actions 46.9 against 30.1), one of 17 to 32 takes 1.1 to 1.2 times as long in fp32, 1.3 to 1.5 in bf16 (20 actions 21.2
+// against 17.5 us, in bf16 21.5 against 15.6, with every switch 33.0 against 20.5).
 constexpr bool is_compiled_count(int A) { return A <= 16 || A == 18; }
+constexpr bool is_larger_count(int A) { return A <= 32; }
 template <typename LT, typename GT>
 int32_t run_compiled_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <typename LT, typename GT>
+int32_t run_larger_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
 template <typename LT, typename GT>
 int32_t run_runtime_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
 
