@@ -369,7 +369,9 @@ int32_t impact_buffer_destroy(impact_buffer* h);
  * of n_fields pointers; a NULL entry leaves that field for a later impact_buffer_append)
  * into it on `stream`, sets its traversal count to 0 and returns the slot in *slot_out.
  * src_location: IMPACT_SRC_DEVICE (one fused copy kernel) or IMPACT_SRC_HOST (one
- * cudaMemcpyAsync per field; use pinned memory to stay asynchronous).
+ * cudaMemcpyAsync per field, or, up to 512 KB of pinned memory on 16-byte boundaries, one kernel
+ * that reads it in place; use pinned memory to stay asynchronous, and leave it as it is until the
+ * stream has passed the push).
  * Returns IMPACT_ERR_FULL, with nothing copied, when no slot is free.
  */
 int32_t impact_buffer_push(impact_buffer* h, const void* const* field_src, int32_t src_location,
