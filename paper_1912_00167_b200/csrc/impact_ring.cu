@@ -14,6 +14,7 @@
 
 #include "impact.h"
 #include "impact_internal.h"
+#include "impact_pinned.h"
 
 namespace impact {
 namespace {
@@ -579,19 +580,6 @@ static int32_t launch_copy(const CopySegments& segs, cudaStream_t stream) {
 // copy per field (four fields, a push of 26 KB 27.6 -> 16.4 us from the call to its end, 500 KB 33 -> 27; 1 MB 43 / 46: larger
 // ones stay with the copy engine).
 constexpr size_t kMostReadInPlace = 512 * 1024;
-// May a kernel read these bytes where they are?  Pinned host memory, mapped for the device, from the first byte to the last;
-// *out is its address there.
-static bool pinned_address(const void* p, size_t bytes, const void** out) {
-    cudaPointerAttributes first = {}, last = {};
-    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();  // (an address that CUDA does not know is no error of this call)
-        return false;
-    }
-    *out = first.devicePointer;
-    return first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer &&
-           static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) == (ptrdiff_t)(bytes - 1);
-}
 // Not in a capture either: what a graph copies at its replays stays a copy of the graph's.
 static bool is_capturing(cudaStream_t stream) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -640,10 +628,9 @@ extern "C" int32_t impact_buffer_push(impact_buffer* h, const void* const* field
             if (field_src[f]) { total += h->field_bytes[f]; in_place = in_place && aligned16(field_src[f]); }
         in_place = in_place && total <= kMostReadInPlace && !is_capturing(cs);
         for (int f = 0; f < h->n_fields && in_place; ++f) {
-            const void* from = nullptr;
             if (!field_src[f]) continue;
-            in_place = pinned_address(field_src[f], h->field_bytes[f], &from);
-            if (in_place) add_segment(segs, from, h->field_ptr(slot, f), h->field_bytes[f]);
+            in_place = pinned_in_one_range(field_src[f], h->field_bytes[f]);
+            if (in_place) add_segment(segs, field_src[f], h->field_ptr(slot, f), h->field_bytes[f]);
         }
         if (in_place) {
             const int32_t st = launch_copy<true>(segs, cs);

@@ -36,6 +36,19 @@ def test_a_stage_is_handed_back_behind_the_whole_warps_reads():
         assert uses and all("hand_back_stage(" in line for line in uses), uses
 
 
+def test_bytes_outside_one_range_are_not_read_in_place(tmp_path):
+    """A kernel reads host memory only where all of it lies in one pinned range: the arithmetic of that."""
+    done = subprocess.run([_host_program(tmp_path, "pinned_check")], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout
+
+
+@pytest.mark.gpu
+def test_what_counts_as_one_pinned_range(tmp_path):
+    """Allocations and registrations, and two registrations with a hole between them (pointers only, nothing is read)."""
+    done = subprocess.run([_host_program(tmp_path, "pinned_check"), "driver"], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout + done.stderr
+
+
 @pytest.mark.gpu
 def test_a_wait_that_gives_up_raises_the_error_word(tmp_path):
     """Waits for a value that nothing ever brings return after their limit and say so in the workspace's error word."""
