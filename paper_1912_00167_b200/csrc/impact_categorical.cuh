@@ -552,10 +552,16 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 // base 2 its log-probabilities overflow and the difference is no number.)
                 if constexpr (kKeepTarget) {
                     // KL = sum_j e^t_j ((zt_j - m_t) - (zl_j - m_l)) / S_t + ln S_l - ln S_t.  What the logits of a row have in
-                    // common cancels before anything is rounded at its size.
+                    // common cancels before anything is rounded at its size.  Differences are taken a sixteenth as large,
+                    // which rounds nothing: where the learner alone masks actions by the type's lowest value they are as
+                    // large as a float gets, and the sum of up to 14 of them, each times at most 1, has to stay one.
+                    static_assert(!kKeepTarget || kA <= 16, "sixteenths");
+                    constexpr float kPart = 1.0f / 16.0f;
                     float2 skl2 = make_float2(0.0f, 0.0f);
+                    const float2 part2 = make_float2(kPart, kPart);
+                    const float2 part_t2 = make_float2(-kPart * m_t, -kPart * m_t), part_l2 = make_float2(-kPart * m_l, -kPart * m_l);
                     auto add_kl = [&](const float2& zt, const float2& zl, int pair) {
-                        const float2 dt = __fadd2_rn(zt, make_float2(-m_t, -m_t)), dl = __fadd2_rn(zl, make_float2(-m_l, -m_l));
+                        const float2 dt = __ffma2_rn(zt, part2, part_t2), dl = __ffma2_rn(zl, part2, part_l2);
                         skl2 = __ffma2_rn(et[pair], __ffma2_rn(dl, make_float2(-1.0f, -1.0f), dt), skl2);
                     };
 #pragma unroll
@@ -568,7 +574,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                     if (kV == 1)  // (the pair's other element is in neither row)
                         add_kl(make_float2(get_element<LT>(row, single_of(r)), kLowest), make_float2(z[NP - 1].x, kLowest), NP - 1);
                     ist = dev::reciprocal(sum_t);
-                    klr = fmaf(skl2.x + skl2.y, ist, __fmul_rn(lgl - lgt, kLn2));
+                    klr = fmaf(skl2.x + skl2.y, __fmul_rn(ist, 1.0f / kPart), __fmul_rn(lgl - lgt, kLn2));
                 } else {  // in natural units, action by action
                     const float lse_t = fmaf(lgt, kLn2, m_t), lse_l = fmaf(lgl, kLn2, m_l);
                     auto add_kl = [&](float zt, float zl) {
