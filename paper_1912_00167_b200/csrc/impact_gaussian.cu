@@ -556,8 +556,8 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
     sh.rot_mask = rl.rot_mask;
     const size_t smem = (size_t)sh.stages * stage;
     static thread_local int configured_device = -1;
-    if (configured_device != di->device) {
-        IMPACT_CUDA_TRY(configure_ring_kernel(kernel, di));
+    if (configured_device != di->device) {  // once per device: room for the largest ring any window setting asks for
+        IMPACT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, di->max_smem_optin - 4096));
         configured_device = di->device;
     }
     sh.n_prefetch = ws_plan(ls.tiles, ls.grid, (size_t)nt * (5 * p.D * sizeof(float) + 16), sh.in_flight, false).prefetch_tiles;
