@@ -845,8 +845,12 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     sh.lanes = ls.lanes;
     const size_t smem = (size_t)sh.stages * stage;
     static thread_local int configured_device = -1;
+    static thread_local size_t own_smem = 0;  // (the kernel's static arrays)
     if (configured_device != di->device) {  // once per device: room for the largest ring any window setting asks for
         IMPACT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, di->max_smem_optin - 4096));
+        cudaFuncAttributes a;
+        IMPACT_CUDA_TRY(cudaFuncGetAttributes(&a, kernel));
+        own_smem = a.sharedSizeBytes;
         configured_device = di->device;
     }
     // (rows wider than 32 actions: the companion gains nothing with fp32 logits and doubles a launch with bf16 ones
@@ -862,14 +866,8 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     } else {
         sh.n_prefetch = plan.prefetch_tiles;
     }
-    // Beside a companion the SM's whole shared memory is laid out as such.  By itself the driver picks the smallest layout that
-    // a block fits; where that leaves less than the kilobyte that any other block needs, the companion of the next launch
-    // cannot become resident beside this one: all its blocks start on the first SMs that come free, whose copy engines then ask
-    // L2 for the whole batch (1024 x 128 steps of 16 actions with every switch 24 us, 8.5 so).  Other launches keep the L1 that
-    // the smallest layout leaves, for the per-step arrays: with the whole of it as shared memory 14 x 2091 steps of 64 actions
-    // take 14.8 us instead of 13.4 (with every switch), 31 x 4000 of 32 actions 22.8 instead of 20.1, in the Gaussian's kernels
-    // 28 012 x 28 of 3 dimensions 19.3 instead of 18.9.
-    IMPACT_CUDA_TRY(launch_laid_out(plan.companion, kernel, dim3((unsigned)ls.grid), dim3(C * 128 + 32), smem, stream, p, sh));
+    const int shared_percent = plan.companion ? percent_beside_companion(smem + own_smem, di) : -1;
+    IMPACT_CUDA_TRY(launch_laid_out(shared_percent, kernel, dim3((unsigned)ls.grid), dim3(C * 128 + 32), smem, stream, p, sh));
     return IMPACT_OK;
 }
 

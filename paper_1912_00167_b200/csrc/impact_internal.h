@@ -18,6 +18,7 @@ struct DeviceInfo {
     int device = -1;
     int sm_count = 0;
     int max_smem_optin = 0;
+    int smem_per_sm = 0;
 };
 // Returns nullptr (and records the error) when no CUDA device is usable.
 const DeviceInfo* current_device_info();
@@ -30,9 +31,9 @@ int64_t option(int32_t which);
 // with grid_dependency_wait(), which returns only once that previous kernel has completed
 // and its writes are visible, so stream order is kept exactly; what is saved is the launch
 // latency between consecutive kernels.
-// whole_smem: the SM's whole shared memory is laid out as such, instead of the smallest layout that a block fits.
+// shared_percent: how much of the SM's shared memory and L1 is laid out as shared memory at least (-1: what a block fits).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_laid_out(bool whole_smem, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+inline cudaError_t launch_laid_out(int shared_percent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                    cudaStream_t stream, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -43,15 +44,15 @@ inline cudaError_t launch_laid_out(bool whole_smem, void (*kernel)(KArgs...), di
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    attr[1].val.sharedMemCarveout = (unsigned int)shared_percent;
     cfg.attrs = attr;
-    cfg.numAttrs = whole_smem ? 2 : 1;
+    cfg.numAttrs = shared_percent >= 0 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_serialized(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                      cudaStream_t stream, Args&&... args) {
-    return launch_laid_out(false, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
+    return launch_laid_out(-1, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
 }
 
 #ifdef __CUDACC__
