@@ -853,12 +853,9 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
         own_smem = a.sharedSizeBytes;
         configured_device = di->device;
     }
-    // (rows wider than 32 actions: the companion gains nothing with fp32 logits and doubles a launch with bf16 ones
-    // -- 27 against 14 us at 65 536 steps --, so such launches ask for their first tiles themselves)
-    // (nor where four groups have a tile each, all of which are asked for at once: 5 to 8 % slower at 600 x 128 steps)
-    const long long rows = p.geo.B * p.geo.T;
-    const bool one_round = C == 4 && 2 * rows < 9 * ls.grid * nt;
-    WsPlan plan = ws_plan(ls.tiles, ls.grid, (size_t)nt * (2 * p.A * sizeof(LT) + 20), sh.in_flight, p.A <= 32 && !one_round);
+    const size_t row_bytes = 2 * p.A * sizeof(LT) + 20;
+    WsPlan plan = ws_plan(ls.tiles, ls.grid, nt * row_bytes, sh.in_flight,
+                          companion_pays(p.A, kLong, C, p.geo.B * p.geo.T, row_bytes, nt, ls.tiles, ls.grid, sh.in_flight, sizeof(GT)));
     if (kIndirect) { plan.companion = false; plan.prefetch_tiles = 0; }  // (addresses unknown on the host)
     if (plan.companion) {
         const int32_t st = launch_companion(p, (int)sizeof(LT), kLong, plan.prefetch_tiles, (int)ls.grid, stream);

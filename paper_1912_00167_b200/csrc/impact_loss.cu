@@ -124,10 +124,8 @@ WsPlan ws_plan(long long tiles, long long grid, size_t tile_bytes, int in_flight
     const bool large_tiles = tile_bytes >= 10 * 1024;
     // (measured on 18 actions: a gain from five tiles per block on -- 8.3 -> 7.6 us at seven --, nothing at three
     // to four, a loss of a quarter of a microsecond at two)
-    // (and up to 28 MB a launch: on 128 steps of 1024 trajectories in fp32 24 actions, 27.8 MB, take 10.1 us with it and 10.6
-    // without, 28 actions, 32 MB, 13.4 and 11.1)
     pl.companion = allow_companion && large_tiles && option(IMPACT_OPT_EARLY_PREFETCH) != 0 && pf >= per_block &&
-                   per_block >= 4 && per_block <= 8 && tiles * (long long)tile_bytes <= 28000000;
+                   per_block >= 4 && per_block <= 8;
     if (!large_tiles) pf = 0;
     if (!pl.companion && pf > in_flight) pf = in_flight;
     if (pf > per_block) pf = per_block;
