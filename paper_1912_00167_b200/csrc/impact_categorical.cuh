@@ -908,8 +908,19 @@ int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream)
         }
         return IMPACT_ERR_UNSUPPORTED;
     }
-    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0) || (!fits && p.tile_aggregates))
+    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0) || (!fits && p.tile_aggregates)) {
+        // Where three groups spill as well (100 bytes a thread and more: 30 and 31 actions with fp32 logits; 32 are read four
+        // at a time and lose nothing by it) and nearly every block has four tiles, four groups have one each: 16 x 4096 steps of
+        // 30 and 31 actions 12.1 and 12.5 us instead of 13.2 and 14.1, with bf16 gradients 11.9 and 12.9 instead of 13.3 and
+        // 14.6.  With fewer tiles three have as much to do (14 x 4096 11.4 on four, 10.6 on three), with more they are faster
+        // (20 x 4096 17.5 and 14.0).
+        if constexpr (A >= 30 && kV < 4 && sizeof(LT) == 4) {
+            const long long tiles = p.geo.B * ((p.geo.T + 127) / 128);
+            if (5 * tiles > 16 * di->sm_count && tiles <= 4 * di->sm_count)
+                return launch_categorical<LT, GT, A, 4, kV, false, true, false>(p, rl, di, stream);
+        }
         return launch_categorical<LT, GT, A, C, kV, false, true, false>(p, rl, di, stream);
+    }
     if (!fits && A > kLongestRows) return IMPACT_ERR_UNSUPPORTED;
     return plain && fits ? launch_categorical<LT, GT, A, CP, kV, true, false, false>(p, rl, di, stream)
                          : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, rl, di, stream);
