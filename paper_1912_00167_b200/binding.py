@@ -10,6 +10,7 @@ import ctypes
 import importlib
 import os
 import struct
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -93,13 +94,12 @@ assert _CALL.size == ctypes.sizeof(impact_loss_call)
 
 _lib = None
 _call_packed = None
-_loss_direct = None  # the direct loss call's arguments checked in native code (csrc/marshal.cpp)
 _vp, _i32, _i64, _f32, _sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_float, ctypes.c_size_t
 
 
 def load_library() -> ctypes.CDLL:
     """Loads libimpact.so; raises if it has not been built (there is no other code path)."""
-    global _lib, _call_packed, _loss_direct
+    global _lib, _call_packed
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -171,11 +171,32 @@ def load_library() -> ctypes.CDLL:
     _call_packed = lib["impact_loss_fwd_bwd_call"]
     _call_packed.restype = _i32
     _call_packed.argtypes = [ctypes.c_char_p, _vp]
-    marshal = importlib.import_module("._marshal", __package__)
-    marshal.bind(ctypes.cast(lib.impact_loss_fwd_bwd_call, _vp).value)
-    _loss_direct = marshal.loss
     _lib = lib
     return lib
+
+
+def _not_served(*args) -> None:
+    """Every direct loss call is checked in Python."""
+
+
+def _bind_loss_direct(*args):
+    """The first direct loss call: finds the native part that checks such a call's arguments (csrc/marshal.cpp).  Nothing else
+    needs it, and a direct call does without as well."""
+    global _loss_direct
+    lib = load_library()
+    try:
+        marshal = importlib.import_module("._marshal", __package__)
+    except ImportError as e:
+        _loss_direct = _not_served
+        warnings.warn(f"{e}: direct loss calls are checked in Python, which takes some 6 us each; rebuild with "
+                      "`python -m paper_1912_00167_b200.build`", RuntimeWarning, stacklevel=3)
+    else:
+        marshal.bind(ctypes.cast(lib.impact_loss_fwd_bwd_call, _vp).value)
+        _loss_direct = marshal.loss
+    return _loss_direct(*args)
+
+
+_loss_direct = _bind_loss_direct
 
 
 def _check(status: int, what: str, allow=()) -> int:
@@ -372,8 +393,6 @@ def impact_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rew
     # The usual call: plain tensors, every argument as it should be, checked in native code.  What that leaves (None) --
     # subclasses, numbers of other types, arguments at fault -- is checked here in a row and packed at once; what still is
     # not as it should be goes the way of a prepared call, which names the argument at fault.
-    if _lib is None:
-        load_library()
     st = _loss_direct(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values, bootstrap_values, coef,
                       loss_terms, dlogits, dvalues, vtarget, advantage, workspace, target_logits_copy,
                       None if stream is None else _stream(stream))

@@ -122,6 +122,34 @@ def _cpu_ring(lib, nbytes):
     return b.ImpactBuffer(N, 2, nbytes, storage=raw[at:at + raw.numel() - 256])
 
 
+def test_nothing_needs_the_native_check_of_direct_calls(lib):
+    """Without the binding's native part the library loads and a direct loss call is checked in Python: it says so once, and
+    names the argument at fault."""
+    import subprocess
+    import sys
+    code = """
+import sys, warnings
+import torch
+sys.modules["paper_1912_00167_b200._marshal"] = None
+import paper_1912_00167_b200 as ip
+assert ip.load_library() is not None and ip.impact_version() > 0
+with warnings.catch_warnings(record=True) as said:
+    warnings.simplefilter("always")
+    z, v = torch.zeros(2, 3, 4), torch.zeros(2, 3)
+    for _ in range(2):
+        try:
+            ip.impact_loss_fwd_bwd(z, z, v, v.int(), v, v, v, v[:, 0], ip.Coefficients(), loss_terms=torch.zeros(8), dlogits=z,
+                                   dvalues=v, workspace=torch.zeros(64, dtype=torch.uint8))
+        except ValueError as e:
+            assert "learner_logits" in str(e), e
+        else:
+            raise SystemExit("served")
+assert len(said) == 1 and "rebuild" in str(said[0].message), said
+"""
+    done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert done.returncode == 0, done.stderr
+
+
 def test_a_slot_view_is_the_slots_bytes_and_nothing_else(lib):
     """Views of every shape and type name the bytes that the library names; a closed buffer and bad places are refused."""
     import torch
