@@ -180,12 +180,13 @@ def _not_served(*args) -> None:
 
 
 def _bind_loss_direct(*args):
-    """The first direct loss call: finds the native part that checks such a call's arguments (csrc/marshal.cpp).  Nothing else
-    needs it, and a direct call does without as well."""
+    """The first direct loss call: finds the native part that checks such a call's arguments (csrc/marshal.cpp), the
+    one built for this Python and this torch.  Nothing else needs it, and a direct call does without as well."""
     global _loss_direct
+    from .build import marshal_name
     lib = load_library()
     try:
-        marshal = importlib.import_module("._marshal", __package__)
+        marshal = importlib.import_module("." + marshal_name(), __package__)
     except ImportError as e:
         _loss_direct = _not_served
         warnings.warn(f"{e}: direct loss calls are checked in Python, which takes some 6 us each; rebuild with "

@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import glob
 import os
+import re
 import subprocess
 import sys
 import sysconfig
@@ -13,7 +14,18 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libimpact.so")
-MARSHAL = os.path.join(PKG, "_marshal.so")
+
+
+def marshal_name() -> str:
+    """The binding's native part, by the Python and the torch that it is built for: it reads torch's objects through headers
+    that are compiled in, so one built for another of either is another module, not this one out of date."""
+    import torch
+    return "_marshal_" + re.sub(r"\W", "_", "%s_torch_%s_%s" % (sysconfig.get_config_var("SOABI"), torch.__version__,
+                                                               (torch.version.git_version or "")[:12]))
+
+
+def marshal_path() -> str:
+    return os.path.join(PKG, marshal_name() + ".so")
 
 
 def sources() -> list[str]:
@@ -21,11 +33,12 @@ def sources() -> list[str]:
 
 
 def needs_build() -> bool:
-    if not (os.path.exists(LIB) and os.path.exists(MARSHAL)):
+    marshal = marshal_path()
+    if not (os.path.exists(LIB) and os.path.exists(marshal)):
         return True
     deps = sources() + glob.glob(os.path.join(CSRC, "*.cpp")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
     deps += glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL)) for d in deps)
+    return any(os.path.getmtime(d) > min(os.path.getmtime(LIB), os.path.getmtime(marshal)) for d in deps)
 
 
 def build_marshal() -> None:
@@ -33,14 +46,16 @@ def build_marshal() -> None:
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    tmp = MARSHAL + ".tmp.%d" % os.getpid()
+    out = marshal_path()
+    tmp = out + ".tmp.%d" % os.getpid()
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fno-gnu-unique", "-DNDEBUG",
+                           "-DIMPACT_MARSHAL=" + marshal_name(),
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), "-I", os.path.join(ROOT, "include"),
                            "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(root, "include"),
                            "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
                            "-isystem", os.path.join(cuda, "include"), os.path.join(CSRC, "marshal.cpp"), "-o", tmp,
                            "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
-    os.replace(tmp, MARSHAL)
+    os.replace(tmp, out)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

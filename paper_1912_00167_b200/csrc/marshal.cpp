@@ -190,7 +190,10 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, g_method
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() {
+// (the module's name says which Python and torch it was built for: IMPACT_MARSHAL, see build.py)
+#define IMPACT_INIT_OF(name) PyInit_##name
+#define IMPACT_INIT(name) IMPACT_INIT_OF(name)
+PyMODINIT_FUNC IMPACT_INIT(IMPACT_MARSHAL)() {
     static const char* const names[kNames] = {"rho_bar", "c_bar", "clip_eps", "vf_coef", "ent_coef", "kl_coef", "lam", "rho_tw",
                                               "is_source", "ratio_mode", "objective", "global_steps"};
     for (int i = 0; i < kNames; ++i)

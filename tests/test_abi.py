@@ -130,8 +130,9 @@ def test_nothing_needs_the_native_check_of_direct_calls(lib):
     code = """
 import sys, warnings
 import torch
-sys.modules["paper_1912_00167_b200._marshal"] = None
 import paper_1912_00167_b200 as ip
+from paper_1912_00167_b200.build import marshal_name
+sys.modules["paper_1912_00167_b200." + marshal_name()] = None
 assert ip.load_library() is not None and ip.impact_version() > 0
 with warnings.catch_warnings(record=True) as said:
     warnings.simplefilter("always")
@@ -148,6 +149,28 @@ assert len(said) == 1 and "rebuild" in str(said[0].message), said
 """
     done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert done.returncode == 0, done.stderr
+
+
+def test_a_native_part_built_for_another_torch_is_not_this_one(lib, monkeypatch):
+    """The module's name says what it was built for: with another torch (or Python) the one that is there counts as missing, is
+    not loaded, and a build makes a new one."""
+    import torch
+    from paper_1912_00167_b200 import binding as b, build
+    assert os.path.exists(build.marshal_path()) and not build.needs_build()
+    name = build.marshal_name()
+    monkeypatch.setattr(b, "_loss_direct", b._bind_loss_direct)
+    assert b._loss_direct(*[None] * 17) is None and b._loss_direct.__module__ == "_marshal"  # (found; it serves no such call)
+    for what, value in (("__version__", "2.12.0"), ("version", type("version", (), dict(git_version="0" * 40)))):
+        with monkeypatch.context() as other:
+            other.setattr(torch, what, value)
+            assert build.marshal_name() != name and build.needs_build()
+            other.setattr(b, "_loss_direct", b._bind_loss_direct)
+            with pytest.warns(RuntimeWarning, match="rebuild"):
+                assert b._loss_direct(*[None] * 17) is None
+            assert b._loss_direct is b._not_served
+    with monkeypatch.context() as other:
+        other.setattr(build.sysconfig, "get_config_var", lambda name: "cpython-313-x86_64-linux-gnu")
+        assert build.marshal_name() != name and build.needs_build()
 
 
 def test_a_slot_view_is_the_slots_bytes_and_nothing_else(lib):
