@@ -28,6 +28,10 @@ def marshal_path() -> str:
     return os.path.join(PKG, marshal_name() + ".so")
 
 
+def _nvcc() -> str:
+    return os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+
+
 def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
@@ -42,18 +46,18 @@ def needs_build() -> bool:
 
 
 def build_marshal() -> None:
-    """The native part of the Python binding (csrc/marshal.cpp), against the headers and libraries of the installed torch."""
+    """The native part of the Python binding (csrc/marshal.cpp), against the headers and libraries of the installed torch.  By
+    nvcc, which knows where CUDA's headers are however it is named."""
     import torch
     root = os.path.dirname(torch.__file__)
-    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     out = marshal_path()
     tmp = out + ".tmp.%d" % os.getpid()
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fno-gnu-unique", "-DNDEBUG",
-                           "-DIMPACT_MARSHAL=" + marshal_name(),
+    subprocess.check_call([_nvcc(), "-O2", "-std=c++17", "-shared", "-cudart", "none", "-Xcompiler", "-fPIC,-fno-gnu-unique",
+                           "-DNDEBUG", "-DIMPACT_MARSHAL=" + marshal_name(),
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), "-I", os.path.join(ROOT, "include"),
                            "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(root, "include"),
                            "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
-                           "-isystem", os.path.join(cuda, "include"), os.path.join(CSRC, "marshal.cpp"), "-o", tmp,
+                           os.path.join(CSRC, "marshal.cpp"), "-o", tmp,
                            "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
     os.replace(tmp, out)
 
@@ -61,7 +65,7 @@ def build_marshal() -> None:
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    nvcc = _nvcc()
     # (no unique symbols: a process that loads two copies of the library -- two versions, say -- would share what each kernel
     # remembers of its own configuration, and the second copy's launches would fail)
     flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xfatbin", "-compress-all",

@@ -151,6 +151,26 @@ assert len(said) == 1 and "rebuild" in str(said[0].message), said
     assert done.returncode == 0, done.stderr
 
 
+def test_the_native_part_builds_with_nvcc_by_any_name(lib, monkeypatch, tmp_path):
+    """A bare name that is found on the path, and a wrapper that lies elsewhere."""
+    import shutil
+    import subprocess
+    from paper_1912_00167_b200 import build
+    real = shutil.which(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))
+    wrapper = tmp_path / "nvcc"
+    wrapper.write_text('#!/bin/sh\nexec "%s" "$@"\n' % real)
+    wrapper.chmod(0o755)
+    monkeypatch.setattr(build, "marshal_path", lambda: str(tmp_path / "made.so"))
+    for name, path in (("nvcc", os.path.dirname(real)), (str(wrapper), None)):
+        monkeypatch.setenv("NVCC", name)
+        if path:
+            monkeypatch.setenv("PATH", path + os.pathsep + os.environ["PATH"])
+        build.build_marshal()
+        names = subprocess.run(["nm", "-D", "--defined-only", build.marshal_path()], capture_output=True, text=True, check=True)
+        assert "PyInit_" + build.marshal_name() in names.stdout
+        os.remove(build.marshal_path())
+
+
 def test_a_native_part_built_for_another_torch_is_not_this_one(lib, monkeypatch):
     """The module's name says what it was built for: with another torch (or Python) the one that is there counts as missing, is
     not loaded, and a build makes a new one."""
