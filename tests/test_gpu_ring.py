@@ -381,6 +381,40 @@ def test_gather_rows_of_every_width(row_bytes, n):
     assert bool((guard[:256] == 0xA5).all()) and bool((guard[256 + n * row_bytes:] == 0xA5).all())
 
 
+@pytest.mark.parametrize("n_cand", [255, 256, 257, 700])
+@pytest.mark.parametrize("ahead", [0, 3])
+def test_device_step_with_more_candidates_than_a_block_has_threads(oracle, n_cand, ahead):
+    """Candidates' tables of up to 512 pointers are asked for as a whole, larger ones candidate by candidate: which candidate
+    lands in which slot, and whose kept pointer comes with the draw, as it is pushed (none ahead) and later."""
+    import ctypes
+    import paper_1912_00167_b200 as ip
+    N, K, n = 5, 1, 13
+    data = torch.arange(n_cand * 16, dtype=torch.int32, device="cuda").view(n_cand, 16)  # (of which a push copies 13)
+    kept = [0x10000 + 64 * c for c in range(n_cand)]  # (handed on, never read)
+    table = torch.tensor([[data[c].data_ptr(), kept[c]] for c in range(n_cand)], dtype=torch.int64, device="cuda")
+    ring, ref = ip.ImpactBuffer(N, K, [4 * n], seed=3, sample_mode=1), oracle.Ring(N, K, 1, seed=3)
+    record = ip.new_loss_inputs_record()
+    push = ring.prepare_device_step(push_sources=table)
+    both = ring.prepare_device_step({"target_logits": 0}, record=record, push_sources=table)
+    ring.device_begin()
+    where, pushed = {}, 0
+    for i in range(ahead + 2 * n_cand + 3):
+        (push if i < ahead else both)()
+        st, slot = ref.push()
+        assert st == 0
+        where[slot] = pushed % n_cand
+        pushed += 1
+        if i < ahead:
+            continue
+        st, slot, k = ref.sample()
+        got = ip.binding.impact_loss_inputs.from_buffer_copy(bytes(record[:ctypes.sizeof(ip.binding.impact_loss_inputs)].tolist()))
+        assert (st, got.status, got.slot, got.k_before) == (0, 0, slot, k)
+        assert got.target_logits == kept[where[slot]]
+        assert torch.equal(ring.slot_view(slot, 0, torch.int32, (n,)), data[where[slot], :n])
+    ring.device_end()
+    ring.close()
+
+
 @pytest.mark.parametrize("row_bytes", [15, 16, 17, 18, 24, 31, 32, 34, 36, 40, 48, 200, 1802])
 @pytest.mark.parametrize("n,offset", [(1, 0), (7, 0), (5000, 0), (40000, 0), (5000, 8), (5000, 4)])
 def test_gather_rows_around_the_granules(row_bytes, n, offset):
