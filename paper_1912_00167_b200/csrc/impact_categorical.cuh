@@ -22,7 +22,8 @@ constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 // itself it would be rounded at its own size before the difference is taken, the largest error of a ratio where actions
 // are few (dvalues' error against 64 bits, two to seven actions: 2.5e-7 to 3.2e-7 that way).
 // (Products and sums are spelled out where the compiler could fuse them one way in one instantiation and another way in
-// the next: every kernel that can serve a call gives the same bits.)
+// the next: every kernel that can serve a call gives the same bits, but for the KL term and its gradient, which flat launches
+// of few actions form from exponentials that they keep and split ones do not; see kKeepTarget.)
 struct Step {
     float l2_theta, l2_target, l_worker;
     float reward, discount, value, value_next;
@@ -118,21 +119,21 @@ __device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss
 template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid_constant__ LaunchForm sh) {
-    constexpr bool kWide = kA == kWideRows, kFixed = kA > 0;
-    constexpr bool kRotated = kV == 4 && (!kFixed || kA % 8 == 0);  // (rows of 4 and 12 actions meet on no bank)
-    constexpr bool kSingles = kV == 1 && kFixed && sizeof(LT) == 4;  // rows element by element
+    constexpr bool kWide = kA == kWideRows;
+    constexpr bool kRotated = kV == 4 && (kWide || kA % 8 == 0);  // (rows of 4 and 12 actions meet on no bank)
+    constexpr bool kSingles = kV == 1 && !kWide && sizeof(LT) == 4;  // rows element by element
     constexpr bool kOdd = kV == 1 && !kSingles;
     constexpr int VW = kV == 1 ? 2 : kV;  // elements of a vector
-    constexpr int NV = (kFixed ? kA : kWideElems) / VW;  // vectors per lane at most
+    constexpr int NV = (kWide ? kWideElems : kA) / VW;  // vectors per lane at most
     constexpr int NP = NV * VW / 2 + (kV == 1 ? 1 : 0);  // pairs: Blackwell's packed fp32 add / mul / fma work on two at once
     constexpr float kLowest = -3.402823466e38f;  // stands for an element that is not there: its exponential is 0
-    static_assert(!kFixed || kA % VW == (kV == 1 ? 1 : 0), "whole vectors");
+    static_assert(kWide || kA % VW == (kV == 1 ? 1 : 0), "whole vectors");
     // The KL term from the target row's own exponentials, kept for the gradient pass too, instead of formed twice again
     // (with the KL term, 100 MB: 7 actions in fp32 25.5 -> 24.9 us, 12 in bf16 20.7 -> 19.2, 14 19.9 -> 18.3).  Not where the
     // registers run short -- 96, the learner's exponentials among them: more actions, the split forms -- nor at 8 to 14
     // actions in fp32, where the term gains 0 to 3 % and calls without it lose as much.
-    constexpr bool kKeepTarget = kFixed && !kPlain && !kLong && kA <= (sizeof(LT) == 2 ? 14 : 7);
-    const int A = kFixed ? kA : p.A;
+    constexpr bool kKeepTarget = !kWide && !kPlain && !kLong && kA <= (sizeof(LT) == 2 ? 14 : 7);
+    const int A = kWide ? p.A : kA;
     const int NT = kWide ? sh.nt : 128;
     const int NTW = NT >> 2;  // rows of a tile that one warp works on
     const int S = sh.stages, W = sh.in_flight;
@@ -320,7 +321,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     const int lrow = wrow + (kWide ? (lane >> log_l) * passes + min(part, passes) : lane);
     const bool owner = kWide ? part < passes : true;
     const int row_vecs = A / VW;  // vectors of a row (odd counts: and one element)
-    const int nvec = kFixed ? NV : (row_vecs + L - 1) >> log_l;  // of the lane with the most
+    const int nvec = kWide ? (row_vecs + L - 1) >> log_l : NV;  // of the lane with the most
     const int rot = kRotated ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
 
     // The tile (in a flat launch only a block's first tile ends early, only its last one can begin late, and from one of
@@ -329,7 +330,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     const unsigned int back = (unsigned int)(C * NT);
     TileRows tl = tile_now(grp);
     // (flat) the place of the lane's step
-    using Steps = typename std::conditional<kFixed && kA <= kLongestRows && !kPlain, unsigned long long, unsigned int>::type;
+    using Steps = typename std::conditional<!kWide && kA <= kLongestRows && !kPlain, unsigned long long, unsigned int>::type;
     const Steps Tn = (Steps)g.T;
     const unsigned int back_traj = kLong ? 0u : (unsigned int)(back / Tn);
     const Steps back_rest = kLong ? (Steps)0 : back - back_traj * Tn;
@@ -455,7 +456,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const int step = (VW * elem) << log_l;
             return kRotated ? ((i * step) ^ (rot * step)) : i * step;
         };
-        auto vec_there = [&](int i) { return kFixed || (kWide ? (i << log_l) + part < row_vecs : i < row_vecs); };
+        auto vec_there = [&](int i) { return !kWide || (i << log_l) + part < row_vecs; };
         // (odd counts) does the row start on an odd element?  Tiles are an even number of rows apart.
         const uint32_t tile_odd = kOdd ? (uint32_t)(kLong ? tl.row0 : br.base) & 1u : 0u;
         auto first_of = [&](int r) { return kOdd ? (int)((tile_odd + (uint32_t)r) & 1u) : 0; };  // of the vectors
@@ -478,7 +479,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             for (int j = 0; j < NP; ++j) z[j] = make_float2(f[2 * j], f[2 * j + 1]);
         };
         // is pair j worked on?  (run-time counts: groups of two pairs up to the last that holds elements; a uniform test)
-        auto pair_used = [&](int j) { return kFixed || (kOdd && j == NP - 1) || (j & ~1) * 2 < nvec * VW; };
+        auto pair_used = [&](int j) { return !kWide || (kOdd && j == NP - 1) || (j & ~1) * 2 < nvec * VW; };
         auto row_max = [&](const float2 (&z)[NP]) {
             float m0 = fmaxf(z[0].x, z[0].y), m1 = m0;
 #pragma unroll
@@ -745,7 +746,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const int first = first_of(r) + part * VW;
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
-                if (!kFixed && kWide && i >= nvec) continue;  // (uniform)
+                if (kWide && i >= nvec) continue;  // (uniform)
                 if (!vec_there(i)) continue;
                 float z[VW], o[VW], zt[VW];
 #pragma unroll
@@ -941,26 +942,25 @@ inline int wide_tile_rows(const BatchGeometry& g, bool aggregates, int A, size_t
     return nt;
 }
 
-template <typename LT, typename GT, int kA, int C, int CP, int kV>
-int32_t run_runtime_form(const CatParams& p, const RowLayout& rl, bool plain, const DeviceInfo* di, cudaStream_t stream) {
+template <typename LT, typename GT, int kV>
+int32_t run_wide_form(const CatParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
+    constexpr int C = 4;
     const bool fits = fits_flat(p.geo);
-    if (splits_trajectories(p.geo, p.tile_aggregates, rl.nt, di, kA == kWideRows ? p.A : 0) || (!fits && p.tile_aggregates)) {
+    if (splits_trajectories(p.geo, p.tile_aggregates, rl.nt, di, p.A) || (!fits && p.tile_aggregates)) {
         if (rl.nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
-        if constexpr (kA == kWideRows) {
-            // Tiles of 64 rows go to three groups: they have 128 registers to a thread and spill nothing (four: 96).
-            // 16 x 4096 steps of 64 actions take 18.7 us instead of 20.4, 31 x 4000 32.0 instead of 35.5.  Four where each
-            // has one tile of the block's, and the ring six stages: 16 x 2048 12.2 us instead of 12.9.
-            const long long tiles = p.geo.B * ((p.geo.T + kMinTileRows - 1) / kMinTileRows);
-            const bool one_each = (tiles + di->sm_count - 1) / di->sm_count == C;
-            if (rl.nt == kMinTileRows &&
-                !(one_each && stages_that_fit(cat_stage_bytes(rl.nt, p.A, sizeof(LT), sizeof(GT)), di->max_smem_optin) >= C + 2))
-                return launch_categorical<LT, GT, kA, 3, kV, false, true, false>(p, rl, di, stream);
-        }
-        return launch_categorical<LT, GT, kA, C, kV, false, true, false>(p, rl, di, stream);
+        // Tiles of 64 rows go to three groups: they have 128 registers to a thread and spill nothing (four: 96).
+        // 16 x 4096 steps of 64 actions take 18.7 us instead of 20.4, 31 x 4000 32.0 instead of 35.5.  Four where each
+        // has one tile of the block's, and the ring six stages: 16 x 2048 12.2 us instead of 12.9.
+        const long long tiles = p.geo.B * ((p.geo.T + kMinTileRows - 1) / kMinTileRows);
+        const bool one_each = (tiles + di->sm_count - 1) / di->sm_count == C;
+        if (rl.nt == kMinTileRows &&
+            !(one_each && stages_that_fit(cat_stage_bytes(rl.nt, p.A, sizeof(LT), sizeof(GT)), di->max_smem_optin) >= C + 2))
+            return launch_categorical<LT, GT, kWideRows, 3, kV, false, true, false>(p, rl, di, stream);
+        return launch_categorical<LT, GT, kWideRows, C, kV, false, true, false>(p, rl, di, stream);
     }
     if (!fits) return IMPACT_ERR_UNSUPPORTED;
-    return plain ? launch_categorical<LT, GT, kA, CP, kV, true, false, false>(p, rl, di, stream)
-                 : launch_categorical<LT, GT, kA, C, kV, false, false, false>(p, rl, di, stream);
+    return is_plain(p) ? launch_categorical<LT, GT, kWideRows, C, kV, true, false, false>(p, rl, di, stream)
+                       : launch_categorical<LT, GT, kWideRows, C, kV, false, false, false>(p, rl, di, stream);
 }
 
 template <typename LT, typename GT, int kV>
@@ -969,7 +969,6 @@ int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t
     const int vecs = p.A / VW;
     RowLayout rl;
     auto settle = [&](int l) { return settle_rows<LT, kV>(rl, p.A, l); };
-    const bool plain = is_plain(p);
     // Rows of more than a lane: the fewest lanes that hold a row and do not meet on the banks more than two at a time.
     rl.nt = wide_tile_rows(p.geo, p.tile_aggregates, p.A, sizeof(LT), sizeof(GT), di);
     int l = 1;
@@ -982,7 +981,7 @@ int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t
         }
         return IMPACT_ERR_UNSUPPORTED;
     }
-    return run_runtime_form<LT, GT, kWideRows, 4, 4, kV>(p, rl, plain, di, stream);
+    return run_wide_form<LT, GT, kV>(p, rl, di, stream);
 }
 
 template <typename LT, typename GT>
