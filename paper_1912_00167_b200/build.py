@@ -52,7 +52,7 @@ def build_marshal() -> None:
     root = os.path.dirname(torch.__file__)
     out = marshal_path()
     tmp = out + ".tmp.%d" % os.getpid()
-    subprocess.check_call([_nvcc(), "-O2", "-std=c++17", "-shared", "-cudart", "none", "-Xcompiler", "-fPIC,-fno-gnu-unique",
+    subprocess.check_call([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O2", "-std=c++17", "-shared", "-cudart", "none", "-Xcompiler", "-fPIC,-fno-gnu-unique",
                            "-DNDEBUG", "-DIMPACT_MARSHAL=" + marshal_name(),
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), "-I", os.path.join(ROOT, "include"),
                            "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(root, "include"),
