@@ -118,15 +118,17 @@ inline int stages_that_fit(size_t stage_bytes, int max_smem) { return (int)((siz
 void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max_smem, long long tiles_per_block,
                    int* stages, int* in_flight);
 // Does a companion (impact_prefetch.cu) pay for a categorical launch of `rows` steps of `row_bytes` inputs each?  (Where
-// ws_plan finds its tiles large and few enough.)  Both sides measured, companion / none, in us:
+// ws_plan finds its tiles large and few enough.)  Both sides measured, companion / none, in us, on inputs that come from HBM;
+// where a program's inputs are still in L2 a companion can only cost (1024 x 128 of 18 actions 7.9 / 7.5, cold 7.5 / 7.9).
 //   Rows wider than 32 actions: no.  It gains nothing with fp32 logits and doubles a launch with bf16 ones (27 / 14 at 65 536
 //   steps).
-//   Split trajectories: up to 28 MB.  Up to 18 actions they gain most, their tiles being spread over the device (16 x 4096 steps
-//   of 9 actions 7.3 / 8.3, of 18 8.5 / 8.8; 31 x 4000 11.1 / 13.6 and 13.1 / 13.5, in bf16 12.8 / 14.8).  More actions: not at
-//   up to four tiles a block (16 x 4096 in bf16 of 24 actions 10.7 / 10.1, of 20 10.1 / 9.1; at 4.3 tiles 20 x 4096 of 24 in fp32
-//   11.4 / 12.1).
+//   Split trajectories: up to 28 MB.  Up to 18 actions they gain, their tiles being spread over the device (31 x 4000 steps of 9
+//   actions 11.1 / 13.6, of 18 13.1 / 13.5, in bf16 12.8 / 14.8); where blocks have fewer than four and a half tiles only small
+//   tiles gain without losing as much on inputs in L2 (16 x 4096 of 9 7.3 / 8.3, in L2 7.7 / 7.8; of 12 7.8 / 8.4 and 7.7 / 8.0;
+//   of 18 8.5 / 8.8 but 9.1 / 8.4).  More actions: not at up to four tiles (16 x 4096 in bf16 of 24 actions 10.7 / 10.1, of 20
+//   10.1 / 9.1; at 4.3 tiles 20 x 4096 of 24 in fp32 11.4 / 12.1).
 //   Whole trajectories, four groups: not where each has about a tile, all of which are asked for at once (600 x 128 of 18 with
-//   every switch 7.1 / 6.8), but for rows of up to 9 actions (9: 5.9 / 6.0).
+//   every switch 7.1 / 6.8; of 9 5.9 / 6.0, in L2 5.9 / 5.7).
 //   Otherwise by the tiles that a block has in flight, behind whose requests the next launch's companion puts its own: three and
 //   more (fp32 logits of up to 23 actions) up to 25.5 MB (1024 x 128 of 20 7.8 / 8.2, 1180 x 128 10.4 / 9.1), with bf16 gradients
 //   28 MB (8.1 / 8.5); two up to 22 MB (800 x 128 of 24 8.0 / 8.2, 900 x 128 10.9 / 9.0; 700 x 128 of 28 8.0 / 8.1, 800 x 128
@@ -135,8 +137,9 @@ inline bool companion_pays(int A, bool split, int groups, long long rows, size_t
                            long long grid, int in_flight, size_t grad_bytes) {
     if (A > 32) return false;
     const long long bytes = rows * (long long)row_bytes;
-    if (split) return bytes <= 28000000 && (A <= 18 || tiles > 4 * grid);
-    if (groups == 4 && A > 9 && 2 * rows < 9 * grid * nt) return false;
+    const bool few_tiles = 2 * rows < 9 * grid * nt;
+    if (split) return bytes <= 28000000 && (A > 18 ? tiles > 4 * grid : !few_tiles || nt * row_bytes <= 15 * 1024);
+    if (groups == 4 && few_tiles) return false;
     return bytes <= (in_flight < 3 ? 22000000 : grad_bytes == 4 ? 25500000 : 28000000);
 }
 // How many tiles per block are asked for in L2 ahead of time, and by whom.

@@ -1,5 +1,6 @@
-// Which launches take a companion, worked out on the host as the launch does: split trajectories of up to 18 actions do, a launch
-// whose groups have a tile each does not, and large ones up to where their companion's requests hold up their own.
+// Which launches take a companion, worked out on the host as the launch does: split trajectories of up to 18 actions do but for
+// few large tiles, a launch whose groups have a tile each does not, and large ones up to where their companion's requests hold
+// up their own.
 #include <stdio.h>
 
 #include "impact_categorical.cuh"
@@ -26,16 +27,18 @@ static void expect(bool want, long long B, long long T, int A, size_t in, size_t
 
 int main() {
     for (int A : {8, 9, 12, 16, 18}) {
-        expect(true, 16, 4096, A, 4, 4, 4, true);
+        expect(A <= 12, 16, 4096, A, 4, 4, 4, true);
+        expect(true, 24, 4096, A, 4, 4, 4, true);
         expect(true, 31, 4000, A, 4, 4, 4, true);
     }
+    expect(true, 16, 4096, 18, 2, 2, 4, true);
     expect(true, 31, 4000, 18, 2, 2, 4, true);
     expect(false, 16, 4096, 20, 2, 2, 3, true);
     expect(false, 16, 4096, 28, 4, 4, 3, true);
     expect(true, 20, 4096, 24, 4, 4, 3, true);
     expect(false, 24, 4096, 33, 2, 2, 4, true);
     expect(false, 600, 128, 18, 4, 4, 4, false);
-    expect(true, 600, 128, 9, 4, 4, 4, false);
+    expect(false, 600, 128, 9, 4, 4, 4, false);
     expect(true, 1024, 128, 18, 4, 4, 5, false);
     expect(true, 1024, 128, 18, 4, 4, 4, false);
     expect(true, 1180, 128, 18, 4, 4, 5, false);
