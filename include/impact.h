@@ -121,9 +121,8 @@ int32_t impact_last_cuda_error(void);
  * used by every later loss call of the process; setting one while another thread is inside a loss call is safe
  * (that call uses the old or the new value).
  *   IMPACT_OPT_EARLY_PREFETCH  1 (default): a loss call whose thread blocks have four to eight tiles each (of at
- *       least 10 KB, in all of 22 to 28 MB at most, rows of at most 32 actions: batches of roughly 75 000 to 150 000
- *       steps of 18 actions, split trajectories of 57 000 steps and more) enqueues
- *       a one-warp-per-block companion kernel right before its loss kernel.  The companion runs beside whatever
+ *       least 10 KB, in all of 22 to 28 MB at most, rows of at most 32 actions: batches of roughly 85 000 to 150 000
+ *       steps of 18 actions) enqueues a one-warp-per-block companion kernel right before its loss kernel.  The companion runs beside whatever
  *       kernel is still busy on the stream, asks L2 for the batch's first tiles, and then waits for the stream's
  *       previous kernel, so stream order is kept exactly; the loss kernel finds its first tiles in L2 instead of
  *       waiting for HBM.  0: no companion; the loss kernel asks for its first tiles itself when it starts.
