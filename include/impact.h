@@ -122,10 +122,11 @@ int32_t impact_last_cuda_error(void);
  * (that call uses the old or the new value).
  *   IMPACT_OPT_EARLY_PREFETCH  1 (default): a loss call whose thread blocks have four to eight tiles each (of at
  *       least 10 KB, in all of 22 to 28 MB at most, rows of at most 32 actions: batches of roughly 85 000 to 150 000
- *       steps of 18 actions) enqueues a one-warp-per-block companion kernel right before its loss kernel.  The companion runs beside whatever
- *       kernel is still busy on the stream, asks L2 for the batch's first tiles, and then waits for the stream's
- *       previous kernel, so stream order is kept exactly; the loss kernel finds its first tiles in L2 instead of
- *       waiting for HBM.  0: no companion; the loss kernel asks for its first tiles itself when it starts.
+ *       steps of 18 actions) enqueues a one-warp-per-block companion kernel right before its loss kernel.  The
+ *       companion runs beside whatever kernel is still busy on the stream, asks L2 for the batch's first tiles, and
+ *       then waits for the stream's previous kernel, so stream order is kept exactly; the loss kernel finds its first
+ *       tiles in L2 instead of waiting for HBM.  0: no companion; the loss kernel asks for its first tiles itself when
+ *       it starts.
  *   IMPACT_OPT_PREFETCH_BYTES  upper bound on the bytes one call asks L2 for ahead of time (default 48 MiB).
  *   IMPACT_OPT_WINDOW_BYTES    bytes of tiles a block keeps in flight from global to shared memory: 0 (default)
  *       lets each launch choose (48 KiB where a block has eight tiles or fewer, 72 KiB beyond), else
