@@ -76,11 +76,12 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 
 // ---- shape of the row passes ------------------------------------------------------------------------------------
 // kA > 0: the action count, known at compile time (1 to 32); a row belongs to one lane, which keeps its exponentials.
-// kA = kWideRows: any count; a row belongs to L = 2 ... 32 lanes that hold up to 32 elements each (vector i of lane g is
-//   the row's vector i L + g), and a warp works on its NT / 4 rows in P = NT / 4 * L / 32 passes.  Row q P + p of the
-//   warp is worked on in pass p by lanes [q L, q L + L) and owned -- for everything that is per step -- by lane q L + p
-//   of them, so results never move between lanes.  The gradient pass forms the exponentials again instead of holding P
-//   rows in registers.  (Fewest lanes: a pass costs a warp about a hundred instructions besides its elements'.)
+// kA < 0: any count above 32; a row belongs to L = 2 ... 16 lanes with -kA vectors each (vector i of lane g is the row's
+//   vector i L + g), known at compile time, of which the last one, for single pairs the last two, may not be there.  A warp
+//   works on 32 / L rows at once, in one pass or in two; row q P + p of the warp is worked on in pass p of P by lanes
+//   [q L, q L + L) and owned -- for everything that is per step -- by lane q L + p of them, so results never move between
+//   lanes.  (Told at run time how many vectors a lane has, up to 32 elements, a warp took 2340 instructions for 32 rows of 64
+//   actions in bf16; so 1760 in one pass, 1500 in two: a million steps 124 -> 86 -> 80 us.)
 //
 // Rows keep their dense layout in shared memory.  kV = 4 or 2: elements per access, where they divide the count.
 // kV = 1 stands for odd counts: a row is then one element and pairs, the element in front where the row starts on an odd
@@ -88,8 +89,6 @@ __device__ __forceinline__ float step_surrogate(const Step& s, const LossScalars
 // time: element by element -- such rows meet on no bank, their pairs on two; 250 000 steps of 9 actions with every
 // switch in use take 11.8 us instead of 12.4.)  Where rows meet on the same banks
 // (pitches with a large power of two), lanes take their vectors in rotated order; maxima and sums do not mind.
-constexpr int kWideRows = -1;
-constexpr int kWideElems = 32;  // elements of a row that a lane holds at most
 __host__ __device__ constexpr bool is_atari(int A) { return A == 4 || A == 6 || A == 9 || A == 18; }
 // Trajectories of 2^32 steps and more that no room for aggregates lets split: with more actions than this they are wider
 // than any device's memory.
@@ -116,17 +115,21 @@ __device__ __forceinline__ LossInputPointers fetch_loss_inputs(const impact_loss
 // kPlain: the configuration of the paper's experiments -- no KL term, the clipped surrogate with the default ratio and
 // importance weights, no optional outputs -- with those branches compiled out.
 //
-template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
+// kKeepLearner: the gradient pass finds the learner row's exponentials in registers, and there is one pass.  Else it forms them
+// again, there may be two, and the forms with every switch have registers enough (with the exponentials kept: 0.82 to 0.9 of
+// the rate).
+template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect, bool kKeepLearner>
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid_constant__ LaunchForm sh) {
-    constexpr bool kWide = kA == kWideRows;
+    constexpr bool kWide = kA < 0;
     constexpr bool kRotated = kV == 4 && (kWide || kA % 8 == 0);  // (rows of 4 and 12 actions meet on no bank)
     constexpr bool kSingles = kV == 1 && !kWide && sizeof(LT) == 4;  // rows element by element
     constexpr bool kOdd = kV == 1 && !kSingles;
     constexpr int VW = kV == 1 ? 2 : kV;  // elements of a vector
-    constexpr int NV = (kWide ? kWideElems : kA) / VW;  // vectors per lane at most
+    constexpr int NV = kWide ? -kA : kA / VW;  // vectors per lane
     constexpr int NP = NV * VW / 2 + (kV == 1 ? 1 : 0);  // pairs: Blackwell's packed fp32 add / mul / fma work on two at once
     constexpr float kLowest = -3.402823466e38f;  // stands for an element that is not there: its exponential is 0
+    constexpr int kSure = kWide ? (kV == 4 ? NV - 1 : NV - 2) : NV;  // vectors that are there whatever the lane
     static_assert(kWide || kA % VW == (kV == 1 ? 1 : 0), "whole vectors");
     // The KL term from the target row's own exponentials, kept for the gradient pass too, instead of formed twice again
     // (with the KL term, 100 MB: 7 actions in fp32 25.5 -> 24.9 us, 12 in bf16 20.7 -> 19.2, 14 19.9 -> 18.3).  Not where the
@@ -315,13 +318,13 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     // the lane's part in the row passes (wide: see above), and the row of a tile that it owns
     const int log_l = kWide ? sh.log_lanes : 0;
     const int L = 1 << log_l;
-    const int passes = kWide ? sh.passes : 1;
     const int part = kWide ? (lane & (L - 1)) : 0;
+    const int passes = kKeepLearner ? 1 : sh.passes;
+    const int my_rows = wrow + (lane >> log_l) * passes;  // the rows that the lane works on: one in each pass
+    const bool owner = part < passes;
     // (a lane that owns no row stands for the one after it: the identity map, in that row's trajectory)
-    const int lrow = wrow + (kWide ? (lane >> log_l) * passes + min(part, passes) : lane);
-    const bool owner = kWide ? part < passes : true;
+    const int lrow = my_rows + (passes == 1 ? (owner ? 0 : 1) : min(part, passes));
     const int row_vecs = A / VW;  // vectors of a row (odd counts: and one element)
-    const int nvec = kWide ? (row_vecs + L - 1) >> log_l : NV;  // of the lane with the most
     const int rot = kRotated ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
 
     // The tile (in a flat launch only a block's first tile ends early, only its last one can begin late, and from one of
@@ -404,7 +407,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
     // lies between a tile's scan and its aggregate and another before the later tiles' are looked at.  (Only here: the other
     // split forms have no register left for it and take up to a sixth longer; and asked for by every warp of the grid at the
     // start, the one line is served 2 us late.)
-    constexpr bool kTagKept = kLong && kWide && C == 3;
+    constexpr bool kTagKept = kLong && kWide;
     const unsigned int kept_tag = kTagKept && gwarp == 0 ? dev::launch_tag(p.counter) : 0u;
     auto tag = [&]() { return kTagKept ? kept_tag : dev::launch_tag(p.counter); };
     int s = grp % S, s_prev = 0;
@@ -420,10 +423,14 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         // between this tile's scan and its gradients (only where tiles are numbered tile-major; the values are first
         // looked at after the scan)
         const long long gtile = (long long)blockIdx.x + (long long)n * gridDim.x;
-        const long long agg_stride = g.tile_major ? 2 * g.B : 2;  // slots between a tile's aggregate and that of the tile after it in time
+        const long long tile_stride = g.tile_major ? g.B : 1;  // from a tile to the one after it in time (and two slots to each)
         const bool peeked = kLong && g.tile_major && gwarp == 0 && tl.r > lane;
-        unsigned long long early_a = 0, early_b = 0;
-        if (peeked) dev::load_aggregate(p.tile_aggregates + 2 * gtile, agg_stride, tl.r - lane, early_a, early_b);
+        unsigned long long* const values_at = kLong && kWide && p.tile_values ? p.tile_values + gtile : nullptr;
+        dev::EarlyLook early = {0, 0, 0};
+        if (peeked) {
+            if (kWide) early = dev::look_at_tile(p.tile_aggregates + 2 * gtile, values_at, tile_stride, 1 + lane);
+            else dev::load_aggregate(p.tile_aggregates + 2 * gtile, 2 * tile_stride, tl.r - lane, early.a, early.b);
+        }
         // every thread waits for the stage itself (a bounded wait: on a time-out the flag is set and the
         // thread goes on with whatever the stage holds, so that all barriers below still pair up)
         if (!stage_wait(&full_bar[s], ph, &abort_s)) atomicExch(p.counter + 1, 1u);
@@ -444,19 +451,18 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                               in_row, wrow, NTW, tl.lo, tl.hi, false);
 
         // ---- row passes (every lane; rows that are not the tile's hold stale bytes and are masked)
-        float2 e[kWide ? 1 : NP];         // the learner row's exponentials, kept for the gradient pass
+        float2 e[kKeepLearner ? NP : 1];  // the learner row's exponentials, kept for the gradient pass
         float2 et[kKeepTarget ? NP : 1];  // (KL term) the target row's
         // Per row: log2 e times the largest logit (m2), log2 of the exponentials' sum (lg); learner: 1 / that sum and the
         // mean logit.  m2 and lg are kept apart: adding them first would round their sum, the largest of the numbers
         // that a log-probability is made of.
         float m2_t = 0.0f, lg_t = 0.0f, m2_l = 0.0f, lg_l = 0.0f, inv_s = 0.0f, mean_z = 0.0f, ent = 0.0f, kl = 0.0f, inv_t = 0.0f;
-        auto row_of = [&](int pass) { return wrow + (kWide ? (lane >> log_l) * passes + pass : lane); };
         // byte offset of the lane's i-th vector from the row's first (of `elem`-byte elements)
         auto vec_at = [&](int i, int elem) {
             const int step = (VW * elem) << log_l;
             return kRotated ? ((i * step) ^ (rot * step)) : i * step;
         };
-        auto vec_there = [&](int i) { return !kWide || (i << log_l) + part < row_vecs; };
+        auto vec_there = [&](int i) { return i < kSure || (i << log_l) + part < row_vecs; };
         // (odd counts) does the row start on an odd element?  Tiles are an even number of rows apart.
         const uint32_t tile_odd = kOdd ? (uint32_t)(kLong ? tl.row0 : br.base) & 1u : 0u;
         auto first_of = [&](int r) { return kOdd ? (int)((tile_odd + (uint32_t)r) & 1u) : 0; };  // of the vectors
@@ -472,27 +478,30 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 for (int j = 0; j < kA; ++j) f[j] = get_element<LT>(row, j);
             }
 #pragma unroll
-            for (int i = 0; i < NV; ++i)
-                if (!kSingles && vec_there(i)) Vec<LT, VW>::ld(at + vec_at(i, (int)sizeof(LT)), f + i * VW);
+            for (int i = 0; i < NV && !kSingles; ++i) {
+                // (a vector that is not there: the lane's first, read again and left out)
+                const bool there = vec_there(i);
+                Vec<LT, VW>::ld(at + (there ? vec_at(i, (int)sizeof(LT)) : 0), f + i * VW);
+#pragma unroll
+                for (int v = 0; v < VW; ++v) f[i * VW + v] = there ? f[i * VW + v] : kLowest;
+            }
             if (kOdd && (!kWide || part == 0)) f[2 * NP - 2] = get_element<LT>(row, single_of(r));
 #pragma unroll
             for (int j = 0; j < NP; ++j) z[j] = make_float2(f[2 * j], f[2 * j + 1]);
         };
-        // is pair j worked on?  (run-time counts: groups of two pairs up to the last that holds elements; a uniform test)
-        auto pair_used = [&](int j) { return !kWide || (kOdd && j == NP - 1) || (j & ~1) * 2 < nvec * VW; };
         auto row_max = [&](const float2 (&z)[NP]) {
             float m0 = fmaxf(z[0].x, z[0].y), m1 = m0;
 #pragma unroll
             for (int j = 1; j < NP; ++j) {
-                if (NP > 9 && !pair_used(j)) continue;
                 if (j & 1) m1 = fmaxf(m1, fmaxf(z[j].x, z[j].y));
                 else m0 = fmaxf(m0, fmaxf(z[j].x, z[j].y));
             }
             return fmaxf(m0, m1);
         };
         const float2 log2e2 = make_float2(kLog2e, kLog2e);
-        for (int pass = 0; pass < (kWide ? passes : 1); ++pass) {
-            const int r = row_of(pass);
+#pragma unroll 1
+        for (int pass = 0; pass < passes; ++pass) {
+            const int r = my_rows + pass;
             float2 z[NP];
             // target row
             load_row(s1, r, z);
@@ -504,7 +513,6 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 const float2 neg_m2 = make_float2(-m2t, -m2t);
 #pragma unroll
                 for (int j = 0; j < NP; ++j) {
-                    if (!pair_used(j)) continue;
                     const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);  // (z - m) log2 e
                     const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
                     sum2 = __fadd2_rn(sum2, ex);
@@ -523,12 +531,11 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 const float2 neg_m2 = make_float2(-m2, -m2);
 #pragma unroll
                 for (int j = 0; j < NP; ++j) {
-                    if (!pair_used(j)) continue;
                     const float2 t2 = __ffma2_rn(z[j], log2e2, neg_m2);
                     const float2 ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
                     sum2 = __fadd2_rn(sum2, ex);
                     sez2 = __ffma2_rn(ex, z[j], sez2);
-                    if constexpr (!kWide) e[j] = ex;
+                    if constexpr (kKeepLearner) e[j] = ex;
                 }
             }
             float sum_l = sum2.x + sum2.y, sez = sez2.x + sez2.y;
@@ -597,7 +604,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                     if (kWide) for (int o = 1; o < L; o <<= 1) klr += __shfl_xor_sync(0xffffffffu, klr, o);
                 }
             }
-            if (!kWide || part == pass) {
+            if (kKeepLearner || part == pass) {
                 m2_t = m2t; lg_t = lgt; m2_l = m2; lg_l = lgl; inv_s = is; mean_z = __fmul_rn(sez, is); kl = klr; inv_t = ist;
                 // H = -sum_j pi_j lp_j = (m - sum_j e_j z_j / S) + ln S: what the logits have in common cancels first
                 ent = fmaf(lgl, kLn2, __fadd_rn(m_l, -mean_z));
@@ -612,10 +619,9 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         st.value = cur.value;
         st.value_next = cur.value_next;
         st.ends = ends_here(tl);
-        const int orow = kWide && !owner ? wrow : lrow;  // (a lane that owns no row looks at the warp's first)
         // (kept finite where the taken action is masked by the type's lowest value: its probability is 0 either way)
-        st.l2_target = dev::max_or_nan(fmaf(get_element<LT>(s1 + orow * in_row, act), kLog2e, -m2_t) - lg_t, kLowest);
-        st.l2_theta = dev::max_or_nan(fmaf(get_element<LT>(s0 + orow * in_row, act), kLog2e, -m2_l) - lg_l, kLowest);
+        st.l2_target = dev::max_or_nan(fmaf(get_element<LT>(s1 + (owner ? lrow : my_rows) * in_row, act), kLog2e, -m2_t) - lg_t, kLowest);
+        st.l2_theta = dev::max_or_nan(fmaf(get_element<LT>(s0 + (owner ? lrow : my_rows) * in_row, act), kLog2e, -m2_l) - lg_l, kLowest);
         float fa, fb;
         const bool truncated = step_map<kPlain>(st, k, fa, fb);
         const bool mine = is_mine(tl);
@@ -625,7 +631,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         int limit = 31 - lane;
         if constexpr (!kLong) {
             const int left = reach - wrow;  // ... counted from the warp's first row
-            limit = min(limit, (kWide ? (left / passes << log_l) + left % passes : left) - lane);
+            limit = min(limit, (passes == 1 ? left << log_l : (left / passes << log_l) + left % passes) - lane);
         }
 
         // the next tile's scalars travel while this tile is worked on
@@ -665,13 +671,15 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                 if (w > gwarp) { lb = fmaf(f.x, lb, f.y); la = f.x * la; }
             }
             const float ma = fa * la, mb = fmaf(fa, lb, fb);
-            if (gtid == 0) dev::publish_tile_aggregate(p.tile_aggregates + 2 * gtile, ma, mb, tag());
+            unsigned long long* const slots = p.tile_aggregates + 2 * gtile;
+            if (gtid == 0) dev::publish_tile_aggregate(slots, ma, mb, tag());
             float carry = 0.0f;
             if (here.r > 0) {  // uniform over the group
                 if (gwarp == 0) {
-                    const float c = dev::compose_later_aggregates(p.tile_aggregates + 2 * gtile, agg_stride, here.r,
-                                                                  tag(), &abort_s, p.counter + 1, peeked, early_a,
-                                                                  early_b);
+                    const float c = kWide ? dev::value_from_later_tiles(slots, values_at, tile_stride, here.r,
+                                                                        tag(), &abort_s, p.counter + 1, early)
+                                          : dev::compose_later_aggregates(slots, 2 * tile_stride, here.r, tag(), &abort_s,
+                                                                          p.counter + 1, peeked, early.a, early.b);
                     if (lane == 0) carry_s[grp] = c;
                 }
                 asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
@@ -679,6 +687,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             }
             adv = fmaf(ma, carry, mb);
             after = fmaf(la, carry, lb);
+            if (kWide && gtid == 0 && values_at) dev::publish_tagged(values_at, adv, tag());
         }
         if constexpr (!kPlain) {
             const float below = __shfl_down_sync(0xffffffffu, adv, 1);
@@ -703,12 +712,15 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         if (n + C >= n_tiles) hand_over_sums();
 
         // ---- gradients: row_j = e_j (ga z_j + gb) [- kl_coef pi_target_j / M], then the taken action's entry
-        const float w1 = __fmul_rn(wpg, k.inv_M), ce = k.ent_over_M, ck = kPlain ? 0.0f : k.kl_over_M;
+        float w1 = __fmul_rn(wpg, k.inv_M);
+        if (kWide && kKeepLearner) w1 = __shfl_sync(0xffffffffu, w1, lane & ~(L - 1));  // (the owner's)
+        const float ce = k.ent_over_M, ck = kPlain ? 0.0f : k.kl_over_M;
         const float ga = __fmul_rn(ce, inv_s), gb = __fmul_rn(__fadd_rn(fmaf(-ce, mean_z, w1), ck), inv_s);
-        for (int pass = 0; pass < (kWide ? passes : 1); ++pass) {
-            const int r = row_of(pass);
+#pragma unroll 1
+        for (int pass = 0; pass < passes; ++pass) {
+            const int r = my_rows + pass;
             float pga = ga, pgb = gb, pm2 = m2_l, plt = kPlain ? 0.0f : __fadd_rn(m2_t, lg_t);
-            if (kWide) {
+            if (!kKeepLearner) {  // (its owner's)
                 const int from = (lane & ~(L - 1)) + pass;
                 pga = __shfl_sync(0xffffffffu, ga, from);
                 pgb = __shfl_sync(0xffffffffu, gb, from);
@@ -723,11 +735,11 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             // the gradient of up to VW neighbouring elements: z and zt in, their places among the lane's elements
             auto grad_of = [&](const float2& z2, const float2& zt2, int pair) {
                 float2 ex;
-                if constexpr (kWide) {
+                if constexpr (kKeepLearner) {
+                    ex = e[pair];
+                } else {
                     const float2 t2 = __ffma2_rn(z2, log2e2, neg_m2);
                     ex = make_float2(dev::exp2_fast(t2.x), dev::exp2_fast(t2.y));
-                } else {
-                    ex = e[pair];
                 }
                 float2 gr = __fmul2_rn(ex, __ffma2_rn(z2, ga2, gb2));
                 if (want_kl) {
@@ -746,7 +758,6 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             const int first = first_of(r) + part * VW;
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
-                if (kWide && i >= nvec) continue;  // (uniform)
                 if (!vec_there(i)) continue;
                 float z[VW], o[VW], zt[VW];
 #pragma unroll
@@ -828,17 +839,17 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
 // ------------------------------------------------------------------------------------------
 // Launch
 // ------------------------------------------------------------------------------------------
-template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect>
+template <typename LT, typename GT, int kA, int C, int kV, bool kPlain, bool kLong, bool kIndirect, bool kKeepLearner = true>
 int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
     const int nt = rl.nt;
-    auto kernel = impact_loss_categorical_kernel<LT, GT, kA, C, kV, kPlain, kLong, kIndirect>;
+    auto kernel = impact_loss_categorical_kernel<LT, GT, kA, C, kV, kPlain, kLong, kIndirect, kKeepLearner>;
     const size_t stage = cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT));
     LaunchShape ls;
     if (!launch_shape(p.geo, nt, kLong, stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di, &ls)) return IMPACT_ERR_UNSUPPORTED;
     LaunchForm sh = {};
     sh.nt = nt;
     sh.log_lanes = rl.log_lanes;
-    sh.passes = (nt / 4 << rl.log_lanes) / 32;
+    sh.passes = rl.passes;
     sh.rot_shift = rl.rot_shift;
     sh.rot_mask = rl.rot_mask;
     sh.stages = ls.stages;
@@ -875,21 +886,21 @@ inline bool is_plain(const CatParams& p) {
            p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
 }
 
-// How a warp's rows on 2^l lanes each meet on the banks, and the rotation that lanes of vectors of four elements take them in.
-// Returns the accesses that still meet.
+// Rows on 2^l lanes each: the rows of a tile, and the rotation that lanes of vectors of four elements take them in, from how a
+// warp's rows meet on the banks.
 template <typename LT, int kV>
-int settle_rows(RowLayout& rl, int A, int l) {
+void settle_rows(RowLayout& rl, int A, int l) {
     constexpr int VW = kV == 1 ? 2 : kV;
     rl.log_lanes = l;
-    const int passes = (rl.nt / 4 << l) / 32, vecs = A / VW;
-    const BankPattern b = bank_pattern(A * sizeof(LT) * (size_t)(passes < 1 ? 1 : passes), 1 << l, VW * (int)sizeof(LT));
+    rl.nt = (128 >> l) * rl.passes;
+    const int vecs = A / VW;
+    const BankPattern b = bank_pattern(A * sizeof(LT) * rl.passes, 1 << l, VW * (int)sizeof(LT));
     rl.rot_mask = 0;
     rl.rot_shift = b.shift;
     if (kV == 4 && vecs % (1 << l) == 0) {
         const int per_lane = vecs >> l;
         while (2 * (rl.rot_mask + 1) <= b.ways && per_lane % (2 * (rl.rot_mask + 1)) == 0) rl.rot_mask = 2 * rl.rot_mask + 1;
     }
-    return b.ways / (rl.rot_mask + 1);
 }
 
 // Consumer groups: four with every switch compiled in; five in the default configuration; six there for small action
@@ -927,61 +938,81 @@ int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream)
                          : launch_categorical<LT, GT, A, C, kV, false, false, false>(p, rl, di, stream);
 }
 
-// Rows of a tile where a row takes more than a lane: tiles of up to 36 KB (a ring of six stages, four of them being worked
-// on).  Few long trajectories are split into tiles of 64 rows, wherever five stages of those fit (up to 44 KB: A = 64 with
-// fp32 logits and bf16 gradients needs 41 KB, and 16 trajectories of 4096 steps take 18.9 us split against 114 on sixteen
-// blocks), or of 128 where narrow types allow it and blocks have two of them (bf16, A = 64: 16 x 4096 16.5 us against 21.5
-// in tiles of 64, 16 x 1000 11.0 against 8.8).
-inline int wide_tile_rows(const BatchGeometry& g, bool aggregates, int A, size_t in_elem, size_t out_elem, const DeviceInfo* di) {
-    int nt = 128;
-    while (nt > 8 && cat_stage_bytes(nt, A, in_elem, out_elem) > 36 * 1024) nt /= 2;
-    const bool few = nt < kMinTileRows || g.B * ((g.T + nt - 1) / nt) < 2 * di->sm_count;
-    if (few && splits_trajectories(g, aggregates, kMinTileRows, di, A) &&
-        stages_that_fit(cat_stage_bytes(kMinTileRows, A, in_elem, out_elem), di->max_smem_optin) > 4)
-        nt = kMinTileRows;
-    return nt;
+// How a row of more than 32 actions is laid on lanes: the fewest that hold it in up to 32 elements each (a row costs a lane
+// some hundred instructions besides its elements'), and the vectors that this makes a lane's: 5 to 8 of four elements, or 10
+// to 16, even numbers of them, of two.
+struct WideWidth {
+    int log_lanes, vectors;
+};
+constexpr int wide_elements(int A) { return A % 4 == 0 ? 4 : 2; }  // of a vector
+constexpr WideWidth wide_width(int A) {
+    const int most = 32 / wide_elements(A), step = most / 8, vecs = A / wide_elements(A);
+    WideWidth w = {1, 5};
+    while ((most << w.log_lanes) < vecs) ++w.log_lanes;
+    while ((w.vectors * step << w.log_lanes) < vecs) ++w.vectors;
+    w.vectors *= step;
+    return w;
+}
+// Rows of a tile where a row takes more than a lane: those of one pass of a group's warps or of two, which share what a tile
+// costs besides its rows.  Split launches, three groups: two passes where the tiles are enough for every SM (16 x 4096 steps of
+// 64 actions in bf16 13.5 us instead of 17.5, of 80 in fp32 20.7 / 28.7; 20 x 300 of 100 7.3 / 6.8) and the ring has a stage for
+// every group.  Whole trajectories, four groups: with two tiles to every SM (bf16, 50 actions: 8.0 us instead of 8.8 at 50 000
+// steps, 30.8 / 34.6 at 400 000, but 7.0 / 6.4 at 25 000) and two stages more than groups.
+inline int wide_tile_rows(const BatchGeometry& g, bool split, int A, size_t in_elem, size_t out_elem, const DeviceInfo* di) {
+    const int one = 128 >> wide_width(A).log_lanes, two = 2 * one;
+    const int fit = stages_that_fit(cat_stage_bytes(two, A, in_elem, out_elem), di->max_smem_optin);
+    if (split) return fit >= 3 && split_tiles(g, two) >= di->sm_count ? two : one;
+    return fit >= 6 && g.B * g.T >= 2ll * two * di->sm_count ? two : one;
 }
 
-template <typename LT, typename GT, int kV>
-int32_t run_wide_form(const CatParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
+template <typename LT, typename GT, int kV, int NV>
+int32_t run_wide_form(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
     constexpr int C = 4;
-    const bool fits = fits_flat(p.geo);
-    if (splits_trajectories(p.geo, p.tile_aggregates, rl.nt, di, p.A) || (!fits && p.tile_aggregates)) {
-        if (rl.nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
-        // Tiles of 64 rows go to three groups: they have 128 registers to a thread and spill nothing (four: 96).
-        // 16 x 4096 steps of 64 actions take 18.7 us instead of 20.4, 31 x 4000 32.0 instead of 35.5.  Four where each
-        // has one tile of the block's, and the ring six stages: 16 x 2048 12.2 us instead of 12.9.
-        const long long tiles = p.geo.B * ((p.geo.T + kMinTileRows - 1) / kMinTileRows);
-        const bool one_each = (tiles + di->sm_count - 1) / di->sm_count == C;
-        if (rl.nt == kMinTileRows &&
-            !(one_each && stages_that_fit(cat_stage_bytes(rl.nt, p.A, sizeof(LT), sizeof(GT)), di->max_smem_optin) >= C + 2))
-            return launch_categorical<LT, GT, kWideRows, 3, kV, false, true, false>(p, rl, di, stream);
-        return launch_categorical<LT, GT, kWideRows, C, kV, false, true, false>(p, rl, di, stream);
+    const int log_lanes = wide_width(p.A).log_lanes, one_pass = 128 >> log_lanes;
+    auto laid_out = [&](int rows) {
+        RowLayout rl;
+        rl.passes = rows / one_pass;
+        settle_rows<LT, kV>(rl, p.A, log_lanes);
+        return rl;
+    };
+    if (p.indirect) {
+        if constexpr (kV == 4 && NV == 8) {
+            if (p.A == 64 && p.geo.T <= 64)
+                return launch_categorical<LT, GT, -NV, C, kV, false, false, true, false>(p, laid_out(one_pass), di, stream);
+        }
+        return IMPACT_ERR_UNSUPPORTED;
+    }
+    const bool fits = fits_flat(p.geo), plain = is_plain(p);
+    // Tiles of few rows keep their maps and values in the workspace's spare slots, as do values alone, where there is room.
+    const int nt = wide_tile_rows(p.geo, true, p.A, sizeof(LT), sizeof(GT), di);
+    const long long tiles = split_tiles(p.geo, nt);
+    const bool room = nt < kMinTileRows ? p.spare_slots && 3 * tiles <= kSpareSlots : p.tile_aggregates != nullptr;
+    if (splits_trajectories(p.geo, room, one_pass, di, p.A) || (!fits && room)) {
+        CatParams q = p;
+        if (nt < kMinTileRows) q.tile_aggregates = p.spare_slots;
+        q.tile_values = nt < kMinTileRows ? p.spare_slots + 2 * tiles : tiles <= kSpareSlots ? p.spare_slots : nullptr;
+        return launch_categorical<LT, GT, -NV, 3, kV, false, true, false, false>(q, laid_out(nt), di, stream);
     }
     if (!fits) return IMPACT_ERR_UNSUPPORTED;
-    return is_plain(p) ? launch_categorical<LT, GT, kWideRows, C, kV, true, false, false>(p, rl, di, stream)
-                       : launch_categorical<LT, GT, kWideRows, C, kV, false, false, false>(p, rl, di, stream);
+    const int rows = wide_tile_rows(p.geo, false, p.A, sizeof(LT), sizeof(GT), di);
+    if (!plain) return launch_categorical<LT, GT, -NV, C, kV, false, false, false, false>(p, laid_out(rows), di, stream);
+    // (fp32 rows take as long as their bytes: one pass)
+    if constexpr (sizeof(LT) == 2 && sizeof(GT) == 2) {
+        if (rows > one_pass) return launch_categorical<LT, GT, -NV, C, kV, true, false, false, false>(p, laid_out(rows), di, stream);
+    }
+    return launch_categorical<LT, GT, -NV, C, kV, true, false, false, true>(p, laid_out(one_pass), di, stream);
 }
 
 template <typename LT, typename GT, int kV>
 int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    constexpr int VW = kV == 1 ? 2 : kV;
-    const int vecs = p.A / VW;
-    RowLayout rl;
-    auto settle = [&](int l) { return settle_rows<LT, kV>(rl, p.A, l); };
-    // Rows of more than a lane: the fewest lanes that hold a row and do not meet on the banks more than two at a time.
-    rl.nt = wide_tile_rows(p.geo, p.tile_aggregates, p.A, sizeof(LT), sizeof(GT), di);
-    int l = 1;
-    while (l < 5 && ((rl.nt / 4 << l) < 32 || ((kWideElems / VW) << l) < vecs || settle(l) > 2)) ++l;
-    settle(l);
-    if (p.indirect) {
-        if constexpr (kV == 4) {
-            if (p.A == 64 && p.geo.T <= 64)
-                return launch_categorical<LT, GT, kWideRows, 4, kV, false, false, true>(p, rl, di, stream);
-        }
-        return IMPACT_ERR_UNSUPPORTED;
+    constexpr int kStep = kV == 4 ? 1 : 2;
+    switch (wide_width(p.A).vectors) {
+        case 5 * kStep: return run_wide_form<LT, GT, kV, 5 * kStep>(p, di, stream);
+        case 6 * kStep: return run_wide_form<LT, GT, kV, 6 * kStep>(p, di, stream);
+        case 7 * kStep: return run_wide_form<LT, GT, kV, 7 * kStep>(p, di, stream);
+        case 8 * kStep: return run_wide_form<LT, GT, kV, 8 * kStep>(p, di, stream);
+        default: return IMPACT_ERR_UNSUPPORTED;
     }
-    return run_wide_form<LT, GT, kV>(p, rl, di, stream);
 }
 
 template <typename LT, typename GT>

@@ -275,6 +275,69 @@ __device__ __forceinline__ float compose_later_aggregates(const unsigned long lo
     return x;
 }
 
+// The same for tiles of few rows, of which a trajectory has hundreds: run by one warp, it looks back from the nearest later
+// tile to the first whose value -- the advantage at its first step, published once it is known -- is there, and composes the
+// maps of the tiles before that.  (A look at all later tiles takes a trip to L2 for every 32 of them: 11 of 375 tiles.)
+// `maps` and `values` point at this tile's slots, the tile j places later has its own 2 * j * stride and j * stride before
+// (values NULL: there is no room for them, and every look goes on to the trajectory's last tile).
+struct EarlyLook {  // what lane l found of the tile l + 1 places later ahead of time
+    unsigned long long a, b, value;
+};
+__device__ __forceinline__ EarlyLook look_at_tile(const unsigned long long* maps, const unsigned long long* values,
+                                                  long long stride, int j) {
+    EarlyLook x;
+    load_aggregate(maps, 2 * stride, j, x.a, x.b);
+    x.value = 0;  // (no tag is 0)
+    if (values) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x.value) : "l"(values - (long long)j * stride) : "memory");
+    return x;
+}
+__device__ __forceinline__ float value_from_later_tiles(const unsigned long long* maps, const unsigned long long* values,
+                                                        long long stride, int r, unsigned int tag, int* abort_flag,
+                                                        unsigned int* error_word, const EarlyLook& early) {
+    const int lane = threadIdx.x & 31;
+    float fa = 1.0f, fb = 0.0f;  // the maps of the tiles looked at so far: what enters the last of them to what enters this tile
+    EarlyLook x = early;
+    for (int base = 1;; base += 32) {
+        const int j = base + lane;
+        int known = j > r ? 2 : 0;  // 1: the tile's map, 2: its value (beyond the trajectory's last tile it is 0)
+        unsigned int needed = 0, have = 0, valued = 0;
+        for (int tries = 0; tries < (1 << 22); ++tries) {
+            if (known == 0) {
+                if (base > 1 || tries > 0) x = look_at_tile(maps, values, stride, j);
+                if ((unsigned int)(x.value >> 32) == tag) known = 2;
+                else if ((unsigned int)(x.a >> 32) == tag && (unsigned int)(x.b >> 32) == tag) known = 1;
+            }
+            valued = __ballot_sync(0xffffffffu, known == 2);
+            have = __ballot_sync(0xffffffffu, known != 0);
+            needed = valued ^ (valued - 1u);  // lanes up to the first of those (all, where there is none)
+            if ((have & needed) == needed) break;
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(abort_flag))) break;
+        }
+        if ((have & needed) != needed) {
+            *reinterpret_cast<volatile int*>(abort_flag) = 1;
+            if (lane == 0) atomicExch(error_word, 1u);
+            return 0.0f;
+        }
+        float a = 1.0f, b = 0.0f;
+        if ((needed >> lane) & 1u) {
+            a = known == 2 ? 0.0f : __uint_as_float((unsigned int)x.a);
+            b = j > r ? 0.0f : __uint_as_float((unsigned int)(known == 2 ? x.value : x.b));
+        }
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float a2 = __shfl_down_sync(0xffffffffu, a, off);
+            const float b2 = __shfl_down_sync(0xffffffffu, b, off);
+            if (lane + off < 32) {  // (a, b) <- (a, b) o (a2, b2): the higher lane's map is applied earlier
+                b = fmaf(a, b2, b);
+                a = a * a2;
+            }
+        }
+        fb = fmaf(fa, __shfl_sync(0xffffffffu, b, 0), fb);
+        fa = fa * __shfl_sync(0xffffffffu, a, 0);
+        if (valued) return fb;
+    }
+}
+
 // Scalars of the loss that the kernels need; filled on the host.
 struct LossScalars {
     float rho_bar, c_bar, clip_lo, clip_hi;

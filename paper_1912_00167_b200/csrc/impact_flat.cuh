@@ -318,7 +318,7 @@ static __device__ __noinline__ void send_rows_general(unsigned char* out, const 
 
 // How the rows of a batch are laid on lanes: rows of a tile, lanes per row, rotation of a lane's vectors.
 struct RowLayout {
-    int nt = 128, log_lanes = 0, rot_shift = 0, rot_mask = 0;
+    int nt = 128, log_lanes = 0, passes = 1, rot_shift = 0, rot_mask = 0;
 };
 
 // Long trajectories go to neighbouring blocks where blocks that own whole ones would leave most of the device idle: the
@@ -327,15 +327,17 @@ struct RowLayout {
 // share of the device that the flat launch keeps busy:
 //   rows of one lane: 0.21 (A = 18, 31 x 4000) 16.3 / 14.6; 0.30 (18, 45 x 1000) 7.5 / 7.3; 0.40 (18, 59 x 4000) 17.1 /
 //   25.6; 0.43 (20, 64 x 1000) 9.4 / 11.1; 0.47 (7, 69 x 4000) 18.2 / 23.6; 0.70 (18, 104 x 4000) 19.9 / 40.2
-//   rows of several lanes (`wide_row` elements, else 0): 0.21 (40, 31 x 4000) 54.9 / 30.2; 0.30 (64, 45 x 1000) 18.5 / 14.3;
-//   0.40 (64, 59 x 4000) 63.7 / 55.9; 0.43 (33, 64 x 1000) 17.8 / 17.5 and (40) 16.6 / 17.1; 0.54 (64, 80 x 1000) 19.4 /
-//   22.3; and with more trajectories than blocks, where whole ones leave most blocks idle for the last of them: 0.54
-//   (64, 160 x 1000) 36.2 / 32.9 and (80) 56.9 / 43.1, but (33) 31.8 / 35.8; 0.68 (64, 200 x 1000) 36.6 / 40.2
+//   rows of several lanes (`wide_row` elements, else 0) in tiles of nt rows, 128 / lanes, each of which takes a group some 0.65
+//   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one 2.4 times its tiles per SM and
+//   3.4 tiles more: (64, 40 x 300) 7.5 / 7.4; (100, 40 x 300) 10.8 / 8.9; (64, 60 x 500) 10.5 / 10.1, in bf16 8.4 / 9.9;
+//   (180, 60 x 500) 22.4 / 25.0; (180, 20 x 100) 7.5 / 6.4; (400, 10 x 50) 8.1 / 5.7; (400, 60 x 100) 12.4 / 13.4;
+//   (100, 16 x 2000) 49 / 19; (64, 160 x 100) 6.0 / 7.7
+inline long long split_tiles(const BatchGeometry& g, int nt) { return g.B * ((g.T + nt - 1) / nt); }
 inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row) {
-    if (g.T <= nt || nt < kMinTileRows || !aggregates) return false;
+    if (g.T <= nt || !aggregates) return false;
     const long long rounds = (g.B + di->sm_count - 1) / di->sm_count;
-    const int percent = wide_row == 0 ? 30 : (wide_row >= 48 && rounds > 1) ? 60 : 45;
-    return 100 * g.B < percent * rounds * di->sm_count;
+    if (wide_row) return 5 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > 12 * split_tiles(g, nt) + 17 * di->sm_count;
+    return 100 * g.B < 30 * rounds * di->sm_count;
 }
 // Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.
 inline bool fits_flat(const BatchGeometry& g) { return g.T < (1ll << 32) - 4096; }

@@ -551,7 +551,6 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
     sh.in_flight = ls.in_flight;
     sh.lanes = ls.lanes;
     sh.log_lanes = rl.log_lanes;
-    sh.passes = 1;
     sh.rot_shift = rl.rot_shift;
     sh.rot_mask = rl.rot_mask;
     const size_t smem = (size_t)sh.stages * stage;
@@ -569,8 +568,9 @@ template <int kD, int C, int CP, int kV>
 int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
     const bool plain = p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
                        p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
-    if (splits_trajectories(p.geo, p.tile_aggregates, rl.nt, di, 0) || !fits_flat(p.geo)) {
-        if (!p.tile_aggregates || rl.nt < kMinTileRows) return IMPACT_ERR_UNSUPPORTED;
+    const bool room = p.tile_aggregates && rl.nt >= kMinTileRows;
+    if (splits_trajectories(p.geo, room, rl.nt, di, 0) || !fits_flat(p.geo)) {
+        if (!room) return IMPACT_ERR_UNSUPPORTED;
         return launch_gaussian<kD, C, kV, false, true>(p, rl, di, stream);
     }
     return plain ? launch_gaussian<kD, CP, kV, true, false>(p, rl, di, stream)

@@ -234,6 +234,7 @@ static int32_t loss_fwd_bwd_impl(
     p.tile_aggregates = (T > kMinTileRows && workspace_bytes >= impact_loss_workspace_bytes(B, T))
                             ? reinterpret_cast<unsigned long long*>(static_cast<char*>(workspace) + kWorkspaceFixedBytes)
                             : nullptr;
+    p.spare_slots = static_cast<unsigned long long*>(workspace);
     p.target_copy = target_logits_copy;
     p.indirect = indirect;
     p.A = A;

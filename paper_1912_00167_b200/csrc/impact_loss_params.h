@@ -14,12 +14,13 @@ namespace impact {
 using dev::LossScalars;
 
 constexpr int kWsMaxStages = 24;      // stages of a persistent kernel's ring at most
-// A workspace: 128 KB that nothing uses any more (they stay, so that its size and the places in it do), the counter words,
-// the tagged rows, the tiles' aggregates where there is room.
-constexpr int kMaxGridBlocks = 4096;  // (32 bytes each of the unused part)
+// A workspace: 128 KB of spare slots for split launches of wide rows, the counter words, the tagged rows, the tiles' aggregates
+// where there is room.
+constexpr int kMaxGridBlocks = 4096;  // (32 bytes each of the first part)
+constexpr long long kSpareSlots = kMaxGridBlocks * 32ll / 8;
 constexpr size_t kCounterBytes = 256; // words: [0] unused, [1] error flag, [2] launch number
 constexpr int kMaxTaggedRows = 1024;  // rows of eight (value, tag) pairs after the counter words: one per block of a persistent kernel
-constexpr int kMinTileRows = 64;      // the smallest tile of a launch that publishes its tiles' aggregates
+constexpr int kMinTileRows = 64;      // the smallest tile that tile_aggregates has room for
 
 // How a batch is laid out over the grid (see impact_flat.cuh).
 struct BatchGeometry {
@@ -46,6 +47,8 @@ struct CatParams {
     unsigned int* counter;
     unsigned long long* tagged_rows;      // rows of (value, launch tag) pairs, see dev::publish_tagged
     unsigned long long* tile_aggregates;  // long launches: two (value, launch tag) pairs per tile (NULL = no room for them)
+    unsigned long long* tile_values;      // long launches of wide rows: a (value, launch tag) pair per tile (NULL = no room)
+    unsigned long long* spare_slots;      // kSpareSlots of the workspace's (NULL = a call without one)
     void* target_copy;  // where the target logits are written as well (NULL = nowhere)
     const impact_loss_inputs* indirect;  // device record that overrides the nine input pointers above (NULL = none)
     BatchGeometry geo;

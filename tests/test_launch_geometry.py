@@ -41,6 +41,11 @@ def test_launches_that_take_a_companion(tmp_path):
     assert done.returncode == 0, done.stdout
 
 
+def test_every_wide_row_has_its_lanes(tmp_path):
+    done = subprocess.run([_host_program(tmp_path, "wide_check")], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout
+
+
 def test_bytes_outside_one_range_are_not_read_in_place(tmp_path):
     """A kernel reads host memory only where all of it lies in one pinned range: the arithmetic of that."""
     done = subprocess.run([_host_program(tmp_path, "pinned_check")], capture_output=True, text=True)
