@@ -433,7 +433,7 @@ int32_t impact_buffer_import_state(impact_buffer* h, const void* blob, size_t bl
  *         a DEVICE array of n_candidates x (n_fields + 1) pointers: for each candidate its n_fields field sources
  *         (NULL = leave the field for the append) and one extra pointer that is remembered with the slot -- the
  *         target network's output for that batch.  Candidates are taken in turn (pushes so far mod n_candidates).
- *         The copy itself is a second kernel enqueued by this call.
+ *         The copy is part of the same kernel.
  *     (2) if inputs_out != NULL: a live slot is drawn, its count goes up, after the K-th traversal it is discarded,
  *         and *inputs_out (DEVICE memory, 16-byte aligned) receives the arguments of the loss call for that batch:
  *         the slot's fields named by `map` (-1 = not kept in the ring: NULL), learner_logits / values /

@@ -845,7 +845,7 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     auto kernel = impact_loss_categorical_kernel<LT, GT, kA, C, kV, kPlain, kLong, kIndirect, kKeepLearner>;
     const size_t stage = cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT));
     LaunchShape ls;
-    if (!launch_shape(p.geo, nt, kLong, stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di, &ls)) return IMPACT_ERR_UNSUPPORTED;
+    if (!launch_shape(p.geo, nt, kLong, stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di, &ls, kIndirect)) return IMPACT_ERR_UNSUPPORTED;
     LaunchForm sh = {};
     sh.nt = nt;
     sh.log_lanes = rl.log_lanes;
@@ -875,7 +875,8 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     } else {
         sh.n_prefetch = plan.prefetch_tiles;
     }
-    const int shared_percent = plan.companion ? percent_beside_companion(smem + own_smem, di) : -1;
+    const int shared_percent = plan.companion ? percent_beside(smem + own_smem, 0, di)
+                               : kIndirect    ? percent_beside(smem + own_smem, kRingStepShared, di) : -1;
     IMPACT_CUDA_TRY(launch_laid_out(shared_percent, kernel, dim3((unsigned)ls.grid), dim3(C * 128 + 32), smem, stream, p, sh));
     return IMPACT_OK;
 }

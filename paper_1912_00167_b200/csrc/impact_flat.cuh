@@ -364,7 +364,7 @@ struct LaunchShape {
     int stages, in_flight, lanes;
 };
 inline bool launch_shape(BatchGeometry& g, int nt, bool is_long, size_t stage_bytes, size_t tile_in_bytes, int groups,
-                         const DeviceInfo* di, LaunchShape* out) {
+                         const DeviceInfo* di, LaunchShape* out, bool cold = false) {
     g.nt = nt;
     g.ntiles = is_long ? (int)((g.T + nt - 1) / nt) : 1;
     if (is_long) {
@@ -383,7 +383,8 @@ inline bool launch_shape(BatchGeometry& g, int nt, bool is_long, size_t stage_by
     if (out->grid > kMaxTaggedRows) return false;  // one tagged row per block
     // tile-major once every block has a trajectory of its own: the aggregates a tile needs are then a round old
     g.tile_major = (is_long && g.B >= out->grid) ? 1 : 0;
-    ws_ring_shape(stage_bytes, tile_in_bytes, groups, di->max_smem_optin, out->tiles_per_block, &out->stages, &out->in_flight);
+    ws_ring_shape(stage_bytes, tile_in_bytes, groups, di->max_smem_optin, out->tiles_per_block, &out->stages, &out->in_flight,
+                  cold);
     if (out->stages < 1 || out->in_flight < 1) return false;
     const int spare = out->stages - out->in_flight;  // producer lanes that request tiles side by side
     out->lanes = spare < 4 ? (spare < 1 ? 1 : spare) : 4;

@@ -83,10 +83,13 @@ int32_t fill_scalars(LossScalars& k, float rho_bar, float c_bar, float clip_eps,
 // first tile's landing is what such a launch waits for).  Beyond the window there is room for the tiles being
 // worked on and being stored.  The barrier protocol needs stages >= in_flight + groups, or exactly one stage per
 // group (then the stage's previous tile is the one the same group worked on last); 0 stages = no valid shape.
+// `cold`: 72 KB whatever the tiles -- no kernel has asked L2 for the inputs of a launch that finds them by a record, and a
+// drawn batch comes from a ring larger than L2 (a step and a loss on 131 072 steps of 18 actions 11.0 us with 48 KB, 10.6 with
+// 72, 11.1 with 96, 11.6 with 32).
 void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max_smem, long long tiles_per_block,
-                   int* stages, int* in_flight) {
+                   int* stages, int* in_flight, bool cold) {
     size_t window = (size_t)option(IMPACT_OPT_WINDOW_BYTES);
-    if (window == 0) window = tiles_per_block <= 8 ? 48 * 1024 : 72 * 1024;
+    if (window == 0) window = tiles_per_block <= 8 && !cold ? 48 * 1024 : 72 * 1024;
     int w = (int)((window + tile_in_bytes - 1) / tile_in_bytes);
     if (w < 2) w = 2;
     if (w > 8) w = 8;

@@ -119,7 +119,7 @@ int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t st
 inline int stages_that_fit(size_t stage_bytes, int max_smem) { return (int)((size_t)(max_smem - 4096) / stage_bytes); }
 // Tiles the producer keeps in flight and stages of the ring, for tiles of `tile_in_bytes` bytes of logits.
 void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max_smem, long long tiles_per_block,
-                   int* stages, int* in_flight);
+                   int* stages, int* in_flight, bool cold = false);
 // Does a companion (impact_prefetch.cu) pay for a categorical launch of `rows` steps of `row_bytes` inputs each?  (Where
 // ws_plan finds its tiles large and few enough.)  Both sides measured, companion / none, in us, on inputs that come from HBM;
 // where a program's inputs are still in L2 a companion can only cost (1024 x 128 of 18 actions 7.9 / 7.5, cold 7.5 / 7.9).
@@ -161,8 +161,9 @@ WsPlan ws_plan(long long tiles, long long grid, size_t tile_bytes, int in_flight
 // through.  With all of it as shared memory: 31 x 4000 steps of 18 actions in bf16 13.4 us instead of 12.8, of 32 in fp32 22.8
 // instead of 20.0 (no companion), 14 x 2091 of 64 with every switch 14.8 instead of 13.4, Gaussian 28 012 x 28 of 3 dimensions
 // 19.3 instead of 18.9.
-inline int percent_beside_companion(size_t smem, const DeviceInfo* di) {
-    const size_t percent = (100 * (smem + 2048) + di->smem_per_sm - 1) / di->smem_per_sm;
+constexpr size_t kRingStepShared = 20 * 1024;  // of a block of the ring's step, which runs between loss launches
+inline int percent_beside(size_t smem, size_t other, const DeviceInfo* di) {
+    const size_t percent = (100 * (smem + other + 2048) + di->smem_per_sm - 1) / di->smem_per_sm;
     return percent < 100 ? (int)percent : 100;
 }
 

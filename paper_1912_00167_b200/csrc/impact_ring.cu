@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "impact.h"
+#include "impact_device.cuh"
 #include "impact_internal.h"
 #include "impact_pinned.h"
 
@@ -206,17 +207,30 @@ __global__ void __launch_bounds__(256) stream_copy_kernel(const uint4* __restric
 // same trace for the same seed.
 struct RingDeviceHeader {
     int32_t write_cursor, read_cursor;
-    uint32_t n_events, tickets;  // tickets: 0 between launches
+    uint32_t n_events, pad;
     uint64_t draws, pushes;
 };
 static_assert(sizeof(RingDeviceHeader) == 32, "read as two 16-byte words");
 constexpr int kEventLog = 4096;  // the most recent push / sample outcomes, for the host to read back
 constexpr int kMaxDeviceSlots = 1024;  // slots a buffer may have for its bookkeeping to go to the device
 
+// What every block of a step reads, in two copies of which a launch reads one and writes the other: the launch's number, odd
+// or even, says which.  `tickets` goes up by 2^kTicketBits with every launch, whatever its grid, and by less with each of its
+// blocks but the one that makes up for them: what it held when a block drew its ticket, shifted, is the launch's number.
+struct RingDeviceState {
+    RingDeviceHeader hd;
+    uint32_t live[kMaxDeviceSlots / 32];  // the slots that hold a batch
+};
+constexpr int kTicketBits = 16;
+struct RingDeviceShared {
+    uint32_t tickets, failed, pad[2];
+    RingDeviceState state[2];
+    const RingDeviceState& current() const { return state[(tickets >> kTicketBits) & 1u]; }
+};
+
 struct RingDeviceView {
-    RingDeviceHeader* hd;
-    int32_t* valid;
-    int32_t* count;
+    RingDeviceShared* shared;
+    int32_t* count;    // per slot: traversals; read and written by one block
     uint64_t* fresh;   // per slot: the extra pointer that came with the batch pushed into it
     int4* events;      // (op, status, slot, k_before); op 1 = push, 2 = sample
     char* storage;
@@ -269,166 +283,223 @@ __device__ __forceinline__ int32_t nth_member(uint32_t word, uint32_t j) {
 // drawn and the inputs of the loss call are resolved into `inputs`.
 //
 // One launch does both.  Every block reads the state for itself (past L1: an earlier launch may have left an older version
-// there) and works out the push's slot and the draw; then it draws a ticket.  The block with the last ticket knows that every
-// block has read the state, so it alone does the bookkeeping and writes the new state -- nothing waits.  The launch is a
-// chain of latencies: its start, the state, the ticket, its end.  So all of the state is asked for at once, what is kept
-// with each slot and the candidates' pointers among it (where they are no more than a block's threads), not only what turns
-// out to be needed; and blocks are few, because their tickets come from one word.  (An iteration of 131 072 steps of 18
-// actions, K = 4, with its loss: 12.1 us; 12.6 with two blocks per SM that asked for the drawn slot's count and pointer and
-// for the candidate's pointers once they knew which.  L2 asked for the drawn slot's fields in here: 12.2.)
+// there) and works out the push's slot; the first block also works out the draw and writes the new state, over the copy that
+// no block of this launch takes anything from, so no block waits for another.  The launch is a chain of latencies: its start,
+// one trip to L2, its end.  So everything that it may need is asked for at once, where there is not too much of it: the
+// candidates' pointers and what is kept with each slot.  (An iteration of 131 072 steps of 18 actions, K = 4, step and loss
+// 12.0 us -> 11.0, of 1 600 steps 7.1 -> 6.2, of 16 384 steps of 9 with a push in each 8.4 -> 7.3; before, every block read all
+// of the state and the one that drew the last ticket wrote it, in blocks of 512 threads that found no room beside a loss
+// launch's.  L2 asked for the drawn slot's fields from here: a grid is complete only when its requests are, 0.3 to 1 us more.)
+//
+// kThreads = 32: a warp per block and 16 KB of shared memory, so that the blocks become resident beside those of the loss
+// launch before, and the loss launch behind beside them: neither's start adds to the chain.  The copy goes through shared
+// memory then, which keeps 16 KB under way with a warp's registers; batches of more than 32 KB to a block go to blocks of 512
+// threads (kStepThreads).  (The next launch is let in behind the wait: before it, 0.1 to 0.4 us more.  The warp's copy through
+// registers or by a loop over the segments: up to 1.2 us more where every step pushes.)
 constexpr int kStepThreads = 512;
-__global__ void __launch_bounds__(kStepThreads) ring_step_kernel(const __grid_constant__ RingDeviceView v, const impact_ring_field_map map,
-                                                                 const void* learner_logits, const float* values,
-                                                                 const float* bootstrap_values, const void* const* sources,
-                                                                 int32_t n_candidates, int32_t do_sample,
-                                                                 impact_loss_inputs* inputs) {
+constexpr int kAheadSlots = 128;       // slots and candidates' pointers that are asked for before it is known which are needed
+constexpr int kStepUnits = 1024;       // 16-byte units of the small form's buffer
+constexpr int kMostSmallUnits = 2048;  // of a block's part of a batch
+
+// A segment's part of the units [u0, u1) of all segments, a segment to every lane, by bulk copies through `buffer` (kStepUnits
+// units).  Returns false if a round's bytes never came.
+__device__ __forceinline__ bool copy_by_warp(const char* src, char* dst, unsigned long long bytes, unsigned long long first,
+                                             unsigned long long u0, unsigned long long u1, uint4* buffer, uint64_t* bar) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long whole_end = first + bytes / 16ull;  // (the last unit may be a part of one)
+    uint32_t parity = 0;
+    for (unsigned long long base = u0; base < u1; base += kStepUnits, parity ^= 1u) {
+        const unsigned long long end = base + kStepUnits < u1 ? base + kStepUnits : u1;
+        const unsigned long long lo = base > first ? base : first, hi = end < whole_end ? end : whole_end;
+        const uint32_t n = lo < hi ? (uint32_t)(hi - lo) * 16u : 0u;
+        uint4* const at = buffer + (lo - base);
+        if (n) dev::bulk_load(at, src + (lo - first) * 16ull, n, bar);
+        const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, n);
+        if (lane == 0) dev::mbarrier_expect_tx(bar, all);
+        bool there = false;
+        for (unsigned int tries = 0; tries < (1u << 22) && !there; ++tries) there = dev::mbarrier_test(bar, parity);
+        if (!__all_sync(0xFFFFFFFFu, there)) return false;
+        if (n) dev::bulk_store(dst + (lo - first) * 16ull, at, n);
+        dev::bulk_store_wait_read();
+        __syncwarp();
+    }
+    if (whole_end >= u0 && whole_end < u1)
+        for (unsigned long long i = bytes & ~15ull; i < bytes; ++i) dst[i] = src[i];
+    return true;
+}
+
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads) ring_step_kernel(const __grid_constant__ RingDeviceView v, const impact_ring_field_map map,
+                                                             const void* learner_logits, const float* values,
+                                                             const float* bootstrap_values, const void* const* sources,
+                                                             int32_t n_candidates, int32_t do_sample,
+                                                             impact_loss_inputs* inputs) {
+    constexpr bool kSmall = kThreads == 32;
+    __shared__ __align__(8) uint64_t bar_s;
+    if (kSmall && threadIdx.x == 0) {
+        dev::mbarrier_init_nofence(&bar_s, 1);
+        dev::fence_mbarrier_init();
+    }
     grid_dependency_wait();
-    __shared__ uint32_t live_s[kMaxDeviceSlots / 32];
-    __shared__ int32_t count_s[kMaxDeviceSlots];
-    __shared__ unsigned long long fresh_s[kMaxDeviceSlots];
+    __shared__ int32_t count_s[kAheadSlots];
+    __shared__ unsigned long long fresh_s[kAheadSlots];
+    __shared__ unsigned long long cand_s[kAheadSlots];
     __shared__ CopySegments plan_s;
-    __shared__ const void* cand_s[kStepThreads];
-    __shared__ int32_t last_s;
+    __shared__ __align__(16) uint4 buffer_s[kSmall ? kStepUnits : 1];
     const int tid = threadIdx.x, lane = tid & 31;
-    const int width = v.n_fields + 1;  // pointers of a candidate
-    const bool all_candidates = sources && (long long)n_candidates * width <= kStepThreads;
-    // (the header by every thread of the first warp: one request)
-    RingDeviceHeader hd;
+    const char* src = nullptr;  // of the lane's segment
+    char* dst = nullptr;
+    unsigned long long bytes = 0, seg_end = 0, units = 0;
     if (tid < 32) {
-        const uint4* const q = reinterpret_cast<const uint4*>(v.hd);
-        const uint4 h0 = __ldcg(q), h1 = __ldcg(q + 1);
-        hd.write_cursor = (int32_t)h0.x; hd.read_cursor = (int32_t)h0.y; hd.n_events = h0.z; hd.tickets = 0;
-        hd.draws = ((uint64_t)h1.y << 32) | h1.x; hd.pushes = ((uint64_t)h1.w << 32) | h1.z;
-    }
-    const void* cand = nullptr;
-    if (all_candidates && tid < n_candidates * width)
-        cand = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(sources) + tid));
-    for (int32_t base = 0; base < kMaxDeviceSlots; base += kStepThreads) {
-        const int32_t s = base + tid;
-        if (base >= v.N) {
-            if (lane == 0) live_s[s >> 5] = 0u;
-            continue;
+        const int width = v.n_fields + 1;  // pointers of a candidate
+        const bool all_candidates = sources && (long long)n_candidates * width <= kAheadSlots, all_slots = v.N <= kAheadSlots;
+        const bool writes = blockIdx.x == 0;
+        unsigned int ticket = 0;
+        if (lane == 0)
+            asm volatile("atom.add.relaxed.gpu.global.u32 %0, [%1], %2;" : "=r"(ticket)
+                         : "l"(&v.shared->tickets), "r"(writes ? (1u << kTicketBits) - (gridDim.x - 1u) : 1u) : "memory");
+        // (both copies; the headers by every thread: one request)
+        const uint4 *const q0 = reinterpret_cast<const uint4*>(&v.shared->state[0].hd), *const q1 = reinterpret_cast<const uint4*>(&v.shared->state[1].hd);
+        const uint4 a0 = __ldcg(q0), b0 = __ldcg(q0 + 1), a1 = __ldcg(q1), b1 = __ldcg(q1 + 1);
+        const uint32_t live0 = __ldcg(v.shared->state[0].live + lane), live1 = __ldcg(v.shared->state[1].live + lane);
+        unsigned long long cand[kAheadSlots / 32], fresh[kAheadSlots / 32];
+        int32_t count[kAheadSlots / 32];
+#pragma unroll
+        for (int i = 0; i < kAheadSlots / 32; ++i) {
+            const int at = i * 32 + lane;
+            cand[i] = all_candidates && at < n_candidates * width ? __ldcg(reinterpret_cast<const unsigned long long*>(sources) + at) : 0ull;
+            const bool slot_there = writes && all_slots && at < v.N;
+            count[i] = slot_there ? __ldcg(v.count + at) : 0;
+            fresh[i] = slot_there ? __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh) + at) : 0ull;
         }
-        const bool there = s < v.N;
-        const int32_t valid = there ? __ldcg(v.valid + s) : 0;
-        const int32_t count = there ? __ldcg(v.count + s) : 0;
-        const unsigned long long fresh = there ? __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh) + s) : 0ull;
-        const uint32_t word = __ballot_sync(0xFFFFFFFFu, valid != 0);
-        if (lane == 0) live_s[s >> 5] = word;
-        if (there) { count_s[s] = count; fresh_s[s] = fresh; }
-    }
-    if (all_candidates) cand_s[tid] = cand;
-    __syncthreads();
-    uint32_t live = 0;
-    int32_t slot = -1, pick = -1, drawn_count = 0;
-    const void* drawn_fresh = nullptr;
-    int first_cand = 0;  // of the candidate's pointers in cand_s
-    if (tid < 32) {
-        live = live_s[lane];
+#pragma unroll
+        for (int i = 0; i < kAheadSlots / 32; ++i) {
+            cand_s[i * 32 + lane] = cand[i];
+            count_s[i * 32 + lane] = count[i];
+            fresh_s[i * 32 + lane] = fresh[i];
+        }
+        const bool odd = ((__shfl_sync(0xFFFFFFFFu, ticket, 0) >> kTicketBits) & 1u) != 0u;
+        const uint4 h0 = odd ? a1 : a0, h1 = odd ? b1 : b0;
+        RingDeviceHeader hd;
+        hd.write_cursor = (int32_t)h0.x; hd.read_cursor = (int32_t)h0.y; hd.n_events = h0.z; hd.pad = 0;
+        hd.draws = ((uint64_t)h1.y << 32) | h1.x; hd.pushes = ((uint64_t)h1.w << 32) | h1.z;
+        uint32_t live = odd ? live1 : live0;
+        __syncwarp();
         const int32_t left = v.N - 32 * lane;  // slots that exist in this lane's word
         const uint32_t exist = left >= 32 ? 0xFFFFFFFFu : (left > 0 ? (1u << left) - 1u : 0u);
+        int32_t slot = -1;
+        int first_cand = 0;  // of the candidate's pointers in cand_s
         if (sources) slot = first_at_or_after(~live & exist, hd.write_cursor);
         if (slot >= 0) {
             const uint64_t c = hd.pushes % (uint64_t)n_candidates;
             if (all_candidates) first_cand = (int)c * width;
-            else if (lane < width) cand_s[lane] = reinterpret_cast<const void*>(__ldcg(reinterpret_cast<const unsigned long long*>(sources) + c * (uint64_t)width + lane));
+            else if (lane < width) cand_s[lane] = __ldcg(reinterpret_cast<const unsigned long long*>(sources) + c * (uint64_t)width + lane);
             __syncwarp();
             if (lane == (slot >> 5)) live |= 1u << (slot & 31);
         }
-        // the draw too is worked out by every block, so that it is done by the time the last one is known
-        const uint32_t n_live = (uint32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
-        if (do_sample && n_live > 0)
-            pick = v.mode == IMPACT_SAMPLE_UNIFORM  // floor(u * live / 2^64)
-                       ? nth_member(live, (uint32_t)__umul64hi(splitmix64_at_dev(v.seed, hd.draws), (uint64_t)n_live))
-                       : first_at_or_after(live, hd.read_cursor);
-        if (pick >= 0) {  // (drawn as it is pushed: nothing is kept with it yet)
-            drawn_count = pick == slot ? 0 : count_s[pick];
-            drawn_fresh = pick == slot ? cand_s[first_cand + v.n_fields] : reinterpret_cast<const void*>(fresh_s[pick]);
-        }
-        if (lane == 0) {
-            int n = 0;
-            unsigned long long units = 0;
-            if (slot >= 0) {
-                for (int f = 0; f < v.n_fields; ++f) {
-                    const void* const from = cand_s[first_cand + f];
-                    if (!from) continue;
-                    plan_s.src[n] = static_cast<const char*>(from);
-                    plan_s.dst[n] = v.storage + (unsigned long long)slot * v.slot_stride + v.field_offset[f];
-                    plan_s.bytes[n] = v.field_bytes[f];
-                    units += (v.field_bytes[f] + 15ull) / 16ull;
-                    plan_s.vec_end[n] = units;
-                    ++n;
-                }
-            }
-            plan_s.n = n;
-            // this block has read all of the state (the release orders those reads before the ticket)
-            unsigned int ticket;
-            asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(ticket) : "l"(&v.hd->tickets) : "memory");
-            last_s = ticket == gridDim.x - 1;
-        }
-    }
-    __syncthreads();
-    if (plan_s.n > 0) copy_segments<false>(plan_s);
-    if (!last_s || tid >= 32) return;
-
-    // ---- the bookkeeping, by the first warp of the last block
-    if (sources) {
         if (slot >= 0) {
-            if (lane == 0) {
-                v.fresh[slot] = reinterpret_cast<uint64_t>(cand_s[first_cand + v.n_fields]);
-                v.valid[slot] = 1;
-                v.count[slot] = 0;
+            const bool mine = lane < v.n_fields;
+            src = mine ? reinterpret_cast<const char*>(cand_s[first_cand + lane]) : nullptr;
+            bytes = src ? v.field_bytes[lane] : 0ull;
+            dst = mine ? v.storage + (unsigned long long)slot * v.slot_stride + v.field_offset[lane] : nullptr;
+            seg_end = (bytes + 15ull) / 16ull;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned long long below = __shfl_up_sync(0xFFFFFFFFu, seg_end, off);
+                if (lane >= off) seg_end += below;
             }
-            hd.write_cursor = (slot + 1) % v.N;
-            hd.pushes += 1;
+            units = __shfl_sync(0xFFFFFFFFu, seg_end, 31);
+            if (!kSmall && mine) {
+                plan_s.src[lane] = src;
+                plan_s.dst[lane] = dst;
+                plan_s.bytes[lane] = bytes;
+                plan_s.vec_end[lane] = seg_end;
+            }
         }
-        if (lane == 0) v.events[hd.n_events % kEventLog] = make_int4(1, slot >= 0 ? IMPACT_OK : IMPACT_ERR_FULL, slot, 0);
-        hd.n_events += 1;
-    }
-    if (do_sample) {
-        if (pick >= 0) {
-            if (v.mode == IMPACT_SAMPLE_UNIFORM) hd.draws += 1;
-            else hd.read_cursor = (pick + 1) % v.N;
-        }
-        if (lane == 0) {
-            int32_t k_before = 0;
-            if (pick >= 0) {
-                k_before = drawn_count;
-                const void* const fresh = drawn_fresh;
-                v.count[pick] = k_before + 1;
-                if (k_before + 1 >= v.K) v.valid[pick] = 0;
-                auto field = [&](int32_t f) -> const void* {
-                    return f >= 0 ? v.storage + (unsigned long long)pick * v.slot_stride + v.field_offset[f] : nullptr;
-                };
-                impact_loss_inputs in;
-                in.learner_logits = learner_logits;
-                in.values = values;
-                in.bootstrap_values = bootstrap_values;
-                in.actions = static_cast<const int32_t*>(field(map.actions));
-                in.rewards = static_cast<const float*>(field(map.rewards));
-                in.discounts = static_cast<const float*>(field(map.discounts));
-                in.worker_logp = static_cast<const float*>(field(map.worker_logp));
-                const void* in_slot = field(map.target_logits);
-                if (k_before == 0 && fresh && in_slot) {  // first traversal: the target network's output is appended now
-                    in.target_logits = fresh;
-                    in.target_logits_copy = const_cast<void*>(in_slot);
-                } else {
-                    in.target_logits = in_slot;
-                    in.target_logits_copy = nullptr;
+        if (!kSmall && lane == 0) plan_s.n = units ? v.n_fields : 0;
+        if (writes) {
+            int32_t pick = -1;
+            const uint32_t n_live = (uint32_t)__reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
+            if (do_sample && n_live > 0)
+                pick = v.mode == IMPACT_SAMPLE_UNIFORM  // floor(u * live / 2^64)
+                           ? nth_member(live, (uint32_t)__umul64hi(splitmix64_at_dev(v.seed, hd.draws), (uint64_t)n_live))
+                           : first_at_or_after(live, hd.read_cursor);
+            const unsigned long long pushed_fresh = slot >= 0 ? cand_s[first_cand + v.n_fields] : 0ull;
+            if (sources) {
+                if (slot >= 0) {
+                    if (lane == 0) {
+                        v.fresh[slot] = pushed_fresh;
+                        v.count[slot] = 0;
+                    }
+                    hd.write_cursor = (slot + 1) % v.N;
+                    hd.pushes += 1;
                 }
-                in.status = IMPACT_OK;
-                in.slot = pick;
-                in.k_before = k_before;
-                in.pad = 0;
-                *inputs = in;
-            } else {
-                inputs->status = IMPACT_ERR_EMPTY;  // the pointers of the previous draw stay in place
+                if (lane == 0) v.events[hd.n_events % kEventLog] = make_int4(1, slot >= 0 ? IMPACT_OK : IMPACT_ERR_FULL, slot, 0);
+                hd.n_events += 1;
             }
-            v.events[hd.n_events % kEventLog] = make_int4(2, pick >= 0 ? IMPACT_OK : IMPACT_ERR_EMPTY, pick, k_before);
+            if (do_sample) {
+                int32_t k_before = 0;
+                unsigned long long kept = 0;
+                if (pick >= 0) {
+                    if (pick == slot) {  // (drawn as it is pushed)
+                        kept = pushed_fresh;
+                    } else {
+                        k_before = all_slots ? count_s[pick] : __ldcg(v.count + pick);
+                        kept = all_slots ? fresh_s[pick] : __ldcg(reinterpret_cast<const unsigned long long*>(v.fresh) + pick);
+                    }
+                    if (v.mode == IMPACT_SAMPLE_UNIFORM) hd.draws += 1;
+                    else hd.read_cursor = (pick + 1) % v.N;
+                    if (k_before + 1 >= v.K && lane == (pick >> 5)) live &= ~(1u << (pick & 31));
+                }
+                if (lane == 0) {
+                    if (pick >= 0) {
+                        v.count[pick] = k_before + 1;
+                        const void* const fresh_at = reinterpret_cast<const void*>(kept);
+                        auto field = [&](int32_t f) -> const void* {
+                            return f >= 0 ? v.storage + (unsigned long long)pick * v.slot_stride + v.field_offset[f] : nullptr;
+                        };
+                        impact_loss_inputs in;
+                        in.learner_logits = learner_logits;
+                        in.values = values;
+                        in.bootstrap_values = bootstrap_values;
+                        in.actions = static_cast<const int32_t*>(field(map.actions));
+                        in.rewards = static_cast<const float*>(field(map.rewards));
+                        in.discounts = static_cast<const float*>(field(map.discounts));
+                        in.worker_logp = static_cast<const float*>(field(map.worker_logp));
+                        const void* in_slot = field(map.target_logits);
+                        if (k_before == 0 && fresh_at && in_slot) {  // first traversal: the target network's output is appended now
+                            in.target_logits = fresh_at;
+                            in.target_logits_copy = const_cast<void*>(in_slot);
+                        } else {
+                            in.target_logits = in_slot;
+                            in.target_logits_copy = nullptr;
+                        }
+                        in.status = IMPACT_OK;
+                        in.slot = pick;
+                        in.k_before = k_before;
+                        in.pad = 0;
+                        *inputs = in;
+                    } else {
+                        inputs->status = IMPACT_ERR_EMPTY;  // the pointers of the previous draw stay in place
+                    }
+                    v.events[hd.n_events % kEventLog] = make_int4(2, pick >= 0 ? IMPACT_OK : IMPACT_ERR_EMPTY, pick, k_before);
+                }
+                hd.n_events += 1;
+            }
+            RingDeviceState* const next = &v.shared->state[odd ? 0 : 1];
+            next->live[lane] = live;
+            if (lane == 0) next->hd = hd;
         }
-        hd.n_events += 1;
     }
-    if (lane == 0) *v.hd = hd;  // (tickets: back to 0)
+    if constexpr (kSmall) {
+        if (units != 0 &&
+            !copy_by_warp(src, dst, bytes, seg_end - (bytes + 15ull) / 16ull, units * blockIdx.x / gridDim.x,
+                          units * (blockIdx.x + 1ull) / gridDim.x, buffer_s, &bar_s) && lane == 0)
+            atomicExch(&v.shared->failed, 1u);
+    } else {
+        __syncthreads();
+        if (plan_s.n > 0) copy_segments<false>(plan_s);
+    }
 }
 
 int blocks_for(unsigned long long work_items, int per_worker, const DeviceInfo* di, int workers = 256) {
@@ -476,19 +547,18 @@ struct impact_buffer {
     char* storage = nullptr;
     bool owns_storage = false;
     // bookkeeping on the device (impact_buffer_device_begin): one allocation, laid out as
-    // [header | valid N | count N | fresh N | events]
+    // [RingDeviceShared | count N | fresh N | events]
     char* device_state = nullptr;
     bool device_mode = false;
     size_t device_state_bytes() const {
-        return align_up16(sizeof(RingDeviceHeader)) + align_up16(sizeof(int32_t) * (size_t)N) * 2 +
+        return align_up16(sizeof(RingDeviceShared)) + align_up16(sizeof(int32_t) * (size_t)N) +
                align_up16(sizeof(uint64_t) * (size_t)N) + sizeof(int4) * (size_t)kEventLog;
     }
     static size_t align_up16(size_t x) { return (x + 15) / 16 * 16; }
     RingDeviceView view() const {
         RingDeviceView v;
         char* p = device_state;
-        v.hd = reinterpret_cast<RingDeviceHeader*>(p); p += align_up16(sizeof(RingDeviceHeader));
-        v.valid = reinterpret_cast<int32_t*>(p); p += align_up16(sizeof(int32_t) * (size_t)N);
+        v.shared = reinterpret_cast<RingDeviceShared*>(p); p += align_up16(sizeof(RingDeviceShared));
         v.count = reinterpret_cast<int32_t*>(p); p += align_up16(sizeof(int32_t) * (size_t)N);
         v.fresh = reinterpret_cast<uint64_t*>(p); p += align_up16(sizeof(uint64_t) * (size_t)N);
         v.events = reinterpret_cast<int4*>(p);
@@ -712,14 +782,16 @@ extern "C" void* impact_buffer_slot_ptr(impact_buffer* h, int32_t slot, int32_t 
 // Brings the host copy of the bookkeeping up to date with the device's (device mode only); synchronises `stream`.
 static int32_t download_state(impact_buffer* h, cudaStream_t cs) {
     const RingDeviceView v = h->view();
-    RingDeviceHeader hd;
-    IMPACT_CUDA_TRY(cudaMemcpyAsync(&hd, v.hd, sizeof(hd), cudaMemcpyDeviceToHost, cs));
-    IMPACT_CUDA_TRY(cudaMemcpyAsync(h->valid.data(), v.valid, sizeof(int32_t) * (size_t)h->N, cudaMemcpyDeviceToHost, cs));
+    RingDeviceShared shared;
+    IMPACT_CUDA_TRY(cudaMemcpyAsync(&shared, v.shared, sizeof(shared), cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaMemcpyAsync(h->count.data(), v.count, sizeof(int32_t) * (size_t)h->N, cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaStreamSynchronize(cs));
-    h->write_cursor = hd.write_cursor;
-    h->read_cursor = hd.read_cursor;
-    h->draws = hd.draws;
+    if (shared.failed) return IMPACT_ERR_CUDA;  // (a copy's bytes never came)
+    const RingDeviceState& now = shared.current();
+    for (int32_t i = 0; i < h->N; ++i) h->valid[i] = (int32_t)((now.live[i >> 5] >> (i & 31)) & 1u);
+    h->write_cursor = now.hd.write_cursor;
+    h->read_cursor = now.hd.read_cursor;
+    h->draws = now.hd.draws;
     return IMPACT_OK;
 }
 
@@ -734,13 +806,14 @@ extern "C" int32_t impact_buffer_device_begin(impact_buffer* h, void* stream) {
     }
     IMPACT_CUDA_TRY(cudaMemsetAsync(h->device_state, 0, h->device_state_bytes(), cs));
     const RingDeviceView v = h->view();
-    RingDeviceHeader hd = {};
-    hd.write_cursor = h->write_cursor;
-    hd.read_cursor = h->read_cursor;
-    hd.draws = h->draws;
+    RingDeviceShared shared = {};
+    RingDeviceState& first = shared.state[0];
+    first.hd.write_cursor = h->write_cursor;
+    first.hd.read_cursor = h->read_cursor;
+    first.hd.draws = h->draws;
+    for (int32_t i = 0; i < h->N; ++i) first.live[i >> 5] |= (h->valid[i] ? 1u : 0u) << (i & 31);
     // (pageable sources: the copies have read them when the calls return)
-    IMPACT_CUDA_TRY(cudaMemcpyAsync(v.hd, &hd, sizeof(hd), cudaMemcpyHostToDevice, cs));
-    IMPACT_CUDA_TRY(cudaMemcpyAsync(v.valid, h->valid.data(), sizeof(int32_t) * (size_t)h->N, cudaMemcpyHostToDevice, cs));
+    IMPACT_CUDA_TRY(cudaMemcpyAsync(v.shared, &shared, sizeof(shared), cudaMemcpyHostToDevice, cs));
     IMPACT_CUDA_TRY(cudaMemcpyAsync(v.count, h->count.data(), sizeof(int32_t) * (size_t)h->N, cudaMemcpyHostToDevice, cs));
     h->device_mode = true;
     return IMPACT_OK;
@@ -775,16 +848,19 @@ extern "C" int32_t impact_buffer_device_step(impact_buffer* h, const impact_ring
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const RingDeviceView v = h->view();
     int blocks = 1;
+    bool small = true;
     if (push_sources) {
         unsigned long long units = 0;
         for (int f = 0; f < h->n_fields; ++f) units += (h->field_bytes[f] + 15) / 16;
         // (a block per SM: most steps find every slot live and copy nothing, and an empty launch should cost as little as
         // possible)
-        blocks = blocks_for(units, 4, di, kStepThreads);
+        small = units <= (unsigned long long)di->sm_count * kMostSmallUnits;
+        blocks = blocks_for(units, 4, di, small ? 32 : kStepThreads);
         if (blocks > di->sm_count) blocks = di->sm_count;
     }
-    IMPACT_CUDA_TRY(launch_serialized(ring_step_kernel, dim3(blocks), dim3(kStepThreads), 0, cs, v, m, learner_logits, values,
-                                      bootstrap_values, push_sources, n_candidates, inputs_out ? 1 : 0, inputs_out));
+    IMPACT_CUDA_TRY(launch_laid_out(100, small ? ring_step_kernel<32> : ring_step_kernel<kStepThreads>, dim3(blocks),
+                                    dim3(small ? 32 : kStepThreads), 0, cs, v, m, learner_logits, values, bootstrap_values, push_sources,
+                                    n_candidates, inputs_out ? 1 : 0, inputs_out));
     return IMPACT_OK;
 }
 
@@ -793,11 +869,12 @@ extern "C" int32_t impact_buffer_device_events(impact_buffer* h, int32_t* events
     if (!h || !h->device_mode || !events_out || !n_out || max_events < 1) return IMPACT_ERR_INVALID_ARG;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const RingDeviceView v = h->view();
-    RingDeviceHeader hd;
+    RingDeviceShared shared;
     std::vector<int4> log((size_t)kEventLog);
-    IMPACT_CUDA_TRY(cudaMemcpyAsync(&hd, v.hd, sizeof(hd), cudaMemcpyDeviceToHost, cs));
+    IMPACT_CUDA_TRY(cudaMemcpyAsync(&shared, v.shared, sizeof(shared), cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaMemcpyAsync(log.data(), v.events, sizeof(int4) * (size_t)kEventLog, cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaStreamSynchronize(cs));
+    const RingDeviceHeader& hd = shared.current().hd;
     uint32_t have = hd.n_events < (uint32_t)kEventLog ? hd.n_events : (uint32_t)kEventLog;
     if (have > (uint32_t)max_events) have = (uint32_t)max_events;
     for (uint32_t i = 0; i < have; ++i) {  // oldest first

@@ -415,6 +415,32 @@ def test_device_step_with_more_candidates_than_a_block_has_threads(oracle, n_can
     ring.close()
 
 
+@pytest.mark.parametrize("sizes", [(13, 5000, 16), (1, 600003, 40), (2500003, 16008), (4800021, 15), (6000007, 48)])
+def test_device_step_copies_batches_of_every_size(sizes):
+    """A block's part of a pushed batch: less than a unit, within one field, over several, more than the buffer holds, and
+    batches that go to the larger blocks; fields that end inside a unit, and one that the candidate leaves out."""
+    import paper_1912_00167_b200 as ip
+    cands = [[torch.randint(0, 256, (n,), dtype=torch.uint8, device="cuda") for n in sizes] for _ in range(3)]
+    storage = torch.full((ip.ImpactBuffer.storage_bytes(3, sizes),), 0xA5, dtype=torch.uint8, device="cuda")
+    ring = ip.ImpactBuffer(3, 1, list(sizes), storage=storage)
+    table = torch.tensor([[0 if (c, f) == (1, 0) else x.data_ptr() for f, x in enumerate(row)] + [0]
+                          for c, row in enumerate(cands)], dtype=torch.int64, device="cuda")
+    push = ring.prepare_device_step(push_sources=table)
+    ring.device_begin()
+    for _ in range(4):  # (the last one finds every slot live)
+        push()
+    want = torch.full_like(storage, 0xA5)
+    for c, row in enumerate(cands):
+        for f, x in enumerate(row):
+            at = ring.slot_ptr(c, f) - storage.data_ptr()
+            if (c, f) != (1, 0):
+                want[at:at + x.numel()] = x
+    assert [e[1] for e in ring.device_events()] == [0, 0, 0, -5]
+    assert torch.equal(storage, want)  # (the bytes between the fields untouched)
+    ring.device_end()
+    ring.close()
+
+
 @pytest.mark.parametrize("row_bytes", [15, 16, 17, 18, 24, 31, 32, 34, 36, 40, 48, 200, 1802])
 @pytest.mark.parametrize("n,offset", [(1, 0), (7, 0), (5000, 0), (40000, 0), (5000, 8), (5000, 4)])
 def test_gather_rows_around_the_granules(row_bytes, n, offset):
