@@ -185,11 +185,8 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             else if (lane == 4) base = IMPACT_IN(rewards);
             else if (lane == 5) base = IMPACT_IN(discounts);
             else if (lane == 6) base = IMPACT_IN(values);
-            const int n_pf = n_tiles < sh.n_prefetch ? n_tiles : sh.n_prefetch;
-            for (int n = 0; n < n_pf; ++n) {
-                const Tile t = tile_at<kLong>(g, br, n, NT);
-                if (base) dev::prefetch_range_l2(base, t.row0 * pitch, (uint32_t)(t.nrows * pitch), total_rows * pitch);
-            }
+            if (lane >= sh.prefetch_arrays) base = nullptr;
+            ask_for_tiles<kLong, 2>(g, br, base, pitch, n_tiles < sh.n_prefetch ? n_tiles : sh.n_prefetch, NT, total_rows);
         }
         // then the barriers
         if (lane < S) {
@@ -873,7 +870,9 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
         const int32_t st = launch_companion(p, (int)sizeof(LT), kLong, plan.prefetch_tiles, (int)ls.grid, stream);
         if (st != IMPACT_OK) return st;
     } else {
-        sh.n_prefetch = plan.prefetch_tiles;
+        const OwnRequests own = own_requests(plan, nt * row_bytes, p.geo.B * p.geo.T, ls.grid, nt, kLong ? 0 : 16 * 1024, kLong ? 0 : 21);
+        sh.n_prefetch = kLong && kA > 0 && kA <= 18 ? 0 : own.tiles;
+        sh.prefetch_arrays = own.slabs_only ? 2 : 7;
     }
     const int shared_percent = plan.companion ? percent_beside(smem + own_smem, 0, di)
                                : kIndirect    ? percent_beside(smem + own_smem, kRingStepShared, di) : -1;

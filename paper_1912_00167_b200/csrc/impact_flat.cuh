@@ -95,6 +95,27 @@ __device__ __forceinline__ int tiles_of_block(const BatchGeometry& g, const Bloc
     return tiles_of_block(g, b, is_long, blockIdx.x, gridDim.x);
 }
 
+// Asks L2 for the block's first n_tiles tiles, lane a for array a's rows of `pitch` bytes (base NULL: none), tile after tile in
+// the order in which the block wants them, so that the memory system sees the requests in that order too.  The first kSlabs
+// arrays are those of logits; of the others, a few bytes to a step, all the tiles' rows are asked for at once where they are
+// neighbours (flat launches): a request takes the copy engine some 35 ns whatever its size.  (A request to each array of each
+// tile: 2500 x 100 steps of 10 actions 10.8 us instead of 10.2, of 12 10.3 instead of 10.0.)
+template <bool kLong, int kSlabs>
+__device__ __forceinline__ void ask_for_tiles(const BatchGeometry& g, const BlockRange& br, const void* base, long long pitch,
+                                              int n_tiles, int nt, long long total_rows) {
+    const bool at_once = !kLong && (int)(threadIdx.x & 31) >= kSlabs;
+    for (int n = 0; n < n_tiles; ++n) {
+        Tile t = tile_at<kLong>(g, br, n, nt);
+        if (at_once) {
+            if (n > 0) break;
+            const Tile first = tile_at<kLong>(g, br, n_tiles - 1, nt);
+            t.nrows += (int)(t.row0 - first.row0);
+            t.row0 = first.row0;
+        }
+        if (base) dev::prefetch_range_l2(base, t.row0 * pitch, (uint32_t)(t.nrows * pitch), total_rows * pitch);
+    }
+}
+
 // A consumer group's tile: which of its rows are the block's (flat) or exist at all (long) -- [lo, hi), empty for a group
 // that has no tile -- and where its first row sits.
 struct TileRows {

@@ -73,11 +73,8 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
             else if (lane == 6) base = p.rewards;
             else if (lane == 7) base = p.discounts;
             else if (lane == 8) base = p.values;
-            const int n_pf = n_tiles < sh.n_prefetch ? n_tiles : sh.n_prefetch;
-            for (int n = 0; n < n_pf; ++n) {
-                const Tile t = tile_at<kLong>(g, br, n, NT);
-                if (base) dev::prefetch_range_l2(base, t.row0 * width, (uint32_t)(t.nrows * width), total_rows * width);
-            }
+            if (lane >= sh.prefetch_arrays) base = nullptr;
+            ask_for_tiles<kLong, 5>(g, br, base, width, n_tiles < sh.n_prefetch ? n_tiles : sh.n_prefetch, NT, total_rows);
         }
         // then the barriers
         if (lane < S) {
@@ -559,7 +556,11 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
         IMPACT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, di->max_smem_optin - 4096));
         configured_device = di->device;
     }
-    sh.n_prefetch = ws_plan(ls.tiles, ls.grid, (size_t)nt * (5 * p.D * sizeof(float) + 16), sh.in_flight, false).prefetch_tiles;
+    const size_t tile_bytes = (size_t)nt * (5 * p.D * sizeof(float) + 16);
+    const OwnRequests own = own_requests(ws_plan(ls.tiles, ls.grid, tile_bytes, sh.in_flight, false), tile_bytes, p.geo.B * p.geo.T,
+                                         ls.grid, nt, 24 * 1024, 12);
+    sh.n_prefetch = own.tiles;
+    sh.prefetch_arrays = own.slabs_only ? 5 : 9;
     IMPACT_CUDA_TRY(launch_serialized(kernel, dim3((unsigned)ls.grid), dim3(C * 128 + 32), smem, stream, p, sh));
     return IMPACT_OK;
 }

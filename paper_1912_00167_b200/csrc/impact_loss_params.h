@@ -83,7 +83,7 @@ struct GaussParams {
 
 // The rest of a launch's shape.
 struct LaunchForm {
-    int nt, stages, in_flight, lanes, n_prefetch;
+    int nt, stages, in_flight, lanes, n_prefetch, prefetch_arrays;
     int log_lanes, passes, rot_shift, rot_mask;  // how rows are laid on lanes (see impact_categorical.cuh)
 };
 
@@ -130,19 +130,21 @@ void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max
 //   tiles gain without losing as much on inputs in L2 (16 x 4096 of 9 7.3 / 8.3, in L2 7.7 / 7.8; of 12 7.8 / 8.4 and 7.7 / 8.0;
 //   of 18 8.5 / 8.8 but 9.1 / 8.4).  More actions: not at up to four tiles (16 x 4096 in bf16 of 24 actions 10.7 / 10.1, of 20
 //   10.1 / 9.1; at 4.3 tiles 20 x 4096 of 24 in fp32 11.4 / 12.1).
-//   Whole trajectories, four groups: not where each has about a tile, all of which are asked for at once (600 x 128 of 18 with
-//   every switch 7.1 / 6.8; of 9 5.9 / 6.0, in L2 5.9 / 5.7).
+//   Whole trajectories: not where a group has about a tile, all of which are asked for at once (600 x 100 of 12 5.6 / 5.5, in L2
+//   5.6 / 4.8; of 24 in bf16 6.8 / 6.0 and 6.7 / 5.1); nor where tiles are small but for large batches (1024 x 128 of 9 6.7 / 7.0, in
+//   L2 6.8 / 6.0; 2500 x 100 with every switch 10.2 / 11.1, in L2 10.4 / 10.4).
 //   Otherwise by the tiles that a block has in flight, behind whose requests the next launch's companion puts its own: three and
 //   more (fp32 logits of up to 23 actions) up to 25.5 MB (1024 x 128 of 20 7.8 / 8.2, 1180 x 128 10.4 / 9.1), with bf16 gradients
 //   28 MB (8.1 / 8.5); two up to 22 MB (800 x 128 of 24 8.0 / 8.2, 900 x 128 10.9 / 9.0; 700 x 128 of 28 8.0 / 8.1, 800 x 128
 //   10.7 / 8.7).
+constexpr size_t kSmallTile = 12 * 1024 + 512;
 inline bool companion_pays(int A, bool split, int groups, long long rows, size_t row_bytes, int nt, long long tiles,
                            long long grid, int in_flight, size_t grad_bytes) {
     if (A > 32) return false;
     const long long bytes = rows * (long long)row_bytes;
     const bool few_tiles = 2 * rows < 9 * grid * nt;
     if (split) return bytes <= 28000000 && (A > 18 ? tiles > 4 * grid : !few_tiles || nt * row_bytes <= 15 * 1024);
-    if (groups == 4 && few_tiles) return false;
+    if (few_tiles || (nt * row_bytes < kSmallTile && bytes < 20000000)) return false;
     return bytes <= (in_flight < 3 ? 22000000 : grad_bytes == 4 ? 25500000 : 28000000);
 }
 // How many tiles per block are asked for in L2 ahead of time, and by whom.
@@ -151,6 +153,29 @@ struct WsPlan {
     bool companion;      // by a companion kernel enqueued before the loss kernel (else by the loss kernel's first warp)
 };
 WsPlan ws_plan(long long tiles, long long grid, size_t tile_bytes, int in_flight, bool allow_companion);
+
+// What the first warp of a launch without a companion asks L2 for: the tiles that it is about to request, while the dependency
+// resolves.  What is not done by then delays the tiles.  In us: nothing / rows of logits / the per-step arrays too.
+//   Nothing where tiles are small: 2500 x 100 steps of 8 actions 9.2 / 9.4 / 10.1, 5243 x 50 of 18 in bf16 11.0 / 11.3 / 11.8,
+//   Gaussian 8000 x 50 of 4 dimensions 14.3 / 16.0 / 16.4.
+//   Nothing where a block has few tiles (fewer than `few` fifths of one) and they are not large: 300 x 50 of 12 3.7 / 4.0 / 4.4, of
+//   18 4.0 / 4.1 / 4.4; 600 x 50 of 18 5.0 / 4.8 / 5.1, but with inputs in L2 4.0 and 5.3 with all; Gaussian 600 x 50 of 8
+//   dimensions 5.7 / 5.8, in L2 4.7 / 5.5, though 512 x 128 7.4 / 6.8 and 5.5 / 6.3.
+//   Rows of logits up to `all_from` bytes to a tile (categorical 16 KB, Gaussian 24): 2500 x 100 of 10 9.8 / 9.5 / 10.2, of 12
+//   10.5 / 9.8 / 10.0, Gaussian 512 x 128 of 8 dimensions 7.4 / 6.7 / 6.8.
+//   All beyond: 2500 x 100 of 32 in bf16 13.8 / 13.7 / 13.0, of 24 with every switch 17.8 / 19.0 / 16.5, 40 x 1000 of 64 12.1 / 11.2 / 10.3.
+//   Split trajectories, whose tiles are asked for one by one: nothing up to 18 actions (16 x 4096 of 18 9.3 / 9.0 / 8.7, in L2 6.4 and 8.7
+//   with all), all beyond (of 24 12.0 / 10.4, in bf16 12.0 / 9.8).
+struct OwnRequests {
+    int tiles;
+    bool slabs_only;
+};
+inline OwnRequests own_requests(const WsPlan& plan, size_t tile_bytes, long long rows, long long grid, int nt, size_t all_from, int few) {
+    const long long tile_rows = grid * nt;
+    OwnRequests r = {plan.prefetch_tiles, tile_bytes < all_from};
+    if (tile_bytes < kSmallTile || (5 * rows < few * tile_rows && tile_bytes < 30 * 1024)) r.tiles = 0;
+    return r;
+}
 
 // The share of the SM's shared memory that a launch with a companion asks to have laid out as such, in percent, for blocks of
 // `smem` bytes: room for a block of the next launch's companion beside one of its own (a kilobyte of either is the system's).

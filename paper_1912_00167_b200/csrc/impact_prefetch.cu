@@ -35,10 +35,8 @@ __global__ void __launch_bounds__(32) impact_prefetch_kernel(const __grid_consta
 #pragma unroll
     for (int a = 0; a < kArrays; ++a)
         if (lane == a) { base = pf.base[a]; pitch = pf.row_bytes[a]; }
-    for (int n = 0; n < n_tiles; ++n) {
-        const Tile t = pf.is_long ? tile_at<true>(pf.geo, br, n, pf.geo.nt) : tile_at<false>(pf.geo, br, n, pf.geo.nt);
-        if (base) dev::prefetch_range_l2(base, t.row0 * pitch, (uint32_t)(t.nrows * pitch), total_rows * pitch);
-    }
+    if (pf.is_long) ask_for_tiles<true, 2>(pf.geo, br, base, pitch, n_tiles, pf.geo.nt, total_rows);
+    else ask_for_tiles<false, 2>(pf.geo, br, base, pitch, n_tiles, pf.geo.nt, total_rows);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
