@@ -179,21 +179,42 @@ def _not_served(*args) -> None:
     """Every direct loss call is checked in Python."""
 
 
-def _bind_loss_direct(*args):
-    """The first direct loss call: finds the native part that checks such a call's arguments (csrc/marshal.cpp), the
-    one built for this Python and this torch.  Nothing else needs it, and a direct call does without as well."""
-    global _loss_direct
+_marshal = None  # (False: not there)
+
+
+def _address(fn) -> int:
+    return ctypes.cast(fn, _vp).value
+
+
+def _find_marshal():
+    """The native part of the binding (csrc/marshal.cpp), the one built for this Python and this torch; None where it is not
+    there.  Every call does without it, more slowly."""
     from .build import marshal_name
     lib = load_library()
     try:
         marshal = importlib.import_module("." + marshal_name(), __package__)
     except ImportError as e:
-        _loss_direct = _not_served
-        warnings.warn(f"{e}: direct loss calls are checked in Python, which takes some 6 us each; rebuild with "
-                      "`python -m paper_1912_00167_b200.build`", RuntimeWarning, stacklevel=3)
-    else:
-        marshal.bind(ctypes.cast(lib.impact_loss_fwd_bwd_call, _vp).value)
-        _loss_direct = marshal.loss
+        warnings.warn(f"{e}: calls are checked and issued in Python, which takes some 1 to 6 us each; rebuild with "
+                      "`python -m paper_1912_00167_b200.build`", RuntimeWarning, stacklevel=4)
+        return None
+    marshal.bind(_address(lib.impact_loss_fwd_bwd_call))
+    marshal.bind_ring(_address(lib.impact_buffer_push), _address(lib.impact_buffer_sample))
+    return marshal
+
+
+def _native():
+    """The same, looked for once."""
+    global _marshal
+    if _marshal is None:
+        _marshal = _find_marshal() or False
+    return _marshal or None
+
+
+def _bind_loss_direct(*args):
+    """The first direct loss call: finds the native part that checks such a call's arguments."""
+    global _loss_direct
+    marshal = _find_marshal()
+    _loss_direct = marshal.loss if marshal else _not_served
     return _loss_direct(*args)
 
 
@@ -249,6 +270,11 @@ def _stream(stream) -> int:
             return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+def _handle_of(stream):
+    """The same for the native part, which takes the current stream for None."""
+    return None if stream is None else _stream(stream)
 
 
 @dataclass
@@ -311,13 +337,19 @@ class PreparedCall:
     the marshalled pointers point into (the C structs and every tensor of the call), so that the call can be
     re-issued for as long as it exists."""
 
-    def __init__(self, fn, args, what, keep):
+    def __init__(self, fn, args, what, keep, native=None):
+        # native: what the binding's native part issues the call from -- (kind, addresses, floats, integers), see csrc/marshal.cpp
+        marshal = _native() if native else None
+        self._capsule = marshal.prepare(native[0], _address(fn), *native[1:]) if marshal else None
+        self._issue = marshal.issue if marshal else None
         # every argument but the last, the stream, as the ctypes object that it is converted to anyway
         conv = [a if a is None or t not in _SIMPLE or isinstance(a, t) else t(a) for a, t in zip(args, fn.argtypes)]
         self._fn, self._args, self._what, self._keep = fn, tuple(conv[:-1]), what, keep
 
     def __call__(self, stream=None) -> None:
-        st = self._fn(*self._args, _stream(stream))
+        st = None if self._capsule is None else self._issue(self._capsule, stream if stream is None else _stream(stream))
+        if st is None:
+            st = self._fn(*self._args, _stream(stream))
         if st != OK:
             _check(st, self._what)
 
@@ -352,7 +384,7 @@ def prepare_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, re
     return PreparedCall(lib.impact_loss_fwd_bwd_call, [ctypes.byref(call), 0], "impact_loss_fwd_bwd_call",
                         (call, learner_logits, target_logits, worker_logp, actions, rewards, discounts, values,
                          bootstrap_values, loss_terms, dlogits, dvalues, vtarget, advantage, workspace,
-                         target_logits_copy))
+                         target_logits_copy), (0, (ctypes.addressof(call),), (), ()))
 
 
 def new_loss_inputs_record(device="cuda") -> torch.Tensor:
@@ -379,7 +411,8 @@ def prepare_loss_fwd_bwd_from_record(record: torch.Tensor, B: int, T: int, A: in
         _dev(advantage, f32, bt, "advantage", True),
         _dev(workspace, torch.uint8, workspace.shape, "workspace"), workspace.numel(), None, record.data_ptr())
     return PreparedCall(lib.impact_loss_fwd_bwd_call, [ctypes.byref(call), 0], "impact_loss_fwd_bwd_call",
-                        (call, record, loss_terms, dlogits, dvalues, vtarget, advantage, workspace))
+                        (call, record, loss_terms, dlogits, dvalues, vtarget, advantage, workspace),
+                        (0, (ctypes.addressof(call),), (), ()))
 
 
 def _fits(t, dtype, shape) -> bool:
@@ -494,7 +527,9 @@ def prepare_loss_fwd_bwd_gaussian(learner_mean, learner_logstd, target_mean, tar
     return PreparedCall(lib.impact_loss_fwd_bwd_gaussian, args, "impact_loss_fwd_bwd_gaussian",
                         (cs, learner_mean, learner_logstd, target_mean, target_logstd, worker_logp, actions, rewards,
                          discounts, values, bootstrap_values, loss_terms, dmean, dlogstd, dvalues, vtarget, advantage,
-                         workspace))
+                         workspace),
+                        (1, (*args[:10], ctypes.addressof(cs), *args[17:24]), tuple(float(x) for x in args[10:13]),
+                         (B, T, D, workspace.numel())))
 
 
 def impact_loss_fwd_bwd_gaussian(learner_mean, learner_logstd, target_mean, target_logstd, worker_logp, actions,
@@ -550,7 +585,7 @@ class ImpactBuffer:
         st = self._lib.impact_buffer_create(N, K, self.n_fields, self._fb, seed, sample_mode,
                                             storage.data_ptr() if storage is not None else None, ctypes.byref(h))
         _check(st, "impact_buffer_create")
-        self._h = h
+        self._h, self._handle = h, h.value
         self._slot = _i32(-1)
         self._k = _i32(-1)
         self._slot_ref, self._k_ref = ctypes.byref(self._slot), ctypes.byref(self._k)
@@ -587,6 +622,12 @@ class ImpactBuffer:
 
     def push(self, fields, stream=None) -> int | None:
         """impact_buffer_push: returns the slot, or None when the buffer is full."""
+        marshal = _marshal or _native()
+        done = marshal.push(self._handle, fields, self.field_bytes, _handle_of(stream)) if marshal else None
+        if done is not None:
+            if done[0] != OK and _check(done[0], "impact_buffer_push", allow=(ERR_FULL,)) == ERR_FULL:
+                return None
+            return done[1]
         host = [t.is_cuda for t in fields if t is not None]
         if any(host) and not all(host):
             raise ValueError("push sources must be all on the device or all on the host")
@@ -599,6 +640,13 @@ class ImpactBuffer:
 
     def sample(self, gather_dst=None, stream=None):
         """impact_buffer_sample: returns (slot, k_before), or None when the buffer is empty."""
+        if gather_dst is None:
+            marshal = _marshal or _native()
+            done = marshal.sample(self._handle, _handle_of(stream)) if marshal else None
+            if done is not None:
+                if done[0] != OK and _check(done[0], "impact_buffer_sample", allow=(ERR_EMPTY,)) == ERR_EMPTY:
+                    return None
+                return done[1:]
         arr = None
         if gather_dst is not None:
             if not all(t is None or t.is_cuda for t in gather_dst):
@@ -681,7 +729,9 @@ class ImpactBuffer:
         args = [self._h, ctypes.byref(fm) if fm is not None else None, ptr(learner_logits), ptr(values),
                 ptr(bootstrap_values), ptr(push_sources), ncand, ptr(record), 0]
         return PreparedCall(self._lib.impact_buffer_device_step, args, "impact_buffer_device_step",
-                            (fm, learner_logits, values, bootstrap_values, push_sources, record))
+                            (fm, learner_logits, values, bootstrap_values, push_sources, record),
+                            (2, (self._h.value, None if fm is None else ctypes.addressof(fm), ptr(learner_logits), ptr(values),
+                                 ptr(bootstrap_values), ptr(push_sources), ptr(record)), (), (ncand,)))
 
     def device_events(self, max_events: int = 4096, stream=None):
         """The most recent (op, status, slot, k_before) outcomes, oldest first (op 1 = push, 2 = sample)."""
@@ -694,7 +744,7 @@ class ImpactBuffer:
     def close(self) -> None:
         if self._h:
             self._lib.impact_buffer_destroy(self._h)
-            self._h = None
+            self._h = self._handle = None
 
     def __del__(self):
         try:

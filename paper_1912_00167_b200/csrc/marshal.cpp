@@ -1,10 +1,12 @@
-// The Python binding's direct loss call in native code: the tensors of one call checked and their addresses handed to
-// impact_loss_fwd_bwd_call.  In Python the checks alone -- type, device, shape and layout of fourteen tensors, an
-// attribute access each -- take four times as long as the launch itself.
+// The Python binding's calls of every iteration in native code: the direct loss call, prepared calls re-issued, the ring's push
+// and sample.  The tensors of a call are checked and their addresses handed to the library's function.  In Python the checks
+// alone -- type, device, shape and layout of fourteen tensors, an attribute access each -- take four times as long as the
+// launch itself, and a prepared call of 25 arguments as long as the launch.
 //
-// A call is served here only if every argument is exactly as it should be: plain dense CUDA tensors (no subclass, no
-// wrapper of a transform, no lazily negated view), coefficients that are Python floats and ints in range.  Anything else
-// gets None, and the caller goes the way that names the argument at fault.  Nothing is kept from one call for the next.
+// A call is served here only if every argument is exactly as it should be: plain dense tensors (no subclass, no wrapper of a
+// transform, no lazily negated view), coefficients that are Python floats and ints in range.  Anything else gets None, and
+// the caller goes the way that names the argument at fault.  Nothing is kept from one call for the next but what a prepared
+// call was prepared with.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -15,6 +17,7 @@
 
 #include <cmath>
 #include <limits>
+#include <new>
 
 #include "impact.h"
 
@@ -23,20 +26,29 @@ namespace {
 using LossCall = int32_t (*)(const impact_loss_call*, void*);
 LossCall g_loss_call = nullptr;
 
-// A plain dense CUDA tensor of the type and shape, contiguous?  Its tensor, or nullptr.
-const at::Tensor* plain_cuda(PyObject* o) {
+// A plain dense tensor of the device's memory (or the host's), contiguous?  Its tensor, or nullptr.
+const at::Tensor* plain(PyObject* o, bool on_host) {
     if (!THPVariable_CheckExact(o)) return nullptr;
     const at::Tensor& t = THPVariable_Unpack(o);
     const c10::TensorImpl* const impl = t.unsafeGetTensorImpl();
-    static const c10::DispatchKeySet bare = c10::DispatchKeySet(c10::DispatchKey::CUDA) |
-                                            c10::getAutocastRelatedKeySetFromBackend(c10::BackendComponent::CUDABit);
-    static const c10::DispatchKeySet with_autograd = bare | c10::getAutogradRelatedKeySetFromBackend(c10::BackendComponent::CUDABit);
+    struct Keys {
+        c10::DispatchKeySet bare, with_autograd;
+        Keys(c10::DispatchKey key, c10::BackendComponent where)
+            : bare(c10::DispatchKeySet(key) | c10::getAutocastRelatedKeySetFromBackend(where)),
+              with_autograd(bare | c10::getAutogradRelatedKeySetFromBackend(where)) {}
+    };
+    static const Keys of_device(c10::DispatchKey::CUDA, c10::BackendComponent::CUDABit);
+    static const Keys of_host(c10::DispatchKey::CPU, c10::BackendComponent::CPUBit);
+    const c10::DispatchKeySet bare = on_host ? of_host.bare : of_device.bare;
+    const c10::DispatchKeySet with_autograd = on_host ? of_host.with_autograd : of_device.with_autograd;
     const c10::DispatchKeySet keys = impl->key_set();
     if ((keys != with_autograd && keys != bare) || !impl->has_storage() || impl->layout() != c10::kStrided ||
         impl->is_python_dispatch() || !impl->is_contiguous())
         return nullptr;
     return &t;
 }
+
+const at::Tensor* plain_cuda(PyObject* o) { return plain(o, false); }
 
 struct Shape {
     int64_t d[3];
@@ -80,6 +92,17 @@ bool integer(PyObject* coef, PyObject* name, int64_t* out) {
 
 enum { kRhoBar, kCBar, kClipEps, kVfCoef, kEntCoef, kKlCoef, kLam, kRhoTw, kIsSource, kRatioMode, kObjective, kGlobalSteps, kNames };
 PyObject* g_names[kNames];
+
+// A stream's handle, None for the current one.  (Numbers only: what else stands for a stream is the caller's to turn into one.)
+bool stream_of(PyObject* o, void** stream) {
+    if (o == Py_None) {
+        *stream = c10::cuda::getCurrentCUDAStream().stream();
+        return true;
+    }
+    if (!PyLong_CheckExact(o)) return false;
+    *stream = PyLong_AsVoidPtr(o);
+    return *stream || !PyErr_Occurred();
+}
 
 bool fill(PyObject* const* a, impact_loss_call* c, void** stream) {
     const at::Tensor* const learner = plain_cuda(a[0]);
@@ -135,14 +158,7 @@ bool fill(PyObject* const* a, impact_loss_call* c, void** stream) {
     c->coef.objective = (int32_t)objective;
     c->coef.global_steps = global_steps;
     c->coef.dlogits_dtype = gt == f32 ? IMPACT_DTYPE_F32 : IMPACT_DTYPE_BF16;
-    if (a[16] == Py_None) {
-        *stream = c10::cuda::getCurrentCUDAStream().stream();
-    } else {
-        if (!PyLong_CheckExact(a[16])) return false;
-        *stream = PyLong_AsVoidPtr(a[16]);
-        if (!*stream && PyErr_Occurred()) return false;
-    }
-    return true;
+    return stream_of(a[16], stream);
 }
 
 // loss(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values, bootstrap_values, coef, loss_terms,
@@ -182,7 +198,187 @@ PyObject* bind(PyObject*, PyObject* address) {
     Py_RETURN_NONE;
 }
 
+// ---- prepared calls: the function's address and its arguments, kept in a capsule that the binding's object holds beside
+// whatever the addresses point into
+struct Prepared {
+    int32_t (*issue)(const Prepared&, void* stream);
+    void* fn;
+    void* p[18];
+    float f[3];
+    int64_t n[4];
+    size_t bytes;
+};
+constexpr const char* kPrepared = "impact prepared call";
+
+int32_t issue_loss(const Prepared& c, void* stream) {
+    return reinterpret_cast<LossCall>(c.fn)(static_cast<const impact_loss_call*>(c.p[0]), stream);
+}
+int32_t issue_gaussian(const Prepared& c, void* stream) {
+    auto in = [&](int i) { return static_cast<const float*>(c.p[i]); };
+    auto out = [&](int i) { return static_cast<float*>(c.p[i]); };
+    return reinterpret_cast<decltype(&impact_loss_fwd_bwd_gaussian)>(c.fn)(
+        in(0), in(1), in(2), in(3), in(4), in(5), in(6), in(7), in(8), in(9), c.f[0], c.f[1], c.f[2],
+        static_cast<const impact_coefficients*>(c.p[10]), c.n[0], c.n[1], (int32_t)c.n[2], out(11), out(12), out(13), out(14), out(15),
+        out(16), c.p[17], c.bytes, stream);
+}
+int32_t issue_step(const Prepared& c, void* stream) {
+    return reinterpret_cast<decltype(&impact_buffer_device_step)>(c.fn)(
+        static_cast<impact_buffer*>(c.p[0]), static_cast<const impact_ring_field_map*>(c.p[1]), c.p[2], static_cast<const float*>(c.p[3]),
+        static_cast<const float*>(c.p[4]), static_cast<const void* const*>(c.p[5]), (int32_t)c.n[0],
+        static_cast<impact_loss_inputs*>(c.p[6]), stream);
+}
+
+// prepare(kind, address of the function, addresses, floats, integers) -> capsule.  kind: 0 loss call, 1 Gaussian loss, 2 step.
+PyObject* prepare(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    static const struct {
+        int32_t (*issue)(const Prepared&, void*);
+        Py_ssize_t addresses, floats, integers;
+    } kinds[] = {{issue_loss, 1, 0, 0}, {issue_gaussian, 18, 3, 4}, {issue_step, 7, 0, 1}};
+    const long kind = n == 5 ? PyLong_AsLong(a[0]) : -1;
+    if (kind < 0 || kind > 2 || !PyTuple_CheckExact(a[2]) || !PyTuple_CheckExact(a[3]) || !PyTuple_CheckExact(a[4]) ||
+        PyTuple_GET_SIZE(a[2]) != kinds[kind].addresses || PyTuple_GET_SIZE(a[3]) != kinds[kind].floats ||
+        PyTuple_GET_SIZE(a[4]) != kinds[kind].integers) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "prepare: not a call's arguments");
+        return nullptr;
+    }
+    Prepared* const c = new (std::nothrow) Prepared();
+    if (!c) return PyErr_NoMemory();
+    c->issue = kinds[kind].issue;
+    c->fn = PyLong_AsVoidPtr(a[1]);
+    for (Py_ssize_t i = 0; i < kinds[kind].addresses; ++i) {
+        PyObject* const v = PyTuple_GET_ITEM(a[2], i);
+        c->p[i] = v == Py_None ? nullptr : PyLong_AsVoidPtr(v);
+    }
+    for (Py_ssize_t i = 0; i < kinds[kind].floats; ++i) c->f[i] = (float)PyFloat_AsDouble(PyTuple_GET_ITEM(a[3], i));
+    for (Py_ssize_t i = 0; i < kinds[kind].integers; ++i) c->n[i] = PyLong_AsLongLong(PyTuple_GET_ITEM(a[4], i));
+    c->bytes = (size_t)c->n[3];
+    PyObject* const capsule = PyErr_Occurred() || !c->fn ? nullptr : PyCapsule_New(c, kPrepared, [](PyObject* o) {
+        delete static_cast<Prepared*>(PyCapsule_GetPointer(o, kPrepared));
+    });
+    if (!capsule) {
+        delete c;
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "no address");
+    }
+    return capsule;
+}
+
+// issue(capsule, stream) -> status, or None: not a stream's handle
+PyObject* issue(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    const Prepared* const c = n == 2 ? static_cast<Prepared*>(PyCapsule_GetPointer(a[0], kPrepared)) : nullptr;
+    if (!c) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "issue takes a prepared call and a stream");
+        return nullptr;
+    }
+    void* stream = nullptr;
+    bool served = false;
+    try {
+        served = stream_of(a[1], &stream);
+    } catch (...) {
+        served = false;
+    }
+    if (!served) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+    int32_t status;
+    Py_BEGIN_ALLOW_THREADS
+    status = c->issue(*c, stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(status);
+}
+
+// ---- the ring's calls
+decltype(&impact_buffer_push) g_push = nullptr;
+decltype(&impact_buffer_sample) g_sample = nullptr;
+
+// push(buffer, fields, bytes of each field, stream) -> (status, slot), or None: not served here
+PyObject* push(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n != 4 || !g_push) {
+        PyErr_SetString(PyExc_TypeError, "push takes 4 arguments, after bind");
+        return nullptr;
+    }
+    constexpr Py_ssize_t kMost = 16;
+    const void* src[kMost] = {};
+    void *buffer = nullptr, *stream = nullptr;
+    int32_t where = IMPACT_SRC_DEVICE;
+    bool served = false;
+    try {
+        served = [&] {
+            if (!PyLong_CheckExact(a[0]) || !(buffer = PyLong_AsVoidPtr(a[0])) || !PyList_CheckExact(a[2])) return false;
+            const bool list = PyList_CheckExact(a[1]);
+            if (!list && !PyTuple_CheckExact(a[1])) return false;
+            const Py_ssize_t fields = PyList_GET_SIZE(a[2]);
+            if (fields > kMost || (list ? PyList_GET_SIZE(a[1]) : PyTuple_GET_SIZE(a[1])) != fields) return false;
+            bool known = false;
+            for (Py_ssize_t f = 0; f < fields; ++f) {
+                PyObject* const o = list ? PyList_GET_ITEM(a[1], f) : PyTuple_GET_ITEM(a[1], f);
+                if (o == Py_None) continue;
+                const at::Tensor* t = plain(o, known && where == IMPACT_SRC_HOST);
+                if (!t && !known && (t = plain(o, true))) where = IMPACT_SRC_HOST;
+                if (!t) return false;
+                known = true;
+                if ((long long)t->nbytes() != PyLong_AsLongLong(PyList_GET_ITEM(a[2], f))) return false;
+                src[f] = t->data_ptr();
+            }
+            return stream_of(a[3], &stream);
+        }();
+    } catch (...) {
+        served = false;
+    }
+    if (!served || PyErr_Occurred()) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+    int32_t status, slot = -1;
+    Py_BEGIN_ALLOW_THREADS
+    status = g_push(static_cast<impact_buffer*>(buffer), src, where, &slot, stream);
+    Py_END_ALLOW_THREADS
+    return Py_BuildValue("(ii)", (int)status, (int)slot);
+}
+
+// sample(buffer, stream) -> (status, slot, k), or None: not served here
+PyObject* sample(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n != 2 || !g_sample) {
+        PyErr_SetString(PyExc_TypeError, "sample takes 2 arguments, after bind");
+        return nullptr;
+    }
+    void *buffer = nullptr, *stream = nullptr;
+    bool served = false;
+    try {
+        served = PyLong_CheckExact(a[0]) && (buffer = PyLong_AsVoidPtr(a[0])) && stream_of(a[1], &stream);
+    } catch (...) {
+        served = false;
+    }
+    if (!served) {
+        PyErr_Clear();
+        Py_RETURN_NONE;
+    }
+    int32_t status, slot = -1, k = -1;
+    Py_BEGIN_ALLOW_THREADS
+    status = g_sample(static_cast<impact_buffer*>(buffer), &slot, &k, nullptr, stream);
+    Py_END_ALLOW_THREADS
+    return Py_BuildValue("(iii)", (int)status, (int)slot, (int)k);
+}
+
+// bind_ring(addresses of impact_buffer_push and impact_buffer_sample)
+PyObject* bind_ring(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    void *push_at = nullptr, *sample_at = nullptr;
+    if (n != 2 || !(push_at = PyLong_AsVoidPtr(a[0])) || !(sample_at = PyLong_AsVoidPtr(a[1]))) {
+        if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "no address");
+        return nullptr;
+    }
+    g_push = reinterpret_cast<decltype(g_push)>(push_at);
+    g_sample = reinterpret_cast<decltype(g_sample)>(sample_at);
+    Py_RETURN_NONE;
+}
+
+#define IMPACT_FAST(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&name)), METH_FASTCALL, nullptr}
 PyMethodDef g_methods[] = {
+    IMPACT_FAST(prepare),
+    IMPACT_FAST(issue),
+    IMPACT_FAST(push),
+    IMPACT_FAST(sample),
+    IMPACT_FAST(bind_ring),
     {"loss", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&loss)), METH_FASTCALL, nullptr},
     {"bind", &bind, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr}};

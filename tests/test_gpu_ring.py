@@ -487,3 +487,112 @@ def test_push_from_host_memory_of_every_kind(sizes, memory):
         for i, (g, w) in enumerate(zip(got, want)):
             assert given[i] is None or torch.equal(g.cpu(), w)
     ring.close()
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_the_rings_calls_and_prepared_calls_issued_natively_or_not(monkeypatch, native):
+    """The binding's native part gives what its Python gives: pushes from either side, of every form of field list, draws,
+    prepared calls on every form of stream; and the same calls are refused."""
+    import paper_1912_00167_b200 as ip
+    from paper_1912_00167_b200 import binding
+    marshal = binding._native()
+    assert marshal is not None
+    served = []
+
+    class Watched:
+        prepare = staticmethod(marshal.prepare)
+
+        @staticmethod
+        def issue(*args):
+            served.append(marshal.issue(*args))
+            return served[-1]
+
+        @staticmethod
+        def push(*args):
+            served.append(marshal.push(*args))
+            return served[-1]
+
+        @staticmethod
+        def sample(*args):
+            served.append(marshal.sample(*args))
+            return served[-1]
+
+    monkeypatch.setattr(binding, "_marshal", Watched if native else False)
+
+    def as_expected(by_native=True):
+        assert [x is not None for x in served] == ([by_native] if native else [])
+        served.clear()
+
+    class Tagged(torch.Tensor):
+        pass
+
+    side = torch.cuda.Stream()
+    ring = ip.ImpactBuffer(2, 1, [400, 24], sample_mode=1)
+    a, b = torch.arange(100, dtype=torch.int32), torch.rand(6)
+    forms = [([a.cuda(), b.cuda()], True), ((a.cuda(), b.cuda()), True), ([a, b], True), ([a.pin_memory(), b.pin_memory()], True),
+             ([None, b.cuda()], True), ([a.cuda().as_subclass(Tagged), b.cuda()], False)]
+    for fields, by_native in forms:
+        for stream in (None, side, side.cuda_stream):
+            torch.cuda.synchronize()
+            slot = ring.push(fields, stream=stream)
+            as_expected(by_native)
+            torch.cuda.synchronize()
+            assert slot in (0, 1)
+            if fields[0] is not None:
+                assert torch.equal(ring.slot_view(slot, 0, torch.int32, (100,)).cpu(), a)
+            assert torch.equal(ring.slot_view(slot, 1, torch.float32, (6,)).cpu(), b)
+            assert ring.sample(stream=stream) == (slot, 0)
+            as_expected()
+    assert ring.sample() is None
+    as_expected()
+    assert ring.push([a.cuda(), b.cuda()]) is not None and ring.push([a.cuda(), b.cuda()]) is not None
+    served.clear()
+    assert ring.push([a.cuda(), b.cuda()]) is None
+    as_expected()
+    for wrong in ([a.cuda(), b], [a.cuda()], [a[:50].cuda(), b.cuda()], [torch.arange(200, dtype=torch.int32).cuda()[::2], b.cuda()]):
+        with pytest.raises(ValueError):
+            ring.push(wrong)
+        as_expected(False)
+    ring.close()
+    for call in (lambda: ring.sample(), lambda: ring.push([a.cuda(), b.cuda()])):
+        with pytest.raises(Exception):
+            call()
+    served.clear()
+
+    # prepared calls
+    B, T, A, D = 5, 20, 6, 3
+    cat = {k: torch.from_numpy(v).cuda() for k, v in ii.categorical_batch(B, T, A, seed=3).items()}
+    gau = {k: torch.from_numpy(v).cuda() for k, v in ii.gaussian_batch(B, T, D, seed=3).items()}
+    ws = ip.new_workspace(B, T)
+    results = []
+    for stream in (None, side, side.cuda_stream):
+        out = dict(loss_terms=torch.zeros(8, device="cuda"), dlogits=torch.zeros(B, T, A, device="cuda"),
+                   dvalues=torch.zeros(B, T, device="cuda"))
+        gout = dict(loss_terms=torch.zeros(8, device="cuda"), dmean=torch.zeros(B, T, D, device="cuda"),
+                    dlogstd=torch.zeros(B, T, D, device="cuda"), dvalues=torch.zeros(B, T, device="cuda"),
+                    vtarget=torch.zeros(B, T, device="cuda"))
+        order = ("learner_logits", "target_logits", "worker_logp", "actions", "rewards", "discounts", "values", "bootstrap_values")
+        gorder = ("learner_mean", "learner_logstd", "target_mean", "target_logstd", "worker_logp", "actions", "rewards",
+                  "discounts", "values", "bootstrap_values")
+        calls = [ip.prepare_loss_fwd_bwd(*[cat[n] for n in order], ip.Coefficients(clip_eps=0.3), workspace=ws, **out),
+                 ip.prepare_loss_fwd_bwd_gaussian(*[gau[n] for n in gorder], ip.Coefficients(clip_eps=0.3, kl_coef=1),
+                                                  workspace=ws, **gout)]
+        torch.cuda.synchronize()
+        for call in calls:
+            call(stream)
+            as_expected()
+        torch.cuda.synchronize()
+        results.append({**out, **{"g" + k: v for k, v in gout.items()}})
+        calls[0].on_stream(0)
+        torch.cuda.synchronize()
+    for r in results[1:]:
+        assert all(torch.equal(r[k], results[0][k]) for k in r)
+    direct = {k: torch.zeros_like(v) for k, v in out.items()}
+    ip.impact_loss_fwd_bwd(*[cat[n] for n in order], ip.Coefficients(clip_eps=0.3), workspace=ws, **direct)
+    gdirect = {k: torch.zeros_like(v) for k, v in gout.items()}
+    binding.load_library().impact_loss_fwd_bwd_gaussian(*calls[1]._args, 0)
+    torch.cuda.synchronize()
+    assert all(torch.equal(direct[k], results[0][k]) for k in direct)
+    assert all(torch.equal(gout[k], results[0]["g" + k]) for k in gdirect)
+    with pytest.raises(ip.ImpactError):  # (the library's own refusal comes back)
+        ip.prepare_loss_fwd_bwd(*[cat[n] for n in order], ip.Coefficients(clip_eps=-1.0), workspace=ws, **out)()
