@@ -18,20 +18,21 @@ __host__ __device__ constexpr size_t gauss_stage_bytes(size_t nt, size_t D) {
 
 namespace {
 
-// exp(x).  Compiled dimensions: one instruction and a rounded product in front of it, whose error grows with |x|.  Others:
+// exp(x).  The MuJoCo tasks' dimensions: one instruction and a rounded product in front of it, whose error grows with |x|.  Others:
 // the accurate function, so that a small standard deviation (log-stds of -2 and less, as a trained policy has) costs its
 // inverse nothing: dmean's error against 64 bits at log-stds of -3 to -2 and 5 dimensions is 5.6e-7 with it, 8.1e-7 without.
-template <bool kFixed>
+__host__ __device__ constexpr bool is_mujoco(int D) { return D == 3 || D == 6 || D == 17; }
+template <bool kFast>
 __device__ __forceinline__ float exp_of(float x) {
-    return kFixed ? dev::exp2_fast(x * 1.4426950408889634f) : expf(x);
+    return kFast ? dev::exp2_fast(x * 1.4426950408889634f) : expf(x);
 }
 
-// kD > 0: the dimension, known at compile time (the MuJoCo tasks of Section 4.3).  kV: dimensions per access to shared
-// memory, where they divide the dimension.
+// kD > 0: the dimension, known at compile time, 1 to 15 and 17: a row belongs to one lane, which keeps z and 1 / sigma where no switch
+// is in use.  kV: dimensions per access to shared memory, where they divide the dimension.
 template <int kD, int C, int kV, bool kPlain, bool kLong>
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_constant__ LaunchForm sh) {
-    constexpr bool kFixed = kD > 0;
+    constexpr bool kFixed = kD > 0, kFast = is_mujoco(kD);
     constexpr float kHalfLog2Pi = 0.91893853320467274178f;
     const int D = kFixed ? kD : p.D;
     const int NT = kFixed ? 128 : sh.nt;
@@ -307,7 +308,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
             Vec<float, kV>::ld(mine_at + 4 * pitch + off, ac);
 #pragma unroll
             for (int v = 0; v < kV; ++v) {
-                const float inv_s = exp_of<kFixed>(-ls[v]), inv_st = exp_of<kFixed>(-lt[v]);
+                const float inv_s = exp_of<kFast>(-ls[v]), inv_st = exp_of<kFast>(-lt[v]);
                 const float z1 = (ac[v] - mu[v]) * inv_s;
                 const float z2 = (ac[v] - mt[v]) * inv_st;
                 lth += (double)fmaf(-0.5f * z1, z1, -ls[v]);
@@ -316,7 +317,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                 if constexpr (kKeep) { z_kept[i * kV + v] = z1; inv_kept[i * kV + v] = inv_s; }
                 if (want_kl) {  // KL(target || learner), per dimension
                     const float dm = (mt[v] - mu[v]) * inv_s;
-                    const float sr = exp_of<kFixed>(lt[v] - ls[v]);  // sigma_target / sigma_learner
+                    const float sr = exp_of<kFast>(lt[v] - ls[v]);  // sigma_target / sigma_learner
                     kl += (ls[v] - lt[v]) + 0.5f * fmaf(sr, sr, dm * dm) - 0.5f;
                 }
             }
@@ -459,7 +460,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                         inv_s = inv_kept[i * kV + v];
                         z = z_kept[i * kV + v];
                     } else {
-                        inv_s = exp_of<kFixed>(-ls[v]);
+                        inv_s = exp_of<kFast>(-ls[v]);
                         z = (ac[v] - mu[v]) * inv_s;  // (a - mu) / sigma
                     }
                     // d log pi / d mu = z / sigma ;  d log pi / d logstd = z^2 - 1 ;  d H / d logstd = 1
@@ -468,7 +469,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                     if (want_kl) {
                         // d KL / d mu = (mu - mu_t) / sigma^2 ; d KL / d logstd = 1 - (sigma_t^2 + (mu_t - mu)^2) / sigma^2
                         const float dm = (mu[v] - mt[v]) * inv_s;
-                        const float sr = exp_of<kFixed>(lt[v] - ls[v]);
+                        const float sr = exp_of<kFast>(lt[v] - ls[v]);
                         gm = fmaf(ck, dm, gm);
                         gs = fmaf(ck, 1.0f - fmaf(sr, sr, dm * dm), gs);
                     }
@@ -519,7 +520,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
     if (grp >= n_tiles) hand_over_sums();
     // ---- one group of the grid (block 0's, the one that runs out of tiles first and so is polling long before the
     // last rows appear) collects every block's row as it appears and writes the loss terms
-    // (in fp64, but for the compiled dimensions on trajectories that fit a tile or are split, which add in fp32 as they
+    // (in fp64, but for the MuJoCo tasks' dimensions on trajectories that fit a tile or are split, which add in fp32 as they
     // always did: fp64 costs 0.15 to 0.3 us at the end of a launch)
     if (blockIdx.x == 0 && grp == n_tiles % C) {
         auto collect = [&](auto zero) {
@@ -528,7 +529,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                                                               k.steps_total, gtid, bar_id, &abort_s))
                 if (gtid == 0) atomicExch(p.counter + 1, 1u);
         };
-        if (!kFixed || (!kLong && g.T > 128)) collect(0.0);
+        if (!kFast || (!kLong && g.T > 128)) collect(0.0);
         else collect(0.0f);
     }
     if (lane == 0) dev::bulk_store_wait_read();  // shared memory must outlive the stores' reads
@@ -565,14 +566,14 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
     return IMPACT_OK;
 }
 
-template <int kD, int C, int CP, int kV>
+template <int kD, int C, int CP, int CL, int kV>
 int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
     const bool plain = p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
                        p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
     const bool room = p.tile_aggregates && rl.nt >= kMinTileRows;
     if (splits_trajectories(p.geo, room, rl.nt, di, 0) || !fits_flat(p.geo)) {
         if (!room) return IMPACT_ERR_UNSUPPORTED;
-        return launch_gaussian<kD, C, kV, false, true>(p, rl, di, stream);
+        return launch_gaussian<kD, CL, kV, false, true>(p, rl, di, stream);
     }
     return plain ? launch_gaussian<kD, CP, kV, true, false>(p, rl, di, stream)
                  : launch_gaussian<kD, C, kV, false, false>(p, rl, di, stream);
@@ -589,10 +590,7 @@ int32_t run_gaussian_width(const GaussParams& p, const DeviceInfo* di, cudaStrea
     if (kV == 4 && vecs % (1 << rl.log_lanes) == 0)
         while (2 * (rl.rot_mask + 1) <= b.ways && (vecs >> rl.log_lanes) % (2 * (rl.rot_mask + 1)) == 0)
             rl.rot_mask = 2 * rl.rot_mask + 1;
-    // (five groups where rows are short, tiles small and a tile's time is arithmetic: D = 1 49.5 -> 43.5 us, 5 70 -> 57 on
-    // 100 to 300 MB; at 12 to 14 dimensions they lose up to a third, at 8 they are even)
-    if (p.D <= 8) return run_gaussian_form<0, 4, 5, kV>(p, rl, di, stream);
-    return run_gaussian_form<0, 3, 3, kV>(p, rl, di, stream);
+    return run_gaussian_form<0, 3, 3, 3, kV>(p, rl, di, stream);
 }
 
 }  // namespace
@@ -600,9 +598,19 @@ int32_t run_gaussian_width(const GaussParams& p, const DeviceInfo* di, cudaStrea
 int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
     const RowLayout rl;
     switch (p.D) {
-        case 3: return run_gaussian_form<3, 4, 4, 1>(p, rl, di, stream);
-        case 6: return run_gaussian_form<6, 4, 4, 2>(p, rl, di, stream);
-        case 17: return run_gaussian_form<17, 3, 3, 1>(p, rl, di, stream);
+        // Consumer groups, with every switch, plain, split.  Where rows are short a tile's time is arithmetic: five (five with every
+        // switch up to five dimensions: 512 x 128 of 1 4.4 us, four 4.6; of 7 6.8 / 6.7).  Longer rows take three, whose ring has
+        // stages enough (8000 x 50 of 15 32.3 us, four 41.7), but four with every switch and split (4000 x 50 of 9 14.2, three 15.3;
+        // 16 x 4096 of 9 9.7 / 12.1, of 17 11.2 / 13.2).  The dimension known at run time: 2500 x 50 of 4 7.6 instead of 6.9, of
+        // 9 12.9 / 9.3, of 13 15.1 / 12.1, with every switch 4000 x 50 of 13 25.9 / 18.0.  16 stays there: rows 64 bytes apart
+        // meet on the banks, and lanes that take their vectors in rotated order do not (35.2 us, 36.2 in order).
+#define IMPACT_FIXED(n, full, plain, split) \
+    case n: return run_gaussian_form<n, full, plain, split, n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1>(p, rl, di, stream)
+        IMPACT_FIXED(1, 5, 5, 4); IMPACT_FIXED(2, 5, 5, 4); IMPACT_FIXED(3, 5, 5, 5); IMPACT_FIXED(4, 5, 5, 4);
+        IMPACT_FIXED(5, 5, 5, 4); IMPACT_FIXED(6, 4, 4, 4); IMPACT_FIXED(7, 4, 5, 4); IMPACT_FIXED(8, 4, 5, 4);
+        IMPACT_FIXED(9, 4, 3, 4); IMPACT_FIXED(10, 4, 3, 4); IMPACT_FIXED(11, 4, 3, 4); IMPACT_FIXED(12, 4, 3, 4);
+        IMPACT_FIXED(13, 4, 3, 4); IMPACT_FIXED(14, 4, 3, 4); IMPACT_FIXED(15, 3, 3, 4); IMPACT_FIXED(17, 3, 3, 4);
+#undef IMPACT_FIXED
         default: break;
     }
     if (p.D % 4 == 0) return run_gaussian_width<4>(p, di, stream);
