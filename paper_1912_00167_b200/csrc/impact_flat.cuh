@@ -350,14 +350,14 @@ struct RowLayout {
 //   25.6; 0.43 (20, 64 x 1000) 9.4 / 11.1; 0.47 (7, 69 x 4000) 18.2 / 23.6; 0.70 (18, 104 x 4000) 19.9 / 40.2
 //   rows of several lanes (`wide_row` elements, else 0) in tiles of nt rows, 128 / lanes, each of which takes a group some 0.65
 //   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one 2.4 times its tiles per SM and
-//   3.4 tiles more: (64, 40 x 300) 7.5 / 7.4; (100, 40 x 300) 10.8 / 8.9; (64, 60 x 500) 10.5 / 10.1, in bf16 8.4 / 9.9;
+//   `cost` / 5 tiles more, 3.4 with the categorical kernel: (64, 40 x 300) 7.5 / 7.4; (100, 40 x 300) 10.8 / 8.9; (64, 60 x 500) 10.5 / 10.1, in bf16 8.4 / 9.9;
 //   (180, 60 x 500) 22.4 / 25.0; (180, 20 x 100) 7.5 / 6.4; (400, 10 x 50) 8.1 / 5.7; (400, 60 x 100) 12.4 / 13.4;
 //   (100, 16 x 2000) 49 / 19; (64, 160 x 100) 6.0 / 7.7
 inline long long split_tiles(const BatchGeometry& g, int nt) { return g.B * ((g.T + nt - 1) / nt); }
-inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row) {
+inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row, int cost = 17) {
     if (g.T <= nt || !aggregates) return false;
     const long long rounds = (g.B + di->sm_count - 1) / di->sm_count;
-    if (wide_row) return 5 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > 12 * split_tiles(g, nt) + 17 * di->sm_count;
+    if (wide_row) return 5 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > 12 * split_tiles(g, nt) + cost * di->sm_count;
     return 100 * g.B < 30 * rounds * di->sm_count;
 }
 // Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.

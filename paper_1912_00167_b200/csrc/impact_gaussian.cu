@@ -27,12 +27,14 @@ __device__ __forceinline__ float exp_of(float x) {
     return kFast ? dev::exp2_fast(x * 1.4426950408889634f) : expf(x);
 }
 
-// kD > 0: the dimension, known at compile time, 1 to 15 and 17: a row belongs to one lane, which keeps z and 1 / sigma where no switch
-// is in use.  kV: dimensions per access to shared memory, where they divide the dimension.
+// kD > 0: the dimension, known at compile time, 1 to 15 and 17: a row belongs to one lane.  kD < 0: -kD vectors per lane, of which a
+// lane may lack the last.  Either keeps z and 1 / sigma where no switch is in use.  kV: dimensions per access to shared memory, where
+// they divide the dimension.
 template <int kD, int C, int kV, bool kPlain, bool kLong>
 __global__ void __launch_bounds__(C * 128 + 32, 1)
 impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_constant__ LaunchForm sh) {
     constexpr bool kFixed = kD > 0, kFast = is_mujoco(kD);
+    constexpr int kVecs = kFixed ? kD / kV : -kD;  // a lane's vectors
     constexpr float kHalfLog2Pi = 0.91893853320467274178f;
     const int D = kFixed ? kD : p.D;
     const int NT = kFixed ? 128 : sh.nt;
@@ -177,7 +179,7 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
     const int gtid = gwarp * 32 + lane;
     const int bar_id = grp + 1;
     const int wrow = gwarp * NTW;  // the warp's first row in a tile
-    constexpr bool kKeep = kFixed && kPlain;  // z and 1 / sigma of the row stay in registers for the gradient pass
+    constexpr bool kKeep = kPlain;  // z and 1 / sigma of the row stay in registers for the gradient pass
     const bool want_kl = !kPlain && (k.kl_coef != 0.0f);
 
     // the lane's part in a row, and the row of a tile that it owns (the first lane of each row; a lane that owns none
@@ -188,7 +190,6 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
     const int my_row = wrow + (kFixed ? lane : (lane >> log_l));
     const bool owner = part == 0;
     const int lrow = my_row + (owner ? 0 : 1);
-    const int n_vecs = kFixed ? kD / kV : (D / kV + L - 1) >> log_l;  // vectors of the lane with the most
     const int rot = (kV == 4 && !kFixed) ? ((lane >> log_l) >> sh.rot_shift) & sh.rot_mask : 0;
 
     // The tile (in a flat launch only a block's first tile ends early, only its last one can begin late, and from one of
@@ -291,13 +292,13 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
             const int step = (kV * 4) << log_l;
             return (kV == 4 && !kFixed) ? ((i * step) ^ (rot * step)) : i * step;
         };
-        auto vec_there = [&](int i) { return kFixed || (i << log_l) + part < D / kV; };
+        auto vec_there = [&](int i) { return kFixed || i < kVecs - 1 || (i << log_l) + part < D / kV; };
 
         // ---- row pass (every lane; rows that are not the tile's hold stale bytes and are masked).  Log-probabilities:
         // D-term sums of magnitude tens that end up in exponents, so they are accumulated in fp64.
         double lth = 0.0, ltg = 0.0;
         float ls_sum = 0.0f, kl = 0.0f;
-        float z_kept[kKeep ? kD : 1], inv_kept[kKeep ? kD : 1];
+        float z_kept[kKeep ? kVecs * kV : 1], inv_kept[kKeep ? kVecs * kV : 1];
         auto row_vec = [&](int i) {
             float mu[kV], ls[kV], mt[kV], lt[kV], ac[kV];
             const int off = vec_at(i);
@@ -322,13 +323,13 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                 }
             }
         };
-        if constexpr (kFixed) {
-#pragma unroll
-            for (int i = 0; i < kD / kV; ++i) row_vec(i);
-        } else {
-#pragma unroll 2
-            for (int i = 0; i < n_vecs; ++i)
-                if (vec_there(i)) row_vec(i);
+        // (lanes that share rows, every switch: eight dimensions at a time; all of them at once took 23.8 us instead of 22.5 at 64
+        // dimensions, 26.4 / 23.2 at 30)
+        constexpr int kUnroll = kFixed || kPlain ? 32 : 8 / kV;
+#pragma unroll kUnroll
+        for (int i = 0; i < kVecs; ++i)
+            if (vec_there(i)) row_vec(i);
+        if constexpr (!kFixed) {
             for (int o = 1; o < L; o <<= 1) {
                 lth += __shfl_xor_sync(0xffffffffu, lth, o);
                 ltg += __shfl_xor_sync(0xffffffffu, ltg, o);
@@ -479,14 +480,9 @@ impact_loss_gaussian_kernel(const __grid_constant__ GaussParams p, const __grid_
                 Vec<float, kV>::st(mine_at + off, om);
                 Vec<float, kV>::st(mine_at + pitch + off, os);
             };
-            if constexpr (kFixed) {
-#pragma unroll
-                for (int i = 0; i < kD / kV; ++i) grad_vec(i);
-            } else {
-#pragma unroll 2
-                for (int i = 0; i < n_vecs; ++i)
-                    if (vec_there(i)) grad_vec(i);
-            }
+#pragma unroll kUnroll
+            for (int i = 0; i < kVecs; ++i)
+                if (vec_there(i)) grad_vec(i);
         }
         if (mine) {
             p.dvalues[here.row0 + lrow] = __fmul_rn(k.dvalue_over_adv, adv);  // V - Vhat = -A
@@ -566,17 +562,32 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
     return IMPACT_OK;
 }
 
+// What a split launch of lanes that share rows costs besides its tiles (see splits_trajectories): 48 x 200 steps of 100 dimensions
+// 14.7 us flat, 13.0 split; 32 x 200 of 40 9.0 / 7.5, of 33 7.4 / 8.2; 10 x 80 of 40 5.1 / 5.6, of 100 7.0 / 5.9.
+constexpr int kGaussSplitCost = 13;
+
 template <int kD, int C, int CP, int CL, int kV>
 int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
     const bool plain = p.k.kl_coef == 0.0f && p.k.objective == IMPACT_OBJECTIVE_CLIPPED_SURROGATE &&
                        p.k.is_source == IMPACT_IS_TARGET_OVER_WORKER && p.k.ratio_mode == IMPACT_RATIO_R3 && !p.vtarget && !p.advantage;
-    const bool room = p.tile_aggregates && rl.nt >= kMinTileRows;
-    if (splits_trajectories(p.geo, room, rl.nt, di, 0) || !fits_flat(p.geo)) {
+    // Tiles of few rows keep their maps in the workspace's spare slots, where there is room: 16 x 4096 steps of 40 dimensions take
+    // 30 us, on one block per trajectory 88; of 100 61 / 196.
+    const bool few_rows = rl.nt < kMinTileRows;
+    const bool room = few_rows ? p.spare_slots && 2 * split_tiles(p.geo, rl.nt) <= kSpareSlots : p.tile_aggregates != nullptr;
+    if (splits_trajectories(p.geo, room, rl.nt, di, rl.log_lanes ? p.D : 0, kGaussSplitCost) || !fits_flat(p.geo)) {
         if (!room) return IMPACT_ERR_UNSUPPORTED;
-        return launch_gaussian<kD, CL, kV, false, true>(p, rl, di, stream);
+        GaussParams q = p;
+        if (few_rows) q.tile_aggregates = p.spare_slots;
+        return launch_gaussian<kD, CL, kV, false, true>(q, rl, di, stream);
     }
-    return plain ? launch_gaussian<kD, CP, kV, true, false>(p, rl, di, stream)
-                 : launch_gaussian<kD, C, kV, false, false>(p, rl, di, stream);
+    if (plain) return launch_gaussian<kD, CP, kV, true, false>(p, rl, di, stream);
+    // Lanes that share rows take four groups where these leave the ring two stages more, one where a vector is one dimension
+    // (26 dimensions 23.2 us, three groups 24.2; 45 27.2 / 29.4; 60, five stages, 26.9 / 23.4).
+    if constexpr (kD < 0) {
+        if (stages_that_fit(gauss_stage_bytes(rl.nt, p.D), di->max_smem_optin) >= (kV == 1 ? 5 : 6))
+            return launch_gaussian<kD, C + 1, kV, false, false>(p, rl, di, stream);
+    }
+    return launch_gaussian<kD, C, kV, false, false>(p, rl, di, stream);
 }
 
 template <int kV>
@@ -590,7 +601,23 @@ int32_t run_gaussian_width(const GaussParams& p, const DeviceInfo* di, cudaStrea
     if (kV == 4 && vecs % (1 << rl.log_lanes) == 0)
         while (2 * (rl.rot_mask + 1) <= b.ways && (vecs >> rl.log_lanes) % (2 * (rl.rot_mask + 1)) == 0)
             rl.rot_mask = 2 * rl.rot_mask + 1;
-    return run_gaussian_form<0, 3, 3, 3, kV>(p, rl, di, stream);
+    // A lane's vectors, the same for many dimensions, are compiled in.  Told at run time they took, on the bytes of 8000 x 50 steps of 17,
+    // 50.3 us instead of 38.5 at 19 dimensions, 51.8 / 35.8 at 37, 47.5 / 36.9 at 63, 35.5 / 35.4 at 32; with every switch on half of
+    // that 34.0 / 24.7 at 23, 23.7 / 22.5 at 64; 300 x 50 of 45 11.2 / 8.2; 16 x 4096 of 23 22.4 / 18.4, of 35 27.0 / 21.7.
+    const int of_lane = (vecs + (1 << rl.log_lanes) - 1) >> rl.log_lanes;
+#define IMPACT_VECS(n) case n: return run_gaussian_form<-(n), 3, 3, 4, kV>(p, rl, di, stream)
+    if constexpr (kV == 4) {
+        switch (of_lane) { IMPACT_VECS(3); IMPACT_VECS(4); IMPACT_VECS(5); }
+    } else if constexpr (kV == 2) {
+        switch (of_lane) { IMPACT_VECS(5); IMPACT_VECS(6); IMPACT_VECS(7); IMPACT_VECS(8); IMPACT_VECS(9); }
+    } else {
+        switch (of_lane) {
+            IMPACT_VECS(10); IMPACT_VECS(11); IMPACT_VECS(12); IMPACT_VECS(13); IMPACT_VECS(14); IMPACT_VECS(15);
+            IMPACT_VECS(16); IMPACT_VECS(17); IMPACT_VECS(18);
+        }
+    }
+#undef IMPACT_VECS
+    return IMPACT_ERR_UNSUPPORTED;  // (no dimension up to 256 gets here)
 }
 
 }  // namespace
@@ -602,8 +629,8 @@ int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t st
         // switch up to five dimensions: 512 x 128 of 1 4.4 us, four 4.6; of 7 6.8 / 6.7).  Longer rows take three, whose ring has
         // stages enough (8000 x 50 of 15 32.3 us, four 41.7), but four with every switch and split (4000 x 50 of 9 14.2, three 15.3;
         // 16 x 4096 of 9 9.7 / 12.1, of 17 11.2 / 13.2).  The dimension known at run time: 2500 x 50 of 4 7.6 instead of 6.9, of
-        // 9 12.9 / 9.3, of 13 15.1 / 12.1, with every switch 4000 x 50 of 13 25.9 / 18.0.  16 stays there: rows 64 bytes apart
-        // meet on the banks, and lanes that take their vectors in rotated order do not (35.2 us, 36.2 in order).
+        // 9 12.9 / 9.3, of 13 15.1 / 12.1, with every switch 4000 x 50 of 13 25.9 / 18.0.  16 is not among them: rows 64 bytes
+        // apart meet on the banks, and lanes that take their vectors in rotated order do not (35.2 us, 36.2 in order).
 #define IMPACT_FIXED(n, full, plain, split) \
     case n: return run_gaussian_form<n, full, plain, split, n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1>(p, rl, di, stream)
         IMPACT_FIXED(1, 5, 5, 4); IMPACT_FIXED(2, 5, 5, 4); IMPACT_FIXED(3, 5, 5, 5); IMPACT_FIXED(4, 5, 5, 4);

@@ -323,6 +323,7 @@ extern "C" int32_t impact_loss_fwd_bwd_gaussian(
     p.tile_aggregates = (T > kMinTileRows && workspace_bytes >= impact_loss_workspace_bytes(B, T))
                             ? reinterpret_cast<unsigned long long*>(static_cast<char*>(workspace) + kWorkspaceFixedBytes)
                             : nullptr;
+    p.spare_slots = static_cast<unsigned long long*>(workspace);
     p.D = D;
     p.geo.B = B;
     p.geo.T = T;

@@ -76,6 +76,7 @@ struct GaussParams {
     unsigned int* counter;
     unsigned long long* tagged_rows;
     unsigned long long* tile_aggregates;
+    unsigned long long* spare_slots;
     BatchGeometry geo;
     LossScalars k;
     int D;
