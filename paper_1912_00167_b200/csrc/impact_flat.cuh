@@ -348,6 +348,9 @@ struct RowLayout {
 // share of the device that the flat launch keeps busy:
 //   rows of one lane: 0.21 (A = 18, 31 x 4000) 16.3 / 14.6; 0.30 (18, 45 x 1000) 7.5 / 7.3; 0.40 (18, 59 x 4000) 17.1 /
 //   25.6; 0.43 (20, 64 x 1000) 9.4 / 11.1; 0.47 (7, 69 x 4000) 18.2 / 23.6; 0.70 (18, 104 x 4000) 19.9 / 40.2
+//   A trajectory of up to three tiles is done before the exchange would be: (18, 16 x 200) 3.8 / 4.8, (18, 44 x 256) 3.9 / 5.1,
+//   (18, 16 x 300) 4.5 / 5.1, in bf16 4.4 / 5.0, 17 dimensions 4.9 / 5.7; of four either: (18, 4 x 400) 4.8 / 5.0, with every
+//   switch 5.4 / 5.0; of five (18, 16 x 600) 5.8 / 4.8
 //   rows of several lanes (`wide_row` elements, else 0) in tiles of nt rows, 128 / lanes, each of which takes a group some 0.65
 //   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one 2.4 times its tiles per SM and
 //   `cost` / 5 tiles more, 3.4 with the categorical kernel: (64, 40 x 300) 7.5 / 7.4; (100, 40 x 300) 10.8 / 8.9; (64, 60 x 500) 10.5 / 10.1, in bf16 8.4 / 9.9;
@@ -358,7 +361,7 @@ inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt,
     if (g.T <= nt || !aggregates) return false;
     const long long rounds = (g.B + di->sm_count - 1) / di->sm_count;
     if (wide_row) return 5 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > 12 * split_tiles(g, nt) + cost * di->sm_count;
-    return 100 * g.B < 30 * rounds * di->sm_count;
+    return g.T > 3ll * nt && 100 * g.B < 30 * rounds * di->sm_count;
 }
 // Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.
 inline bool fits_flat(const BatchGeometry& g) { return g.T < (1ll << 32) - 4096; }
