@@ -150,7 +150,8 @@ int64_t impact_get_option(int32_t option);
  * the tiles of a trajectory that is worked on by several thread blocks at once).  A workspace
  * with the fixed part only -- impact_loss_workspace_bytes(1, 1) -- serves every batch too: long
  * trajectories are then swept by one thread block each, which is slower when there are few of
- * them.  Returns 0 for non-positive sizes.
+ * them (but for rows of which a tile has fewer than 64: up to 16384 words of the fixed part link
+ * theirs).  Returns 0 for non-positive sizes.
  */
 size_t impact_loss_workspace_bytes(int64_t B, int64_t T);
 
