@@ -420,14 +420,11 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         // between this tile's scan and its gradients (only where tiles are numbered tile-major; the values are first
         // looked at after the scan)
         const long long gtile = (long long)blockIdx.x + (long long)n * gridDim.x;
-        const long long tile_stride = g.tile_major ? g.B : 1;  // from a tile to the one after it in time (and two slots to each)
-        const bool peeked = kLong && g.tile_major && gwarp == 0 && tl.r > lane;
-        unsigned long long* const values_at = kLong && kWide && p.tile_values ? p.tile_values + gtile : nullptr;
-        dev::EarlyLook early = {0, 0, 0};
-        if (peeked) {
-            if (kWide) early = dev::look_at_tile(p.tile_aggregates + 2 * gtile, values_at, tile_stride, 1 + lane);
-            else dev::load_aggregate(p.tile_aggregates + 2 * gtile, 2 * tile_stride, tl.r - lane, early.a, early.b);
-        }
+        const long long agg_stride = g.tile_major ? 2 * g.B : 2;  // slots between a tile's aggregate and that of the tile after it in time
+        // (rows of several lanes are never split where there are as many trajectories as blocks)
+        const bool peeked = kLong && !kWide && g.tile_major && gwarp == 0 && tl.r > lane;
+        unsigned long long early_a = 0, early_b = 0;
+        if (peeked) dev::load_aggregate(p.tile_aggregates + 2 * gtile, agg_stride, tl.r - lane, early_a, early_b);
         // every thread waits for the stage itself (a bounded wait: on a time-out the flag is set and the
         // thread goes on with whatever the stage holds, so that all barriers below still pair up)
         if (!stage_wait(&full_bar[s], ph, &abort_s)) atomicExch(p.counter + 1, 1u);
@@ -673,10 +670,13 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             float carry = 0.0f;
             if (here.r > 0) {  // uniform over the group
                 if (gwarp == 0) {
-                    const float c = kWide ? dev::value_from_later_tiles(slots, values_at, tile_stride, here.r,
-                                                                        tag(), &abort_s, p.counter + 1, early)
-                                          : dev::compose_later_aggregates(slots, 2 * tile_stride, here.r, tag(), &abort_s,
-                                                                          p.counter + 1, peeked, early.a, early.b);
+                    float c;
+                    if (kWide && p.block_values)
+                        c = dev::value_from_later_tiles(slots, p.block_values + 4 * (here.traj * (g.ntiles / 32)), here.r, ma, mb,
+                                                        tag(), &abort_s, p.counter + 1);
+                    else
+                        c = dev::compose_later_aggregates(slots, agg_stride, here.r, tag(), &abort_s, p.counter + 1, peeked,
+                                                          early_a, early_b);
                     if (lane == 0) carry_s[grp] = c;
                 }
                 asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
@@ -684,7 +684,6 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
             }
             adv = fmaf(ma, carry, mb);
             after = fmaf(la, carry, lb);
-            if (kWide && gtid == 0 && values_at) dev::publish_tagged(values_at, adv, tag());
         }
         if constexpr (!kPlain) {
             const float below = __shfl_down_sync(0xffffffffu, adv, 1);
@@ -843,6 +842,7 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     const size_t stage = cat_stage_bytes(nt, p.A, sizeof(LT), sizeof(GT));
     LaunchShape ls;
     if (!launch_shape(p.geo, nt, kLong, stage, 2 * (size_t)nt * p.A * sizeof(LT), C, di, &ls, kIndirect)) return IMPACT_ERR_UNSUPPORTED;
+    if (kA < 0) p.geo.tile_major = 0;  // (a trajectory's tiles side by side, as value_from_later_tiles looks for them)
     LaunchForm sh = {};
     sh.nt = nt;
     sh.log_lanes = rl.log_lanes;
@@ -983,14 +983,15 @@ int32_t run_wide_form(const CatParams& p, const DeviceInfo* di, cudaStream_t str
         return IMPACT_ERR_UNSUPPORTED;
     }
     const bool fits = fits_flat(p.geo), plain = is_plain(p);
-    // Tiles of few rows keep their maps and values in the workspace's spare slots, as do values alone, where there is room.
+    // Tiles of few rows keep their maps and their blocks' values in the workspace's spare slots, as do blocks' values alone, where
+    // there is room.  (A block of 32 tiles takes four slots.)
     const int nt = wide_tile_rows(p.geo, true, p.A, sizeof(LT), sizeof(GT), di);
     const long long tiles = split_tiles(p.geo, nt);
     const bool room = nt < kMinTileRows ? p.spare_slots && 3 * tiles <= kSpareSlots : p.tile_aggregates != nullptr;
     if (splits_trajectories(p.geo, room, one_pass, di, p.A) || (!fits && room)) {
         CatParams q = p;
         if (nt < kMinTileRows) q.tile_aggregates = p.spare_slots;
-        q.tile_values = nt < kMinTileRows ? p.spare_slots + 2 * tiles : tiles <= kSpareSlots ? p.spare_slots : nullptr;
+        q.block_values = nt < kMinTileRows ? p.spare_slots + 2 * tiles : tiles <= kSpareSlots ? p.spare_slots : nullptr;
         return launch_categorical<LT, GT, -NV, 3, kV, false, true, false, false>(q, laid_out(nt), di, stream);
     }
     if (!fits) return IMPACT_ERR_UNSUPPORTED;

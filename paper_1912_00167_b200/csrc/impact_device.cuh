@@ -228,6 +228,20 @@ __device__ __forceinline__ void load_aggregate(const unsigned long long* mine, l
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(va), "=l"(vb) : "l"(mine - (long long)j * stride) : "memory");
 }
 
+// A chunk's maps, the one that is applied first in lane 0, which gets the whole.
+__device__ __forceinline__ void compose_in_time_order(float& a, float& b) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float a2 = __shfl_down_sync(0xffffffffu, a, off);
+        const float b2 = __shfl_down_sync(0xffffffffu, b, off);
+        if (lane + off < 32) {  // (a, b) <- (a2, b2) o (a, b): the higher lane's map is applied later
+            b = fmaf(a2, b, b2);
+            a = a2 * a;
+        }
+    }
+}
+
 // Run by one warp: `mine` points at this tile's pair of slots; tile j (1 = the nearest later tile ... r = the
 // trajectory's last) has its slots at mine - j * stride.  Reads their aggregates (a lane each, 32 at a time,
 // waiting -- bounded -- until a pair carries this launch's tag), composes them in time order and returns the
@@ -259,83 +273,83 @@ __device__ __forceinline__ float compose_later_aggregates(const unsigned long lo
             a = __uint_as_float((unsigned int)va);
             b = __uint_as_float((unsigned int)vb);
         }
-        // compose over the warp: lane l ends up with map_{l+31} o ... o map_l; lane 0's is the chunk's
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float a2 = __shfl_down_sync(0xffffffffu, a, off);
-            const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-            if (lane + off < 32) {  // (a, b) <- (a2, b2) o (a, b): the higher lane's map is applied later
-                b = fmaf(a2, b, b2);
-                a = a2 * a;
-            }
-        }
+        compose_in_time_order(a, b);
         const float ca = __shfl_sync(0xffffffffu, a, 0), cb = __shfl_sync(0xffffffffu, b, 0);
         x = fmaf(ca, x, cb);
     }
     return x;
 }
 
-// The same for tiles of few rows, of which a trajectory has hundreds: run by one warp, it looks back from the nearest later
-// tile to the first whose value -- the advantage at its first step, published once it is known -- is there, and composes the
-// maps of the tiles before that.  (A look at all later tiles takes a trip to L2 for every 32 of them: 11 of 375 tiles.)
-// `maps` and `values` point at this tile's slots, the tile j places later has its own 2 * j * stride and j * stride before
-// (values NULL: there is no room for them, and every look goes on to the trajectory's last tile).
-struct EarlyLook {  // what lane l found of the tile l + 1 places later ahead of time
-    unsigned long long a, b, value;
-};
-__device__ __forceinline__ EarlyLook look_at_tile(const unsigned long long* maps, const unsigned long long* values,
-                                                  long long stride, int j) {
-    EarlyLook x;
-    load_aggregate(maps, 2 * stride, j, x.a, x.b);
-    x.value = 0;  // (no tag is 0)
-    if (values) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x.value) : "l"(values - (long long)j * stride) : "memory");
-    return x;
-}
-__device__ __forceinline__ float value_from_later_tiles(const unsigned long long* maps, const unsigned long long* values,
-                                                        long long stride, int r, unsigned int tag, int* abort_flag,
-                                                        unsigned int* error_word, const EarlyLook& early) {
+// The same, with the same bits, for tiles of few rows, of which a trajectory has hundreds (a look at all later tiles takes a
+// trip to L2 for every 32 of them: 11 of 375).  Tiles are counted from the trajectory's end, this one is number r; its blocks of
+// 32 are the chunks above.  The last tile of a block leads it: it publishes the block's map, finds what enters the block -- a
+// lane per earlier block, from the nearest whose value is known -- and publishes the value that leaves it.  The other tiles
+// wait for the maps between them and their block's first and for the one value that enters it, so that a trajectory's tiles do
+// not all ask for the same lines.  A block's maps are always composed as the one tree and applied to what leaves the block
+// before, so the bits do not depend on what had been published by when.
+// `blocks`: four slots per whole block of this trajectory -- the block's map, the value that leaves it, none.  (own_a, own_b):
+// this tile's map, in lane 0.
+__device__ __forceinline__ float value_from_later_tiles(const unsigned long long* mine, unsigned long long* blocks, int r,
+                                                        float own_a, float own_b, unsigned int tag, int* abort_flag,
+                                                        unsigned int* error_word) {
     const int lane = threadIdx.x & 31;
-    float fa = 1.0f, fb = 0.0f;  // the maps of the tiles looked at so far: what enters the last of them to what enters this tile
-    EarlyLook x = early;
-    for (int base = 1;; base += 32) {
-        const int j = base + lane;
-        int known = j > r ? 2 : 0;  // 1: the tile's map, 2: its value (beyond the trajectory's last tile it is 0)
-        unsigned int needed = 0, have = 0, valued = 0;
-        for (int tries = 0; tries < (1 << 22); ++tries) {
-            if (known == 0) {
-                if (base > 1 || tries > 0) x = look_at_tile(maps, values, stride, j);
-                if ((unsigned int)(x.value >> 32) == tag) known = 2;
-                else if ((unsigned int)(x.a >> 32) == tag && (unsigned int)(x.b >> 32) == tag) known = 1;
-            }
-            valued = __ballot_sync(0xffffffffu, known == 2);
-            have = __ballot_sync(0xffffffffu, known != 0);
-            needed = valued ^ (valued - 1u);  // lanes up to the first of those (all, where there is none)
-            if ((have & needed) == needed) break;
-            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(abort_flag))) break;
+    const int block = r >> 5, part = r & 31;
+    const bool leads = part == 31;
+    auto tagged = [&](unsigned long long v) { return (unsigned int)(v >> 32) == tag; };  // (no tag is 0)
+    auto number = [](unsigned long long v) { return __uint_as_float((unsigned int)v); };
+    auto gave_up = [&]() {
+        *reinterpret_cast<volatile int*>(abort_flag) = 1;
+        if (lane == 0) atomicExch(error_word, 1u);
+        return 0.0f;
+    };
+    // the block's maps in front of this tile's, and what enters the block
+    const bool map = lane < part, value = lane == 31 && !leads && block > 0;
+    const unsigned long long* const at = map ? mine - 2 * (part - lane) : blocks + 4 * (block - 1) + 2;
+    unsigned long long va = 0, vb = 0;
+    bool there = !map && !value, all = false;
+    for (int tries = 0; tries < (1 << 22); ++tries) {
+        if (!there) {
+            load_aggregate(at, 0, 0, va, vb);
+            there = tagged(va) && (value || tagged(vb));
         }
-        if ((have & needed) != needed) {
-            *reinterpret_cast<volatile int*>(abort_flag) = 1;
-            if (lane == 0) atomicExch(error_word, 1u);
-            return 0.0f;
-        }
-        float a = 1.0f, b = 0.0f;
-        if ((needed >> lane) & 1u) {
-            a = known == 2 ? 0.0f : __uint_as_float((unsigned int)x.a);
-            b = j > r ? 0.0f : __uint_as_float((unsigned int)(known == 2 ? x.value : x.b));
-        }
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float a2 = __shfl_down_sync(0xffffffffu, a, off);
-            const float b2 = __shfl_down_sync(0xffffffffu, b, off);
-            if (lane + off < 32) {  // (a, b) <- (a, b) o (a2, b2): the higher lane's map is applied earlier
-                b = fmaf(a, b2, b);
-                a = a * a2;
-            }
-        }
-        fb = fmaf(fa, __shfl_sync(0xffffffffu, b, 0), fb);
-        fa = fa * __shfl_sync(0xffffffffu, a, 0);
-        if (valued) return fb;
+        all = __all_sync(0xffffffffu, there);
+        if (all || __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(abort_flag))) break;
     }
+    if (!all) return gave_up();
+    float x = block > 0 && !leads ? number(__shfl_sync(0xffffffffu, va, 31)) : 0.0f;
+    float a = map ? number(va) : 1.0f, b = map ? number(vb) : 0.0f;
+    if (leads) {
+        own_a = __shfl_sync(0xffffffffu, own_a, 0);
+        own_b = __shfl_sync(0xffffffffu, own_b, 0);
+        float ba = map ? a : own_a, bb = map ? b : own_b;
+        compose_in_time_order(ba, bb);
+        if (lane == 0) publish_tile_aggregate(blocks + 4 * block, ba, bb, tag);
+        if (block > 0) {
+            unsigned int needed = 0, have = 0, valued = 0;
+            int known = lane >= block ? 2 : 0;  // 1: the map of the block, lane + 1 before this one, 2: the value that leaves it
+            unsigned long long vx = 0, none = 0;
+            for (int tries = 0; tries < (1 << 22); ++tries) {
+                if (known < 2 && lane < block) {
+                    load_aggregate(blocks + 4 * (block - 1 - lane), 0, 0, va, vb);
+                    load_aggregate(blocks + 4 * (block - 1 - lane) + 2, 0, 0, vx, none);
+                    known = tagged(vx) ? 2 : tagged(va) && tagged(vb) ? 1 : 0;
+                }
+                valued = __ballot_sync(0xffffffffu, known == 2);
+                have = __ballot_sync(0xffffffffu, known != 0);
+                needed = valued ^ (valued - 1u);  // lanes up to the first of those
+                if (valued && (have & needed) == needed) break;
+                if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(abort_flag))) break;
+            }
+            if (!valued || (have & needed) != needed) return gave_up();
+            int n = __ffs((int)valued) - 1;
+            x = n < block ? number(__shfl_sync(0xffffffffu, vx, n)) : 0.0f;
+            while (--n >= 0) x = fmaf(number(__shfl_sync(0xffffffffu, va, n)), x, number(__shfl_sync(0xffffffffu, vb, n)));
+        }
+        if (lane == 0) publish_tagged(blocks + 4 * block + 2, fmaf(ba, x, bb), tag);
+    }
+    if (part == 0) return x;
+    compose_in_time_order(a, b);
+    return fmaf(__shfl_sync(0xffffffffu, a, 0), x, __shfl_sync(0xffffffffu, b, 0));
 }
 
 // Scalars of the loss that the kernels need; filled on the host.

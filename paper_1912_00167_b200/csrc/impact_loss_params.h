@@ -47,7 +47,7 @@ struct CatParams {
     unsigned int* counter;
     unsigned long long* tagged_rows;      // rows of (value, launch tag) pairs, see dev::publish_tagged
     unsigned long long* tile_aggregates;  // long launches: two (value, launch tag) pairs per tile (NULL = no room for them)
-    unsigned long long* tile_values;      // long launches of wide rows: a (value, launch tag) pair per tile (NULL = no room)
+    unsigned long long* block_values;     // long launches of wide rows: see dev::value_from_later_tiles (NULL = no room)
     unsigned long long* spare_slots;      // kSpareSlots of the workspace's (NULL = a call without one)
     void* target_copy;  // where the target logits are written as well (NULL = nowhere)
     const impact_loss_inputs* indirect;  // device record that overrides the nine input pointers above (NULL = none)

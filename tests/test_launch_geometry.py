@@ -67,6 +67,13 @@ def test_a_wait_that_gives_up_raises_the_error_word(tmp_path):
 
 
 @pytest.mark.gpu
+def test_what_comes_after_a_tile_has_the_same_bits_wherever_it_is_found(tmp_path):
+    """Values published or not, near or far, or no room for them."""
+    done = subprocess.run([_host_program(tmp_path, "lookback_check")], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout + done.stderr
+
+
+@pytest.mark.gpu
 def test_the_reciprocal_is_as_good_as_a_rounded_one(tmp_path):
     done = subprocess.run([_host_program(tmp_path, "reciprocal_check")], capture_output=True, text=True)
     assert done.returncode == 0, done.stdout + done.stderr
