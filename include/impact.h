@@ -445,6 +445,10 @@ int32_t impact_buffer_import_state(impact_buffer* h, const void* blob, size_t bl
  *         pointers of the previous draw stay in place.
  *     A loss call reads the record through impact_loss_call.inputs_on_device.  All steps and the loss calls that
  *     use their records belong on ONE stream.
+ *     Waits inside a step are bounded.  One that runs out twice leaves the batch whole, but memory that belongs to other
+ *     kernels may have been written to: _device_end, _device_events, impact_buffer_live and _export_state then report
+ *     IMPACT_ERR_CUDA (impact_last_cuda_error: cudaErrorTimeout).  _device_end brings the bookkeeping back and leaves
+ *     device mode all the same.
  *   impact_buffer_device_events  the most recent outcomes, oldest first, as (op, status, slot, k_before) quadruples
  *                                of int32 (op 1 = push, 2 = sample; up to 4096 are kept); synchronises `stream`.
  */

@@ -16,6 +16,7 @@
 #include "impact_device.cuh"
 #include "impact_internal.h"
 #include "impact_pinned.h"
+#include "impact_ring_copy.cuh"
 
 namespace impact {
 namespace {
@@ -223,7 +224,7 @@ struct RingDeviceState {
 };
 constexpr int kTicketBits = 16;
 struct RingDeviceShared {
-    uint32_t tickets, failed, pad[2];
+    uint32_t tickets, failed, pad[2];  // failed: see copy_by_warp
     RingDeviceState state[2];
     const RingDeviceState& current() const { return state[(tickets >> kTicketBits) & 1u]; }
 };
@@ -298,35 +299,7 @@ __device__ __forceinline__ int32_t nth_member(uint32_t word, uint32_t j) {
 // registers or by a loop over the segments: up to 1.2 us more where every step pushes.)
 constexpr int kStepThreads = 512;
 constexpr int kAheadSlots = 128;       // slots and candidates' pointers that are asked for before it is known which are needed
-constexpr int kStepUnits = 1024;       // 16-byte units of the small form's buffer
 constexpr int kMostSmallUnits = 2048;  // of a block's part of a batch
-
-// A segment's part of the units [u0, u1) of all segments, a segment to every lane, by bulk copies through `buffer` (kStepUnits
-// units).  Returns false if a round's bytes never came.
-__device__ __forceinline__ bool copy_by_warp(const char* src, char* dst, unsigned long long bytes, unsigned long long first,
-                                             unsigned long long u0, unsigned long long u1, uint4* buffer, uint64_t* bar) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long whole_end = first + bytes / 16ull;  // (the last unit may be a part of one)
-    uint32_t parity = 0;
-    for (unsigned long long base = u0; base < u1; base += kStepUnits, parity ^= 1u) {
-        const unsigned long long end = base + kStepUnits < u1 ? base + kStepUnits : u1;
-        const unsigned long long lo = base > first ? base : first, hi = end < whole_end ? end : whole_end;
-        const uint32_t n = lo < hi ? (uint32_t)(hi - lo) * 16u : 0u;
-        uint4* const at = buffer + (lo - base);
-        if (n) dev::bulk_load(at, src + (lo - first) * 16ull, n, bar);
-        const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, n);
-        if (lane == 0) dev::mbarrier_expect_tx(bar, all);
-        bool there = false;
-        for (unsigned int tries = 0; tries < (1u << 22) && !there; ++tries) there = dev::mbarrier_test(bar, parity);
-        if (!__all_sync(0xFFFFFFFFu, there)) return false;
-        if (n) dev::bulk_store(dst + (lo - first) * 16ull, at, n);
-        dev::bulk_store_wait_read();
-        __syncwarp();
-    }
-    if (whole_end >= u0 && whole_end < u1)
-        for (unsigned long long i = bytes & ~15ull; i < bytes; ++i) dst[i] = src[i];
-    return true;
-}
 
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads) ring_step_kernel(const __grid_constant__ RingDeviceView v, const impact_ring_field_map map,
@@ -494,7 +467,7 @@ __global__ void __launch_bounds__(kThreads) ring_step_kernel(const __grid_consta
     if constexpr (kSmall) {
         if (units != 0 &&
             !copy_by_warp(src, dst, bytes, seg_end - (bytes + 15ull) / 16ull, units * blockIdx.x / gridDim.x,
-                          units * (blockIdx.x + 1ull) / gridDim.x, buffer_s, &bar_s) && lane == 0)
+                          units * (blockIdx.x + 1ull) / gridDim.x, buffer_s, &bar_s, kCopyTries) && lane == 0)
             atomicExch(&v.shared->failed, 1u);
     } else {
         __syncthreads();
@@ -779,20 +752,26 @@ extern "C" void* impact_buffer_slot_ptr(impact_buffer* h, int32_t slot, int32_t 
     return h->field_ptr(slot, field);
 }
 
-// Brings the host copy of the bookkeeping up to date with the device's (device mode only); synchronises `stream`.
-static int32_t download_state(impact_buffer* h, cudaStream_t cs) {
+// A step's wait has run out, twice: the batch is whole, but copies that it had asked for may have come late.
+static int32_t status_of(const RingDeviceShared& shared) {
+    return shared.failed ? record_cuda_error(cudaErrorTimeout) : IMPACT_OK;
+}
+
+// Brings the host copy of the bookkeeping up to date with the device's (device mode only) whatever status_of says; synchronises
+// `stream`.
+static int32_t download_state(impact_buffer* h, cudaStream_t cs, bool* brought_back) {
     const RingDeviceView v = h->view();
     RingDeviceShared shared;
     IMPACT_CUDA_TRY(cudaMemcpyAsync(&shared, v.shared, sizeof(shared), cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaMemcpyAsync(h->count.data(), v.count, sizeof(int32_t) * (size_t)h->N, cudaMemcpyDeviceToHost, cs));
     IMPACT_CUDA_TRY(cudaStreamSynchronize(cs));
-    if (shared.failed) return IMPACT_ERR_CUDA;  // (a copy's bytes never came)
+    *brought_back = true;
     const RingDeviceState& now = shared.current();
     for (int32_t i = 0; i < h->N; ++i) h->valid[i] = (int32_t)((now.live[i >> 5] >> (i & 31)) & 1u);
     h->write_cursor = now.hd.write_cursor;
     h->read_cursor = now.hd.read_cursor;
     h->draws = now.hd.draws;
-    return IMPACT_OK;
+    return status_of(shared);
 }
 
 extern "C" int32_t impact_buffer_device_begin(impact_buffer* h, void* stream) {
@@ -821,10 +800,10 @@ extern "C" int32_t impact_buffer_device_begin(impact_buffer* h, void* stream) {
 
 extern "C" int32_t impact_buffer_device_end(impact_buffer* h, void* stream) {
     if (!h || !h->device_mode) return IMPACT_ERR_INVALID_ARG;
-    const int32_t st = download_state(h, static_cast<cudaStream_t>(stream));
-    if (st != IMPACT_OK) return st;
-    h->device_mode = false;
-    return IMPACT_OK;
+    bool brought_back = false;
+    const int32_t st = download_state(h, static_cast<cudaStream_t>(stream), &brought_back);
+    if (brought_back) h->device_mode = false;
+    return st;
 }
 
 extern "C" int32_t impact_buffer_device_step(impact_buffer* h, const impact_ring_field_map* map,
@@ -882,13 +861,14 @@ extern "C" int32_t impact_buffer_device_events(impact_buffer* h, int32_t* events
         events_out[4 * i + 0] = e.x; events_out[4 * i + 1] = e.y; events_out[4 * i + 2] = e.z; events_out[4 * i + 3] = e.w;
     }
     *n_out = (int32_t)have;
-    return IMPACT_OK;
+    return status_of(shared);
 }
 
 extern "C" int32_t impact_buffer_live(const impact_buffer* h) {
     if (!h) return IMPACT_ERR_INVALID_ARG;
     if (h->device_mode) {
-        const int32_t st = download_state(const_cast<impact_buffer*>(h), nullptr);
+        bool brought_back = false;
+        const int32_t st = download_state(const_cast<impact_buffer*>(h), nullptr, &brought_back);
         if (st != IMPACT_OK) return st;
     }
     int32_t live = 0;
@@ -904,7 +884,8 @@ extern "C" size_t impact_buffer_state_bytes(const impact_buffer* h) {
 extern "C" int32_t impact_buffer_export_state(const impact_buffer* h, void* blob, size_t blob_bytes) {
     if (!h || !blob || blob_bytes < impact_buffer_state_bytes(h)) return IMPACT_ERR_INVALID_ARG;
     if (h->device_mode) {  // the device holds the truth: fetch it (default stream; synchronises)
-        const int32_t st = download_state(const_cast<impact_buffer*>(h), nullptr);
+        bool brought_back = false;
+        const int32_t st = download_state(const_cast<impact_buffer*>(h), nullptr, &brought_back);
         if (st != IMPACT_OK) return st;
     }
     StateHeader hd;

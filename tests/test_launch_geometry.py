@@ -67,8 +67,15 @@ def test_a_wait_that_gives_up_raises_the_error_word(tmp_path):
 
 
 @pytest.mark.gpu
+def test_a_ring_step_whose_wait_gives_up_leaves_a_whole_batch(tmp_path):
+    """...and a handle that is told so goes on."""
+    done = subprocess.run([_host_program(tmp_path, "ring_check")], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout + done.stderr
+
+
+@pytest.mark.gpu
 def test_what_comes_after_a_tile_has_the_same_bits_wherever_it_is_found(tmp_path):
-    """Values published or not, near or far, or no room for them."""
+    """Values published or not, near or far."""
     done = subprocess.run([_host_program(tmp_path, "lookback_check")], capture_output=True, text=True)
     assert done.returncode == 0, done.stdout + done.stderr
 
