@@ -427,7 +427,9 @@ int32_t impact_buffer_import_state(impact_buffer* h, const void* blob, size_t bl
  *                                first time) and switches the handle to device mode: impact_buffer_push, _sample and
  *                                _import_state are refused until impact_buffer_device_end, which brings the
  *                                bookkeeping back to the host (synchronises `stream`).  impact_buffer_live and
- *                                _export_state keep working (they fetch the device's copy; synchronising).
+ *                                _export_state keep working: they fetch the device's copy by way of the default stream and
+ *                                wait for that, so a step that is under way on another stream may or may not be in it.
+ *                                Wait for the steps' stream first where it matters.
  *   impact_buffer_device_step    one step on `stream`, in this order:
  *     (1) if push_sources != NULL: the next of n_candidates worker batches goes into the first free slot at or after
  *         the write cursor; with every slot live nothing happens (IMPACT_ERR_FULL in the event log).  push_sources is

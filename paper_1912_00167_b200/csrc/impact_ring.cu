@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256) stream_copy_kernel(const uint4* __restric
 // same trace for the same seed.
 struct RingDeviceHeader {
     int32_t write_cursor, read_cursor;
-    uint32_t n_events, pad;
+    uint32_t n_events, steps;  // steps: launches so far
     uint64_t draws, pushes;
 };
 static_assert(sizeof(RingDeviceHeader) == 32, "read as two 16-byte words");
@@ -226,7 +226,9 @@ constexpr int kTicketBits = 16;
 struct RingDeviceShared {
     uint32_t tickets, failed, pad[2];  // failed: see copy_by_warp
     RingDeviceState state[2];
-    const RingDeviceState& current() const { return state[(tickets >> kTicketBits) & 1u]; }
+    // As the last launch that is complete left it, for the host.  (`tickets` goes up at a launch's start, the copy that it
+    // writes is there at its end.)
+    const RingDeviceState& current() const { return state[(int32_t)(state[1].hd.steps - state[0].hd.steps) > 0 ? 1 : 0]; }
 };
 
 struct RingDeviceView {
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(kThreads) ring_step_kernel(const __grid_consta
         const bool odd = ((__shfl_sync(0xFFFFFFFFu, ticket, 0) >> kTicketBits) & 1u) != 0u;
         const uint4 h0 = odd ? a1 : a0, h1 = odd ? b1 : b0;
         RingDeviceHeader hd;
-        hd.write_cursor = (int32_t)h0.x; hd.read_cursor = (int32_t)h0.y; hd.n_events = h0.z; hd.pad = 0;
+        hd.write_cursor = (int32_t)h0.x; hd.read_cursor = (int32_t)h0.y; hd.n_events = h0.z; hd.steps = h0.w + 1u;
         hd.draws = ((uint64_t)h1.y << 32) | h1.x; hd.pushes = ((uint64_t)h1.w << 32) | h1.z;
         uint32_t live = odd ? live1 : live0;
         __syncwarp();

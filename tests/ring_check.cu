@@ -1,4 +1,5 @@
-// The ring's step where its waits run out.  The copy of a batch whose wait is given no look at all: every byte of it is there and
+// What the host takes for the bookkeeping's present state at every moment of a step (no GPU).
+// With an argument, the ring's step where its waits run out.  The copy of a batch whose wait is given no look at all: every byte of it is there and
 // none beside it.  A handle whose step has said that copies may have come late: it is told, gets its bookkeeping back and
 // goes on outside device mode.  Returns the number of checks that fail (255 at most).
 #include "impact_ring.cu"
@@ -102,9 +103,39 @@ static void handle_that_was_told() {
     check(impact_buffer_destroy(h) == IMPACT_OK, "destroy", 0);
 }
 
-int main() {
-    copies();
-    handle_that_was_told();
+// Block 0 draws the ticket that makes up for the others' at any place among them, and writes the other copy at its end.
+static void states() {
+    for (uint32_t blocks : {1u, 2u, 148u})
+        for (uint32_t first : {0u, 65534u, 0xFFFFFFFEu}) {
+            RingDeviceShared s = {};
+            s.tickets = first << kTicketBits;
+            s.state[first & 1].hd.steps = first;
+            s.state[~first & 1].hd.steps = first - 1;  // (a buffer of no steps has 0 in both)
+            if (first == 0) s.state[1].hd.steps = 0;
+            for (uint32_t n = first; n != first + 5; ++n) {
+                const uint32_t odd = (s.tickets >> kTicketBits) & 1u;
+                for (uint32_t place : {0u, blocks / 2, blocks - 1}) {  // block 0's among the tickets
+                    RingDeviceShared at = s;
+                    for (uint32_t i = 0; i < blocks; ++i) {
+                        check(((at.tickets >> kTicketBits) & 1u) == odd, "copy that a block reads", n);
+                        at.tickets += i == place ? (1u << kTicketBits) - (blocks - 1) : 1u;
+                        check(at.current().hd.steps == n, "state in a step", n);
+                    }
+                }
+                s.tickets += 1u << kTicketBits;
+                s.state[odd ^ 1u].hd = s.state[odd].hd;
+                s.state[odd ^ 1u].hd.steps += 1;
+                check(s.current().hd.steps == n + 1, "state behind a step", n);
+            }
+        }
+}
+
+int main(int argc, char**) {
+    states();
+    if (argc > 1) {
+        copies();
+        handle_that_was_told();
+    }
     printf("%d wrong\n", bad);
     return bad > 255 ? 255 : bad;
 }

@@ -52,6 +52,11 @@ def test_bytes_outside_one_range_are_not_read_in_place(tmp_path):
     assert done.returncode == 0, done.stdout
 
 
+def test_the_host_finds_the_state_that_the_last_step_left(tmp_path):
+    done = subprocess.run([_host_program(tmp_path, "ring_check")], capture_output=True, text=True)
+    assert done.returncode == 0, done.stdout
+
+
 @pytest.mark.gpu
 def test_what_counts_as_one_pinned_range(tmp_path):
     """Allocations and registrations, and two registrations with a hole between them (pointers only, nothing is read)."""
@@ -69,7 +74,7 @@ def test_a_wait_that_gives_up_raises_the_error_word(tmp_path):
 @pytest.mark.gpu
 def test_a_ring_step_whose_wait_gives_up_leaves_a_whole_batch(tmp_path):
     """...and a handle that is told so goes on."""
-    done = subprocess.run([_host_program(tmp_path, "ring_check")], capture_output=True, text=True)
+    done = subprocess.run([_host_program(tmp_path, "ring_check"), "steps"], capture_output=True, text=True)
     assert done.returncode == 0, done.stdout + done.stderr
 
 
