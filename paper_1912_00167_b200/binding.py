@@ -360,6 +360,26 @@ class PreparedCall:
             _check(st, self._what)
 
 
+class _PreparedStep(PreparedCall):
+    """A prepared call on a buffer's handle, for as long as the buffer is open (the call keeps it from being collected)."""
+
+    def __init__(self, ring, *args):
+        super().__init__(*args)
+        self._ring = ring
+
+    def _open(self):
+        if not self._ring._h:
+            _check(ERR_INVALID_ARG, self._what)
+
+    def __call__(self, stream=None) -> None:
+        self._open()
+        super().__call__(stream)
+
+    def on_stream(self, cuda_stream: int) -> None:
+        self._open()
+        super().on_stream(cuda_stream)
+
+
 def prepare_loss_fwd_bwd(learner_logits, target_logits, worker_logp, actions, rewards, discounts, values,
                          bootstrap_values, coef: Coefficients, *, loss_terms, dlogits, dvalues,
                          vtarget=None, advantage=None, workspace, target_logits_copy=None) -> PreparedCall:
@@ -728,10 +748,10 @@ class ImpactBuffer:
         ptr = lambda t: None if t is None else t.data_ptr()
         args = [self._h, ctypes.byref(fm) if fm is not None else None, ptr(learner_logits), ptr(values),
                 ptr(bootstrap_values), ptr(push_sources), ncand, ptr(record), 0]
-        return PreparedCall(self._lib.impact_buffer_device_step, args, "impact_buffer_device_step",
-                            (fm, learner_logits, values, bootstrap_values, push_sources, record),
-                            (2, (self._h.value, None if fm is None else ctypes.addressof(fm), ptr(learner_logits), ptr(values),
-                                 ptr(bootstrap_values), ptr(push_sources), ptr(record)), (), (ncand,)))
+        return _PreparedStep(self, self._lib.impact_buffer_device_step, args, "impact_buffer_device_step",
+                             (fm, learner_logits, values, bootstrap_values, push_sources, record),
+                             (2, (self._h.value, None if fm is None else ctypes.addressof(fm), ptr(learner_logits), ptr(values),
+                                  ptr(bootstrap_values), ptr(push_sources), ptr(record)), (), (ncand,)))
 
     def device_events(self, max_events: int = 4096, stream=None):
         """The most recent (op, status, slot, k_before) outcomes, oldest first (op 1 = push, 2 = sample)."""

@@ -213,6 +213,38 @@ def test_a_slot_view_is_the_slots_bytes_and_nothing_else(lib):
         ring.slot_view(0, 0, torch.float32, (5, 7))
 
 
+@pytest.mark.parametrize("native", [True, False])
+def test_a_prepared_step_keeps_its_buffer_and_ends_with_it(lib, monkeypatch, native):
+    """The call holds the handle by its address: the buffer is there for as long as the call is, and a closed one is refused
+    before anything looks at the handle."""
+    import gc
+    import torch
+    import weakref
+    from paper_1912_00167_b200 import binding as b
+    if not native:
+        monkeypatch.setattr(b, "_marshal", False)
+    ring = _cpu_ring(lib, [4 * 35, 24])
+    step = ring.prepare_device_step({"rewards": 0}, record=torch.zeros(128, dtype=torch.uint8))
+    assert (step._capsule is not None) == native
+    ref = weakref.ref(ring)
+    del ring
+    gc.collect()
+    assert ref() is not None and ref()._h
+    for call in (step, step.on_stream):
+        with pytest.raises(b.ImpactError):  # (the library's own: not in device mode)
+            call(0)
+    ref().close()
+
+    def issued(*args):
+        raise AssertionError("a closed buffer's handle")
+
+    step._fn = step._issue = issued
+    for call in (step, step.on_stream):
+        with pytest.raises(b.ImpactError) as e:
+            call(0)
+        assert e.value.status == b.ERR_INVALID_ARG
+
+
 def test_a_slot_view_does_not_depend_on_earlier_ones(lib):
     """A first view, or the buffer itself, made under inference mode leaves later views ordinary tensors that autograd may
     save."""
