@@ -352,15 +352,18 @@ struct RowLayout {
 //   (18, 16 x 300) 4.5 / 5.1, in bf16 4.4 / 5.0, 17 dimensions 4.9 / 5.7; of four either: (18, 4 x 400) 4.8 / 5.0, with every
 //   switch 5.4 / 5.0; of five (18, 16 x 600) 5.8 / 4.8
 //   rows of several lanes (`wide_row` elements, else 0) in tiles of nt rows, 128 / lanes, each of which takes a group some 0.65
-//   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one 2.4 times its tiles per SM and
-//   `cost` / 5 tiles more, 3.4 with the categorical kernel: (64, 40 x 300) 7.5 / 7.4; (100, 40 x 300) 10.8 / 8.9; (64, 60 x 500) 10.5 / 10.1, in bf16 8.4 / 9.9;
-//   (180, 60 x 500) 22.4 / 25.0; (180, 20 x 100) 7.5 / 6.4; (400, 10 x 50) 8.1 / 5.7; (400, 60 x 100) 12.4 / 13.4;
-//   (100, 16 x 2000) 49 / 19; (64, 160 x 100) 6.0 / 7.7
+//   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one twice its tiles per SM
+//   (`slope` tenths) and 2.5 tiles more (`cost`): (64, 16 x 300) 6.6 / 5.6, (64, 32 x 300) 6.9 / 6.2, (64, 50 x 300) 7.5 / 7.8; with every
+//   switch (60, 20 x 300) 9.1 / 6.4, (60, 38 x 500) 12.1 / 9.1; (40, 20 x 200) 5.1 / 5.1, (40, 40 x 200) 5.4 / 5.7; (60, 50 x 500) 10.3 /
+//   8.4, in bf16 8.6 / 7.6; (64, 54 x 1000) 16.0 / 11.2, (64, 58 x 1000) 16.2 / 15.5, inputs in L2 13.6 / 14.4; (64, 62 x 2000) 29.2 /
+//   26.1; (64, 66 x 4000) 54.3 / 48.8; (100, 40 x 100) 6.3 / 6.2; (100, 58 x 1000) 27.2 / 20.8; (180, 50 x 100) 7.3 / 7.6; (400, 40 x 50)
+//   8.0 / 7.9; (64, 160 x 100) 6.0 / 7.7
 inline long long split_tiles(const BatchGeometry& g, int nt) { return g.B * ((g.T + nt - 1) / nt); }
-inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row, int cost = 17) {
+inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row, int slope = 20,
+                                int cost = 25) {
     if (g.T <= nt || !aggregates) return false;
     const long long rounds = (g.B + di->sm_count - 1) / di->sm_count;
-    if (wide_row) return 5 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > 12 * split_tiles(g, nt) + cost * di->sm_count;
+    if (wide_row) return 10 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > slope * split_tiles(g, nt) + cost * di->sm_count;
     return g.T > 3ll * nt && 100 * g.B < 30 * rounds * di->sm_count;
 }
 // Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.

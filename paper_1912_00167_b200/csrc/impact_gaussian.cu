@@ -562,9 +562,9 @@ int32_t launch_gaussian(GaussParams p, const RowLayout& rl, const DeviceInfo* di
     return IMPACT_OK;
 }
 
-// What a split launch of lanes that share rows costs besides its tiles (see splits_trajectories): 48 x 200 steps of 100 dimensions
-// 14.7 us flat, 13.0 split; 32 x 200 of 40 9.0 / 7.5, of 33 7.4 / 8.2; 10 x 80 of 40 5.1 / 5.6, of 100 7.0 / 5.9.
-constexpr int kGaussSplitCost = 13;
+// What a split launch of lanes that share rows costs (see splits_trajectories): 48 x 200 steps of 100 dimensions 14.7 us
+// flat, 13.0 split; 32 x 200 of 40 9.0 / 7.5, of 33 7.4 / 8.2; 10 x 80 of 40 5.1 / 5.6, of 100 7.0 / 5.9.
+constexpr int kGaussSplitSlope = 24, kGaussSplitCost = 26;
 
 template <int kD, int C, int CP, int CL, int kV>
 int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const DeviceInfo* di, cudaStream_t stream) {
@@ -574,7 +574,7 @@ int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const Devic
     // 30 us, on one block per trajectory 88; of 100 61 / 196.
     const bool few_rows = rl.nt < kMinTileRows;
     const bool room = few_rows ? p.spare_slots && 2 * split_tiles(p.geo, rl.nt) <= kSpareSlots : p.tile_aggregates != nullptr;
-    if (splits_trajectories(p.geo, room, rl.nt, di, rl.log_lanes ? p.D : 0, kGaussSplitCost) || !fits_flat(p.geo)) {
+    if (splits_trajectories(p.geo, room, rl.nt, di, rl.log_lanes ? p.D : 0, kGaussSplitSlope, kGaussSplitCost) || !fits_flat(p.geo)) {
         if (!room) return IMPACT_ERR_UNSUPPORTED;
         GaussParams q = p;
         if (few_rows) q.tile_aggregates = p.spare_slots;

@@ -39,6 +39,17 @@ int main() {
                         }
                     }
     }
+    // where either way of working on few trajectories was found the faster one by a twentieth and more
+    const struct { int A; long long B, T; bool split; } found[] = {
+        {60, 20, 300, true}, {60, 32, 300, true}, {64, 28, 300, true}, {60, 38, 500, true}, {60, 50, 500, true}, {64, 54, 1000, true},
+        {36, 50, 1000, true}, {100, 50, 300, true}, {100, 58, 1000, true}, {64, 62, 2000, true}, {64, 66, 4000, true}, {100, 20, 100, true},
+        {40, 50, 300, false}, {40, 40, 200, false}, {64, 40, 200, false}, {100, 50, 100, false}, {64, 160, 100, false}, {180, 58, 100, false}};
+    for (const auto& f : found) {
+        BatchGeometry g = {};
+        g.B = f.B;
+        g.T = f.T;
+        check(splits_trajectories(g, true, 128 >> wide_width(f.A).log_lanes, &di, f.A) == f.split, "split", f.A, f.B * f.T);
+    }
     printf("%d\n", bad);
     return bad > 255 ? 255 : bad;
 }
