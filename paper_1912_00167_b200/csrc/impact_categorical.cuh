@@ -920,7 +920,7 @@ int32_t run_fixed(const CatParams& p, const DeviceInfo* di, cudaStream_t stream)
         }
         return IMPACT_ERR_UNSUPPORTED;
     }
-    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0) || (!fits && p.tile_aggregates)) {
+    if (splits_trajectories(p.geo, p.tile_aggregates, 128, di, 0, 0, 0, plain) || (!fits && p.tile_aggregates)) {
         // Where three groups spill as well (100 bytes a thread and more: 30 and 31 actions with fp32 logits; 32 are read four
         // at a time and lose nothing by it) and nearly every block has four tiles, four groups have one each: 16 x 4096 steps of
         // 30 and 31 actions 12.1 and 12.5 us instead of 13.2 and 14.1, with bf16 gradients 11.9 and 12.9 instead of 13.3 and

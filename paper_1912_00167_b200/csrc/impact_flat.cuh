@@ -350,7 +350,9 @@ struct RowLayout {
 //   25.6; 0.43 (20, 64 x 1000) 9.4 / 11.1; 0.47 (7, 69 x 4000) 18.2 / 23.6; 0.70 (18, 104 x 4000) 19.9 / 40.2
 //   A trajectory of up to three tiles is done before the exchange would be: (18, 16 x 200) 3.8 / 4.8, (18, 44 x 256) 3.9 / 5.1,
 //   (18, 16 x 300) 4.5 / 5.1, in bf16 4.4 / 5.0, 17 dimensions 4.9 / 5.7; of four either: (18, 4 x 400) 4.8 / 5.0, with every
-//   switch 5.4 / 5.0; of five (18, 16 x 600) 5.8 / 4.8
+//   switch 5.4 / 5.0; of five (18, 16 x 600) 5.8 / 4.8.  With every switch (not `plain`) one or two trajectories of three tiles are
+//   split: (18, 1 x 300) 5.0 / 4.7, (18, 2 x 384) 5.0 / 4.8, (32, 1 x 300) 5.6 / 5.4, (6, 1 x 300) 4.2 / 4.2, 17 dimensions 5.7 / 5.3; but
+//   (18, 4 x 300) 4.4 / 4.9, (6, 4 x 384) 3.6 / 4.3
 //   rows of several lanes (`wide_row` elements, else 0) in tiles of nt rows, 128 / lanes, each of which takes a group some 0.65
 //   us whatever the width: a flat launch takes as long as the busiest block's tiles, a split one twice its tiles per SM
 //   (`slope` tenths) and 2.5 tiles more (`cost`): (64, 16 x 300) 6.6 / 5.6, (64, 32 x 300) 6.9 / 6.2, (64, 50 x 300) 7.5 / 7.8; with every
@@ -360,11 +362,11 @@ struct RowLayout {
 //   8.0 / 7.9; (64, 160 x 100) 6.0 / 7.7
 inline long long split_tiles(const BatchGeometry& g, int nt) { return g.B * ((g.T + nt - 1) / nt); }
 inline bool splits_trajectories(const BatchGeometry& g, bool aggregates, int nt, const DeviceInfo* di, int wide_row, int slope = 20,
-                                int cost = 25) {
+                                int cost = 25, bool plain = true) {
     if (g.T <= nt || !aggregates) return false;
     const long long rounds = (g.B + di->sm_count - 1) / di->sm_count;
     if (wide_row) return 10 * ((rounds * g.T + nt - 1) / nt) * di->sm_count > slope * split_tiles(g, nt) + cost * di->sm_count;
-    return g.T > 3ll * nt && 100 * g.B < 30 * rounds * di->sm_count;
+    return g.T > (plain || g.B > 2 ? 3ll : 2ll) * nt && 100 * g.B < 30 * rounds * di->sm_count;
 }
 // Flat launches count a trajectory's steps in 32 bits, but for the form of the fewest actions with every switch compiled in.
 inline bool fits_flat(const BatchGeometry& g) { return g.T < (1ll << 32) - 4096; }

@@ -574,7 +574,7 @@ int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const Devic
     // 30 us, on one block per trajectory 88; of 100 61 / 196.
     const bool few_rows = rl.nt < kMinTileRows;
     const bool room = few_rows ? p.spare_slots && 2 * split_tiles(p.geo, rl.nt) <= kSpareSlots : p.tile_aggregates != nullptr;
-    if (splits_trajectories(p.geo, room, rl.nt, di, rl.log_lanes ? p.D : 0, kGaussSplitSlope, kGaussSplitCost) || !fits_flat(p.geo)) {
+    if (splits_trajectories(p.geo, room, rl.nt, di, rl.log_lanes ? p.D : 0, kGaussSplitSlope, kGaussSplitCost, plain) || !fits_flat(p.geo)) {
         if (!room) return IMPACT_ERR_UNSUPPORTED;
         GaussParams q = p;
         if (few_rows) q.tile_aggregates = p.spare_slots;

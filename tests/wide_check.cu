@@ -50,6 +50,15 @@ int main() {
         g.T = f.T;
         check(splits_trajectories(g, true, 128 >> wide_width(f.A).log_lanes, &di, f.A) == f.split, "split", f.A, f.B * f.T);
     }
+    // (rows of one lane, tiles of 128: trajectories of three tiles stay whole, but for one or two with every switch)
+    for (long long B : {1ll, 2ll, 3ll, 44ll})
+        for (long long T : {200ll, 256ll, 257ll, 384ll, 385ll, 600ll})
+            for (bool plain : {false, true}) {
+                BatchGeometry g = {};
+                g.B = B;
+                g.T = T;
+                check(splits_trajectories(g, true, 128, &di, 0, 0, 0, plain) == (T > (plain || B > 2 ? 384 : 256)), "split of three", (int)B, T);
+            }
     printf("%d\n", bad);
     return bad > 255 ? 255 : bad;
 }
