@@ -420,11 +420,11 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
         // between this tile's scan and its gradients (only where tiles are numbered tile-major; the values are first
         // looked at after the scan)
         const long long gtile = (long long)blockIdx.x + (long long)n * gridDim.x;
-        const long long agg_stride = g.tile_major ? 2 * g.B : 2;  // slots between a tile's aggregate and that of the tile after it in time
+        const long long tile_stride = g.tile_major ? g.B : 1;  // from a tile to the one after it in time (and two slots to each)
         // (rows of several lanes are never split where there are as many trajectories as blocks)
         const bool peeked = kLong && !kWide && g.tile_major && gwarp == 0 && tl.r > lane;
         unsigned long long early_a = 0, early_b = 0;
-        if (peeked) dev::load_aggregate(p.tile_aggregates + 2 * gtile, agg_stride, tl.r - lane, early_a, early_b);
+        if (peeked) dev::load_aggregate(p.tile_aggregates + 2 * gtile, 2 * tile_stride, tl.r - lane, early_a, early_b);
         // every thread waits for the stage itself (a bounded wait: on a time-out the flag is set and the
         // thread goes on with whatever the stage holds, so that all barriers below still pair up)
         if (!stage_wait(&full_bar[s], ph, &abort_s)) atomicExch(p.counter + 1, 1u);
@@ -675,7 +675,7 @@ impact_loss_categorical_kernel(const __grid_constant__ CatParams p, const __grid
                         c = dev::value_from_later_tiles(slots, p.block_values + 4 * (here.traj * (g.ntiles / 32)), here.r, ma, mb,
                                                         tag(), &abort_s, p.counter + 1);
                     else
-                        c = dev::compose_later_aggregates(slots, agg_stride, here.r, tag(), &abort_s, p.counter + 1, peeked,
+                        c = dev::compose_later_aggregates(slots, 2 * tile_stride, here.r, tag(), &abort_s, p.counter + 1, peeked,
                                                           early_a, early_b);
                     if (lane == 0) carry_s[grp] = c;
                 }
