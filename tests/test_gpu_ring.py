@@ -381,11 +381,11 @@ def test_gather_rows_of_every_width(row_bytes, n):
     assert bool((guard[:256] == 0xA5).all()) and bool((guard[256 + n * row_bytes:] == 0xA5).all())
 
 
-@pytest.mark.parametrize("n_cand", [255, 256, 257, 700])
+@pytest.mark.parametrize("n_cand", [63, 64, 65, 255, 256, 257, 700])
 @pytest.mark.parametrize("ahead", [0, 3])
-def test_device_step_with_more_candidates_than_a_block_has_threads(oracle, n_cand, ahead):
-    """Candidates' tables of up to 512 pointers are asked for as a whole, larger ones candidate by candidate: which candidate
-    lands in which slot, and whose kept pointer comes with the draw, as it is pushed (none ahead) and later."""
+def test_device_step_with_small_and_large_tables_of_candidates(oracle, n_cand, ahead):
+    """Candidates' tables of up to 128 pointers, two to a candidate, are asked for as a whole, larger ones candidate by candidate:
+    which candidate lands in which slot, and whose kept pointer comes with the draw, as it is pushed (none ahead) and later."""
     import ctypes
     import paper_1912_00167_b200 as ip
     N, K, n = 5, 1, 13
@@ -412,6 +412,43 @@ def test_device_step_with_more_candidates_than_a_block_has_threads(oracle, n_can
         assert got.target_logits == kept[where[slot]]
         assert torch.equal(ring.slot_view(slot, 0, torch.int32, (n,)), data[where[slot], :n])
     ring.device_end()
+    ring.close()
+
+
+@pytest.mark.parametrize("N", [31, 32, 33, 127, 128, 129, 1000, 1024])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_device_step_on_small_and_large_rings(oracle, N, mode):
+    """What is kept with up to 128 slots is asked for as a whole, with more for the slot that is drawn: draws in rings that fill
+    up, have slots discarded and filled again, each with its count and the pointer that came with its batch."""
+    import ctypes
+    import paper_1912_00167_b200 as ip
+    K, n_cand, size = 2, 7, ctypes.sizeof(ip.binding.impact_loss_inputs)
+    data = torch.zeros(16, dtype=torch.int32, device="cuda")
+    kept = [0x10000 + 64 * c for c in range(n_cand)]  # (handed on, never read)
+    table = torch.tensor([[data.data_ptr(), k] for k in kept], dtype=torch.int64, device="cuda")
+    ring, ref = ip.ImpactBuffer(N, K, [64], seed=9, sample_mode=mode), oracle.Ring(N, K, mode, seed=9)
+    record = ip.new_loss_inputs_record()
+    push = ring.prepare_device_step(push_sources=table)
+    draw = ring.prepare_device_step({"target_logits": 0}, record=record)
+    ring.device_begin()
+    in_slot, pushed = {}, 0
+    # all slots filled, then more draws than pushes, and the ring filled again
+    for ahead in [True] * (N - 1) + [i % 3 == 0 for i in range(90)] + [True] * 40 + [False] * 40:
+        (push if ahead else draw)()
+        if ahead:
+            st, slot = ref.push()
+            if st == 0:
+                in_slot[slot] = kept[pushed % n_cand]
+                pushed += 1
+            continue
+        st, slot, k = ref.sample()
+        got = ip.binding.impact_loss_inputs.from_buffer_copy(bytes(record[:size].tolist()))
+        assert (st, got.status) in ((ref.OK, 0), (ref.EMPTY, -4))
+        if st == 0:
+            assert (got.slot, got.k_before) == (slot, k)
+            assert got.target_logits == (in_slot[slot] if k == 0 else ring.slot_ptr(slot, 0))
+    ring.device_end()
+    assert ring.live() == ref.live()
     ring.close()
 
 
@@ -589,10 +626,12 @@ def test_the_rings_calls_and_prepared_calls_issued_natively_or_not(monkeypatch, 
         assert all(torch.equal(r[k], results[0][k]) for k in r)
     direct = {k: torch.zeros_like(v) for k, v in out.items()}
     ip.impact_loss_fwd_bwd(*[cat[n] for n in order], ip.Coefficients(clip_eps=0.3), workspace=ws, **direct)
-    gdirect = {k: torch.zeros_like(v) for k, v in gout.items()}
-    binding.load_library().impact_loss_fwd_bwd_gaussian(*calls[1]._args, 0)
+    wanted = {k: v.clone() for k, v in gout.items()}
+    for v in gout.values():
+        v.fill_(float("nan"))
+    assert binding.load_library().impact_loss_fwd_bwd_gaussian(*calls[1]._args, 0) == 0
     torch.cuda.synchronize()
     assert all(torch.equal(direct[k], results[0][k]) for k in direct)
-    assert all(torch.equal(gout[k], results[0]["g" + k]) for k in gdirect)
+    assert all(torch.equal(gout[k], wanted[k]) for k in wanted)
     with pytest.raises(ip.ImpactError):  # (the library's own refusal comes back)
         ip.prepare_loss_fwd_bwd(*[cat[n] for n in order], ip.Coefficients(clip_eps=-1.0), workspace=ws, **out)()
