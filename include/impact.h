@@ -120,17 +120,17 @@ int32_t impact_last_cuda_error(void);
  * result.  (The paper prescribes no kernel design, so these have no counterpart there.)  A value set here is
  * used by every later loss call of the process; setting one while another thread is inside a loss call is safe
  * (that call uses the old or the new value).
- *   IMPACT_OPT_EARLY_PREFETCH  1 (default): a loss call whose thread blocks have four to eight tiles each (of at
- *       least 10 KB, in all of 22 to 28 MB at most, rows of at most 32 actions: batches of roughly 85 000 to 150 000
- *       steps of 18 actions) enqueues a one-warp-per-block companion kernel right before its loss kernel.  The
- *       companion runs beside whatever kernel is still busy on the stream, asks L2 for the batch's first tiles, and
+ *   IMPACT_OPT_EARLY_PREFETCH  1 (default): a loss call whose thread blocks have four to sixteen tiles each (of at
+ *       least 12.5 KB, or of 10 KB from 20 MB on, in all of 22 to 28 MB at most, rows of at most 32 actions: batches of
+ *       roughly 85 000 to 150 000 steps of 18 actions) enqueues a one-warp-per-block companion kernel right before its
+ *       loss kernel.  The companion runs beside whatever kernel is still busy on the stream, asks L2 for the batch's first tiles, and
  *       then waits for the stream's previous kernel, so stream order is kept exactly; the loss kernel finds its first
  *       tiles in L2 instead of waiting for HBM.  0: no companion; the loss kernel asks for its first tiles itself when
- *       it starts.
+ *       it starts, where they are large enough for that to pay.
  *   IMPACT_OPT_PREFETCH_BYTES  upper bound on the bytes one call asks L2 for ahead of time (default 48 MiB).
  *   IMPACT_OPT_WINDOW_BYTES    bytes of tiles a block keeps in flight from global to shared memory: 0 (default)
- *       lets each launch choose (48 KiB where a block has eight tiles or fewer, 72 KiB beyond), else
- *       16 KiB .. 160 KiB.
+ *       lets each launch choose (48 KiB where a block has eight tiles or fewer, 72 KiB beyond and where the inputs come
+ *       by a record on the device), else 16 KiB .. 160 KiB.
  * impact_set_option returns IMPACT_ERR_INVALID_ARG for an unknown option or a value out of range;
  * impact_get_option returns -1 for an unknown option.
  */

@@ -864,7 +864,7 @@ int32_t launch_categorical(CatParams p, const RowLayout& rl, const DeviceInfo* d
     }
     const size_t row_bytes = 2 * p.A * sizeof(LT) + 20;
     WsPlan plan = ws_plan(ls.tiles, ls.grid, nt * row_bytes, sh.in_flight,
-                          companion_pays(p.A, kLong, C, p.geo.B * p.geo.T, row_bytes, nt, ls.tiles, ls.grid, sh.in_flight, sizeof(GT)));
+                          companion_pays(p.A, kLong, p.geo.B * p.geo.T, row_bytes, nt, ls.tiles, ls.grid, sh.in_flight, sizeof(GT)));
     if (kIndirect) { plan.companion = false; plan.prefetch_tiles = 0; }  // (addresses unknown on the host)
     if (plan.companion) {
         const int32_t st = launch_companion(p, (int)sizeof(LT), kLong, plan.prefetch_tiles, (int)ls.grid, stream);

@@ -139,7 +139,7 @@ void ws_ring_shape(size_t stage_bytes, size_t tile_in_bytes, int groups, int max
 //   28 MB (8.1 / 8.5); two up to 22 MB (800 x 128 of 24 8.0 / 8.2, 900 x 128 10.9 / 9.0; 700 x 128 of 28 8.0 / 8.1, 800 x 128
 //   10.7 / 8.7).
 constexpr size_t kSmallTile = 12 * 1024 + 512;
-inline bool companion_pays(int A, bool split, int groups, long long rows, size_t row_bytes, int nt, long long tiles,
+inline bool companion_pays(int A, bool split, long long rows, size_t row_bytes, int nt, long long tiles,
                            long long grid, int in_flight, size_t grad_bytes) {
     if (A > 32) return false;
     const long long bytes = rows * (long long)row_bytes;
@@ -187,7 +187,7 @@ inline OwnRequests own_requests(const WsPlan& plan, size_t tile_bytes, long long
 // through.  With all of it as shared memory: 31 x 4000 steps of 18 actions in bf16 13.4 us instead of 12.8, of 32 in fp32 22.8
 // instead of 20.0 (no companion), 14 x 2091 of 64 with every switch 14.8 instead of 13.4, Gaussian 28 012 x 28 of 3 dimensions
 // 19.3 instead of 18.9.
-constexpr size_t kRingStepShared = 20 * 1024;  // of a block of the ring's step, which runs between loss launches
+constexpr size_t kRingStepShared = 20 * 1024;  // of a one-warp block of the ring's step, which runs between loss launches
 inline int percent_beside(size_t smem, size_t other, const DeviceInfo* di) {
     const size_t percent = (100 * (smem + other + 2048) + di->smem_per_sm - 1) / di->smem_per_sm;
     return percent < 100 ? (int)percent : 100;

@@ -291,13 +291,16 @@ __device__ __forceinline__ int32_t nth_member(uint32_t word, uint32_t j) {
 // one trip to L2, its end.  So everything that it may need is asked for at once, where there is not too much of it: the
 // candidates' pointers and what is kept with each slot.  (An iteration of 131 072 steps of 18 actions, K = 4, step and loss
 // 12.0 us -> 11.0, of 1 600 steps 7.1 -> 6.2, of 16 384 steps of 9 with a push in each 8.4 -> 7.3; before, every block read all
-// of the state and the one that drew the last ticket wrote it, in blocks of 512 threads that found no room beside a loss
-// launch's.  L2 asked for the drawn slot's fields from here: a grid is complete only when its requests are, 0.3 to 1 us more.)
+// of the state and the one that drew the last ticket wrote it, in blocks of 512 threads.  Rings and tables of which there is too
+// much take another trip: a step that pushes nothing on 128, 129, 512, 1024 slots 2.6, 2.7, 2.9, 2.9 us, then 3.3, 3.3, 3.4, 3.7;
+// 126, 132, 510 pointers 2.6, 2.7, 2.7, then 3.4.  L2 asked for the drawn slot's fields from here: a grid is complete only when its requests are, 0.3 to 1 us more.)
 //
 // kThreads = 32: a warp per block and 16 KB of shared memory, so that the blocks become resident beside those of the loss
-// launch before, and the loss launch behind beside them: neither's start adds to the chain.  The copy goes through shared
-// memory then, which keeps 16 KB under way with a warp's registers; batches of more than 32 KB to a block go to blocks of 512
-// threads (kStepThreads).  (The next launch is let in behind the wait: before it, 0.1 to 0.4 us more.  The warp's copy through
+// launch before, and the loss launch behind beside them, where that leaves them kRingStepShared: neither's start adds to the
+// chain then.  (It does but for 18 actions in fp32 in the default configuration, whose 12 stages take 217 KB of an SM.)  The copy
+// goes through shared memory, which keeps 16 KB under way with a warp's registers; batches of more than 32 KB to a block, the
+// 131 072 steps above among them, go to blocks of 512 threads (kStepThreads), which find no registers beside a loss launch's.
+// (The next launch is let in behind the wait: before it, 0.1 to 0.4 us more.  The warp's copy through
 // registers or by a loop over the segments: up to 1.2 us more where every step pushes.)
 constexpr int kStepThreads = 512;
 constexpr int kAheadSlots = 128;       // slots and candidates' pointers that are asked for before it is known which are needed

@@ -19,7 +19,7 @@ static void expect(bool want, long long B, long long T, int A, size_t in, size_t
     bool got = !want;
     if (launch_shape(g, 128, split, cat_stage_bytes(128, A, in, out), 2 * 128 * A * in, groups, &di, &ls))
         got = ws_plan(ls.tiles, ls.grid, 128 * (2 * A * in + 20), ls.in_flight,
-                      companion_pays(A, split, groups, B * T, 2 * A * in + 20, 128, ls.tiles, ls.grid, ls.in_flight, out)).companion;
+                      companion_pays(A, split, B * T, 2 * A * in + 20, 128, ls.tiles, ls.grid, ls.in_flight, out)).companion;
     if (got == want) return;
     ++bad;
     printf("B=%lld T=%lld A=%d in=%zu out=%zu groups=%d split=%d: %d\n", B, T, A, in, out, groups, (int)split, (int)got);
