@@ -1038,11 +1038,4 @@ int32_t run_larger_count(const CatParams& p, const DeviceInfo* di, cudaStream_t 
     }
 }
 
-template <typename LT, typename GT>
-int32_t run_runtime_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    if (p.A % 4 == 0) return run_runtime_width<LT, GT, 4>(p, di, stream);
-    if (p.A % 2 == 0) return run_runtime_width<LT, GT, 2>(p, di, stream);
-    return run_runtime_width<LT, GT, 1>(p, di, stream);
-}
-
 }  // namespace impact

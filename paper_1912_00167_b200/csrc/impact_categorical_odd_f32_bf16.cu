@@ -1,0 +1,7 @@
+// The categorical loss kernels for fp32 logits and bf16 gradients, odd counts above 32 (one translation
+// unit per pair of types and kind of count, so that they compile side by side and a first launch loads few of them).
+#include "impact_categorical.cuh"
+
+namespace impact {
+template int32_t run_runtime_width<float, __nv_bfloat16, 1>(const CatParams&, const DeviceInfo*, cudaStream_t);
+}  // namespace impact

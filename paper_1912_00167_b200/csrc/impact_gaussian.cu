@@ -590,59 +590,93 @@ int32_t run_gaussian_form(const GaussParams& p, const RowLayout& rl, const Devic
     return launch_gaussian<kD, C, kV, false, false>(p, rl, di, stream);
 }
 
+// Lanes that share rows: the rows of a tile, the lanes of a row, the rotation that lanes of vectors of four take them in.
 template <int kV>
-int32_t run_gaussian_width(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
+RowLayout rows_on_lanes(int D) {
     RowLayout rl;
-    while (rl.nt > 8 && gauss_stage_bytes(rl.nt, p.D) > gauss_stage_cap) rl.nt /= 2;
+    while (rl.nt > 8 && gauss_stage_bytes(rl.nt, D) > gauss_stage_cap) rl.nt /= 2;
     while ((rl.nt / 4 << rl.log_lanes) < 32) ++rl.log_lanes;
-    const BankPattern b = bank_pattern(p.D * sizeof(float), 1 << rl.log_lanes, kV * 4);
+    const BankPattern b = bank_pattern(D * sizeof(float), 1 << rl.log_lanes, kV * 4);
     rl.rot_shift = b.shift;
-    const int vecs = p.D / kV;
+    const int vecs = D / kV;
     if (kV == 4 && vecs % (1 << rl.log_lanes) == 0)
         while (2 * (rl.rot_mask + 1) <= b.ways && (vecs >> rl.log_lanes) % (2 * (rl.rot_mask + 1)) == 0)
             rl.rot_mask = 2 * rl.rot_mask + 1;
-    // A lane's vectors, the same for many dimensions, are compiled in.  Told at run time they took, on the bytes of 8000 x 50 steps of 17,
-    // 50.3 us instead of 38.5 at 19 dimensions, 51.8 / 35.8 at 37, 47.5 / 36.9 at 63, 35.5 / 35.4 at 32; with every switch on half of
-    // that 34.0 / 24.7 at 23, 23.7 / 22.5 at 64; 300 x 50 of 45 11.2 / 8.2; 16 x 4096 of 23 22.4 / 18.4, of 35 27.0 / 21.7.
-    const int of_lane = (vecs + (1 << rl.log_lanes) - 1) >> rl.log_lanes;
-#define IMPACT_VECS(n) case n: return run_gaussian_form<-(n), 3, 3, 4, kV>(p, rl, di, stream)
-    if constexpr (kV == 4) {
-        switch (of_lane) { IMPACT_VECS(3); IMPACT_VECS(4); IMPACT_VECS(5); }
-    } else if constexpr (kV == 2) {
-        switch (of_lane) { IMPACT_VECS(5); IMPACT_VECS(6); IMPACT_VECS(7); IMPACT_VECS(8); IMPACT_VECS(9); }
-    } else {
-        switch (of_lane) {
-            IMPACT_VECS(10); IMPACT_VECS(11); IMPACT_VECS(12); IMPACT_VECS(13); IMPACT_VECS(14); IMPACT_VECS(15);
-            IMPACT_VECS(16); IMPACT_VECS(17); IMPACT_VECS(18);
-        }
-    }
-#undef IMPACT_VECS
-    return IMPACT_ERR_UNSUPPORTED;  // (no dimension up to 256 gets here)
+    return rl;
+}
+template <int kV>
+int vectors_of_a_lane(int D) {
+    const int log_lanes = rows_on_lanes<kV>(D).log_lanes;
+    return (D / kV + (1 << log_lanes) - 1) >> log_lanes;
 }
 
 }  // namespace
 
-int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
-    const RowLayout rl;
-    switch (p.D) {
-        // Consumer groups, with every switch, plain, split.  Where rows are short a tile's time is arithmetic: five (five with every
-        // switch up to five dimensions: 512 x 128 of 1 4.4 us, four 4.6; of 7 6.8 / 6.7).  Longer rows take three, whose ring has
-        // stages enough (8000 x 50 of 15 32.3 us, four 41.7), but four with every switch and split (4000 x 50 of 9 14.2, three 15.3;
-        // 16 x 4096 of 9 9.7 / 12.1, of 17 11.2 / 13.2).  The dimension known at run time: 2500 x 50 of 4 7.6 instead of 6.9, of
-        // 9 12.9 / 9.3, of 13 15.1 / 12.1, with every switch 4000 x 50 of 13 25.9 / 18.0.  16 is not among them: rows 64 bytes
-        // apart meet on the banks, and lanes that take their vectors in rotated order do not (35.2 us, 36.2 in order).
+// The kernels are compiled in units of a few dimensions each, by files that say which and include this one: the first launch of
+// a unit's kernels loads the whole unit (all dimensions in one took 45 ms).
+#ifndef IMPACT_GAUSSIAN_PART
+#define IMPACT_GAUSSIAN_PART 0
+#endif
+constexpr int kGaussPart = IMPACT_GAUSSIAN_PART;  // (0: this file by itself)
+
+#if IMPACT_GAUSSIAN_PART < 3
+// Consumer groups, with every switch, plain, split.  Where rows are short a tile's time is arithmetic: five (five with every
+// switch up to five dimensions: 512 x 128 of 1 4.4 us, four 4.6; of 7 6.8 / 6.7).  Longer rows take three, whose ring has
+// stages enough (8000 x 50 of 15 32.3 us, four 41.7), but four with every switch and split (4000 x 50 of 9 14.2, three 15.3;
+// 16 x 4096 of 9 9.7 / 12.1, of 17 11.2 / 13.2).  The dimension known at run time: 2500 x 50 of 4 7.6 instead of 6.9, of
+// 9 12.9 / 9.3, of 13 15.1 / 12.1, with every switch 4000 x 50 of 13 25.9 / 18.0.  16 is not among them: rows 64 bytes
+// apart meet on the banks, and lanes that take their vectors in rotated order do not (35.2 us, 36.2 in order).
 #define IMPACT_FIXED(n, full, plain, split) \
-    case n: return run_gaussian_form<n, full, plain, split, n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1>(p, rl, di, stream)
-        IMPACT_FIXED(1, 5, 5, 4); IMPACT_FIXED(2, 5, 5, 4); IMPACT_FIXED(3, 5, 5, 5); IMPACT_FIXED(4, 5, 5, 4);
-        IMPACT_FIXED(5, 5, 5, 4); IMPACT_FIXED(6, 4, 4, 4); IMPACT_FIXED(7, 4, 5, 4); IMPACT_FIXED(8, 4, 5, 4);
+    case n: return run_gaussian_form<n, full, plain, split, n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1>(p, RowLayout(), di, stream)
+template <>
+int32_t run_gaussian_part<kGaussPart>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    switch (p.D) {
+#if IMPACT_GAUSSIAN_PART == 0
+        IMPACT_FIXED(3, 5, 5, 5); IMPACT_FIXED(6, 4, 4, 4); IMPACT_FIXED(17, 3, 3, 4);
+#elif IMPACT_GAUSSIAN_PART == 1
+        IMPACT_FIXED(1, 5, 5, 4); IMPACT_FIXED(2, 5, 5, 4); IMPACT_FIXED(4, 5, 5, 4); IMPACT_FIXED(5, 5, 5, 4);
+        IMPACT_FIXED(7, 4, 5, 4); IMPACT_FIXED(8, 4, 5, 4);
+#else
         IMPACT_FIXED(9, 4, 3, 4); IMPACT_FIXED(10, 4, 3, 4); IMPACT_FIXED(11, 4, 3, 4); IMPACT_FIXED(12, 4, 3, 4);
-        IMPACT_FIXED(13, 4, 3, 4); IMPACT_FIXED(14, 4, 3, 4); IMPACT_FIXED(15, 3, 3, 4); IMPACT_FIXED(17, 3, 3, 4);
-#undef IMPACT_FIXED
-        default: break;
+        IMPACT_FIXED(13, 4, 3, 4); IMPACT_FIXED(14, 4, 3, 4); IMPACT_FIXED(15, 3, 3, 4);
+#endif
+        default: return IMPACT_ERR_UNSUPPORTED;
     }
-    if (p.D % 4 == 0) return run_gaussian_width<4>(p, di, stream);
-    if (p.D % 2 == 0) return run_gaussian_width<2>(p, di, stream);
-    return run_gaussian_width<1>(p, di, stream);
 }
+#undef IMPACT_FIXED
+#else
+// A lane's vectors, the same for many dimensions, are compiled in.  Told at run time they took, on the bytes of 8000 x 50 steps of 17,
+// 50.3 us instead of 38.5 at 19 dimensions, 51.8 / 35.8 at 37, 47.5 / 36.9 at 63, 35.5 / 35.4 at 32; with every switch on half of
+// that 34.0 / 24.7 at 23, 23.7 / 22.5 at 64; 300 x 50 of 45 11.2 / 8.2; 16 x 4096 of 23 22.4 / 18.4, of 35 27.0 / 21.7.
+#define IMPACT_VECS(n) case n: return run_gaussian_form<-(n), 3, 3, 4, kV>(p, rows_on_lanes<kV>(p.D), di, stream)
+template <>
+int32_t run_gaussian_part<kGaussPart>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    constexpr int kV = kGaussPart == 3 ? 4 : kGaussPart == 4 ? 2 : 1;
+    switch (vectors_of_a_lane<kV>(p.D)) {
+#if IMPACT_GAUSSIAN_PART == 3
+        IMPACT_VECS(3); IMPACT_VECS(4); IMPACT_VECS(5);
+#elif IMPACT_GAUSSIAN_PART == 4
+        IMPACT_VECS(5); IMPACT_VECS(6); IMPACT_VECS(7); IMPACT_VECS(8); IMPACT_VECS(9);
+#elif IMPACT_GAUSSIAN_PART == 5
+        IMPACT_VECS(10); IMPACT_VECS(11); IMPACT_VECS(12); IMPACT_VECS(13);
+#else
+        IMPACT_VECS(14); IMPACT_VECS(15); IMPACT_VECS(16); IMPACT_VECS(17); IMPACT_VECS(18);
+#endif
+        default: return IMPACT_ERR_UNSUPPORTED;  // (no dimension up to 256 gets here)
+    }
+}
+#undef IMPACT_VECS
+#endif
+
+#if IMPACT_GAUSSIAN_PART == 0
+int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream) {
+    if (is_mujoco(p.D)) return run_gaussian_part<0>(p, di, stream);
+    if (p.D <= 8) return run_gaussian_part<1>(p, di, stream);
+    if (p.D <= 15) return run_gaussian_part<2>(p, di, stream);
+    if (p.D % 4 == 0) return run_gaussian_part<3>(p, di, stream);
+    if (p.D % 2 == 0) return run_gaussian_part<4>(p, di, stream);
+    return vectors_of_a_lane<1>(p.D) <= 13 ? run_gaussian_part<5>(p, di, stream) : run_gaussian_part<6>(p, di, stream);
+}
+#endif
 
 }  // namespace impact

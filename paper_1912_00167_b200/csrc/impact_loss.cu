@@ -167,8 +167,10 @@ extern "C" int32_t impact_loss_workspace_status(const void* workspace, size_t wo
 
 template <typename LT, typename GT>
 static int32_t run_categorical(const CatParams& p, const DeviceInfo* di, cudaStream_t s) {
-    return is_compiled_count(p.A) ? run_compiled_count<LT, GT>(p, di, s)
-           : is_larger_count(p.A) ? run_larger_count<LT, GT>(p, di, s) : run_runtime_count<LT, GT>(p, di, s);
+    if (is_compiled_count(p.A)) return run_compiled_count<LT, GT>(p, di, s);
+    if (is_larger_count(p.A)) return run_larger_count<LT, GT>(p, di, s);
+    if (p.A % 4 == 0) return run_runtime_width<LT, GT, 4>(p, di, s);
+    return p.A % 2 == 0 ? run_runtime_width<LT, GT, 2>(p, di, s) : run_runtime_width<LT, GT, 1>(p, di, s);
 }
 static int32_t run_typed(const CatParams& p, bool logits_bf16, bool grads_bf16, const DeviceInfo* di, cudaStream_t s) {
     if (!logits_bf16 && !grads_bf16) return run_categorical<float, float>(p, di, s);

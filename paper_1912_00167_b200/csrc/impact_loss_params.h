@@ -111,10 +111,19 @@ template <typename LT, typename GT>
 int32_t run_compiled_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
 template <typename LT, typename GT>
 int32_t run_larger_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
-template <typename LT, typename GT>
-int32_t run_runtime_count(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <typename LT, typename GT, int kV>  // more than 32 actions, of which kV are read at a time (1: odd counts)
+int32_t run_runtime_width(const CatParams& p, const DeviceInfo* di, cudaStream_t stream);
 
 int32_t run_gaussian(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <int kPart>  // (one specialisation per translation unit, see impact_gaussian.cu)
+int32_t run_gaussian_part(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<0>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<1>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<2>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<3>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<4>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<5>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
+template <> int32_t run_gaussian_part<6>(const GaussParams& p, const DeviceInfo* di, cudaStream_t stream);
 
 // Stages of a ring that a block has room for; 4 KB are left for static shared memory.
 inline int stages_that_fit(size_t stage_bytes, int max_smem) { return (int)((size_t)(max_smem - 4096) / stage_bytes); }
